@@ -14,7 +14,6 @@ bool fwd_tc_available();
 
 namespace {
 
-constexpr int kMaxDevices = 64;
 int g_sm_count[kMaxDevices] = {};      // per device ordinal; filled on first use (a benign race: every writer stores the same value)
 thread_local char g_detail[256] = "";
 
@@ -246,8 +245,9 @@ static gka_status fwd_impl(const gka_desc *desc, const void *q, const void *k, c
         a.ws.decay = w.decay;
         a.tile_hh = w.hh;
         a.tile_hu = w.hu;
-    } else {
-        if (wants_tensor_path(desc)) return GKA_ERR_CUDA;   // no driver entry point for tensor maps
+    } else if (wants_tensor_path(desc)) {
+        return GKA_ERR_CUDA;   // no driver entry point for tensor maps
+    } else if (desc->d_k < 64) {
         a.plan.set(desc->B * desc->heads, chunks_of(desc->T), G);
         a.ws = carve_workspace(desc->workspace, G, simt_dim(desc), simt_dim(desc));
     }
@@ -259,6 +259,8 @@ static gka_status fwd_impl(const gka_desc *desc, const void *q, const void *k, c
     if (err != cudaSuccess) return cuda_result(err, "gka_fwd_chunked (validation pass)");
     if (tensor_path)
         err = launch_fwd_tc(a, stream);
+    else if (desc->d_k >= 64)
+        err = launch_fwd_recur(a, desc->io_dtype, sm_count(), desc->workspace, desc->workspace_bytes, stream);
     else
         err = launch_fwd_simt(a, desc->d_k, desc->io_dtype, stream);
     return cuda_result(err, tensor_path ? "gka_fwd_chunked (tensor-core path)" : "gka_fwd_chunked (fp32 path)");

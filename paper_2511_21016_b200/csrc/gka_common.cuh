@@ -11,6 +11,7 @@
 namespace gka {
 
 constexpr int kChunk = 64;            // tokens per chunk (C)
+constexpr int kMaxDevices = 64;       // device ordinals for which per-device values are cached
 constexpr int kMaxWorkItems = 296;    // upper bound on persistent work items (2 per SM on 148 SMs)
 // Division of an index below 2^31 by a divisor fixed for a launch, as a multiplication: with l = ceil(log2 d),
 // k = 31 + l and M = floor(2^k / d) + 1, floor(n M / 2^k) = floor(n / d) for every n < 2^31 (the excess
@@ -176,6 +177,15 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
+// 1 / x for x well inside the normal range (the weight schedule of Algorithm 1 divides by 4 - rho^2 omega, between 2 and 4):
+// the hardware's approximation and one Newton step, within one unit in the last place.  Unlike a division it has no rare
+// branch, so the compiler schedules the code around it as one block.
+__device__ __forceinline__ float recip(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return fmaf(r, fmaf(-x, r, 1.f), r);
+}
+
 // Wait for an mbarrier phase with a time limit (about a second).  The wait sleeps in hardware
 // (try_wait with a suspend-time hint), so a waiting warp leaves the issue slots to working warps.
 // Returns false if the phase did not complete in time; the caller records GKA_ERR_TIMEOUT and
@@ -224,6 +234,7 @@ struct FwdArgs {
 };
 
 // Launchers implemented in the kernel translation units.  Each returns a cudaError_t.
+cudaError_t launch_fwd_recur(const FwdArgs &a, int io_dtype, int sms, void *ws, size_t ws_bytes, cudaStream_t stream);
 cudaError_t launch_fwd_simt(const FwdArgs &a, int d, int io_dtype, cudaStream_t stream);
 // cross-item scan of the summaries; after_summary: launched as a programmatic dependent of the summary kernel
 cudaError_t launch_fwd_scan(const FwdArgs &a, int st, cudaStream_t stream, bool after_summary);
