@@ -37,7 +37,7 @@
  *   - bf16 I/O with GKA_PREC_NATIVE and T >= 16 runs on the tensor cores (tiles of 128 tokens x 128 channels; head
  *     dimension 64 is zero-extended on chip and skips the zero channels in the contractions over the channels, about
  *     0.83 of the time of 128); f32 I/O, GKA_PREC_HIGH, T < 16 and head dimensions 16 and
- *     32 run in fp32 arithmetic on the CUDA cores (16 and 32 zero-extended to 64 on chip in the chunked calls; the
+ *     32 run in fp32 arithmetic on the CUDA cores (16 and 32: an explicit H_t per token in the registers of a few lanes; the
  *     decode calls handle them with one warp per (sequence, head) pair).
  */
 #ifndef GKA_H_
@@ -112,7 +112,7 @@ typedef struct {
  * states of the cross-chunk state scan (one fp32 state per work segment) and, on the bf16
  * tensor-core path, the bf16 copies of the initial H and U of every 128-token tile plus its
  * ||H||_F^2 (64 KB + 4 B per tile; Section 4.2.1 stores the initial state of every chunk as well).
- * The fp32 path carries the states on chip and stores none per chunk.
+ * The fp32 path stores the start states of its sequence segments, with head dimensions 16 and 32 one state per 32 tokens.
  * Returns 0 if the descriptor is invalid.  Pure host arithmetic; no CUDA call.
  */
 size_t gka_fwd_workspace_bytes(const gka_desc *desc, int chunk);

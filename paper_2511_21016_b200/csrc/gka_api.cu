@@ -110,8 +110,6 @@ constexpr int kMinTensorT = 16;
 bool wants_tensor_path(const gka_desc *d) {
     return d->io_dtype == GKA_BF16 && d->precision == GKA_PREC_NATIVE && (d->d_k == 128 || d->d_k == 64) && d->T >= kMinTensorT;
 }
-// head dimension the fp32 kernels work with on chip: 16 and 32 are zero-extended to 64
-int simt_dim(const gka_desc *d) { return d->d_k <= 64 ? 64 : 128; }
 long long work_units(const gka_desc *d) {
     return (long long)d->B * d->heads * (wants_tensor_path(d) ? tiles_of(d->T) : chunks_of(d->T));
 }
@@ -147,7 +145,8 @@ const char *gka_status_string(int status) {
 size_t gka_fwd_workspace_bytes(const gka_desc *desc, int chunk) {
     if (check_fwd_shape(desc, chunk) != GKA_OK) return 0;
     if (wants_tensor_path(desc)) return tc_workspace_bytes_for(work_items_cap(desc, chunk), work_units(desc));
-    return workspace_bytes_for(work_items_cap(desc, chunk), simt_dim(desc), simt_dim(desc));
+    if (desc->d_k < 64) return small_workspace_bytes_for((long long)desc->B * desc->heads, desc->T, desc->d_k);
+    return workspace_bytes_for(work_items_cap(desc, chunk), desc->d_k, desc->d_v);
 }
 
 int gka_fwd_num_work_items(const gka_desc *desc, int chunk) {
@@ -241,15 +240,11 @@ static gka_status fwd_impl(const gka_desc *desc, const void *q, const void *k, c
         const TcWorkspace w = carve_tc_workspace(desc->workspace, G, a.plan.NC);
         a.ws.start = w.start;
         a.ws.delta = w.delta;
-        a.ws.cur = nullptr;
         a.ws.decay = w.decay;
         a.tile_hh = w.hh;
         a.tile_hu = w.hu;
     } else if (wants_tensor_path(desc)) {
         return GKA_ERR_CUDA;   // no driver entry point for tensor maps
-    } else if (desc->d_k < 64) {
-        a.plan.set(desc->B * desc->heads, chunks_of(desc->T), G);
-        a.ws = carve_workspace(desc->workspace, G, simt_dim(desc), simt_dim(desc));
     }
     a.ev_start = reinterpret_cast<cudaEvent_t>(desc->profile_start);
     a.ev_stop = reinterpret_cast<cudaEvent_t>(desc->profile_stop);
@@ -262,7 +257,7 @@ static gka_status fwd_impl(const gka_desc *desc, const void *q, const void *k, c
     else if (desc->d_k >= 64)
         err = launch_fwd_recur(a, desc->io_dtype, sm_count(), desc->workspace, desc->workspace_bytes, stream);
     else
-        err = launch_fwd_simt(a, desc->d_k, desc->io_dtype, stream);
+        err = launch_fwd_small(a, desc->io_dtype, desc->workspace, stream);
     return cuda_result(err, tensor_path ? "gka_fwd_chunked (tensor-core path)" : "gka_fwd_chunked (fp32 path)");
 }
 

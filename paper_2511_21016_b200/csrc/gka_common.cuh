@@ -70,12 +70,10 @@ struct WorkPlan {
     __host__ __device__ bool cut_in(int i) const { return (lo(i) % N) != 0; }
 };
 
-// Workspace layout (floats): start states [G][st], summaries [G][st], running masters [G][st],
-// decay products [G].  st = d_k*d_k + d_v*d_k.
+// State scan of the tensor-core path (floats): start states [G][st], summaries [G][st], decay products [G].
 struct Workspace {
     float *start;
     float *delta;
-    float *cur;
     float *decay;
 };
 
@@ -83,20 +81,18 @@ __host__ __device__ inline size_t state_floats(int dk, int dv) {
     return (size_t)dk * dk + (size_t)dv * dk;
 }
 
+// fp32 path, head dimensions 64 and 128: room for 3 G segment states and G floats more (gka_recur.cu lays it out)
 inline size_t workspace_bytes_for(int G, int dk, int dv) {
     size_t st = state_floats(dk, dv);
     size_t fl = 3 * (size_t)G * st + (size_t)G;
     return ((fl * sizeof(float) + 255) / 256) * 256;
 }
 
-inline Workspace carve_workspace(void *base, int G, int dk, int dv) {
-    size_t st = state_floats(dk, dv);
-    Workspace w;
-    w.start = reinterpret_cast<float *>(base);
-    w.delta = w.start + (size_t)G * st;
-    w.cur = w.delta + (size_t)G * st;
-    w.decay = w.cur + (size_t)G * st;
-    return w;
+// Head dimensions 16 and 32: one state per 32-token chunk of every sequence, and the chunks' decays.
+constexpr int kSmallChunk = 32;
+__host__ __device__ constexpr int small_chunks_of(int T) { return (T + kSmallChunk - 1) / kSmallChunk; }
+inline size_t small_workspace_bytes_for(long long pairs, int T, int d) {
+    return (((size_t)pairs * small_chunks_of(T) * (state_floats(d, d) + 1) * sizeof(float) + 255) / 256) * 256;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -235,9 +231,7 @@ struct FwdArgs {
 
 // Launchers implemented in the kernel translation units.  Each returns a cudaError_t.
 cudaError_t launch_fwd_recur(const FwdArgs &a, int io_dtype, int sms, void *ws, size_t ws_bytes, cudaStream_t stream);
-cudaError_t launch_fwd_simt(const FwdArgs &a, int d, int io_dtype, cudaStream_t stream);
-// cross-item scan of the summaries; after_summary: launched as a programmatic dependent of the summary kernel
-cudaError_t launch_fwd_scan(const FwdArgs &a, int st, cudaStream_t stream, bool after_summary);
+cudaError_t launch_fwd_small(const FwdArgs &a, int io_dtype, void *ws, cudaStream_t stream);
 cudaError_t launch_decode(float *state, const void *q, const void *k, const void *v,
                           const float *gate, const float *lam, int n_iter, void *out, int nseq,
                           int heads, int d, int io_dtype, unsigned flags, const float *beta, const float *alpha, int *device_status,

@@ -566,6 +566,58 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     if (t < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
 }
 
+// Scan over work items: the start state of item i (when its range starts inside a sequence) is the
+// fold  state <- decay_j * state + delta_j  over the items j < i that hold the earlier part of the
+// same sequence, starting from the sequence's initial state.  A sequence spans few items, so every
+// item folds its own short chain independently: blockIdx.y = item, four state elements per thread.
+__global__ void fwd_scan(FwdArgs a) {
+    // programmatic dependent of the summary kernel, and the state kernel one of this kernel: both may be scheduled early,
+    // and each waits here for its producer
+    constexpr int st = 2 * D * D;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const WorkPlan &P = a.plan;
+    const int i = blockIdx.y + 1;
+    __shared__ int s_j0, s_seq;           // the chain is found once per block (64-bit divisions are slow)
+    if (threadIdx.x == 0) {
+        int j0 = -1;
+        if (P.cut_in(i)) {
+            // first item of the chain: the one whose range holds the start of this sequence (its last run
+            // begins there, whatever sequence the item itself started in)
+            const long long seq_start = (P.lo(i) / P.N) * P.N;
+            j0 = i - 1;
+            while (P.lo(j0) > seq_start) --j0;
+        }
+        s_j0 = j0;
+        s_seq = (int)(P.lo(i) / P.N);
+    }
+    __syncthreads();
+    const int j0 = s_j0, seq = s_seq;
+    if (j0 < 0) return;
+    const int e = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+    if (e >= st) return;
+    float4 carry = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (a.state_in) {
+        const int dd = 2 * a.d * a.d;
+        if (dd == st) {
+            carry = *reinterpret_cast<const float4 *>(a.state_in + (size_t)seq * st + e);
+        } else {
+            // the workspace holds states zero-extended to the on-chip head dimension
+            const int which = e / (D * D), row = (e / D) % D, col = e % D;
+            if (row < a.d && col < a.d) carry = *reinterpret_cast<const float4 *>(a.state_in + (size_t)seq * dd + (size_t)which * a.d * a.d + (size_t)row * a.d + col);
+        }
+    }
+    for (int j = j0; j < i; ++j) {
+        const float dcy = a.ws.decay[j];
+        const float4 d = *reinterpret_cast<const float4 *>(a.ws.delta + (size_t)j * st + e);
+        carry.x = fmaf(dcy, carry.x, d.x);
+        carry.y = fmaf(dcy, carry.y, d.y);
+        carry.z = fmaf(dcy, carry.z, d.z);
+        carry.w = fmaf(dcy, carry.w, d.w);
+    }
+    *reinterpret_cast<float4 *>(a.ws.start + (size_t)i * st + e) = carry;
+}
+
 }  // namespace
 
 bool fwd_tc_available() { return get_encode_fn() != nullptr; }
@@ -602,8 +654,16 @@ cudaError_t launch_fwd_tc(const FwdArgs &a_in, cudaStream_t stream) {
         if (err != cudaSuccess) return err;
         fwd_tc_summary_kernel<<<a.plan.G, kThreadsState, KV_SMEM, stream>>>(tmK, tmV, a);
         if (a.start_from_scan) {
-            err = launch_fwd_scan(a, (int)state_floats(D, D), stream, true);
-            if (err != cudaSuccess) return err;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(2 * D * D / 4 / 256, (unsigned)(a.plan.G - 1));
+            cfg.blockDim = dim3(256);
+            cfg.stream = stream;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[0].val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            if ((err = cudaLaunchKernelEx(&cfg, fwd_scan, a)) != cudaSuccess) return err;
         }
         a.after_summary = 1;
     }
