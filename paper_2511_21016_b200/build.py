@@ -8,6 +8,7 @@ import sys
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libgka.so")
+BINDING = os.path.join(_HERE, "_gka_torch.so")      # native marshalling of the torch binding, linked against libgka.so
 SOURCES = ["gka_api.cu", "gka_fwd_small.cu", "gka_decode.cu", "gka_recur.cu", "gka_decode_small.cu", "gka_tc_state.cu", "gka_tc_solve.cu", "gka_noalloc.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xptxas", "-v"]
@@ -19,16 +20,29 @@ def _nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(BINDING):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
     deps.append(os.path.join(os.path.dirname(_HERE), "include", "gka.h"))
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _binding_command() -> list:
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    return ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+            "-isystem", os.path.join(root, "include"), "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"),
+            "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include"),
+            os.path.join(CSRC, "gka_torch.cpp"), "-o", BINDING, "-L" + os.path.join(root, "lib"), "-L" + _HERE,
+            "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-lgka", "-Wl,-rpath,$ORIGIN"]
+
+
 def build_library(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu of the library into libgka.so (object files under build/)."""
+    """Compile every .cu of the library into libgka.so (object files under build/) and the torch binding beside it."""
     if not force and not _stale():
         return LIB
     obj_dir = os.path.join(_HERE, "build")
@@ -51,6 +65,7 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
         raise RuntimeError("nvcc failed")
     cmd = [_nvcc(), "-shared", "-o", LIB, *objs, "-lcudart"]
     subprocess.check_call(cmd)
+    subprocess.check_call(_binding_command())
     return LIB
 
 

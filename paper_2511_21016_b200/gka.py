@@ -1,8 +1,12 @@
-"""Thin ctypes binding of the GKA C ABI (include/gka.h).
+"""Thin binding of the GKA C ABI (include/gka.h).
 
 Argument marshalling only: every step of the path runs in the CUDA kernels of
 ``libgka.so``.  PyTorch is used for device memory and streams.  There is no CPU
 fallback: if the library is missing or a call fails, an exception is raised.
+
+The calls that a program makes for every batch or token are marshalled by ``_gka_torch.so`` (csrc/gka_torch.cpp): checked
+and filled into a descriptor in Python they cost 17 to 40 us of host time, more than the kernels of a small call.  What it
+does not take as it is comes back as None, and the ctypes form below converts it or raises.
 """
 from __future__ import annotations
 
@@ -95,6 +99,21 @@ def load_library():
         lib.gka_status_string.restype = ctypes.c_char_p
         _lib = lib
     return _lib
+
+
+_native = None
+
+
+def _load_native():
+    """Load _gka_torch.so, the native marshalling (built in-tree beside libgka.so).  Raises if it is missing."""
+    global _native
+    if _native is None:
+        load_library()
+        if not os.path.exists(os.path.join(_HERE, "_gka_torch.so")):
+            raise FileNotFoundError("_gka_torch.so is missing: build it with `python -m paper_2511_21016_b200.build`")
+        from . import _gka_torch
+        _native = _gka_torch
+    return _native
 
 
 def status_string(status: int) -> str:
@@ -201,6 +220,12 @@ def gka_fwd_chunked(q, k, v, gate, lam, n_iter, chunk=64, out=None, state_out=No
 
     Returns (out, state_out).  Work is enqueued on ``stream`` (default: torch's current stream).
     """
+    r = (_native or _load_native()).fwd_chunked(q, k, v, gate, lam, n_iter, chunk, out, state_out, state_in, workspace, precision,
+                                                flags, fro_out, device_status, stream, profile_events, beta, alpha)
+    if r is not None:
+        if r.__class__ is int:
+            raise GkaError(r, "gka_fwd_chunked")
+        return r
     if q.dim() != 4:
         raise ValueError(f"q: expected [B, T, heads, d], got shape {tuple(q.shape)}")
     B, T, heads, d = q.shape
@@ -235,6 +260,12 @@ def gka_solve_chunked(rhs, k, gate, lam, n_iter, chunk=64, out=None, *, state_in
 
     With rhs = q this is the iterate the forward multiplies by U_t; with rhs = dL/dx it is dL/dq.
     """
+    r = (_native or _load_native()).solve_chunked(rhs, k, gate, lam, n_iter, chunk, out, state_in, workspace, precision, flags,
+                                                  device_status, stream, beta)
+    if r is not None:
+        if r.__class__ is int:
+            raise GkaError(r, "gka_solve_chunked")
+        return r
     if rhs.dim() != 4:
         raise ValueError(f"rhs: expected [B, T, heads, d], got shape {tuple(rhs.shape)}")
     B, T, heads, d = rhs.shape
@@ -266,6 +297,12 @@ def gka_fwd_chunked_host(q, k, v, gate, lam, n_iter, chunk, out, state_out, *, s
                          precision=GKA_PREC_NATIVE, flags=0, stream=None, device_status=None):
     """Host-buffer forward: q, k, v, gate, lam, out, state_out are (pinned) CPU tensors; staging and
     workspace are CUDA byte tensors.  Copies and kernels are enqueued on the stream; no synchronisation."""
+    rc = (_native or _load_native()).fwd_chunked_host(q, k, v, gate, lam, n_iter, chunk, out, state_out, staging, workspace,
+                                                      precision, flags, stream, device_status)
+    if rc == GKA_OK:
+        return out, state_out
+    if rc is not None:
+        raise GkaError(rc, "gka_fwd_chunked_host")
     if q.dim() != 4:
         raise ValueError(f"q: expected [B, T, heads, d], got shape {tuple(q.shape)}")
     B, T, heads, d = q.shape
@@ -324,6 +361,12 @@ def gka_fwd_chunked_noalloc(q, k, v, gate, lam, n_iter, chunk=64, out=None, stat
 def gka_decode_step(state, q, k, v, gate, lam, n_iter, out=None, *, flags=0, device_status=None,
                     stream=None, profile_events=None, beta=None, alpha=None):
     """One recurrent step.  state: [N,heads,2*d*d] f32, updated in place; q,k,v: [N,heads,d]."""
+    r = (_native or _load_native()).decode_step(state, q, k, v, gate, lam, n_iter, out, flags, device_status, stream,
+                                                profile_events, beta, alpha)
+    if r is not None:
+        if r.__class__ is int:
+            raise GkaError(r, "gka_decode_step")
+        return r
     if q.dim() != 3:
         raise ValueError(f"q: expected [N, heads, d], got shape {tuple(q.shape)}")
     N, heads, d = q.shape
@@ -349,6 +392,12 @@ def gka_decode_tokens(state, q, k, v, gate, lam, n_iter, out=None, *, flags=0, d
                       stream=None, profile_events=None, beta=None, alpha=None):
     """The recurrent step over T consecutive tokens.  state: [N,heads,2*d*d] f32, updated in place;
     q,k,v: [N,T,heads,d]; gate, lam (beta, alpha): [N,T,heads]."""
+    r = (_native or _load_native()).decode_tokens(state, q, k, v, gate, lam, n_iter, out, flags, device_status, stream,
+                                                  profile_events, beta, alpha)
+    if r is not None:
+        if r.__class__ is int:
+            raise GkaError(r, "gka_decode_tokens")
+        return r
     if q.dim() != 4:
         raise ValueError(f"q: expected [N, T, heads, d], got shape {tuple(q.shape)}")
     N, T, heads, d = q.shape
