@@ -227,6 +227,7 @@ static gka_status fwd_impl(const gka_desc *desc, const void *q, const void *k, c
     a.d = desc->d_k;
     a.divH.set((unsigned)desc->heads);
     a.n_iter = n_iter;
+    a.sms = sm_count();
     a.flags = desc->flags;
     a.solve_only = solve_only ? 1 : 0;
     a.start_from_scan = 0;
@@ -255,7 +256,7 @@ static gka_status fwd_impl(const gka_desc *desc, const void *q, const void *k, c
     if (tensor_path)
         err = launch_fwd_tc(a, stream);
     else if (desc->d_k >= 64)
-        err = launch_fwd_recur(a, desc->io_dtype, sm_count(), desc->workspace, desc->workspace_bytes, stream);
+        err = launch_fwd_recur(a, desc->io_dtype, desc->workspace, desc->workspace_bytes, stream);
     else
         err = launch_fwd_small(a, desc->io_dtype, desc->workspace, stream);
     return cuda_result(err, tensor_path ? "gka_fwd_chunked (tensor-core path)" : "gka_fwd_chunked (fp32 path)");
@@ -291,7 +292,7 @@ gka_status gka_decode_step(const gka_desc *desc, float *state, const void *q, co
                                   reinterpret_cast<cudaEvent_t>(desc->profile_stop), reinterpret_cast<cudaStream_t>(desc->stream));
     else
         err = launch_decode(state, q, k, v, gate, lam, n_iter, out, desc->B, desc->heads,
-                                    desc->d_k, desc->io_dtype, desc->flags, desc->beta, desc->alpha, desc->device_status,
+                                    desc->d_k, desc->io_dtype, desc->flags, desc->beta, desc->alpha, desc->device_status, sm_count(),
                                     reinterpret_cast<cudaEvent_t>(desc->profile_start),
                                     reinterpret_cast<cudaEvent_t>(desc->profile_stop),
                                     reinterpret_cast<cudaStream_t>(desc->stream));
@@ -318,7 +319,7 @@ gka_status gka_decode_tokens(const gka_desc *desc, float *state, const void *q, 
     else
         err = launch_decode_multi(state, q, k, v, gate, lam, n_iter, out, desc->B, desc->T, desc->heads,
                                           desc->d_k, desc->io_dtype, desc->flags, desc->beta, desc->alpha,
-                                          desc->device_status,
+                                          desc->device_status, sm_count(),
                                           reinterpret_cast<cudaEvent_t>(desc->profile_start),
                                           reinterpret_cast<cudaEvent_t>(desc->profile_stop),
                                           reinterpret_cast<cudaStream_t>(desc->stream));

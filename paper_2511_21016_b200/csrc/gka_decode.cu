@@ -11,6 +11,7 @@
 //   - ||H_t||_F is a block reduction, Algorithm 1 runs with L = ||H_t||_F + lambda_t,
 //     mu = lambda_t; row sums are reduced with warp shuffles inside the 8-lane groups.
 #include "gka_common.cuh"
+#include "gka_tc_util.cuh"
 
 namespace gka {
 namespace {
@@ -42,6 +43,10 @@ decode_kernel(float *__restrict__ state, const IoT *__restrict__ q, const IoT *_
     float *gH = state + (size_t)head * (2 * D * D);
     float *gU = gH + D * D;
 
+    // Programmatic launch in stream order: the blocks of the next decode step may take their SMs while this one drains, and
+    // wait here, before their first access to memory, until the kernels before them are complete and visible.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
     // ---- kick off the bulk copy of U_old
     const uint32_t bar_addr = smem_u32(bar);
     if (tid == 0) {
@@ -49,6 +54,7 @@ decode_kernel(float *__restrict__ state, const IoT *__restrict__ q, const IoT *_
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (tid == 0) {
         constexpr uint32_t bytes = D * D * sizeof(float);
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_addr), "r"(bytes)
@@ -130,26 +136,25 @@ decode_kernel(float *__restrict__ state, const IoT *__restrict__ q, const IoT *_
     int cur = 0;
     for (int it = 0; it < n_iter; ++it) {
         const float *xs = sX + cur * D;
-        float xc[CG][4];
+        omega = 4.f * recip(4.f - rho2 * omega);
+        const float step = s0 * omega, mom = omega - 1.f;
+        uint64_t acc[RPT];
 #pragma unroll
         for (int n = 0; n < CG; ++n) {
-            float4 t4 = *reinterpret_cast<const float4 *>(xs + 4 * (lane8 + 8 * n));
-            xc[n][0] = t4.x; xc[n][1] = t4.y; xc[n][2] = t4.z; xc[n][3] = t4.w;
+            const ulonglong2 x2 = *reinterpret_cast<const ulonglong2 *>(xs + 4 * (lane8 + 8 * n));
+#pragma unroll
+            for (int m = 0; m < RPT; ++m) {
+                const uint64_t h0 = tcu::f2_pack(Hr[m][n].x, Hr[m][n].y), h1 = tcu::f2_pack(Hr[m][n].z, Hr[m][n].w);
+                acc[m] = n == 0 ? tcu::f2_mul(h0, x2.x) : tcu::f2_fma(h0, x2.x, acc[m]);
+                acc[m] = tcu::f2_fma(h1, x2.y, acc[m]);
+            }
         }
-        omega = 4.f / (4.f - rho2 * omega);
-        const float step = s0 * omega, mom = omega - 1.f;
         float sm[RPT];
 #pragma unroll
         for (int m = 0; m < RPT; ++m) {
-            float s = 0.f;
-#pragma unroll
-            for (int n = 0; n < CG; ++n) {
-                s = fmaf(Hr[m][n].x, xc[n][0], s);
-                s = fmaf(Hr[m][n].y, xc[n][1], s);
-                s = fmaf(Hr[m][n].z, xc[n][2], s);
-                s = fmaf(Hr[m][n].w, xc[n][3], s);
-            }
-            sm[m] = s;
+            float lo, hi;
+            tcu::f2_unpack(acc[m], lo, hi);
+            sm[m] = lo + hi;
         }
         float tot;
         const bool hi4 = (lane8 & 4) != 0;
@@ -228,34 +233,44 @@ decode_kernel(float *__restrict__ state, const IoT *__restrict__ q, const IoT *_
 template <int D, typename IoT>
 cudaError_t launch_typed(float *state, const void *q, const void *k, const void *v, const float *gate,
                          const float *lam, int n_iter, void *out, int nheads_total, unsigned flags, const float *beta, const float *alpha,
-                         int *device_status, cudaEvent_t ev_start, cudaEvent_t ev_stop, cudaStream_t stream) {
-    const size_t smem = (size_t)(D * D + 5 * D + 16) * sizeof(float) + 16;
+                         int *device_status, int sms, cudaEvent_t ev_start, cudaEvent_t ev_stop, cudaStream_t stream) {
+    const size_t smem = spread_smem((size_t)(D * D + 5 * D + 16) * sizeof(float) + 16, nheads_total, sms);
     auto kernel = (beta || alpha) ? decode_kernel<D, IoT, true> : decode_kernel<D, IoT, false>;
-    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemLimit limit[2];
+    cudaError_t err = limit[(beta || alpha) ? 1 : 0].raise(kernel);
     if (err != cudaSuccess) return err;
     if (ev_start) cudaEventRecord(ev_start, stream);
-    kernel<<<nheads_total, kThreads, smem, stream>>>(
-        state, reinterpret_cast<const IoT *>(q), reinterpret_cast<const IoT *>(k),
-        reinterpret_cast<const IoT *>(v), gate, lam, n_iter, reinterpret_cast<IoT *>(out), flags, beta, alpha,
-        device_status);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = ev_start ? 0 : 1;
+    cfg.gridDim = dim3((unsigned)nheads_total);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    err = cudaLaunchKernelEx(&cfg, kernel, state, reinterpret_cast<const IoT *>(q), reinterpret_cast<const IoT *>(k),
+                             reinterpret_cast<const IoT *>(v), gate, lam, n_iter, reinterpret_cast<IoT *>(out), flags, beta,
+                             alpha, device_status);
     if (ev_stop) cudaEventRecord(ev_stop, stream);
-    return cudaGetLastError();
+    return err;
 }
 
 }  // namespace
 
 cudaError_t launch_decode(float *state, const void *q, const void *k, const void *v, const float *gate,
                           const float *lam, int n_iter, void *out, int nseq, int heads, int d,
-                          int io_dtype, unsigned flags, const float *beta, const float *alpha, int *device_status, cudaEvent_t ev_start, cudaEvent_t ev_stop, cudaStream_t stream) {
+                          int io_dtype, unsigned flags, const float *beta, const float *alpha, int *device_status, int sms, cudaEvent_t ev_start, cudaEvent_t ev_stop, cudaStream_t stream) {
     const int total = nseq * heads;
     if (d == 128) {
         return io_dtype == GKA_BF16
-                   ? launch_typed<128, __nv_bfloat16>(state, q, k, v, gate, lam, n_iter, out, total, flags, beta, alpha, device_status, ev_start, ev_stop, stream)
-                   : launch_typed<128, float>(state, q, k, v, gate, lam, n_iter, out, total, flags, beta, alpha, device_status, ev_start, ev_stop, stream);
+                   ? launch_typed<128, __nv_bfloat16>(state, q, k, v, gate, lam, n_iter, out, total, flags, beta, alpha, device_status, sms, ev_start, ev_stop, stream)
+                   : launch_typed<128, float>(state, q, k, v, gate, lam, n_iter, out, total, flags, beta, alpha, device_status, sms, ev_start, ev_stop, stream);
     }
     return io_dtype == GKA_BF16
-               ? launch_typed<64, __nv_bfloat16>(state, q, k, v, gate, lam, n_iter, out, total, flags, beta, alpha, device_status, ev_start, ev_stop, stream)
-               : launch_typed<64, float>(state, q, k, v, gate, lam, n_iter, out, total, flags, beta, alpha, device_status, ev_start, ev_stop, stream);
+               ? launch_typed<64, __nv_bfloat16>(state, q, k, v, gate, lam, n_iter, out, total, flags, beta, alpha, device_status, sms, ev_start, ev_stop, stream)
+               : launch_typed<64, float>(state, q, k, v, gate, lam, n_iter, out, total, flags, beta, alpha, device_status, sms, ev_start, ev_stop, stream);
 }
 
 }  // namespace gka

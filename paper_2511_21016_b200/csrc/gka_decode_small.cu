@@ -16,6 +16,8 @@ decode_small_kernel(float *__restrict__ state, const IoT *__restrict__ q, const 
                     const IoT *__restrict__ v, const float *__restrict__ gate, const float *__restrict__ lam,
                     int n_iter, IoT *__restrict__ out, unsigned flags, const float *__restrict__ beta,
                     const float *__restrict__ alpha, int T, int heads, int npairs) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");           // programmatic launch in stream order, as in gka_decode.cu
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int lane = threadIdx.x & 31;
     const int sh = blockIdx.x * (kThreadsSmall / 32) + (threadIdx.x >> 5);   // (sequence, head) pair of this warp
     if (sh >= npairs) return;
@@ -100,11 +102,20 @@ cudaError_t launch_small_typed(float *state, const void *q, const void *k, const
     const int npairs = nseq * heads;
     const int blocks = (npairs + kThreadsSmall / 32 - 1) / (kThreadsSmall / 32);
     if (ev_start) cudaEventRecord(ev_start, stream);
-    decode_small_kernel<D, IoT><<<blocks, kThreadsSmall, 0, stream>>>(
-        state, reinterpret_cast<const IoT *>(q), reinterpret_cast<const IoT *>(k), reinterpret_cast<const IoT *>(v), gate, lam,
-        n_iter, reinterpret_cast<IoT *>(out), flags, beta, alpha, T, heads, npairs);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = ev_start ? 0 : 1;
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kThreadsSmall);
+    cfg.stream = stream;
+    const cudaError_t err = cudaLaunchKernelEx(
+        &cfg, decode_small_kernel<D, IoT>, state, reinterpret_cast<const IoT *>(q), reinterpret_cast<const IoT *>(k),
+        reinterpret_cast<const IoT *>(v), gate, lam, n_iter, reinterpret_cast<IoT *>(out), flags, beta, alpha, T, heads, npairs);
     if (ev_stop) cudaEventRecord(ev_stop, stream);
-    return cudaGetLastError();
+    return err;
 }
 
 }  // namespace

@@ -100,6 +100,7 @@ template <int D, typename IoT>
 __global__ void __launch_bounds__(32 * kSumWarps) small_summary(SmallArgs a) {
     constexpr int E = D * D / 32;
     __shared__ __align__(16) Chunk<D> sm[kSumWarps];
+    asm volatile("griddepcontrol.wait;" ::: "memory");           // whatever wrote the inputs (programmatic launch)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int warp = threadIdx.x >> 5, l = threadIdx.x & 31;
     const long long w = (long long)blockIdx.x * kSumWarps + warp;
@@ -549,11 +550,11 @@ cudaError_t launch_typed(const SmallArgs &a, cudaEvent_t ev_start, cudaEvent_t e
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
+    cfg.numAttrs = 1;
     cfg.stream = stream;
     cfg.gridDim = dim3((unsigned)((units + kSumWarps - 1) / kSumWarps));
     cfg.blockDim = dim3(32 * kSumWarps);
     if ((err = cudaLaunchKernelEx(&cfg, small_summary<D, IoT>, a)) != cudaSuccess) return err;
-    cfg.numAttrs = 1;
     cfg.gridDim = dim3((unsigned)((elements / 4 + 127) / 128), (unsigned)(a.pairs < 65535 ? a.pairs : 65535));
     cfg.blockDim = dim3(elements / 4 < 128 ? elements / 4 : 128);
     if ((err = cudaLaunchKernelEx(&cfg, small_scan, a, st, elements)) != cudaSuccess) return err;

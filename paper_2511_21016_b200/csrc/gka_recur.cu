@@ -23,8 +23,6 @@
 // The forward splits every sequence into P segments of L tokens (and a segment into F parts) so that the blocks fill the
 // device; recur_summary computes what a segment adds to the state, recur_scan folds that into the start state of every
 // segment, and a block of a later part first folds the tokens of its segment that come before it.
-#include <atomic>
-
 #include "gka_common.cuh"
 #include "gka_tc_util.cuh"
 
@@ -542,7 +540,8 @@ __global__ void __launch_bounds__(Rc<D>::NT, Rc<D>::kMinBlocks) recur_kernel(Rec
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (tid < 16) sm.S[tid] = 0.f;
-    asm volatile("griddepcontrol.wait;" ::: "memory");           // the scan's start states (no effect on a plain launch)
+    asm volatile("griddepcontrol.wait;" ::: "memory");           // programmatic launch: the scan's start states, or the inputs
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const float *const start = s > 0 ? a.seg + ((size_t)pair * (a.P - 1) + s - 1) * 2 * D * D
                                      : (a.state_in ? a.state_in + (size_t)pair * 2 * D * D : nullptr);
     if (tid == 0 && start) bulk_in(start);
@@ -637,6 +636,7 @@ __global__ void __launch_bounds__(256, 1) recur_summary(RecurArgs a) {
     constexpr int TR = D / 16, G4 = TR / 4, NS = kSumTokens;
     __shared__ __align__(16) IoT sK[2][NS][D], sV[2][NS][D];
     __shared__ float sG[2][NS], sB[2][NS];
+    asm volatile("griddepcontrol.wait;" ::: "memory");           // whatever wrote the inputs (programmatic launch)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
     const int pair = blockIdx.x / (a.P - 1), s = blockIdx.x % (a.P - 1);
@@ -782,6 +782,7 @@ cudaError_t launch_typed(RecurArgs a, long long pairs, int sms, void *ws, size_t
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
+    cfg.numAttrs = 1;
     cfg.stream = stream;
     if (a.P > 1) {
         cfg.gridDim = dim3((unsigned)(pairs * (a.P - 1)));
@@ -790,23 +791,16 @@ cudaError_t launch_typed(RecurArgs a, long long pairs, int sms, void *ws, size_t
         const int n4 = (int)(st / (a.solve_only ? 2 : 1)) / 4;       // the solve alone needs no U
         cfg.gridDim = dim3((n4 + 127) / 128, (unsigned)pairs);
         cfg.blockDim = dim3(128);
-        cfg.numAttrs = 1;
         if ((err = cudaLaunchKernelEx(&cfg, recur_scan, a, (int)st)) != cudaSuccess) return err;
     }
-    constexpr size_t smem = Rc<D>::kSmem;
-    static std::atomic<bool> ready[kMaxDevices];                      // shared-memory limit raised on this device
-    int dev = 0;
-    if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
-    if (dev >= kMaxDevices || !ready[dev].load(std::memory_order_relaxed)) {
-        err = cudaFuncSetAttribute(recur_kernel<D, IoT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (err != cudaSuccess) return err;
-        if (dev < kMaxDevices) ready[dev].store(true, std::memory_order_relaxed);
-    }
+    const size_t smem = spread_smem(Rc<D>::kSmem, pairs * a.P * a.F, sms);
+    static SmemLimit limit;
+    if ((err = limit.raise(recur_kernel<D, IoT>)) != cudaSuccess) return err;
     if (ev_start) cudaEventRecord(ev_start, stream);
     cfg.gridDim = dim3((unsigned)(pairs * a.P * a.F));
     cfg.blockDim = dim3(Rc<D>::NT);
     cfg.dynamicSmemBytes = smem;
-    cfg.numAttrs = a.P > 1 && !ev_start ? 1 : 0;
+    cfg.numAttrs = ev_start ? 0 : 1;
     err = cudaLaunchKernelEx(&cfg, recur_kernel<D, IoT>, a);
     if (ev_stop) cudaEventRecord(ev_stop, stream);
     return err;
@@ -823,23 +817,23 @@ cudaError_t launch_any(const RecurArgs &a, int d, int io_dtype, long long pairs,
 
 }  // namespace
 
-cudaError_t launch_fwd_recur(const FwdArgs &f, int io_dtype, int sms, void *ws, size_t ws_bytes, cudaStream_t stream) {
+cudaError_t launch_fwd_recur(const FwdArgs &f, int io_dtype, void *ws, size_t ws_bytes, cudaStream_t stream) {
     RecurArgs a = {};
     a.q = f.q; a.k = f.k; a.v = f.v; a.gate = f.gate; a.lam = f.lam; a.beta = f.beta; a.alpha = f.alpha; a.out = f.out;
     a.state_in = f.state_in; a.state_out = f.state_out; a.fro_out = f.fro_out; a.device_status = f.device_status;
     a.T = f.T; a.heads = f.heads; a.n_iter = f.n_iter; a.flags = f.flags; a.solve_only = f.solve_only;
-    return launch_any(a, f.d, io_dtype, (long long)f.B * f.heads, sms, ws, ws_bytes, f.ev_start, f.ev_stop, stream);
+    return launch_any(a, f.d, io_dtype, (long long)f.B * f.heads, f.sms, ws, ws_bytes, f.ev_start, f.ev_stop, stream);
 }
 
 cudaError_t launch_decode_multi(float *state, const void *q, const void *k, const void *v, const float *gate,
                                 const float *lam, int n_iter, void *out, int nseq, int T, int heads, int d, int io_dtype,
-                                unsigned flags, const float *beta, const float *alpha, int *device_status,
+                                unsigned flags, const float *beta, const float *alpha, int *device_status, int sms,
                                 cudaEvent_t ev_start, cudaEvent_t ev_stop, cudaStream_t stream) {
     RecurArgs a = {};
     a.q = q; a.k = k; a.v = v; a.gate = gate; a.lam = lam; a.beta = beta; a.alpha = alpha; a.out = out;
     a.state_in = state; a.state_out = state; a.device_status = device_status;
     a.T = T; a.heads = heads; a.n_iter = n_iter; a.flags = flags;
-    return launch_any(a, d, io_dtype, (long long)nseq * heads, 0, nullptr, 0, ev_start, ev_stop, stream);
+    return launch_any(a, d, io_dtype, (long long)nseq * heads, sms, nullptr, 0, ev_start, ev_stop, stream);
 }
 
 }  // namespace gka

@@ -1106,12 +1106,10 @@ cudaError_t launch_fwd_solve(const FwdArgs &a, cudaStream_t stream) {
     const bool half = a.d == 64;
     auto kernel = extra ? (half ? fwd_tc_solve_kernel<true, true> : fwd_tc_solve_kernel<true, false>)
                         : (half ? fwd_tc_solve_kernel<false, true> : fwd_tc_solve_kernel<false, false>);
-    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SOLVE_SMEM);
+    static SmemLimit limit[2][2];
+    cudaError_t err = limit[extra][half].raise(kernel, (int)SOLVE_SMEM);
     if (err != cudaSuccess) return err;
-    int dev = 0, sms = 0;
-    if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
-    if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return err;
-    const long long want = ntiles < sms ? ntiles : (long long)sms;   // one persistent block per SM, two tiles in flight each
+    const long long want = ntiles < a.sms ? ntiles : (long long)a.sms;   // one persistent block per SM, two tiles in flight each
     if (a.ev_start) cudaEventRecord(a.ev_start, stream);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(want < 1 ? 1 : want));

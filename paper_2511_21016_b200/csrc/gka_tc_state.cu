@@ -69,8 +69,9 @@ __global__ void __launch_bounds__(kThreadsState, 1)
 fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, FwdArgs a) {
     const WorkPlan &P = a.plan;
     const int item = blockIdx.x;
-    // the state kernel may be launched as a programmatic dependent: its blocks may take the SMs that this grid
-    // leaves and run their prologue; they wait for this grid's completion before they read a summary
+    // Programmatic launch in stream order: wait for whatever wrote the inputs, then let the state kernel's blocks take the SMs
+    // that this grid leaves and run their prologue; they wait for this grid's completion before they read a summary.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (!P.cut_out(item)) return;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -262,7 +263,10 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     unsigned char *smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     const uint32_t sb = smem_u32(smem), bars = smem_u32(&s_bars[0]);
     const int t = threadIdx.x, l = t & 31;
-    // the solve kernel is launched as a programmatic dependent of this one
+    // The call's first kernel waits for whatever wrote its inputs (behind a summary or scan kernel only the summaries are
+    // waited for, further down); the solve kernel is launched as a programmatic dependent of this one and reads inputs
+    // before it waits, hence this order.
+    if (!a.after_summary) asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (t == 0) {
@@ -639,51 +643,41 @@ cudaError_t launch_fwd_tc(const FwdArgs &a_in, cudaStream_t stream) {
     // work items) would make every block re-read its whole chain, so the scan kernel materialises the start
     // states once instead.
     a.start_from_scan = longest > 4 ? 1 : 0;
-    int sms_here = 0, dev_here = 0;
-    if ((err = cudaGetDevice(&dev_here)) != cudaSuccess) return err;
-    if ((err = cudaDeviceGetAttribute(&sms_here, cudaDevAttrMultiProcessorCount, dev_here)) != cudaSuccess) return err;
     // two blocks per work item (one per master) where no sequence is cut and the blocks still fit one per SM
-    a.state_split = (!any_cut && 2 * a.plan.G <= sms_here) ? 1 : 0;
+    a.state_split = (!any_cut && 2 * a.plan.G <= a.sms) ? 1 : 0;
     alignas(64) CUtensorMap tmK, tmV, tmS;      // boxes of 128 tokens x 64 channels; per-tile bf16 state copies
     const int cols = a.heads * a.d;
     if (!make_tile_map(&tmK, a.k, a.B, a.T, cols, NT) || !make_tile_map(&tmV, a.v, a.B, a.T, cols, NT) ||
         !make_state_map(&tmS, a.tile_hu, (unsigned long long)a.plan.NC * 256ull))
         return cudaErrorInvalidValue;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cfg.stream = stream;
+    static SmemLimit summary_limit, state_limit[2];
     if (any_cut) {
-        err = cudaFuncSetAttribute(fwd_tc_summary_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KV_SMEM);
-        if (err != cudaSuccess) return err;
-        fwd_tc_summary_kernel<<<a.plan.G, kThreadsState, KV_SMEM, stream>>>(tmK, tmV, a);
+        if ((err = summary_limit.raise(fwd_tc_summary_kernel, (int)KV_SMEM)) != cudaSuccess) return err;
+        cfg.gridDim = dim3((unsigned)a.plan.G);
+        cfg.blockDim = dim3(kThreadsState);
+        cfg.dynamicSmemBytes = KV_SMEM;
+        if ((err = cudaLaunchKernelEx(&cfg, fwd_tc_summary_kernel, tmK, tmV, a)) != cudaSuccess) return err;
         if (a.start_from_scan) {
-            cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(2 * D * D / 4 / 256, (unsigned)(a.plan.G - 1));
             cfg.blockDim = dim3(256);
-            cfg.stream = stream;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            attr[0].val.programmaticStreamSerializationAllowed = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
+            cfg.dynamicSmemBytes = 0;
             if ((err = cudaLaunchKernelEx(&cfg, fwd_scan, a)) != cudaSuccess) return err;
         }
         a.after_summary = 1;
     }
     auto state_kernel = a.state_split ? fwd_tc_state_kernel<true> : fwd_tc_state_kernel<false>;
-    err = cudaFuncSetAttribute(state_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ST_SMEM);
-    if (err != cudaSuccess) return err;
-    {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(a.plan.G * (a.state_split ? 2 : 1)));
-        cfg.blockDim = dim3(kThreadsStateK);
-        cfg.dynamicSmemBytes = ST_SMEM;
-        cfg.stream = stream;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = a.after_summary ? 1 : 0;
-        err = cudaLaunchKernelEx(&cfg, state_kernel, tmK, tmV, tmS, a);
-        if (err != cudaSuccess) return err;
-    }
+    if ((err = state_limit[a.state_split].raise(state_kernel, (int)ST_SMEM)) != cudaSuccess) return err;
+    cfg.gridDim = dim3((unsigned)(a.plan.G * (a.state_split ? 2 : 1)));
+    cfg.blockDim = dim3(kThreadsStateK);
+    cfg.dynamicSmemBytes = ST_SMEM;
+    if ((err = cudaLaunchKernelEx(&cfg, state_kernel, tmK, tmV, tmS, a)) != cudaSuccess) return err;
     return launch_fwd_solve(a, stream);
 }
 
