@@ -60,9 +60,14 @@ constexpr int CT = kSlots * ST;            // compute threads
 // Warpgroups: 0 = helpers (gate scalars, TMA: one warp per slot, MMA issue), 1 = score warps (the masked-score
 // epilogue of both slots, one warp per TMEM lane quadrant), 2 and 3 = the compute warps of slot 0 and slot 1.
 constexpr int kThreadsSolve = 256 + CT;
-constexpr int kRegsLaunch = 128, kRegsCompute = 200, kRegsScore = 64, kRegsHelper = 48;   // register split after setmaxnreg
+// register split after setmaxnreg; with head dimension 64 the iterate takes half the registers
+constexpr int kRegsLaunch = 128, kRegsHelper = 48;
+__host__ __device__ constexpr int regs_compute(bool half) { return half ? 152 : 200; }
+__host__ __device__ constexpr int regs_score(bool half) { return half ? 160 : 64; }
 static_assert(kThreadsSolve * kRegsLaunch <= 65536, "launch registers");
-static_assert(CT * kRegsCompute + 128 * kRegsScore + 128 * kRegsHelper <= kThreadsSolve * kRegsLaunch, "register split exceeds the launch allocation");
+static_assert(CT * regs_compute(false) + 128 * regs_score(false) + 128 * kRegsHelper <= kThreadsSolve * kRegsLaunch &&
+                  CT * regs_compute(true) + 128 * regs_score(true) + 128 * kRegsHelper <= kThreadsSolve * kRegsLaunch,
+              "register split exceeds the launch allocation");
 
 // ---- shared memory map (bytes; operand buffers 1024-byte aligned): three operand tiles per slot, then the scalars
 constexpr uint32_t BUF_A = 0;                  // keys (Khat)
@@ -88,7 +93,7 @@ struct SlotScalars {
 };
 constexpr uint32_t SC_BYTES = (sizeof(SlotScalars) + 127) / 128 * 128;
 constexpr uint32_t SOLVE_SMEM = OFF_SC + kSlots * SC_BYTES + 1024;   // + slack for the 1024-byte alignment of the base
-static_assert(SOLVE_SMEM + 2048 <= 232448, "shared memory budget");
+static_assert(SOLVE_SMEM + 4096 <= 232448, "shared memory budget");
 
 // ---- TMEM columns: shared score accumulator S (P overwrites it in place); per slot the residual / output
 // accumulator R and the bf16 operand E
@@ -213,7 +218,7 @@ __device__ __forceinline__ void prod_kk(bool half, uint32_t d, uint32_t a_base, 
     else mma8_kk<ACC0, 8>(d, a_base, b_base, kIdescKK);
 }
 // The products of one request.  kb, hb, cb: descriptor bases (shared address >> 4) of the slot's buffers.
-__device__ __forceinline__ void issue_batch(int op, bool half, uint32_t kb, uint32_t hb, uint32_t cb, uint32_t tm_S, uint32_t tm_R,
+__device__ __forceinline__ void issue_batch(int op, bool half, bool split, uint32_t kb, uint32_t hb, uint32_t cb, uint32_t tm_S, uint32_t tm_R,
                                             uint32_t tm_E, uint32_t bar_s, uint32_t bar_r, uint32_t bar_sc) {
     switch (op) {
         case OP_FROB:    // Gram matrix Khat Khat^T and Khat H_0
@@ -224,7 +229,7 @@ __device__ __forceinline__ void issue_batch(int op, bool half, uint32_t kb, uint
         case OP_ITER1:   // S = E Khat^T, R += E H_0^T (the second runs under the masked-score epilogue)
             prod_ek<0>(half, tm_S, tm_E, kb);
             mma_commit(bar_sc);
-            if (half) mma_commit(bar_s);     // (the slot's compute warps take part in the masked-score epilogue)
+            if (split) mma_commit(bar_s);    // (the slot's compute warps take part in the masked-score epilogue)
             prod_ek<1>(half, tm_R, tm_E, hb);
             break;
         case OP_ITER2:   // R += P Khat
@@ -253,10 +258,10 @@ struct Ctx {
 
 // Masked scores of 16 keys: S (fp32, 16 columns) -> P (packed bf16 pairs in 8 registers).  EXACT: per-element factor
 // 2^(ac_c - G_j) (strongly decaying tiles, whose keys are not pre-scaled); KEYF: key j's column times ks[j] (the pass
-// whose P meets the unscaled V); DIAG: keys i <= l of the 32-key block are visible (i0: first key of this half).
+// whose P meets the unscaled V); DIAG: mk masks the keys i <= l of the 32-key block.
 template <bool EXACT, bool KEYF, bool DIAG>
 __device__ __forceinline__ void p_half(const uint32_t (&r)[16], uint32_t (&pk)[8], const float *G2h, const float *ksh,
-                                       float ac_c, int l, int i0) {
+                                       float ac_c, const uint32_t *mk) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
         float p0 = __uint_as_float(r[2 * u]), p1 = __uint_as_float(r[2 * u + 1]);
@@ -269,11 +274,19 @@ __device__ __forceinline__ void p_half(const uint32_t (&r)[16], uint32_t (&pk)[8
             p0 *= f.x;
             p1 *= f.y;
         }
-        if (DIAG) {
-            p0 = (i0 + 2 * u <= l) ? p0 : 0.f;
-            p1 = (i0 + 2 * u + 1 <= l) ? p1 : 0.f;
-        }
         pk[u] = pack_bf16(p0, p1);
+        if (DIAG) pk[u] &= mk[u];
+    }
+}
+// The keys of the diagonal block that token l of a lane quadrant sees, as masks of the packed pairs 2 u, 2 u + 1: a table in
+// shared memory (rows of 20 words: no bank conflict), fetched while the scores are on their way.  Selecting before the
+// conversion took four instructions per pair, on a scheduler that the update warps of the other slot keep busy.
+struct DiagMasks { uint32_t row[32][20]; };
+__device__ __forceinline__ void diag_masks(const DiagMasks &m, int l, uint32_t (&mk)[16]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(&m.row[l][4 * i]);
+        mk[4 * i] = v.x; mk[4 * i + 1] = v.y; mk[4 * i + 2] = v.z; mk[4 * i + 3] = v.w;
     }
 }
 // Masked-score epilogue of token c = 32 q + l: key blocks below q need no mask, block q is the diagonal block, the
@@ -282,15 +295,17 @@ __device__ __forceinline__ void p_half(const uint32_t (&r)[16], uint32_t (&pk)[8
 // first.
 template <bool EXACT, bool KEYF>
 __device__ __forceinline__ void p_convert(const Ctx &cx, const GateScalars *gs, float ac_c, int kb, const uint32_t (&ra)[16],
-                                          const uint32_t (&rb)[16]) {
+                                          const uint32_t (&rb)[16], const DiagMasks &dm) {
     uint32_t pa[8], pb[8];
     const float *G2kb = gs->G2 + 32 * kb, *kskb = gs->ks + 32 * kb;
+    uint32_t mk[16];
     if (kb == cx.q) {
-        p_half<EXACT, KEYF, true>(ra, pa, G2kb, kskb, ac_c, cx.l, 0);
-        p_half<EXACT, KEYF, true>(rb, pb, G2kb + 16, kskb + 16, ac_c, cx.l, 16);
+        diag_masks(dm, cx.l, mk);
+        p_half<EXACT, KEYF, true>(ra, pa, G2kb, kskb, ac_c, mk);
+        p_half<EXACT, KEYF, true>(rb, pb, G2kb + 16, kskb + 16, ac_c, mk + 8);
     } else {
-        p_half<EXACT, KEYF, false>(ra, pa, G2kb, kskb, ac_c, cx.l, 0);
-        p_half<EXACT, KEYF, false>(rb, pb, G2kb + 16, kskb + 16, ac_c, cx.l, 16);
+        p_half<EXACT, KEYF, false>(ra, pa, G2kb, kskb, ac_c, mk);
+        p_half<EXACT, KEYF, false>(rb, pb, G2kb + 16, kskb + 16, ac_c, mk + 8);
     }
     TMEM_ST8(cx.tm_s + 32 * kb, pa);
     TMEM_ST8(cx.tm_s + 32 * kb + 8, pb);
@@ -301,21 +316,71 @@ __device__ __forceinline__ void p_convert(const Ctx &cx, const GateScalars *gs, 
 __device__ __forceinline__ int p_split(int q) { return (q + 2) >> 1; }
 // The masked-score epilogue of an iteration for the key blocks kb0 <= kb < kb1 of this thread's token.
 template <bool EXACT>
-__device__ __forceinline__ void p_epilogue_blocks(const Ctx &cx, const GateScalars *gs, float ac_c, int kb0, int kb1) {
+__device__ __forceinline__ void p_epilogue_blocks(const Ctx &cx, const GateScalars *gs, float ac_c, int kb0, int kb1, const DiagMasks &dm) {
 #pragma unroll 1
     for (int kb = kb0; kb < kb1; ++kb) {
         uint32_t ra[16], rb[16];
         TMEM_LD16(cx.tm_s + 32 * kb, ra);
         TMEM_LD16(cx.tm_s + 32 * kb + 16, rb);
         tmem_wait_ld();
-        p_convert<EXACT, false>(cx, gs, ac_c, kb, ra, rb);
+        p_convert<EXACT, false>(cx, gs, ac_c, kb, ra, rb, dm);
     }
     tmem_wait_st();
 }
-template <bool EXACT, bool KEYF, bool SPLIT>
-__device__ __forceinline__ void p_epilogue_t(const Ctx &cx, const GateScalars *gs, float ac_c) {
+// The same for all key blocks of lane quadrant Q, as straight-line code.
+template <int Q, int KB>
+__device__ __forceinline__ void p_block(const Ctx &cx, const DiagMasks &dm, const uint32_t (&r)[32]) {
+    uint32_t mk[16];
+    if constexpr (KB == Q) diag_masks(dm, cx.l, mk);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        uint32_t pk[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            pk[u] = pack_bf16(__uint_as_float(r[16 * h + 2 * u]), __uint_as_float(r[16 * h + 2 * u + 1]));
+            if constexpr (KB == Q) pk[u] &= mk[8 * h + u];
+        }
+        TMEM_ST8(cx.tm_s + 32 * KB + 8 * h, pk);
+    }
+}
+// AHEAD: with the registers for it (head dimension 64) every block's load is in flight at once.
+template <int Q, bool AHEAD>
+__device__ __forceinline__ void p_blocks(const Ctx &cx, const DiagMasks &dm) {
+    uint32_t r[AHEAD ? Q + 1 : 1][32];
+    if constexpr (AHEAD) {
+#pragma unroll
+        for (int kb = 0; kb <= Q; ++kb) TMEM_LD32(cx.tm_s + 32 * kb, r[kb]);
+        tmem_wait_ld();
+    } else {
+        TMEM_LD32(cx.tm_s, r[0]);
+        tmem_wait_ld();
+    }
+    p_block<Q, 0>(cx, dm, r[0]);
+    if constexpr (Q > 0) {
+        if constexpr (!AHEAD) { TMEM_LD32(cx.tm_s + 32, r[0]); tmem_wait_ld(); }
+        p_block<Q, 1>(cx, dm, r[AHEAD ? 1 : 0]);
+    }
+    if constexpr (Q > 1) {
+        if constexpr (!AHEAD) { TMEM_LD32(cx.tm_s + 64, r[0]); tmem_wait_ld(); }
+        p_block<Q, 2>(cx, dm, r[AHEAD ? 2 : 0]);
+    }
+    if constexpr (Q > 2) {
+        if constexpr (!AHEAD) { TMEM_LD32(cx.tm_s + 96, r[0]); tmem_wait_ld(); }
+        p_block<Q, 3>(cx, dm, r[AHEAD ? 3 : 0]);
+    }
+}
+template <bool EXACT, bool KEYF, bool SPLIT, bool AHEAD>
+__device__ __forceinline__ void p_epilogue_t(const Ctx &cx, const GateScalars *gs, float ac_c, const DiagMasks &dm) {
     if (!KEYF && SPLIT) {     // an iteration: the upper key blocks are left to the token's compute warp
-        p_epilogue_blocks<EXACT>(cx, gs, ac_c, 0, p_split(cx.q));
+        p_epilogue_blocks<EXACT>(cx, gs, ac_c, 0, p_split(cx.q), dm);
+        return;
+    }
+    if (!KEYF && !EXACT) {
+        if (cx.q == 0) p_blocks<0, AHEAD>(cx, dm);
+        else if (cx.q == 1) p_blocks<1, AHEAD>(cx, dm);
+        else if (cx.q == 2) p_blocks<2, AHEAD>(cx, dm);
+        else p_blocks<3, AHEAD>(cx, dm);
+        tmem_wait_st();
         return;
     }
     if (KEYF) {      // (the product of an iteration leaves out the rows whose key block is above the diagonal instead)
@@ -334,14 +399,14 @@ __device__ __forceinline__ void p_epilogue_t(const Ctx &cx, const GateScalars *g
         TMEM_LD16(cx.tm_s + 32 * kb, ra);
         TMEM_LD16(cx.tm_s + 32 * kb + 16, rb);
         tmem_wait_ld();
-        p_convert<EXACT, KEYF>(cx, gs, ac_c, kb, ra, rb);
+        p_convert<EXACT, KEYF>(cx, gs, ac_c, kb, ra, rb, dm);
     }
     tmem_wait_st();
 }
-template <bool KEYF, bool SPLIT>
-__device__ __forceinline__ void p_epilogue(const Ctx &cx, const GateScalars *gs, bool exact, float ac_c) {
-    if (exact) p_epilogue_t<true, KEYF, SPLIT>(cx, gs, ac_c);
-    else p_epilogue_t<false, KEYF, SPLIT>(cx, gs, ac_c);
+template <bool KEYF, bool SPLIT, bool AHEAD>
+__device__ __forceinline__ void p_epilogue(const Ctx &cx, const GateScalars *gs, bool exact, float ac_c, const DiagMasks &dm) {
+    if (exact) p_epilogue_t<true, KEYF, SPLIT, AHEAD>(cx, gs, ac_c, dm);
+    else p_epilogue_t<false, KEYF, SPLIT, AHEAD>(cx, gs, ac_c, dm);
 }
 
 // Sum over one 32-key block of the squared Gram entries of the earlier keys (decayed when the keys are not
@@ -393,7 +458,8 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     __shared__ uint32_t s_tmem_base;
     __shared__ int s_abort;
     __shared__ __align__(16) uint32_t s_req[4];     // per slot: requests posted (warps), Gram matrices read (warps)
-    __shared__ uint32_t s_sinfo[2];                 // score event n (parity): slot | read pass << 1 | gate buffer << 2 | (n + 1) << 8
+    __shared__ __align__(16) DiagMasks dm;
+    __shared__ uint32_t s_sinfo[2];                 // score event n (parity): slot | read pass << 1 | gate buffer << 2 | per-element factors << 3 | (n + 1) << 8
 
     unsigned char *smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     const int tid = threadIdx.x;
@@ -410,6 +476,10 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bars + 8 * i), "r"(per_warp ? ST / 32 : 1));
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    for (int i = tid; i < 32 * 16; i += kThreadsSolve) {
+        const int ml = i >> 4, u = i & 15;
+        dm.row[ml][u] = (2 * u <= ml ? 0x0000FFFFu : 0u) | (2 * u + 1 <= ml ? 0xFFFF0000u : 0u);
     }
     if (tid < 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&s_tmem_base))
@@ -431,7 +501,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     const bool mix = alpha_p != nullptr && !solve_only;   // alpha-connection: the read uses alpha x + (1 - alpha) q
     // Head dimension 64: the slot's compute warps, idle while the slot has the score tile, convert the upper key blocks of
     // the masked scores of an iteration (with 128 channels this measured slower: the warps come later to their update)
-    constexpr bool SPLIT = HALF;
+    constexpr bool SPLIT = false;
     constexpr bool half = HALF;                           // head dimension 64: channels 64..127 are zero, their k-steps are left out
 
     // The helper warps come first: when a scheduler changes warps it prefers the oldest eligible one, and the thread
@@ -552,16 +622,21 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 bool gave_up = false;
                 uint32_t sev = 0;                       // score events so far
                 const uint32_t sinfo_addr = smem_u32(&s_sinfo[0]);
+                auto buffer_info = [&](int sl) -> uint32_t {      // gate buffer of the slot's tile, and whether it needs per-element factors
+                    const uint32_t buf = (sl ? til1 : til0) & 1u;
+                    const int *const ex = reinterpret_cast<const SlotScalars *>(smem + OFF_SC + sl * SC_BYTES)->exact;
+                    return (buf << 2) | (*reinterpret_cast<const volatile int *>(ex + buf) != 0 ? 8u : 0u);
+                };
                 auto issue = [&](int sl, int o) {
                     const uint32_t sbb = bars + 8 * (sl * B_PER_SLOT);
                     const uint32_t sl14 = base14 + ((sl * SLOT_BYTES) >> 4);
                     if (o == OP_ITER1 || o == OP_OUT_S) {   // tell the score warps whose scores come next
                         ++sev;
-                        const uint32_t info = (uint32_t)sl | (o == OP_OUT_S ? 2u : 0u) | (((sl ? til1 : til0) & 1u) << 2) | (sev << 8);
+                        const uint32_t info = (uint32_t)sl | (o == OP_OUT_S ? 2u : 0u) | buffer_info(sl) | (sev << 8);
                         asm volatile("st.volatile.shared::cta.u32 [%0], %1;" ::"r"(sinfo_addr + 4u * ((sev - 1u) & 1u)), "r"(info) : "memory");
                     }
                     fence_after();
-                    issue_batch(o, half, sl14 + (BUF_A >> 4), sl14 + (BUF_B >> 4), sl14 + (BUF_C >> 4), tmem + TM_S, tmem + tm_r_of(sl),
+                    issue_batch(o, half, SPLIT, sl14 + (BUF_A >> 4), sl14 + (BUF_B >> 4), sl14 + (BUF_C >> 4), tmem + TM_S, tmem + tm_r_of(sl),
                                 tmem + tm_e_of(sl), sbb + 8 * B_MMA_S, sbb + 8 * B_MMA_R, bars + 8 * B_SC);
                 };
                 // Bookkeeping of a request of slot sl that has just been issued, together with its follow-up (ITER2 after
@@ -643,7 +718,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                         const uint32_t thr_t = t ? thr1 : thr0;
                         const uint32_t n_kb = t14 + (BUF_A >> 4), n_tmE = tmem + tm_e_of(t);
                         const uint32_t n_barS = bars + 8 * (t * B_PER_SLOT + B_MMA_S);
-                        const uint32_t n_info = (uint32_t)t | (((t ? til1 : til0) & 1u) << 2) | ((sev + 1u) << 8);
+                        const uint32_t n_info = (uint32_t)t | buffer_info(t) | ((sev + 1u) << 8);
                         const uint32_t n_sinfo = sinfo_addr + 4u * (sev & 1u);
                         uint32_t c_t = 0u;
                         for (int polls = 0;;) {
@@ -710,7 +785,8 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         // The masked-score epilogue of both slots: S (fp32) -> P (packed bf16) in place, for the scores of an iteration
         // and for those of the read.  These warps hold no iterate, so they are not short of registers, and the compute
         // warps go from their update straight to the wait for the accumulator.
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsScore));
+        if constexpr (HALF) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(regs_score(true)));
+        else asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(regs_score(false)));
         Ctx cx;
         cx.l = tid & 31;
         cx.q = (tid >> 5) & 3;
@@ -721,8 +797,8 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         const long long n_events = (long long)n_mine * per_tile;
         int reads0 = 0, reads1 = 0;         // read passes seen per slot (= tiles done)
         for (long long ev = 0; ev < n_events; ++ev) {
-            // The issuing thread announces an event before it issues the score product: whose scores, which pass; the
-            // scalars the epilogue needs are fetched while the product runs.
+            // The issuing thread announces an event before it issues the score product: whose scores, which pass, which gate
+            // buffer, per-element factors or not.
             uint32_t info = 0u;
             if (cx.l == 0) {
                 for (int polls = 0;; ++polls) {
@@ -736,10 +812,9 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             }
             info = __shfl_sync(0xffffffffu, info, 0);
             const int sl_ = (int)(info & 1u);
-            const SlotScalars *const scs = reinterpret_cast<const SlotScalars *>(smem + OFF_SC + sl_ * SC_BYTES);
-            const GateScalars *const gs = &scs->g[(info >> 2) & 1u];
-            const bool exact = scs->exact[(info >> 2) & 1u] != 0;
-            const float ac_c = gs->ac[cx.c];
+            const GateScalars *const gs = &reinterpret_cast<const SlotScalars *>(smem + OFF_SC + sl_ * SC_BYTES)->g[(info >> 2) & 1u];
+            const bool exact = (info & 8u) != 0u;
+            const float ac_c = exact ? gs->ac[cx.c] : 0.f;
             wait_bar(bars + 8 * B_SC, (uint32_t)(ev & 1), abort_addr);
             fence_after();
             if (info & 2u) {
@@ -753,16 +828,16 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     tma_load_tile3(&tmK, sbase + sl_ * SLOT_BYTES + BUF_A, bar_k, tn.h * a.d, tile_x_hi(tn.h, a.d, a.heads), tn.n * NT, tn.b);
                 }
                 if (sl_) ++reads1; else ++reads0;
-                p_epilogue<true, SPLIT>(cx, gs, exact, ac_c);
+                p_epilogue<true, SPLIT, HALF>(cx, gs, exact, ac_c, dm);
             } else {
-                p_epilogue<false, SPLIT>(cx, gs, exact, ac_c);
+                p_epilogue<false, SPLIT, HALF>(cx, gs, exact, ac_c, dm);
             }
             fence_before();
             warp_post(smem_u32(&s_req[sl_]), cx.l);          // -> ITER2 / OUT_O of that slot
         }
     } else {
         // ================================= compute threads =================================
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsCompute));
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(regs_compute(HALF)));
         const int slot = (tid >> 7) - 2;
         Ctx cx;
         cx.l = tid & 31;
@@ -922,7 +997,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 if (a.fro_out && valid) a.fro_out[ti.tok0 + (size_t)c * a.heads] = fc;
             }
             wait_bar(sb + 8 * B_LD_Q, (uint32_t)(j & 1), abort_addr);   // q tile has landed
-            // ---- x_0: R = q, E_0 = czb q, xs = E_0
+            // ---- x_0: R = q, E_0 = czb q; xs takes an increment when it is next read from the operand columns
 #pragma unroll
             for (int g16 = 0; g16 < NG16; ++g16) {
                 uint32_t rr[16], pk[8];
@@ -935,9 +1010,8 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                         const float qa = bf16_lo(qq[u]), qb = bf16_hi(qq[u]);
                         rr[8 * h2 + 2 * u] = __float_as_uint(qa);
                         rr[8 * h2 + 2 * u + 1] = __float_as_uint(qb);
-                        const uint32_t p = pack_bf16(czb * qa, czb * qb);
-                        pk[4 * h2 + u] = p;
-                        xs[8 * g16 + 4 * h2 + u] = f2_pack(bf16_lo(p), bf16_hi(p));
+                        pk[4 * h2 + u] = pack_bf16(czb * qa, czb * qb);
+                        xs[8 * g16 + 4 * h2 + u] = 0ull;
                     }
                 }
                 TMEM_ST16(cx.tm_r + 16 * g16, rr);
@@ -953,21 +1027,23 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             }
             for (int it = 0; it < a.n_iter; ++it) {
                 const bool last = it + 1 == a.n_iter;
-                omega = 4.f / (4.f - rho2 * omega);              // weight schedule
+                omega = 4.f * recip(4.f - rho2 * omega);         // weight schedule
                 const float beta = omega - 1.f, cz = czb * omega;
                 const uint64_t beta2 = f2_pack(beta, beta), cz2 = f2_pack(cz, cz), lz2 = f2_pack(lz, lz);
                 // this warp's share of the masked-score epilogue (the upper key blocks of its tokens)
                 if (SPLIT) {
                     wait_s();
-                    if (exact) p_epilogue_blocks<true>(cx, gs, gs->ac[c], p_split(cx.q), cx.q + 1);
-                    else p_epilogue_blocks<false>(cx, gs, 0.f, p_split(cx.q), cx.q + 1);
+                    if (exact) p_epilogue_blocks<true>(cx, gs, gs->ac[c], p_split(cx.q), cx.q + 1, dm);
+                    else p_epilogue_blocks<false>(cx, gs, 0.f, p_split(cx.q), cx.q + 1, dm);
                     fence_before();
                     arrive_rdy();                                // -> ITER2 (with the score warps' posts)
                 }
                 wait_r();
                 if (last) after_last_h0_product();
-                // e_new = beta e_old + cz (R + lz xs) as bf16, xs += e_new (the value the operand holds).  Sixteen
-                // channels at a time; the next group's loads are in flight while a group is computed.
+                // xs += e_old (the value the operand held), e_new = beta e_old + cz (R + lz xs) as bf16.  Sixteen channels at
+                // a time; the next group's loads are in flight while a group is computed.  (Adding e_new at once would unpack
+                // every increment twice: 9 instead of 7 instructions per pair of channels in code that runs once per
+                // iteration and does not fit the first-level instruction cache.)
                 {
                     uint32_t ra[16], rb[16], ea[8], eb[8];
                     TMEM_LD16(cx.tm_r, ra);
@@ -987,15 +1063,15 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 #pragma unroll
                         for (int u = 0; u < 8; ++u) {
                             const int i = 8 * g + u;
+                            const uint64_t eo = f2_pack(bf16_lo(e[u]), bf16_hi(e[u]));
+                            xs[i] = f2_add(xs[i], eo);
                             const uint64_t res = f2_fma(lz2, xs[i], f2_pack(__uint_as_float(r[2 * u]), __uint_as_float(r[2 * u + 1])));
-                            const uint64_t en = f2_fma(cz2, res, f2_mul(beta2, f2_pack(bf16_lo(e[u]), bf16_hi(e[u]))));
                             float ea_, eb_;
-                            f2_unpack(en, ea_, eb_);
+                            f2_unpack(f2_fma(cz2, res, f2_mul(beta2, eo)), ea_, eb_);
                             pk[u] = pack_bf16(ea_, eb_);
-                            xs[i] = f2_add(xs[i], f2_pack(bf16_lo(pk[u]), bf16_hi(pk[u])));
                         }
                         TMEM_ST8(cx.tm_e + 8 * g, pk);
-                                        if (g < NG16 - 1) tmem_wait_ld();
+                        if (g < NG16 - 1) tmem_wait_ld();
                     }
                     if (!last) {
                         tmem_wait_st();
@@ -1004,7 +1080,16 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     }
                 }
             }
-            // ---- final iterate
+            // ---- final iterate: the last increment
+            tmem_wait_st();
+#pragma unroll
+            for (int g = 0; g < NG16; g += 4) {
+                uint32_t e[32];
+                TMEM_LD32(cx.tm_e + 8 * g, e);
+                tmem_wait_ld();
+#pragma unroll
+                for (int u = 0; u < 32; ++u) xs[8 * g + u] = f2_add(xs[8 * g + u], f2_pack(bf16_lo(e[u]), bf16_hi(e[u])));
+            }
             if (solve_only) {
                 // the solve is the result: x_c = -xs / zt_c as bf16, staged in the q buffer and stored by TMA
                 const float izc = gs->iz[c];
