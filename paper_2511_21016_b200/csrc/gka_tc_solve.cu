@@ -30,19 +30,25 @@
 // product reads only its B operand (keys, H_0, U_0, values) from shared memory and leaves half of the shared-memory
 // bandwidth to everything else.  Shared memory per slot: keys, H_0 (later U_0), q (later V, then the result).
 //
-// Warp roles: 4 compute warps per slot, a thread owns one token (one TMEM lane) and all 128 channels of its
-// iterate in registers; 4 score warps (one per TMEM lane quadrant) run the masked-score epilogue of both slots; one
-// warp prepares the gate scalars one tile ahead; one thread per slot issues that slot's TMA stores and the loads that
-// follow them; one thread issues every tcgen05.mma for both slots.  Requests to the issuing thread are counters in
-// shared memory (one count per warp), completion comes back through tcgen05.commit mbarriers.  What bounds the
-// iterations is the turn of a slot on the score tile (score product, epilogue, second product); stores to tensor
-// memory (about 40 bytes per cycle per SM) are the scarce resource of the epilogues.
+// Warp roles: 4 compute warps per slot, a thread owns one token (one TMEM lane) and all 128 channels of its iterate in
+// registers, and masks its own scores; one warp prepares the gate scalars one tile ahead; one thread per slot issues that
+// slot's TMA stores and the loads that follow them; one thread issues every tcgen05.mma for both slots.  Requests to the
+// issuing thread are counters in shared memory (one count per warp), completion comes back through tcgen05.commit mbarriers.
+// What bounds the iterations is the turn of a slot on the score tile (score product, epilogue, second product), and in it how
+// fast a warp that has been woken gets through its instructions: what the warps of a block execute per iteration does not fit
+// the first-level instruction cache, so the number of instructions between two hand-overs counts more than their kind.
+// Hence the increment is added to the iterate when it is next unpacked, the diagonal block is masked after the conversion,
+// and there are no separate warps for the scores (as a third party they had to be told whose scores come next, started
+// cold, and shared every scheduler with two update warps).  B = 4, 16 heads, T = 4096, 10 / 30 iterations: 406 / 794 us per
+// call before, 351 / 681 with these.
 //
 // Head dimension 64 arrives zero-extended to 128 channels (the upper TMA box reads zeros).  The kernel instantiated
 // with HALF leaves out what the zero channels would contribute: contractions over the channels take four k-steps
-// instead of eight, and the passes of the compute warps over the channels stop at channel 64.  Its turns on the score
-// tile are shorter, so the masked-score epilogue weighs more: there the slot's compute warps, idle during the turn,
-// convert the upper key blocks of their tokens and the score warps the lower ones.
+// instead of eight, products into R have 64 columns, and the passes of the compute warps stop at channel 64.  R and E then
+// take half of their columns, which leaves room for a score tile per slot: nothing is handed from slot to slot, so a slot is
+// one chain of its four compute warps, and one of their threads issues the slot's products (no issuing thread: a request no
+// longer waits for a thread that serves both slots).  B = 4, 16 heads, T = 2048, 10 / 30 iterations: 179 / 353 us per call with
+// the shared score tile, 153 / 292 with this.
 #include <cuda.h>
 
 #include "gka_common.cuh"
@@ -57,17 +63,11 @@ constexpr int NT = kTile;                  // tokens per tile: one per TMEM lane
 constexpr int kSlots = 2;
 constexpr int ST = 128;                    // compute threads per slot
 constexpr int CT = kSlots * ST;            // compute threads
-// Warpgroups: 0 = helpers (gate scalars, TMA: one warp per slot, MMA issue), 1 = score warps (the masked-score
-// epilogue of both slots, one warp per TMEM lane quadrant), 2 and 3 = the compute warps of slot 0 and slot 1.
-constexpr int kThreadsSolve = 256 + CT;
-// register split after setmaxnreg; with head dimension 64 the iterate takes half the registers
-constexpr int kRegsLaunch = 128, kRegsHelper = 48;
-__host__ __device__ constexpr int regs_compute(bool half) { return half ? 152 : 200; }
-__host__ __device__ constexpr int regs_score(bool half) { return half ? 160 : 64; }
+// Warpgroups: 0 = helpers (gate scalars, TMA: one warp per slot, MMA issue), 1 and 2 = the compute warps of slot 0 and slot 1.
+constexpr int kThreadsSolve = 128 + CT;
+constexpr int kRegsLaunch = 168, kRegsCompute = 216, kRegsHelper = 72;   // register split after setmaxnreg (128 channels)
 static_assert(kThreadsSolve * kRegsLaunch <= 65536, "launch registers");
-static_assert(CT * regs_compute(false) + 128 * regs_score(false) + 128 * kRegsHelper <= kThreadsSolve * kRegsLaunch &&
-                  CT * regs_compute(true) + 128 * regs_score(true) + 128 * kRegsHelper <= kThreadsSolve * kRegsLaunch,
-              "register split exceeds the launch allocation");
+static_assert(CT * kRegsCompute + 128 * kRegsHelper <= kThreadsSolve * kRegsLaunch, "register split exceeds the launch allocation");
 
 // ---- shared memory map (bytes; operand buffers 1024-byte aligned): three operand tiles per slot, then the scalars
 constexpr uint32_t BUF_A = 0;                  // keys (Khat)
@@ -89,7 +89,6 @@ struct GateScalars {       // per token of a tile, from the gates and the other 
 struct SlotScalars {
     GateScalars g[2];
     float carry[2][4];     // per-warp totals (a, b) of the affine scan
-    int exact[2];          // the tile of gate buffer 0 / 1 decays below 2^-60 (per-element factors in the score epilogue)
 };
 constexpr uint32_t SC_BYTES = (sizeof(SlotScalars) + 127) / 128 * 128;
 constexpr uint32_t SOLVE_SMEM = OFF_SC + kSlots * SC_BYTES + 1024;   // + slack for the 1024-byte alignment of the base
@@ -97,9 +96,13 @@ static_assert(SOLVE_SMEM + 4096 <= 232448, "shared memory budget");
 
 // ---- TMEM columns: shared score accumulator S (P overwrites it in place); per slot the residual / output
 // accumulator R and the bf16 operand E
-constexpr uint32_t TM_S = 0;
-__host__ __device__ constexpr uint32_t tm_r_of(int s) { return 128u + 128u * (uint32_t)s; }
+// (128 channels), or, with head dimension 64, where R and E take half of the columns, a score tile per slot
+__host__ __device__ constexpr uint32_t tm_s_of(bool half, int s) { return half ? 128u * (uint32_t)s : 0u; }
+__host__ __device__ constexpr uint32_t tm_r_of(bool half, int s) { return half ? 256u + 64u * (uint32_t)s : 128u + 128u * (uint32_t)s; }
 __host__ __device__ constexpr uint32_t tm_e_of(int s) { return 384u + 64u * (uint32_t)s; }
+// products whose result goes to R have as many columns as there are channels
+__host__ __device__ constexpr uint32_t idesc_r_kk(bool half) { return make_idesc(128, half ? 64 : 128, 0, 0); }
+__host__ __device__ constexpr uint32_t idesc_r_pm(bool half) { return make_idesc(128, half ? 64 : 128, 0, 1); }
 
 enum {                 // per slot
     B_LD_K = 0,        // K tile has landed (TMA)
@@ -116,8 +119,8 @@ enum {                 // per slot
     B_PER_SLOT
 };
 constexpr int B_DRAIN = kSlots * B_PER_SLOT;   // every product is complete (before the tensor memory is given back)
-constexpr int B_SC = B_DRAIN + 1;              // tcgen05.commit: a score product of either slot is complete (-> score warps)
-constexpr int B_COUNT = B_SC + 1;
+constexpr int B_SC = B_DRAIN + 1;              // + slot: tcgen05.commit, a score product of the slot is complete
+constexpr int B_COUNT = B_SC + kSlots;
 
 // Requests a slot makes to the issuing thread: every warp of the slot adds one to the slot's request counter in
 // shared memory (a poll of both counters is one 40-cycle load, where a test of an mbarrier phase takes 100 cycles);
@@ -161,6 +164,12 @@ __device__ __forceinline__ void wait_bar(uint32_t bar, uint32_t parity, uint32_t
 __device__ __forceinline__ void warp_post(uint32_t addr, int lane) {
     __syncwarp();
     if (lane == 0) asm volatile("red.release.cta.shared::cta.add.u32 [%0], 1;" ::"r"(addr) : "memory");
+}
+// The same where the warp has written tensor memory only: tcgen05.wait::st and tcgen05.fence::before_thread_sync order that
+// for the thread that issues the products, and the count itself need not wait for anything else.
+__device__ __forceinline__ void warp_post_tmem(uint32_t addr, int lane) {
+    __syncwarp();
+    if (lane == 0) asm volatile("red.relaxed.cta.shared::cta.add.u32 [%0], 1;" ::"r"(addr) : "memory");
 }
 // one arrival per warp, after every lane's writes and fences
 __device__ __forceinline__ void warp_arrive(uint32_t bar, int lane) {
@@ -208,42 +217,41 @@ __device__ __forceinline__ void mma8_ek(uint32_t d, uint32_t e_tmem, uint32_t b_
 // The contractions over the channels: with head dimension 64 (zero-extended on chip) the channels 64..127 of every
 // operand are zero, and the four k-steps over them are left out.
 template <int ACC0>
-__device__ __forceinline__ void prod_ek(bool half, uint32_t d, uint32_t e_tmem, uint32_t b_base) {
-    if (half) mma8_ek<ACC0, 4>(d, e_tmem, b_base, kIdescKK);
-    else mma8_ek<ACC0, 8>(d, e_tmem, b_base, kIdescKK);
+__device__ __forceinline__ void prod_ek(bool half, uint32_t d, uint32_t e_tmem, uint32_t b_base, uint32_t idesc) {
+    if (half) mma8_ek<ACC0, 4>(d, e_tmem, b_base, idesc);
+    else mma8_ek<ACC0, 8>(d, e_tmem, b_base, idesc);
 }
 template <int ACC0>
-__device__ __forceinline__ void prod_kk(bool half, uint32_t d, uint32_t a_base, uint32_t b_base) {
-    if (half) mma8_kk<ACC0, 4>(d, a_base, b_base, kIdescKK);
-    else mma8_kk<ACC0, 8>(d, a_base, b_base, kIdescKK);
+__device__ __forceinline__ void prod_kk(bool half, uint32_t d, uint32_t a_base, uint32_t b_base, uint32_t idesc) {
+    if (half) mma8_kk<ACC0, 4>(d, a_base, b_base, idesc);
+    else mma8_kk<ACC0, 8>(d, a_base, b_base, idesc);
 }
 // The products of one request.  kb, hb, cb: descriptor bases (shared address >> 4) of the slot's buffers.
-__device__ __forceinline__ void issue_batch(int op, bool half, bool split, uint32_t kb, uint32_t hb, uint32_t cb, uint32_t tm_S, uint32_t tm_R,
+__device__ __forceinline__ void issue_batch(int op, bool half, uint32_t kb, uint32_t hb, uint32_t cb, uint32_t tm_S, uint32_t tm_R,
                                             uint32_t tm_E, uint32_t bar_s, uint32_t bar_r, uint32_t bar_sc) {
     switch (op) {
         case OP_FROB:    // Gram matrix Khat Khat^T and Khat H_0
-            prod_kk<0>(half, tm_S, kb, kb);
-            prod_kk<0>(half, tm_R, kb, hb);
+            prod_kk<0>(half, tm_S, kb, kb, kIdescKK);
+            prod_kk<0>(half, tm_R, kb, hb, idesc_r_kk(half));
             mma_commit(bar_s);
             break;
         case OP_ITER1:   // S = E Khat^T, R += E H_0^T (the second runs under the masked-score epilogue)
-            prod_ek<0>(half, tm_S, tm_E, kb);
+            prod_ek<0>(half, tm_S, tm_E, kb, kIdescKK);
             mma_commit(bar_sc);
-            if (split) mma_commit(bar_s);    // (the slot's compute warps take part in the masked-score epilogue)
-            prod_ek<1>(half, tm_R, tm_E, hb);
+            prod_ek<1>(half, tm_R, tm_E, hb, idesc_r_kk(half));
             break;
         case OP_ITER2:   // R += P Khat
-            mma8_pm_rows(tm_R, tm_S, kb, kIdescPM);
+            mma8_pm_rows(tm_R, tm_S, kb, idesc_r_pm(half));
             mma_commit(bar_r);
             break;
         case OP_OUT_S:   // scores of the final iterate: S = X_hi Khat^T + X_lo Khat^T (X_lo sits in the first columns of R)
-            prod_ek<0>(half, tm_S, tm_E, kb);
-            prod_ek<1>(half, tm_S, tm_R, kb);
+            prod_ek<0>(half, tm_S, tm_E, kb, kIdescKK);
+            prod_ek<1>(half, tm_S, tm_R, kb, kIdescKK);
             mma_commit(bar_sc);
-            prod_ek<0>(half, tm_R, tm_E, hb);   // O = X_hi U_0^T (runs under the masked-score epilogue; X_lo has been read)
+            prod_ek<0>(half, tm_R, tm_E, hb, idesc_r_kk(half));   // O = X_hi U_0^T (runs under the masked-score epilogue; X_lo has been read)
             break;
         case OP_OUT_O:   // O += P V
-            mma8_pm(tm_R, tm_S, cb, kIdescPM);
+            mma8_pm(tm_R, tm_S, cb, idesc_r_pm(half));
             mma_commit(bar_r);
             break;
         default:
@@ -310,23 +318,6 @@ __device__ __forceinline__ void p_convert(const Ctx &cx, const GateScalars *gs, 
     TMEM_ST8(cx.tm_s + 32 * kb, pa);
     TMEM_ST8(cx.tm_s + 32 * kb + 8, pb);
 }
-// Head dimension 64: key blocks of the masked scores that a token's score warp converts in an iteration; the token's
-// compute warp, which has nothing else to do until the product that consumes the masked scores is complete, converts
-// the rest.
-__device__ __forceinline__ int p_split(int q) { return (q + 2) >> 1; }
-// The masked-score epilogue of an iteration for the key blocks kb0 <= kb < kb1 of this thread's token.
-template <bool EXACT>
-__device__ __forceinline__ void p_epilogue_blocks(const Ctx &cx, const GateScalars *gs, float ac_c, int kb0, int kb1, const DiagMasks &dm) {
-#pragma unroll 1
-    for (int kb = kb0; kb < kb1; ++kb) {
-        uint32_t ra[16], rb[16];
-        TMEM_LD16(cx.tm_s + 32 * kb, ra);
-        TMEM_LD16(cx.tm_s + 32 * kb + 16, rb);
-        tmem_wait_ld();
-        p_convert<EXACT, false>(cx, gs, ac_c, kb, ra, rb, dm);
-    }
-    tmem_wait_st();
-}
 // The same for all key blocks of lane quadrant Q, as straight-line code.
 template <int Q, int KB>
 __device__ __forceinline__ void p_block(const Ctx &cx, const DiagMasks &dm, const uint32_t (&r)[32]) {
@@ -343,38 +334,29 @@ __device__ __forceinline__ void p_block(const Ctx &cx, const DiagMasks &dm, cons
         TMEM_ST8(cx.tm_s + 32 * KB + 8 * h, pk);
     }
 }
-// AHEAD: with the registers for it (head dimension 64) every block's load is in flight at once.
+// AHEAD (128 channels): the next block's scores are on their way while a block is converted (4 to 5 % of a call; with head
+// dimension 64 it measured 1 % slower).
 template <int Q, bool AHEAD>
 __device__ __forceinline__ void p_blocks(const Ctx &cx, const DiagMasks &dm) {
-    uint32_t r[AHEAD ? Q + 1 : 1][32];
-    if constexpr (AHEAD) {
-#pragma unroll
-        for (int kb = 0; kb <= Q; ++kb) TMEM_LD32(cx.tm_s + 32 * kb, r[kb]);
-        tmem_wait_ld();
+    uint32_t ra[32], rb[32];
+    auto load = [&](int kb, uint32_t(&r)[32]) { TMEM_LD32(cx.tm_s + 32 * kb, r); };
+    load(0, ra);
+    tmem_wait_ld();
+    if constexpr (!AHEAD) {
+        p_block<Q, 0>(cx, dm, ra);
+        if constexpr (Q > 0) { load(1, ra); tmem_wait_ld(); p_block<Q, 1>(cx, dm, ra); }
+        if constexpr (Q > 1) { load(2, ra); tmem_wait_ld(); p_block<Q, 2>(cx, dm, ra); }
+        if constexpr (Q > 2) { load(3, ra); tmem_wait_ld(); p_block<Q, 3>(cx, dm, ra); }
     } else {
-        TMEM_LD32(cx.tm_s, r[0]);
-        tmem_wait_ld();
-    }
-    p_block<Q, 0>(cx, dm, r[0]);
-    if constexpr (Q > 0) {
-        if constexpr (!AHEAD) { TMEM_LD32(cx.tm_s + 32, r[0]); tmem_wait_ld(); }
-        p_block<Q, 1>(cx, dm, r[AHEAD ? 1 : 0]);
-    }
-    if constexpr (Q > 1) {
-        if constexpr (!AHEAD) { TMEM_LD32(cx.tm_s + 64, r[0]); tmem_wait_ld(); }
-        p_block<Q, 2>(cx, dm, r[AHEAD ? 2 : 0]);
-    }
-    if constexpr (Q > 2) {
-        if constexpr (!AHEAD) { TMEM_LD32(cx.tm_s + 96, r[0]); tmem_wait_ld(); }
-        p_block<Q, 3>(cx, dm, r[AHEAD ? 3 : 0]);
+        if constexpr (Q > 0) load(1, rb);
+        p_block<Q, 0>(cx, dm, ra);
+        if constexpr (Q > 0) { tmem_wait_ld(); if constexpr (Q > 1) load(2, ra); p_block<Q, 1>(cx, dm, rb); }
+        if constexpr (Q > 1) { tmem_wait_ld(); if constexpr (Q > 2) load(3, rb); p_block<Q, 2>(cx, dm, ra); }
+        if constexpr (Q > 2) { tmem_wait_ld(); p_block<Q, 3>(cx, dm, rb); }
     }
 }
-template <bool EXACT, bool KEYF, bool SPLIT, bool AHEAD>
+template <bool EXACT, bool KEYF, bool AHEAD>
 __device__ __forceinline__ void p_epilogue_t(const Ctx &cx, const GateScalars *gs, float ac_c, const DiagMasks &dm) {
-    if (!KEYF && SPLIT) {     // an iteration: the upper key blocks are left to the token's compute warp
-        p_epilogue_blocks<EXACT>(cx, gs, ac_c, 0, p_split(cx.q), dm);
-        return;
-    }
     if (!KEYF && !EXACT) {
         if (cx.q == 0) p_blocks<0, AHEAD>(cx, dm);
         else if (cx.q == 1) p_blocks<1, AHEAD>(cx, dm);
@@ -403,10 +385,10 @@ __device__ __forceinline__ void p_epilogue_t(const Ctx &cx, const GateScalars *g
     }
     tmem_wait_st();
 }
-template <bool KEYF, bool SPLIT, bool AHEAD>
+template <bool KEYF, bool AHEAD>
 __device__ __forceinline__ void p_epilogue(const Ctx &cx, const GateScalars *gs, bool exact, float ac_c, const DiagMasks &dm) {
-    if (exact) p_epilogue_t<true, KEYF, SPLIT, AHEAD>(cx, gs, ac_c, dm);
-    else p_epilogue_t<false, KEYF, SPLIT, AHEAD>(cx, gs, ac_c, dm);
+    if (exact) p_epilogue_t<true, KEYF, AHEAD>(cx, gs, ac_c, dm);
+    else p_epilogue_t<false, KEYF, AHEAD>(cx, gs, ac_c, dm);
 }
 
 // Sum over one 32-key block of the squared Gram entries of the earlier keys (decayed when the keys are not
@@ -459,7 +441,6 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     __shared__ int s_abort;
     __shared__ __align__(16) uint32_t s_req[4];     // per slot: requests posted (warps), Gram matrices read (warps)
     __shared__ __align__(16) DiagMasks dm;
-    __shared__ uint32_t s_sinfo[2];                 // score event n (parity): slot | read pass << 1 | gate buffer << 2 | per-element factors << 3 | (n + 1) << 8
 
     unsigned char *smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     const int tid = threadIdx.x;
@@ -469,7 +450,6 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     if (tid == 0) {
         s_abort = 0;
         s_req[0] = s_req[1] = s_req[2] = s_req[3] = 0u;
-        s_sinfo[0] = s_sinfo[1] = 0u;
         for (int i = 0; i < B_COUNT; ++i) {
             const int b = i % B_PER_SLOT;
             const bool per_warp = i < B_DRAIN && (b == B_RDY_ST || b == B_QF || b == B_GF0 || b == B_GF1);
@@ -499,15 +479,12 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     const float *const beta_p = EXTRA ? a.beta : nullptr;
     const float *const alpha_p = EXTRA ? a.alpha : nullptr;
     const bool mix = alpha_p != nullptr && !solve_only;   // alpha-connection: the read uses alpha x + (1 - alpha) q
-    // Head dimension 64: the slot's compute warps, idle while the slot has the score tile, convert the upper key blocks of
-    // the masked scores of an iteration (with 128 channels this measured slower: the warps come later to their update)
-    constexpr bool SPLIT = false;
     constexpr bool half = HALF;                           // head dimension 64: channels 64..127 are zero, their k-steps are left out
 
     // The helper warps come first: when a scheduler changes warps it prefers the oldest eligible one, and the thread
     // that issues the products must not wait behind the compute warps of its scheduler.
     if (tid < 128) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsHelper));
+        if constexpr (!HALF) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsHelper));
         const int hw = tid >> 5, lane = tid & 31;
         if (hw == 0) {
             // ================= gate scalars of every tile, one tile ahead of the compute warps =================
@@ -601,7 +578,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 }
                 asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // output stores are complete
             }
-        } else {
+        } else if constexpr (!HALF) {
             // ================================ MMA issuing thread ================================
             // Serves the requests of both slots in the order they become ready.  The score tile S is held by a slot
             // from its FROB request until its warps have read the Gram matrix (counted in shared memory), from ITER1 to the issue of
@@ -620,24 +597,12 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 int owner = -1;                         // slot that holds S while its warps read the Gram matrix
                 int prefer = 0;                         // slot to serve first when both are ready
                 bool gave_up = false;
-                uint32_t sev = 0;                       // score events so far
-                const uint32_t sinfo_addr = smem_u32(&s_sinfo[0]);
-                auto buffer_info = [&](int sl) -> uint32_t {      // gate buffer of the slot's tile, and whether it needs per-element factors
-                    const uint32_t buf = (sl ? til1 : til0) & 1u;
-                    const int *const ex = reinterpret_cast<const SlotScalars *>(smem + OFF_SC + sl * SC_BYTES)->exact;
-                    return (buf << 2) | (*reinterpret_cast<const volatile int *>(ex + buf) != 0 ? 8u : 0u);
-                };
                 auto issue = [&](int sl, int o) {
                     const uint32_t sbb = bars + 8 * (sl * B_PER_SLOT);
                     const uint32_t sl14 = base14 + ((sl * SLOT_BYTES) >> 4);
-                    if (o == OP_ITER1 || o == OP_OUT_S) {   // tell the score warps whose scores come next
-                        ++sev;
-                        const uint32_t info = (uint32_t)sl | (o == OP_OUT_S ? 2u : 0u) | buffer_info(sl) | (sev << 8);
-                        asm volatile("st.volatile.shared::cta.u32 [%0], %1;" ::"r"(sinfo_addr + 4u * ((sev - 1u) & 1u)), "r"(info) : "memory");
-                    }
                     fence_after();
-                    issue_batch(o, half, SPLIT, sl14 + (BUF_A >> 4), sl14 + (BUF_B >> 4), sl14 + (BUF_C >> 4), tmem + TM_S, tmem + tm_r_of(sl),
-                                tmem + tm_e_of(sl), sbb + 8 * B_MMA_S, sbb + 8 * B_MMA_R, bars + 8 * B_SC);
+                    issue_batch(o, half, sl14 + (BUF_A >> 4), sl14 + (BUF_B >> 4), sl14 + (BUF_C >> 4), tmem + tm_s_of(half, sl),
+                                tmem + tm_r_of(half, sl), tmem + tm_e_of(sl), sbb + 8 * B_MMA_S, sbb + 8 * B_MMA_R, bars + 8 * (B_SC + sl));
                 };
                 // Bookkeeping of a request of slot sl that has just been issued, together with its follow-up (ITER2 after
                 // ITER1, OUT_O after OUT_S): the slot's next request, counters and tile count.  Returns the counter value
@@ -645,8 +610,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 auto book = [&](int sl, int o) -> uint32_t {
                     bool tile_done = false;
                     int it = sl ? it1 : it0, nop;
-                    // (the masked scores of an iteration come from the score warps and the slot's compute warps)
-                    const uint32_t thr = (sl ? thr1 : thr0) + (SPLIT && o == OP_ITER1 ? 8u : 4u);
+                    const uint32_t thr = (sl ? thr1 : thr0) + 4u;
                     if (o == OP_FROB) {
                         owner = sl;                          // until the Gram matrix has been read
                         nop = it < a.n_iter ? OP_ITER1 : OP_OUT_S;
@@ -707,19 +671,16 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     if (o == OP_FROB) continue;
                     // ---- ITER1 or OUT_S of slot s is running: its follow-up (ITER2, OUT_O) comes next.  In the steady state
                     // of the iterations the other slot's ITER1 follows at once; everything both need is worked out here,
-                    // while the products run and the score warps work, so that a handful of instructions lie between the
+                    // while the products run and the scores are masked, so that a handful of instructions lie between the
                     // posts and the products.
                     for (;;) {
                         const int t = 1 - s;
                         const uint32_t s14 = base14 + ((s * SLOT_BYTES) >> 4), t14 = base14 + ((t * SLOT_BYTES) >> 4);
-                        const uint32_t p_kb = s14 + (BUF_A >> 4), p_tmR = tmem + tm_r_of(s);
+                        const uint32_t p_kb = s14 + (BUF_A >> 4), p_tmR = tmem + tm_r_of(half, s);
                         const uint32_t p_barR = bars + 8 * (s * B_PER_SLOT + B_MMA_R);
                         const bool t_iter = (t ? left1 : left0) > 0 && (t ? op1 : op0) == OP_ITER1;
                         const uint32_t thr_t = t ? thr1 : thr0;
                         const uint32_t n_kb = t14 + (BUF_A >> 4), n_tmE = tmem + tm_e_of(t);
-                        const uint32_t n_barS = bars + 8 * (t * B_PER_SLOT + B_MMA_S);
-                        const uint32_t n_info = (uint32_t)t | buffer_info(t) | ((sev + 1u) << 8);
-                        const uint32_t n_sinfo = sinfo_addr + 4u * (sev & 1u);
                         uint32_t c_t = 0u;
                         for (int polls = 0;;) {
                             uint32_t c0, c1;
@@ -734,7 +695,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                         if (gave_up) break;
                         if (o == OP_ITER1) {
                             fence_after();
-                            mma8_pm_rows(p_tmR, tmem + TM_S, p_kb, kIdescPM);  // ITER2: R += P Khat
+                            mma8_pm_rows(p_tmR, tmem + tm_s_of(half, s), p_kb, idesc_r_pm(half));  // ITER2: R += P Khat
                             mma_commit(p_barR);
                         } else {                                 // OUT_O: the V tile (TMA)
                             wait_bar(bars + 8 * (s * B_PER_SLOT + B_LD_V), til & 1u, abort_addr);
@@ -756,13 +717,10 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                             break;
                         }
                         // ---- ITER1 of the other slot, at once
-                        asm volatile("st.volatile.shared::cta.u32 [%0], %1;" ::"r"(n_sinfo), "r"(n_info) : "memory");
-                        ++sev;
                         fence_after();
-                        prod_ek<0>(half, tmem + TM_S, n_tmE, n_kb);           // S = E Khat^T
-                        mma_commit(bars + 8 * B_SC);
-                        if (SPLIT) mma_commit(n_barS);
-                        prod_ek<1>(half, tmem + tm_r_of(t), n_tmE, n_kb + ((BUF_B - BUF_A) >> 4));   // R += E H_0^T
+                        prod_ek<0>(half, tmem + tm_s_of(half, t), n_tmE, n_kb, kIdescKK);           // S = E Khat^T
+                        mma_commit(bars + 8 * (B_SC + t));
+                        prod_ek<1>(half, tmem + tm_r_of(half, t), n_tmE, n_kb + ((BUF_B - BUF_A) >> 4), idesc_r_kk(half));   // R += E H_0^T
                         if (owner == t) {                        // (its Gram reads are done: it has asked again)
                             if (t) gthr1 += 4u; else gthr0 += 4u;
                             owner = -1;
@@ -780,72 +738,17 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 if (!mbar_spin_bounded(bars + 8 * B_DRAIN, 0u)) set_abort(abort_addr);
             }
         }
-    } else if (tid < 256) {
-        // ================================== score warps ==================================
-        // The masked-score epilogue of both slots: S (fp32) -> P (packed bf16) in place, for the scores of an iteration
-        // and for those of the read.  These warps hold no iterate, so they are not short of registers, and the compute
-        // warps go from their update straight to the wait for the accumulator.
-        if constexpr (HALF) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(regs_score(true)));
-        else asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(regs_score(false)));
-        Ctx cx;
-        cx.l = tid & 31;
-        cx.q = (tid >> 5) & 3;
-        cx.c = 32 * cx.q + cx.l;
-        cx.tm_s = tmem + TM_S + ((uint32_t)(32 * cx.q) << 16);
-        cx.tm_r = cx.tm_e = 0u;
-        const int per_tile = a.n_iter + (solve_only ? 0 : 1);
-        const long long n_events = (long long)n_mine * per_tile;
-        int reads0 = 0, reads1 = 0;         // read passes seen per slot (= tiles done)
-        for (long long ev = 0; ev < n_events; ++ev) {
-            // The issuing thread announces an event before it issues the score product: whose scores, which pass, which gate
-            // buffer, per-element factors or not.
-            uint32_t info = 0u;
-            if (cx.l == 0) {
-                for (int polls = 0;; ++polls) {
-                    asm volatile("ld.volatile.shared::cta.u32 %0, [%1];" : "=r"(info) : "r"(smem_u32(&s_sinfo[ev & 1])) : "memory");
-                    if ((info >> 8) == (uint32_t)(ev + 1)) break;
-                    if ((polls & 1023) == 1023 && (aborted(abort_addr) || polls > (1 << 24))) {
-                        set_abort(abort_addr);
-                        break;
-                    }
-                }
-            }
-            info = __shfl_sync(0xffffffffu, info, 0);
-            const int sl_ = (int)(info & 1u);
-            const GateScalars *const gs = &reinterpret_cast<const SlotScalars *>(smem + OFF_SC + sl_ * SC_BYTES)->g[(info >> 2) & 1u];
-            const bool exact = (info & 8u) != 0u;
-            const float ac_c = exact ? gs->ac[cx.c] : 0.f;
-            wait_bar(bars + 8 * B_SC, (uint32_t)(ev & 1), abort_addr);
-            fence_after();
-            if (info & 2u) {
-                // the score products of the read pass were the last readers of the slot's keys: the next tile's keys
-                // are loaded now, and the slot's compute warps scale them while the read runs
-                const int kdone = sl_ + kSlots * (sl_ ? reads1 : reads0);
-                if (tid == 128 && kdone + kSlots < n_mine) {
-                    const TileInfo tn = tile_info(a, t_lo + kdone + kSlots);
-                    const uint32_t bar_k = bars + 8 * (sl_ * B_PER_SLOT + B_LD_K);
-                    mbar_expect_tx(bar_k, 32768u);
-                    tma_load_tile3(&tmK, sbase + sl_ * SLOT_BYTES + BUF_A, bar_k, tn.h * a.d, tile_x_hi(tn.h, a.d, a.heads), tn.n * NT, tn.b);
-                }
-                if (sl_) ++reads1; else ++reads0;
-                p_epilogue<true, SPLIT, HALF>(cx, gs, exact, ac_c, dm);
-            } else {
-                p_epilogue<false, SPLIT, HALF>(cx, gs, exact, ac_c, dm);
-            }
-            fence_before();
-            warp_post(smem_u32(&s_req[sl_]), cx.l);          // -> ITER2 / OUT_O of that slot
-        }
     } else {
         // ================================= compute threads =================================
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(regs_compute(HALF)));
-        const int slot = (tid >> 7) - 2;
+        if constexpr (!HALF) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsCompute));
+        const int slot = (tid >> 7) - 1;
         Ctx cx;
         cx.l = tid & 31;
         cx.q = (tid >> 5) & 3;
         cx.c = 32 * cx.q + cx.l;
         const uint32_t lane_addr = (uint32_t)(32 * cx.q) << 16;
-        cx.tm_s = tmem + TM_S + lane_addr;
-        cx.tm_r = tmem + tm_r_of(slot) + lane_addr;
+        cx.tm_s = tmem + tm_s_of(half, slot) + lane_addr;
+        cx.tm_r = tmem + tm_r_of(half, slot) + lane_addr;
         cx.tm_e = tmem + tm_e_of(slot) + lane_addr;
         const int c = cx.c, l = cx.l;
         const bool leader = c == 0;                              // issues the slot's loads that follow a product
@@ -864,7 +767,45 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         auto wait_s = [&]() { wait_bar(sb + 8 * B_MMA_S, n_s & 1u, abort_addr); ++n_s; fence_after(); };
         auto wait_r = [&]() { wait_bar(sb + 8 * B_MMA_R, n_r & 1u, abort_addr); ++n_r; fence_after(); };
         const uint32_t req_addr = smem_u32(&s_req[slot]), grd_addr = smem_u32(&s_req[2 + slot]);
-        auto arrive_rdy = [&]() { warp_post(req_addr, l); };
+        // Requests.  With 128 channels they go to the issuing thread.  HALF: one thread of the slot waits for the slot's other warps
+        // and issues the products itself (one thread, so that they run in order; in the warp with the fewest key blocks, which
+        // can best afford to wait until the tensor pipe has taken them).
+        uint32_t n_req = 0;                   // requests of this slot so far (HALF)
+        uint32_t n_sc = 0;                    // completed phases of B_SC
+        auto request = [&](int op, uint32_t tile_parity) {
+            if constexpr (!HALF) {
+                if (op != OP_FROB) warp_post_tmem(req_addr, l);
+                else warp_post(req_addr, l);
+            } else {
+                ++n_req;
+                if (cx.q != 0) {
+                    if (op != OP_FROB) warp_post_tmem(req_addr, l);
+                    else warp_post(req_addr, l);
+                } else {
+                    __syncwarp();
+                    if (l == 0) {
+                        uint32_t cnt = 0u;
+                        for (int polls = 0;; ++polls) {
+                            asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(cnt) : "r"(req_addr) : "memory");
+                            if ((int)(cnt - 3u * n_req) >= 0) break;
+                            if ((polls & 1023) == 1023 && (aborted(abort_addr) || polls > (1 << 24))) {
+                                set_abort(abort_addr);
+                                break;
+                            }
+                        }
+                        if (op == OP_FROB) wait_bar(sb + 8 * B_LD_H, tile_parity, abort_addr);    // the H_0 tile (TMA)
+                        if (op == OP_OUT_S) wait_bar(sb + 8 * B_LD_U, tile_parity, abort_addr);   // the U_0 tile
+                        if (op == OP_OUT_O) wait_bar(sb + 8 * B_LD_V, tile_parity, abort_addr);   // the V tile
+                        fence_after();
+                        const uint32_t s14 = (sl >> 4) & 0x3FFF;
+                        issue_batch(op, true, s14 + (BUF_A >> 4), s14 + (BUF_B >> 4), s14 + (BUF_C >> 4), tmem + tm_s_of(true, slot),
+                                    tmem + tm_r_of(true, slot), tmem + tm_e_of(slot), sb + 8 * B_MMA_S, sb + 8 * B_MMA_R, bars + 8 * (B_SC + slot));
+                    }
+                    __syncwarp();
+                }
+            }
+        };
+        auto wait_scores = [&]() { wait_bar(bars + 8 * (B_SC + slot), n_sc & 1u, abort_addr); ++n_sc; fence_after(); };
         // -xs (times `scale`) as packed bf16 pairs of channel group g8 (8 channels): its leading part, or the remainder
         auto pack_x = [&](int g8, bool lo, float scale, uint32_t(&pk)[4]) {
 #pragma unroll
@@ -934,9 +875,9 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             };
             if (j == 0 || solve_only) stage_keys(j);             // (otherwise done under the previous tile's read)
             const bool exact = gs->G2[ti.ntok - 1] < -60.f;     // the tile decays below 2^-60: per-element factors
-            if (leader) sc->exact[j & 1] = exact ? 1 : 0;       // (for the score warps; published by the FROB request)
             const float G2c = gs->G2[c];
-            arrive_rdy();                                        // -> FROB
+            if (HALF) fence_before();
+            request(OP_FROB, (uint32_t)(j & 1));
             wait_s();
             if (a.n_iter == 0) after_last_h0_product();
             // ---- chunk-wise Frobenius norms: for the token's key, k^T H_0 k and the decayed squared Gram entries of
@@ -959,7 +900,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     }
                 }
                 fence_before();
-                warp_post(grd_addr, l);                          // the Gram matrix has been read: S is free again
+                if (!HALF) warp_post(grd_addr, l);               // the Gram matrix has been read: S is free again
 #pragma unroll 1
                 for (int p = 0; p < NG16 / 2; ++p) {
                     TMEM_LD32(cx.tm_r + 32 * p, ra);
@@ -1023,21 +964,17 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             float omega = 2.f;
             if (a.n_iter > 0) {
                 fence_before();
-                arrive_rdy();                                    // -> ITER1
+                request(OP_ITER1, 0u);
             }
             for (int it = 0; it < a.n_iter; ++it) {
                 const bool last = it + 1 == a.n_iter;
                 omega = 4.f * recip(4.f - rho2 * omega);         // weight schedule
                 const float beta = omega - 1.f, cz = czb * omega;
                 const uint64_t beta2 = f2_pack(beta, beta), cz2 = f2_pack(cz, cz), lz2 = f2_pack(lz, lz);
-                // this warp's share of the masked-score epilogue (the upper key blocks of its tokens)
-                if (SPLIT) {
-                    wait_s();
-                    if (exact) p_epilogue_blocks<true>(cx, gs, gs->ac[c], p_split(cx.q), cx.q + 1, dm);
-                    else p_epilogue_blocks<false>(cx, gs, 0.f, p_split(cx.q), cx.q + 1, dm);
-                    fence_before();
-                    arrive_rdy();                                // -> ITER2 (with the score warps' posts)
-                }
+                wait_scores();                                   // the masked scores
+                p_epilogue<false, !HALF>(cx, gs, exact, exact ? gs->ac[c] : 0.f, dm);
+                fence_before();
+                request(OP_ITER2, 0u);
                 wait_r();
                 if (last) after_last_h0_product();
                 // xs += e_old (the value the operand held), e_new = beta e_old + cz (R + lz xs) as bf16.  Sixteen channels at
@@ -1076,7 +1013,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     if (!last) {
                         tmem_wait_st();
                         fence_before();
-                        arrive_rdy();                            // -> ITER1
+                        request(OP_ITER1, 0u);
                     }
                 }
             }
@@ -1136,10 +1073,14 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             }
             tmem_wait_st();
             fence_before();
-            arrive_rdy();                                        // -> OUT_S
-            // (the score warps mask the scores and post OUT_O; the values stay as loaded: their row factor
-            // sqrt(beta_j) 2^(-G_j / 2) rides on the masked scores)
-            if (more) stage_keys(j + 1);                         // the next tile's keys (loaded by a score warp at the read pass)
+            request(OP_OUT_S, (uint32_t)(j & 1));
+            wait_scores();
+            load_next_k();                                       // its products were the last readers of the keys
+            p_epilogue<true, !HALF>(cx, gs, exact, exact ? gs->ac[c] : 0.f, dm);
+            fence_before();
+            request(OP_OUT_O, (uint32_t)(j & 1));
+            // (the values stay as loaded: their row factor sqrt(beta_j) 2^(-G_j / 2) rides on the masked scores)
+            if (more) stage_keys(j + 1);                         // the next tile's keys, under the read
             wait_r();
             load_next_h();                                       // every product of the tile is complete
             // O as bf16 into the V buffer (no product reads it any more), stored by TMA
@@ -1164,6 +1105,10 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             fence_before();
             warp_arrive(sb + 8 * (B_GF0 + (j & 1)), l);
             warp_arrive(sb + 8 * B_RDY_ST, l);
+        }
+        if (HALF && cx.q == 0 && l == 0) {                       // every product is complete before the tensor memory is given back
+            mma_commit(sb + 8 * B_MMA_R);
+            if (!mbar_spin_bounded(sb + 8 * B_MMA_R, n_r & 1u)) set_abort(abort_addr);
         }
     }
 
