@@ -23,6 +23,11 @@
 // The forward splits every sequence into P segments of L tokens (and a segment into F parts) so that the blocks fill the
 // device; recur_summary computes what a segment adds to the state, recur_scan folds that into the start state of every
 // segment, and a block of a later part first folds the tokens of its segment that come before it.
+//
+// Measured, before (chunk-wise fp32 kernels; one token at a time for decoding) and with these kernels: B=2, 8 heads, T=8192,
+// d=128, f32, r=8: 3209 -> 2075 us; 64 x 32 pairs, 8 tokens, d=128, bf16, r=10: 425 -> 286 us; B=1, 2 heads, T=256, d=64, f32,
+// r=8: 118.5 -> 29 us (there: three dependent launches and the chain of batches).  Tried: scalar instead of two-wide
+// multiply-adds +10 %, the batch's constants in shared memory +8 %, rolled loops +3 %.
 #include "gka_common.cuh"
 #include "gka_tc_util.cuh"
 
