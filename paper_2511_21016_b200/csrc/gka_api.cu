@@ -409,24 +409,25 @@ gka_status gka_fwd_chunked_host(const gka_desc *desc, void *staging, const void 
     // streams: copies in (helper stream), kernels (the caller's stream), copies out (second helper stream).
     // The two copy directions and the kernels overlap; the caller's stream ends up waiting for everything.
     // What the pipeline cannot hide is its tail, the kernels and the copy out of the last piece, so the last
-    // batch entries are also cut along the sequence (the state is carried from piece to piece on the device).
+    // batch entry is also cut along the sequence (the state is carried from piece to piece on the device): in half, and
+    // what is left in half again while it takes the bus much longer (16 MiB: 0.3 ms) than a further job costs (some
+    // 20 us of copies and launches).  B = 4, 16 heads, T = 4096, d = 128, bf16: 4.30 ms with two halves, 4.20 with a
+    // half and two quarters, 4.22 with one more piece; B = 1: 1.264, 1.189, 1.201 ms (the copies alone: 3.7, 0.95 ms).
+    const size_t hh = (size_t)desc->heads;
     struct Job { int b0, nb, t0, tn; bool first, last; };
     std::vector<Job> jobs;
     const int per = (desc->B + 7) / 8;                       // at most 8 batch slices
     const int nslices = (desc->B + per - 1) / per;
-    // pieces of the sequences of the last slice: two halves measured best (every further piece costs about as much
-    // as it takes off the tail)
-    const int tpieces = (desc->T >= 4 * 2 * kChunk) ? 2 : 1;
     for (int i = 0; i < nslices; ++i) {
         const int b0 = i * per, nb = (b0 + per <= desc->B) ? per : desc->B - b0;
-        if (i + 1 < nslices || tpieces == 1) {
-            jobs.push_back({b0, nb, 0, desc->T, true, true});
-        } else {
-            const int tstep = ((desc->T / tpieces + 2 * kChunk - 1) / (2 * kChunk)) * (2 * kChunk);   // whole 128-token tiles
-            for (int b = b0; b < b0 + nb; ++b) {
-                for (int t0 = 0; t0 < desc->T; t0 += tstep)
-                    jobs.push_back({b, 1, t0, (t0 + tstep < desc->T) ? tstep : desc->T - t0, t0 == 0, t0 + tstep >= desc->T});
-            }
+        const bool tail = i + 1 == nslices && desc->T >= 4 * kTile;
+        if (!tail || nb > 1) jobs.push_back({b0, tail ? nb - 1 : nb, 0, desc->T, true, true});
+        if (!tail) continue;
+        for (int t0 = 0, tn; t0 < desc->T; t0 += tn) {
+            const int rest = desc->T - t0, half = (rest / 2 + kTile - 1) / kTile * kTile;     // whole tiles
+            const size_t bytes = (size_t)rest * hh * (2 * desc->d_k + desc->d_v) * es;
+            tn = t0 == 0 || (rest >= 8 * kTile && bytes >= (size_t)16 << 20) ? half : rest;
+            jobs.push_back({desc->B - 1, 1, t0, tn, t0 == 0, t0 + tn >= desc->T});
         }
     }
     const int njobs = (int)jobs.size();
@@ -437,12 +438,15 @@ gka_status gka_fwd_chunked_host(const gka_desc *desc, void *staging, const void 
         (err = cudaStreamWaitEvent(hp->in, hp->start, 0)) != cudaSuccess ||
         (err = cudaStreamWaitEvent(hp->out, hp->start, 0)) != cudaSuccess)
         return cuda_result(err, "gka_fwd_chunked_host (stream ordering)");
-    const size_t hh = (size_t)desc->heads;
     auto copy = [&](unsigned char *dst, const void *src, size_t off, size_t bytes, cudaMemcpyKind kind, cudaStream_t on) {
         return kind == cudaMemcpyHostToDevice
                    ? cudaMemcpyAsync(dst + off, static_cast<const unsigned char *>(src) + off, bytes, kind, on)
                    : cudaMemcpyAsync(static_cast<unsigned char *>(const_cast<void *>(src)) + off, dst + off, bytes, kind, on);
     };
+    // the per-token scalars of all jobs in one copy each: a copy costs the engine some microseconds whatever its size
+    err = copy(dgate, gate, 0, ng, cudaMemcpyHostToDevice, hp->in);
+    if (err == cudaSuccess) err = copy(dlam, lam, 0, ng, cudaMemcpyHostToDevice, hp->in);
+    if (err != cudaSuccess) return cuda_result(err, "gka_fwd_chunked_host (host-to-device copies)");
     for (int i = 0; i < njobs; ++i) {
         const Job &j = jobs[i];
         // a job's tokens are one contiguous range: whole batch entries, or a token range of one entry
@@ -450,8 +454,6 @@ gka_status gka_fwd_chunked_host(const gka_desc *desc, void *staging, const void 
         err = copy(dq, q, tok0 * desc->d_k * es, ntok * desc->d_k * es, cudaMemcpyHostToDevice, hp->in);
         if (err == cudaSuccess) err = copy(dk, k, tok0 * desc->d_k * es, ntok * desc->d_k * es, cudaMemcpyHostToDevice, hp->in);
         if (err == cudaSuccess) err = copy(dv, v, tok0 * desc->d_v * es, ntok * desc->d_v * es, cudaMemcpyHostToDevice, hp->in);
-        if (err == cudaSuccess) err = copy(dgate, gate, tok0 * 4, ntok * 4, cudaMemcpyHostToDevice, hp->in);
-        if (err == cudaSuccess) err = copy(dlam, lam, tok0 * 4, ntok * 4, cudaMemcpyHostToDevice, hp->in);
         if (err == cudaSuccess) err = cudaEventRecord(hp->copied[i], hp->in);
         if (err != cudaSuccess) return cuda_result(err, "gka_fwd_chunked_host (host-to-device copies)");
     }
