@@ -234,7 +234,7 @@ static gka_status fwd_impl(const gka_desc *desc, const void *q, const void *k, c
     a.state_split = 0;
     a.after_summary = 0;
     const bool tensor_path = wants_tensor_path(desc) && fwd_tc_available();
-    a.tile_hh = nullptr;
+    a.tile_hh = a.tile_hh2 = nullptr;
     a.tile_hu = nullptr;
     if (tensor_path) {
         a.plan.set(desc->B * desc->heads, tiles_of(desc->T), G, false);

@@ -223,11 +223,12 @@ struct FwdArgs {
     int sms;               // of the current device
     int after_summary;     // tensor path: the main kernel is launched as a programmatic dependent of the summary kernel
     int start_from_scan;   // tensor path: start states were materialised by the scan kernel (long chains of summaries)
-    int state_split;       // tensor path, no sequence cut: two blocks per work item in the state kernel, one for H, one for U
+    int state_split;       // tensor path, no sequence cut: 2^state_split blocks per work item in the state kernel
     int solve_only;        // write the solve x_t = CH(H_t + lambda_t I, q_t, r) itself instead of U_t x_t (v unused)
     WorkPlan plan;
     Workspace ws;
     float *tile_hh;        // tensor path: ||H_0||_F^2 of every 128-token tile
+    float *tile_hh2;       // its second term, where two blocks keep H (or nullptr)
     unsigned char *tile_hu; // tensor path: bf16 H_0, U_0 of every 128-token tile
     cudaEvent_t ev_start, ev_stop;   // optional, recorded around the main kernel (host side only)
 };

@@ -106,6 +106,12 @@ __device__ __forceinline__ void tma_load_tile3(const CUtensorMap *map, uint32_t 
                 "r"(dst + 16384 * hf), "l"(reinterpret_cast<uint64_t>(map)), "r"(hf ? x_hi : x), "r"(y), "r"(z), "r"(bar)
             : "memory");
 }
+__device__ __forceinline__ void tma_load_box3(const CUtensorMap *map, uint32_t dst, uint32_t bar, int x, int y, int z) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::
+            "r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar)
+        : "memory");
+}
 // column of the second box of head h's tile: the head's upper 64 channels, or past the tensor for head dimension 64
 __host__ __device__ __forceinline__ int tile_x_hi(int h, int d, int heads) { return d == 128 ? h * 128 + 64 : heads * d; }
 __device__ __forceinline__ void tma_load_tile2(const CUtensorMap *map, uint32_t dst, uint32_t bar, int y) {

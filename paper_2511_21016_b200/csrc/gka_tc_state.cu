@@ -44,10 +44,11 @@ constexpr uint32_t KV_SMEM = NS * STAGE + 1024;          // + slack for the 1024
 constexpr uint32_t ST_SMEM = KV_SMEM;
 
 // rows of the K and V tiles of a stage times f[j]
-__device__ __forceinline__ void scale_kv(unsigned char *stage, const float *f, int t, bool with_v = true) {
+// (boxes of 64 channels: K 0 and 1, V 2 and 3; those whose bit is set in `boxes`)
+__device__ __forceinline__ void scale_kv(unsigned char *stage, const float *f, int t, uint32_t boxes = 15u) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-        if (i >= 4 && !with_v) break;              // (the K tile is the first half of the stage)
+        if (!(boxes >> (i >> 1) & 1u)) continue;
         const int qi = t + CT * i;                 // 16-byte group index in the 64 KB stage
         const float fj = f[(qi & 1023) >> 3];      // row of this group (K and V tiles alike)
         uint4 v = *reinterpret_cast<const uint4 *>(stage + qi * 16);
@@ -243,15 +244,15 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 // increments dH = K~^T K~, dU = V~^T K~ into one of two TMEM buffers, one tile ahead of their use; per tile a thread
 // stores the bf16 copies of its part of the tile-initial H_0, U_0 (and adds up ||H_0||_F^2), then advances its
 // masters: H <- zeta H + dH, U <- zeta U + dU.  The warp that issues the products also turns the gates into the row
-// factors and the tile's decay, two tiles ahead, so that the compute warps meet no scan.  SPLIT: two blocks per work
-// item, one keeps H (and loads only the keys), one keeps U.
+// factors and the tile's decay, two tiles ahead, so that the compute warps meet no scan.  PARTS: blocks per work
+// item; with two, one keeps H (and loads only the keys), one keeps U; with four, each keeps 64 columns of one of them.
 // ------------------------------------------------------------------------------------------------------------
 // TB_STG0 + stage: one barrier per stage, like the loads.  (With a single barrier the compute warps could complete two
 // phases, tiles m + 1 and m + 2, while the TMA thread was still held up behind tile m's store; the phase parity it
 // then polled looked incomplete, and the compute warps in turn waited for the load that only this thread issues.)
 enum { TB_KV0 = 0, TB_D0 = NS, TB_D1, TB_STG0, TB_COUNT = TB_STG0 + NS };
 
-template <bool SPLIT>
+template <int PARTS>
 __global__ void __launch_bounds__(kThreadsStateK, 1)
 fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                     const __grid_constant__ CUtensorMap tmS, FwdArgs a) {
@@ -286,10 +287,13 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     const uint32_t tmem = s_tmem_base;
     const WorkPlan &P = a.plan;
     // With no sequence cut and few work items the masters are split: two blocks per item, one advances H (and needs
-    // only the keys), one U.  Each handles the masters w_lo <= which < w_hi.
-    const int item = SPLIT ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
-    const int w_lo = SPLIT ? (int)(blockIdx.x & 1) : 0, w_hi = SPLIT ? w_lo + 1 : 2;
+    // only the keys), one U; four blocks: 64 columns each of H and U.  A block handles the masters w_lo <= which < w_hi.
+    const int item = (int)(blockIdx.x / PARTS);
+    const int w_lo = PARTS == 4 ? (int)(blockIdx.x >> 1 & 1) : PARTS == 2 ? (int)(blockIdx.x & 1) : 0, w_hi = PARTS > 1 ? w_lo + 1 : 2;
     const bool do_h = w_lo == 0, do_u = w_hi == 2;
+    const int half = PARTS == 4 ? (int)(blockIdx.x & 1) : 0;             // columns 64 half .. of the masters
+    constexpr int CW = PARTS == 4 ? 16 : 32;                             // columns of a thread
+    const uint32_t boxes = PARTS < 4 ? (do_u ? 15u : 3u) : (do_u ? 12u + (1u << half) : 3u);     // of K and V: loaded and scaled
     const long long f_lo = P.lo(item), f_hi = P.lo(item + 1);
     const int n_mine = (int)(f_hi - f_lo);
     const uint32_t base14 = (sb >> 4) & 0x3FFF;
@@ -320,6 +324,12 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             auto issue_tma = [&](int m) {
                 const Pos p = pos_of(m);
                 const uint32_t dst = sb + (uint32_t)(m % NS) * STAGE, bar = bars + 8 * (TB_KV0 + m % NS);
+                if (PARTS == 4 && do_u) {                // V and the keys' own 64 channels
+                    mbar_expect_tx(bar, 49152u);
+                    tma_load_box3(&tmK, dst + 16384 * half, bar, p.h * a.d + 64 * half, p.n * NT, p.b);
+                    tma_load_tile3(&tmV, dst + 32768, bar, p.h * a.d, tile_x_hi(p.h, a.d, a.heads), p.n * NT, p.b);
+                    return;
+                }
                 mbar_expect_tx(bar, do_u ? 65536u : 32768u);
                 tma_load_tile3(&tmK, dst, bar, p.h * a.d, tile_x_hi(p.h, a.d, a.heads), p.n * NT, p.b);
                 if (do_u) tma_load_tile3(&tmV, dst + 32768, bar, p.h * a.d, tile_x_hi(p.h, a.d, a.heads), p.n * NT, p.b);
@@ -331,7 +341,7 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 wait(TB_STG0 + m % NS, (uint32_t)((m / NS) & 1));
                 const uint32_t src = sb + (uint32_t)(m % NS) * STAGE;
                 for (int which = w_lo; which < w_hi; ++which)
-                    for (int hf = 0; hf < 2; ++hf)
+                    for (int hf = half; hf < (PARTS == 4 ? half + 1 : 2); ++hf)
                         asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::
                                          "l"(reinterpret_cast<uint64_t>(&tmS)), "r"(64 * hf), "r"((int)((f_lo + m) * 256 + 128 * which)),
                                      "r"(src + 32768 * which + 16384 * hf)
@@ -404,8 +414,10 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 fence_after();
                 const uint32_t kb = base14 + (uint32_t)(m % NS) * (STAGE >> 4), vb = kb + (32768u >> 4);
                 const uint32_t tm_d = tmem + 256 * (m & 1);
-                if (do_h) mma8_mm<0>(tm_d, kb, kb, kIdescMM);              // dH = K~^T K~
-                if (do_u) mma8_mm<0>(tm_d + 128, vb, kb, kIdescMM);        // dU = V~^T K~
+                constexpr uint32_t idesc = PARTS == 4 ? make_idesc(128, 64, 1, 1) : kIdescMM;
+                const uint32_t bb = kb + (16384u >> 4) * half;
+                if (do_h) mma8_mm<0>(tm_d, kb, bb, idesc);                 // dH = K~^T K~
+                if (do_u) mma8_mm<0>(tm_d + 128, vb, bb, idesc);           // dU = V~^T K~
                 mma_commit(bars + 8 * (TB_D0 + (m & 1)));
             }
             __syncwarp();
@@ -416,9 +428,10 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         }
     } else if (n_mine > 0) {
         // ================================= compute threads =================================
-        const int q = (t >> 5) & 3, cq = t >> 7, c = 32 * q + l;
+        const int q = (t >> 5) & 3, cq = t >> 7, c = 32 * q + l, col0 = 64 * half + CW * cq;     // row, first column
         const uint32_t lane_addr = (uint32_t)(32 * q) << 16;
         const size_t st = state_floats(D, D);
+        float *const hh_out = half ? a.tile_hh2 : a.tile_hh;
         // first item of the chain of summaries behind this block's start state
         int chain_j0 = item;
         if (P.cut_in(item)) {
@@ -429,14 +442,14 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         // Tile m: rows scaled in place by the row factors (prepared by the issuing warp), products posted.
         auto prepare = [&](int m) {
             wait(TB_KV0 + m % NS, (uint32_t)((m / NS) & 1));
-            scale_kv(smem + (size_t)(m % NS) * STAGE, s_w[m % 3], t, do_u);
+            scale_kv(smem + (size_t)(m % NS) * STAGE, s_w[m % 3], t, boxes);
             fence_async_smem();
             fence_before();
             if (t == 0) *reinterpret_cast<volatile int *>(&s_req) = m;
             asm volatile("bar.sync 3, 544;" ::: "memory");       // hand the tile to the issuing warp
         };
 
-        float mH[32], mU[32];
+        float mH[CW], mU[CW];
         asm volatile("bar.sync 3, 544;" ::: "memory");           // the factors of the first two tiles are published
         prepare(0);
         // summaries and start states are read after this point only
@@ -453,19 +466,19 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 const float *s0 = (chained && a.start_from_scan) ? a.ws.start + (size_t)item * st
                                   : (a.state_in ? a.state_in + (size_t)p.seq * st : nullptr);
                 const int j0 = (chained && !a.start_from_scan) ? chain_j0 : 0, j1 = (chained && !a.start_from_scan) ? item : 0;
-                const size_t e = (size_t)c * D + 32 * cq;
+                const size_t e = (size_t)c * D + col0;
                 // the caller's state has head dimension a.d (rows and columns from a.d on are zero on chip); the scan
                 // kernel's start states are in the on-chip layout
                 const bool ext = s0 != nullptr && !(chained && a.start_from_scan);
-                const float *const s0e = ext ? a.state_in + (size_t)p.seq * 2 * a.d * a.d + (size_t)c * a.d + 32 * cq : nullptr;
-                const bool in_ext = c < a.d && 32 * cq < a.d;
+                const float *const s0e = ext ? a.state_in + (size_t)p.seq * 2 * a.d * a.d + (size_t)c * a.d + col0 : nullptr;
+                const bool in_ext = c < a.d && col0 < a.d;
 #pragma unroll
                 for (int which = 0; which < 2; ++which) {
                     if (which < w_lo || which >= w_hi) continue;
-                    float(&mm)[32] = which ? mU : mH;
+                    float(&mm)[CW] = which ? mU : mH;
                     const size_t eo = e + which * (size_t)D * D;
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
+                    for (int i = 0; i < CW / 4; ++i) {
                         const float4 v4 = ext ? (in_ext ? *reinterpret_cast<const float4 *>(s0e + which * (size_t)a.d * a.d + 4 * i)
                                                         : make_float4(0.f, 0.f, 0.f, 0.f))
                                           : (s0 ? *reinterpret_cast<const float4 *>(s0 + eo + 4 * i) : make_float4(0.f, 0.f, 0.f, 0.f));
@@ -475,7 +488,7 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                         // summaries come from the kernel this one may overlap with as its programmatic dependent: ordinary loads
                         const float dj = *reinterpret_cast<const volatile float *>(a.ws.decay + j);
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) {
+                        for (int i = 0; i < CW / 4; ++i) {
                             const float4 dd = *(reinterpret_cast<const float4 *>(a.ws.delta + (size_t)j * st + eo) + i);
                             mm[4 * i + 0] = fmaf(dj, mm[4 * i + 0], dd.x);
                             mm[4 * i + 1] = fmaf(dj, mm[4 * i + 1], dd.y);
@@ -494,10 +507,10 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 #pragma unroll
             for (int which = 0; which < 2; ++which) {
                 if (which < w_lo || which >= w_hi) continue;
-                float(&mm)[32] = which ? mU : mH;
+                float(&mm)[CW] = which ? mU : mH;
                 float hs = 0.f;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
+                for (int i = 0; i < CW / 8; ++i) {
                     uint32_t pk[4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
@@ -505,7 +518,7 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                         if (which == 0) hs = fmaf(v0, v0, fmaf(v1, v1, hs));
                         pk[u] = pack_bf16(v0, v1);
                     }
-                    *reinterpret_cast<uint4 *>(stg + 32768 * which + tile_off(c, 4 * cq + i)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                    *reinterpret_cast<uint4 *>(stg + 32768 * which + tile_off(c, col0 / 8 + i)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
                 }
                 if (which == 0) {
 #pragma unroll
@@ -519,9 +532,9 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 }
                 // advance the master: zeta m + increment
 #pragma unroll
-                for (int piece = 0; piece < 2; ++piece) {
+                for (int piece = 0; piece < CW / 16; ++piece) {
                     uint32_t r[16];
-                    TMEM_LD16(tmem + 256 * (m & 1) + 128 * which + lane_addr + 32 * cq + 16 * piece, r);
+                    TMEM_LD16(tmem + 256 * (m & 1) + 128 * which + lane_addr + CW * cq + 16 * piece, r);
                     tmem_wait_ld();
 #pragma unroll
                     for (int i = 0; i < 16; ++i) mm[16 * piece + i] = fmaf(decay, mm[16 * piece + i], __uint_as_float(r[i]));
@@ -529,14 +542,14 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             }
             fence_before();
             // ---- final state of the sequence
-            if (p.seq_end && a.state_out && c < a.d && 32 * cq < a.d) {      // in the caller's layout (head dimension a.d)
-                float *so = a.state_out + (size_t)p.seq * 2 * a.d * a.d + (size_t)c * a.d + 32 * cq;
+            if (p.seq_end && a.state_out && c < a.d && col0 < a.d) {      // in the caller's layout (head dimension a.d)
+                float *so = a.state_out + (size_t)p.seq * 2 * a.d * a.d + (size_t)c * a.d + col0;
 #pragma unroll
                 for (int which = 0; which < 2; ++which) {
                     if (which < w_lo || which >= w_hi) continue;
-                    const float(&mm)[32] = which ? mU : mH;
+                    const float(&mm)[CW] = which ? mU : mH;
 #pragma unroll
-                    for (int i = 0; i < 8; ++i)
+                    for (int i = 0; i < CW / 4; ++i)
                         *reinterpret_cast<float4 *>(so + which * (size_t)a.d * a.d + 4 * i) = make_float4(mm[4 * i], mm[4 * i + 1], mm[4 * i + 2], mm[4 * i + 3]);
                 }
             }
@@ -547,7 +560,7 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 float hh = 0.f;
 #pragma unroll
                 for (int i = 0; i < 16; ++i) hh += s_red[(m - 1) % 3][i];
-                a.tile_hh[tile - 1] = hh;
+                hh_out[tile - 1] = hh;
             }
         }
         if (t == 0) *reinterpret_cast<volatile int *>(&s_req) = -1;
@@ -557,7 +570,7 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 float hh = 0.f;
 #pragma unroll
                 for (int i = 0; i < 16; ++i) hh += s_red[m % 3][i];
-                a.tile_hh[f_lo + m] = hh;
+                hh_out[f_lo + m] = hh;
             }
             if (s_abort != 0 && a.device_status) atomicExch(a.device_status, (int)GKA_ERR_TIMEOUT);
         }
@@ -645,6 +658,14 @@ cudaError_t launch_fwd_tc(const FwdArgs &a_in, cudaStream_t stream) {
     a.start_from_scan = longest > 4 ? 1 : 0;
     // two blocks per work item (one per master) where no sequence is cut and the blocks still fit one per SM
     a.state_split = (!any_cut && 2 * a.plan.G <= a.sms) ? 1 : 0;
+    // Four blocks per item, 64 columns of one master each, where those still fit one per SM (at head dimension 64 the upper half
+    // would be zeros): a block scales and packs less per tile.  B=4, 8 heads, T=2048, r = 30 / r = 0: 226 -> 218 / 76 -> 68 us for
+    // the call; B=3, 8 heads, T=1999, r = 30: 205 -> 200.  The second half of ||H_0||_F^2 goes to the summaries' place, which
+    // nothing else uses when no sequence is cut.
+    if (a.state_split && 4 * a.plan.G <= a.sms && a.d == D && a.plan.NC <= (long long)a.plan.G * (long long)state_floats(D, D)) {
+        a.state_split = 2;
+        a.tile_hh2 = a.ws.delta;
+    }
     alignas(64) CUtensorMap tmK, tmV, tmS;      // boxes of 128 tokens x 64 channels; per-tile bf16 state copies
     const int cols = a.heads * a.d;
     if (!make_tile_map(&tmK, a.k, a.B, a.T, cols, NT) || !make_tile_map(&tmV, a.v, a.B, a.T, cols, NT) ||
@@ -657,7 +678,7 @@ cudaError_t launch_fwd_tc(const FwdArgs &a_in, cudaStream_t stream) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cfg.stream = stream;
-    static SmemLimit summary_limit, state_limit[2];
+    static SmemLimit summary_limit, state_limit[3];
     if (any_cut) {
         if ((err = summary_limit.raise(fwd_tc_summary_kernel, (int)KV_SMEM)) != cudaSuccess) return err;
         cfg.gridDim = dim3((unsigned)a.plan.G);
@@ -672,9 +693,9 @@ cudaError_t launch_fwd_tc(const FwdArgs &a_in, cudaStream_t stream) {
         }
         a.after_summary = 1;
     }
-    auto state_kernel = a.state_split ? fwd_tc_state_kernel<true> : fwd_tc_state_kernel<false>;
+    auto state_kernel = a.state_split == 2 ? fwd_tc_state_kernel<4> : a.state_split ? fwd_tc_state_kernel<2> : fwd_tc_state_kernel<1>;
     if ((err = state_limit[a.state_split].raise(state_kernel, (int)ST_SMEM)) != cudaSuccess) return err;
-    cfg.gridDim = dim3((unsigned)(a.plan.G * (a.state_split ? 2 : 1)));
+    cfg.gridDim = dim3((unsigned)(a.plan.G << a.state_split));
     cfg.blockDim = dim3(kThreadsStateK);
     cfg.dynamicSmemBytes = ST_SMEM;
     if ((err = cudaLaunchKernelEx(&cfg, state_kernel, tmK, tmV, tmS, a)) != cudaSuccess) return err;
