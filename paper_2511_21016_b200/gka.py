@@ -272,7 +272,7 @@ def gka_solve_chunked(rhs, k, gate, lam, n_iter, chunk=64, out=None, *, state_in
     _expect_tokens(rhs, k, None, gate, lam, out, names=("rhs", "k", "v", "x_out"), beta=beta)
     _expect("state_in", state_in, torch.float32, (B, heads, 2 * d * d))
     _expect("device_status", device_status, torch.int32, (1,))
-    _check_cuda(rhs, k, gate, lam, out, state_in, workspace, device_status)
+    _check_cuda(rhs, k, gate, lam, out, state_in, workspace, device_status, beta)
     if out is None:
         out = torch.empty_like(rhs)
     if workspace is None:

@@ -194,6 +194,44 @@ def test_binding_rejects_mismatched_tensors():
         gka.gka_fwd_chunked_noalloc(q, q, q, g, g.double(), 1)
 
 
+def test_every_tensor_is_checked_for_its_device(monkeypatch):
+    """A host tensor among a device call's arguments would be read or written at its host address by the kernels: what the
+    native marshalling does not take as it is has every one of its tensors checked (the marshalling is made to refuse)."""
+    import torch
+
+    class Refuses:
+        def __getattr__(self, name):
+            return lambda *a: None
+
+    class Checked(Exception):
+        pass
+
+    def check(*ts):
+        raise Checked([t for t in ts if t is not None])
+
+    monkeypatch.setattr(gka, "_native", Refuses())
+    monkeypatch.setattr(gka, "_check_cuda", check)
+    B, T, H, d = 2, 4, 3, 64
+    vec, scalar, state = (lambda: torch.zeros(B, T, H, d)), (lambda: torch.ones(B, T, H)), (lambda: torch.zeros(B, H, 2 * d * d))
+    status, ws = torch.zeros(1, dtype=torch.int32), torch.zeros(256, dtype=torch.uint8)
+    fwd = [vec(), vec(), vec(), scalar(), scalar()]
+    fwd_kw = dict(out=vec(), state_out=state(), state_in=state(), workspace=ws, fro_out=scalar(), device_status=status, beta=scalar(), alpha=scalar())
+    solve_kw = dict(out=vec(), state_in=state(), workspace=ws, device_status=status, beta=scalar())
+    dec_kw = dict(out=vec(), device_status=status, beta=scalar(), alpha=scalar())
+    one = lambda t: t[:, 0].contiguous()
+    calls = [
+        (lambda *a, **kw: gka.gka_fwd_chunked(*a, 1, **kw), fwd, fwd_kw),
+        (lambda *a, **kw: gka.gka_solve_chunked(*a, 1, **kw), [vec(), vec(), scalar(), scalar()], solve_kw),
+        (lambda *a, **kw: gka.gka_decode_tokens(*a, 1, **kw), [state()] + fwd, dec_kw),
+        (lambda *a, **kw: gka.gka_decode_step(*a, 1, **kw), [state()] + [one(t) for t in fwd],
+         {n: t if n == "device_status" else one(t) for n, t in dec_kw.items()}),
+    ]
+    for call, args, kw in calls:
+        with pytest.raises(Checked) as e:
+            call(*args, **kw)
+        assert {id(t) for t in e.value.args[0]} == {id(t) for t in args + list(kw.values())}
+
+
 def test_synth_substreams_and_distributions():
     cfg = synth.shrink(synth.CONFIGS[1], B=2, heads=3, T=128)
     full = synth.make_inputs(cfg)
