@@ -4,7 +4,7 @@
 // A call from Python spends its time before the first launch: with the checks and the descriptor in Python a decode step
 // took 17 us of host time and a forward 33 to 40, more than the kernels of a small call.  Every function takes its
 // arguments by position and returns the result, the library's status (an int) if the call failed, or None if an argument
-// does not fit as it is; the Python wrapper then goes through its own checks, which convert it or say what is wrong.
+// does not fit as it is; the Python wrapper then says what is wrong, or converts it and calls once more.
 #define PY_SSIZE_T_CLEAN
 #include <torch/csrc/autograd/python_variable.h>
 

@@ -6,7 +6,7 @@ fallback: if the library is missing or a call fails, an exception is raised.
 
 The calls that a program makes for every batch or token are marshalled by ``_gka_torch.so`` (csrc/gka_torch.cpp): checked
 and filled into a descriptor in Python they cost 17 to 40 us of host time, more than the kernels of a small call.  What it
-does not take as it is comes back as None, and the ctypes form below converts it or raises.
+does not take as it is comes back as None; the wrapper then says what is wrong, or converts it and calls again.
 """
 from __future__ import annotations
 
@@ -182,6 +182,40 @@ def make_desc(B, T, heads, d_k, d_v, io_dtype, precision=GKA_PREC_NATIVE, flags=
     return d
 
 
+def _int(x) -> int:
+    """A number as the C int it becomes in the descriptor or the call."""
+    return ctypes.c_int(int(x)).value
+
+
+def _flags(x) -> int:
+    return ctypes.c_uint(int(x)).value
+
+
+def _events(pair):
+    return None if pair is None else tuple(None if e is None else int(e) for e in pair)
+
+
+def _bytes(t):
+    """Scratch as the bytes it consists of."""
+    return t if t is None or t.dtype == torch.uint8 else t.reshape(-1).view(torch.uint8)
+
+
+def _expect_workspace(q, chunk, precision):
+    """Raise GkaError where no workspace can be made for this call because its shape is not supported."""
+    B, T, heads, d = q.shape
+    desc = make_desc(B, T, heads, d, d, _io_code(q), precision)
+    if load_library().gka_fwd_workspace_bytes(ctypes.byref(desc), chunk) == 0:
+        raise GkaError(2, "gka_fwd_workspace_bytes")
+
+
+def _again(where, call, *args):
+    """Second call of the native marshalling, with arguments that have been checked and converted."""
+    r = call(*args)
+    if r is None:
+        raise TypeError(f"{where}: an argument is of a type that the call does not take")
+    return r
+
+
 def gka_fwd_workspace_bytes(B, T, heads, d, io_dtype=GKA_BF16, chunk=64) -> int:
     desc = make_desc(B, T, heads, d, d, io_dtype)
     return int(load_library().gka_fwd_workspace_bytes(ctypes.byref(desc), chunk))
@@ -220,38 +254,28 @@ def gka_fwd_chunked(q, k, v, gate, lam, n_iter, chunk=64, out=None, state_out=No
 
     Returns (out, state_out).  Work is enqueued on ``stream`` (default: torch's current stream).
     """
-    r = (_native or _load_native()).fwd_chunked(q, k, v, gate, lam, n_iter, chunk, out, state_out, state_in, workspace, precision,
-                                                flags, fro_out, device_status, stream, profile_events, beta, alpha)
-    if r is not None:
-        if r.__class__ is int:
-            raise GkaError(r, "gka_fwd_chunked")
-        return r
-    if q.dim() != 4:
-        raise ValueError(f"q: expected [B, T, heads, d], got shape {tuple(q.shape)}")
-    B, T, heads, d = q.shape
-    _expect_tokens(q, k, v, gate, lam, out, fro_out=fro_out, beta=beta, alpha=alpha)
-    _expect("state_out", state_out, torch.float32, (B, heads, 2 * d * d))
-    _expect("state_in", state_in, torch.float32, (B, heads, 2 * d * d))
-    _expect("device_status", device_status, torch.int32, (1,))
-    _check_cuda(q, k, v, gate, lam, out, state_out, state_in, workspace, fro_out, device_status, beta, alpha)
-    if out is None:
-        out = torch.empty_like(v)
-    if state_out is None:
-        state_out = torch.empty(B, heads, 2 * d * d, dtype=torch.float32, device=q.device)
-    if workspace is None:
-        workspace = alloc_workspace(B, T, heads, d, q.device, chunk, _io_code(q), precision)
-    elif workspace.dtype != torch.uint8:
-        raise ValueError("workspace: expected a uint8 tensor")
-    if stream is None:
-        stream = torch.cuda.current_stream(q.device).cuda_stream
-    desc = make_desc(B, T, heads, d, v.shape[-1], _io_code(q), precision, flags, stream, workspace,
-                     state_in, device_status, fro_out, profile_events, beta, alpha)
-    rc = load_library().gka_fwd_chunked(ctypes.byref(desc), q.data_ptr(), k.data_ptr(), v.data_ptr(),
-                                        gate.data_ptr(), lam.data_ptr(), int(n_iter), int(chunk),
-                                        out.data_ptr(), _ptr(state_out))
-    if rc != GKA_OK:
-        raise GkaError(rc, "gka_fwd_chunked")
-    return out, state_out
+    call = (_native or _load_native()).fwd_chunked
+    r = call(q, k, v, gate, lam, n_iter, chunk, out, state_out, state_in, workspace, precision, flags, fro_out, device_status,
+             stream, profile_events, beta, alpha)
+    if r is None:
+        if q.dim() != 4:
+            raise ValueError(f"q: expected [B, T, heads, d], got shape {tuple(q.shape)}")
+        B, T, heads, d = q.shape
+        _expect_tokens(q, k, v, gate, lam, out, fro_out=fro_out, beta=beta, alpha=alpha)
+        _expect("state_out", state_out, torch.float32, (B, heads, 2 * d * d))
+        _expect("state_in", state_in, torch.float32, (B, heads, 2 * d * d))
+        _expect("device_status", device_status, torch.int32, (1,))
+        _check_cuda(q, k, v, gate, lam, out, state_out, state_in, workspace, fro_out, device_status, beta, alpha)
+        precision, chunk = _int(precision), _int(chunk)
+        if workspace is None:
+            _expect_workspace(q, chunk, precision)
+        elif workspace.dtype != torch.uint8:
+            raise ValueError("workspace: expected a uint8 tensor")
+        r = _again("gka_fwd_chunked", call, q, k, v, gate, lam, _int(n_iter), chunk, out, state_out, state_in, workspace, precision,
+                   _flags(flags), fro_out, device_status, stream, _events(profile_events), beta, alpha)
+    if r.__class__ is int:
+        raise GkaError(r, "gka_fwd_chunked")
+    return r
 
 
 def gka_solve_chunked(rhs, k, gate, lam, n_iter, chunk=64, out=None, *, state_in=None, workspace=None,
@@ -260,32 +284,24 @@ def gka_solve_chunked(rhs, k, gate, lam, n_iter, chunk=64, out=None, *, state_in
 
     With rhs = q this is the iterate the forward multiplies by U_t; with rhs = dL/dx it is dL/dq.
     """
-    r = (_native or _load_native()).solve_chunked(rhs, k, gate, lam, n_iter, chunk, out, state_in, workspace, precision, flags,
-                                                  device_status, stream, beta)
-    if r is not None:
-        if r.__class__ is int:
-            raise GkaError(r, "gka_solve_chunked")
-        return r
-    if rhs.dim() != 4:
-        raise ValueError(f"rhs: expected [B, T, heads, d], got shape {tuple(rhs.shape)}")
-    B, T, heads, d = rhs.shape
-    _expect_tokens(rhs, k, None, gate, lam, out, names=("rhs", "k", "v", "x_out"), beta=beta)
-    _expect("state_in", state_in, torch.float32, (B, heads, 2 * d * d))
-    _expect("device_status", device_status, torch.int32, (1,))
-    _check_cuda(rhs, k, gate, lam, out, state_in, workspace, device_status, beta)
-    if out is None:
-        out = torch.empty_like(rhs)
-    if workspace is None:
-        workspace = alloc_workspace(B, T, heads, d, rhs.device, chunk, _io_code(rhs), precision)
-    if stream is None:
-        stream = torch.cuda.current_stream(rhs.device).cuda_stream
-    desc = make_desc(B, T, heads, d, d, _io_code(rhs), precision, flags, stream, workspace, state_in, device_status,
-                     beta=beta)
-    rc = load_library().gka_solve_chunked(ctypes.byref(desc), rhs.data_ptr(), k.data_ptr(), gate.data_ptr(),
-                                          lam.data_ptr(), int(n_iter), int(chunk), out.data_ptr())
-    if rc != GKA_OK:
-        raise GkaError(rc, "gka_solve_chunked")
-    return out
+    call = (_native or _load_native()).solve_chunked
+    r = call(rhs, k, gate, lam, n_iter, chunk, out, state_in, workspace, precision, flags, device_status, stream, beta)
+    if r is None:
+        if rhs.dim() != 4:
+            raise ValueError(f"rhs: expected [B, T, heads, d], got shape {tuple(rhs.shape)}")
+        B, T, heads, d = rhs.shape
+        _expect_tokens(rhs, k, None, gate, lam, out, names=("rhs", "k", "v", "x_out"), beta=beta)
+        _expect("state_in", state_in, torch.float32, (B, heads, 2 * d * d))
+        _expect("device_status", device_status, torch.int32, (1,))
+        _check_cuda(rhs, k, gate, lam, out, state_in, workspace, device_status, beta)
+        precision, chunk = _int(precision), _int(chunk)
+        if workspace is None:
+            _expect_workspace(rhs, chunk, precision)
+        r = _again("gka_solve_chunked", call, rhs, k, gate, lam, _int(n_iter), chunk, out, state_in, _bytes(workspace), precision,
+                   _flags(flags), device_status, stream, beta)
+    if r.__class__ is int:
+        raise GkaError(r, "gka_solve_chunked")
+    return r
 
 
 def gka_fwd_host_staging_bytes(B, T, heads, d, io_dtype) -> int:
@@ -297,34 +313,28 @@ def gka_fwd_chunked_host(q, k, v, gate, lam, n_iter, chunk, out, state_out, *, s
                          precision=GKA_PREC_NATIVE, flags=0, stream=None, device_status=None):
     """Host-buffer forward: q, k, v, gate, lam, out, state_out are (pinned) CPU tensors; staging and
     workspace are CUDA byte tensors.  Copies and kernels are enqueued on the stream; no synchronisation."""
-    rc = (_native or _load_native()).fwd_chunked_host(q, k, v, gate, lam, n_iter, chunk, out, state_out, staging, workspace,
-                                                      precision, flags, stream, device_status)
-    if rc == GKA_OK:
-        return out, state_out
-    if rc is not None:
-        raise GkaError(rc, "gka_fwd_chunked_host")
-    if q.dim() != 4:
-        raise ValueError(f"q: expected [B, T, heads, d], got shape {tuple(q.shape)}")
-    B, T, heads, d = q.shape
-    if out is None:
-        raise ValueError("out: the host-buffer call writes into a caller-provided CPU tensor")
-    _expect_tokens(q, k, v, gate, lam, out)
-    _expect("state_out", state_out, torch.float32, (B, heads, 2 * d * d))
-    _expect("device_status", device_status, torch.int32, (1,))
-    for t in (q, k, v, gate, lam, out, state_out):
-        if t is not None and (t.is_cuda or not t.is_contiguous()):
-            raise ValueError("host-buffer call takes contiguous CPU tensors")
-    _check_cuda(staging, workspace, device_status)
-    need = gka_fwd_host_staging_bytes(B, T, heads, d, _io_code(q))
-    if staging.dtype != torch.uint8 or staging.numel() < need:
-        raise ValueError(f"staging: expected a uint8 tensor of at least {need} bytes")
-    if stream is None:
-        stream = torch.cuda.current_stream(staging.device).cuda_stream
-    desc = make_desc(B, T, heads, d, v.shape[-1], _io_code(q), precision, flags, stream, workspace,
-                     device_status=device_status)
-    rc = load_library().gka_fwd_chunked_host(ctypes.byref(desc), staging.data_ptr(), q.data_ptr(),
-                                             k.data_ptr(), v.data_ptr(), gate.data_ptr(), lam.data_ptr(),
-                                             int(n_iter), int(chunk), out.data_ptr(), _ptr(state_out))
+    call = (_native or _load_native()).fwd_chunked_host
+    rc = call(q, k, v, gate, lam, n_iter, chunk, out, state_out, staging, workspace, precision, flags, stream, device_status)
+    if rc is None:
+        if q.dim() != 4:
+            raise ValueError(f"q: expected [B, T, heads, d], got shape {tuple(q.shape)}")
+        B, T, heads, d = q.shape
+        if out is None:
+            raise ValueError("out: the host-buffer call writes into a caller-provided CPU tensor")
+        _expect_tokens(q, k, v, gate, lam, out)
+        _expect("state_out", state_out, torch.float32, (B, heads, 2 * d * d))
+        _expect("device_status", device_status, torch.int32, (1,))
+        for t in (q, k, v, gate, lam, out, state_out):
+            if t is not None and (t.is_cuda or not t.is_contiguous()):
+                raise ValueError("host-buffer call takes contiguous CPU tensors")
+        _check_cuda(staging, workspace, device_status)
+        need = gka_fwd_host_staging_bytes(B, T, heads, d, _io_code(q))
+        if staging.dtype != torch.uint8 or staging.numel() < need:
+            raise ValueError(f"staging: expected a uint8 tensor of at least {need} bytes")
+        if workspace is None:
+            raise GkaError(5, "gka_fwd_chunked_host")
+        rc = _again("gka_fwd_chunked_host", call, q, k, v, gate, lam, _int(n_iter), _int(chunk), out, state_out, staging,
+                    _bytes(workspace), _int(precision), _flags(flags), stream, device_status)
     if rc != GKA_OK:
         raise GkaError(rc, "gka_fwd_chunked_host")
     return out, state_out
@@ -361,62 +371,42 @@ def gka_fwd_chunked_noalloc(q, k, v, gate, lam, n_iter, chunk=64, out=None, stat
 def gka_decode_step(state, q, k, v, gate, lam, n_iter, out=None, *, flags=0, device_status=None,
                     stream=None, profile_events=None, beta=None, alpha=None):
     """One recurrent step.  state: [N,heads,2*d*d] f32, updated in place; q,k,v: [N,heads,d]."""
-    r = (_native or _load_native()).decode_step(state, q, k, v, gate, lam, n_iter, out, flags, device_status, stream,
-                                                profile_events, beta, alpha)
-    if r is not None:
-        if r.__class__ is int:
-            raise GkaError(r, "gka_decode_step")
-        return r
-    if q.dim() != 3:
-        raise ValueError(f"q: expected [N, heads, d], got shape {tuple(q.shape)}")
-    N, heads, d = q.shape
-    _expect_tokens(q, k, v, gate, lam, out, beta=beta, alpha=alpha)
-    _expect("state", state, torch.float32, (N, heads, 2 * d * d))
-    _expect("device_status", device_status, torch.int32, (1,))
-    _check_cuda(state, q, k, v, gate, lam, out, device_status, beta, alpha)
-    if out is None:
-        out = torch.empty_like(v)
-    if stream is None:
-        stream = torch.cuda.current_stream(q.device).cuda_stream
-    desc = make_desc(N, 1, heads, d, v.shape[-1], _io_code(q), GKA_PREC_NATIVE, flags, stream,
-                     device_status=device_status, profile_events=profile_events, beta=beta, alpha=alpha)
-    rc = load_library().gka_decode_step(ctypes.byref(desc), state.data_ptr(), q.data_ptr(),
-                                        k.data_ptr(), v.data_ptr(), gate.data_ptr(), lam.data_ptr(),
-                                        int(n_iter), out.data_ptr())
-    if rc != GKA_OK:
-        raise GkaError(rc, "gka_decode_step")
-    return out
+    call = (_native or _load_native()).decode_step
+    r = call(state, q, k, v, gate, lam, n_iter, out, flags, device_status, stream, profile_events, beta, alpha)
+    if r is None:
+        if q.dim() != 3:
+            raise ValueError(f"q: expected [N, heads, d], got shape {tuple(q.shape)}")
+        N, heads, d = q.shape
+        _expect_tokens(q, k, v, gate, lam, out, beta=beta, alpha=alpha)
+        _expect("state", state, torch.float32, (N, heads, 2 * d * d))
+        _expect("device_status", device_status, torch.int32, (1,))
+        _check_cuda(state, q, k, v, gate, lam, out, device_status, beta, alpha)
+        r = _again("gka_decode_step", call, state, q, k, v, gate, lam, _int(n_iter), out, _flags(flags), device_status, stream,
+                   _events(profile_events), beta, alpha)
+    if r.__class__ is int:
+        raise GkaError(r, "gka_decode_step")
+    return r
 
 
 def gka_decode_tokens(state, q, k, v, gate, lam, n_iter, out=None, *, flags=0, device_status=None,
                       stream=None, profile_events=None, beta=None, alpha=None):
     """The recurrent step over T consecutive tokens.  state: [N,heads,2*d*d] f32, updated in place;
     q,k,v: [N,T,heads,d]; gate, lam (beta, alpha): [N,T,heads]."""
-    r = (_native or _load_native()).decode_tokens(state, q, k, v, gate, lam, n_iter, out, flags, device_status, stream,
-                                                  profile_events, beta, alpha)
-    if r is not None:
-        if r.__class__ is int:
-            raise GkaError(r, "gka_decode_tokens")
-        return r
-    if q.dim() != 4:
-        raise ValueError(f"q: expected [N, T, heads, d], got shape {tuple(q.shape)}")
-    N, T, heads, d = q.shape
-    _expect_tokens(q, k, v, gate, lam, out, beta=beta, alpha=alpha)
-    _expect("state", state, torch.float32, (N, heads, 2 * d * d))
-    _expect("device_status", device_status, torch.int32, (1,))
-    _check_cuda(state, q, k, v, gate, lam, out, device_status, beta, alpha)
-    if out is None:
-        out = torch.empty_like(v)
-    if stream is None:
-        stream = torch.cuda.current_stream(q.device).cuda_stream
-    desc = make_desc(N, T, heads, d, v.shape[-1], _io_code(q), GKA_PREC_NATIVE, flags, stream,
-                     device_status=device_status, profile_events=profile_events, beta=beta, alpha=alpha)
-    rc = load_library().gka_decode_tokens(ctypes.byref(desc), state.data_ptr(), q.data_ptr(),
-                                          k.data_ptr(), v.data_ptr(), gate.data_ptr(), lam.data_ptr(),
-                                          int(n_iter), out.data_ptr())
-    if rc != GKA_OK:
-        raise GkaError(rc, "gka_decode_tokens")
-    return out
+    call = (_native or _load_native()).decode_tokens
+    r = call(state, q, k, v, gate, lam, n_iter, out, flags, device_status, stream, profile_events, beta, alpha)
+    if r is None:
+        if q.dim() != 4:
+            raise ValueError(f"q: expected [N, T, heads, d], got shape {tuple(q.shape)}")
+        N, T, heads, d = q.shape
+        _expect_tokens(q, k, v, gate, lam, out, beta=beta, alpha=alpha)
+        _expect("state", state, torch.float32, (N, heads, 2 * d * d))
+        _expect("device_status", device_status, torch.int32, (1,))
+        _check_cuda(state, q, k, v, gate, lam, out, device_status, beta, alpha)
+        r = _again("gka_decode_tokens", call, state, q, k, v, gate, lam, _int(n_iter), out, _flags(flags), device_status, stream,
+                   _events(profile_events), beta, alpha)
+    if r.__class__ is int:
+        raise GkaError(r, "gka_decode_tokens")
+    return r
 
 
 def gka_selftest_bounded_wait(device_status, polls=4096, stream=None):

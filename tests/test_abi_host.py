@@ -232,6 +232,39 @@ def test_every_tensor_is_checked_for_its_device(monkeypatch):
         assert {id(t) for t in e.value.args[0]} == {id(t) for t in args + list(kw.values())}
 
 
+def test_arguments_that_need_a_conversion_reach_the_native_call(monkeypatch):
+    """What the native marshalling refuses is converted and handed to it again: numpy numbers, a list of events, scratch of
+    another type; what it still refuses is a TypeError."""
+    import torch
+    seen = []
+
+    class TakesIntegersOnly:
+        def __getattr__(self, name):
+            def call(*a):
+                seen.append(a)
+                plain = (int, type(None), tuple, torch.Tensor)
+                ok = all(type(x) in plain for x in a) and all(x.dtype != torch.int16 for x in a if isinstance(x, torch.Tensor))
+                return (0 if name == "fwd_chunked_host" else "done") if ok else None
+            return call
+
+    monkeypatch.setattr(gka, "_native", TakesIntegersOnly())
+    monkeypatch.setattr(gka, "_check_cuda", lambda *a: None)
+    q, g, st = torch.zeros(2, 4, 3, 64), torch.ones(2, 4, 3), torch.zeros(2, 3, 2 * 64 * 64)
+    assert gka.gka_fwd_chunked(q, q, q, g, g, np.int64(3), np.int32(64), flags=np.uint32(1), precision=np.int8(1), profile_events=[5, None]) == "done"
+    assert seen[-1][5:7] == (3, 64) and seen[-1][11:13] == (1, 1) and seen[-1][16] == (5, None)
+    assert gka.gka_solve_chunked(q, q, g, g, 3, workspace=torch.zeros(128, dtype=torch.int16)) == "done"
+    assert seen[-1][8].dtype == torch.uint8 and seen[-1][8].numel() == 256
+    assert gka.gka_decode_step(st, q[:, 0], q[:, 0], q[:, 0], g[:, 0], g[:, 0], np.int64(2)) == "done"
+    assert gka.gka_decode_tokens(st, q, q, q, g, g, np.int64(2)) == "done"
+    need = gka.gka_fwd_host_staging_bytes(2, 4, 3, 64, gka.GKA_F32)
+    staging = torch.zeros(need, dtype=torch.uint8)
+    assert gka.gka_fwd_chunked_host(q, q, q, g, g, np.int64(2), 64, q, st, staging=staging, workspace=torch.zeros(8, dtype=torch.int16))[0] is q
+    with pytest.raises(TypeError):
+        gka.gka_decode_tokens(st, q, q, q, g, g, 2, stream="0")
+    with pytest.raises(gka.GkaError):       # no workspace can be made: an unsupported head dimension
+        gka.gka_fwd_chunked(q[..., :48].contiguous(), *[q[..., :48].contiguous()] * 2, g, g, np.int64(3))
+
+
 def test_synth_substreams_and_distributions():
     cfg = synth.shrink(synth.CONFIGS[1], B=2, heads=3, T=128)
     full = synth.make_inputs(cfg)
