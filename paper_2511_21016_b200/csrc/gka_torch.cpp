@@ -105,13 +105,25 @@ gka_desc describe(const Tensor &q, int64_t B, int64_t T, int precision, long lon
     d.stream = stream == Py_None ? static_cast<void *>(c10::cuda::getCurrentCUDAStream(device).stream()) : address(stream);
     return d;
 }
+// Where the caller names a stream, what a call allocates (scratch above all, which is given back when the call returns, with its
+// kernels still to run) belongs to that stream: a block of the current stream's pool could go to other work of the current
+// stream at once.
+struct OnStream {
+    c10::cuda::OptionalCUDAStreamGuard guard;
+    OnStream(PyObject *stream, const gka_desc &d, int device) {
+        if (stream == Py_None) return;
+        const cudaStream_t s = static_cast<cudaStream_t>(d.stream);
+        guard.reset_stream(s == nullptr || s == cudaStreamLegacy ? c10::cuda::getDefaultCUDAStream(device)
+                                                                 : c10::cuda::getStreamFromExternal(s, device));
+    }
+};
 void events(gka_desc &d, PyObject *o) {
     if (o == Py_None) return;
     if (!PyTuple_Check(o) || PyTuple_GET_SIZE(o) != 2) throw Bad();
     d.profile_start = address(PyTuple_GET_ITEM(o, 0));
     d.profile_stop = address(PyTuple_GET_ITEM(o, 1));
 }
-// The workspace given by the caller, or one of this call (a block of torch's allocator, ordered on the current stream)
+// The workspace given by the caller, or one of this call
 Tensor workspace(gka_desc &d, PyObject *o, int chunk, const Tensor &q) {
     Tensor w;
     if (o == Py_None) {
@@ -164,6 +176,7 @@ template <int DIM> PyObject *decode(PyObject *const *a, Py_ssize_t n) {
         events(d, a[11]);
         d.beta = tk.scalar(a[12], true);
         d.alpha = tk.scalar(a[13], true);
+        const OnStream on(a[10], d, tk.q.get_device());
         Tensor out = like(a[7], tk.q);
         const int rc = unlocked([&] {
             return DIM == 4 ? gka_decode_tokens(&d, state, tk.q.data_ptr(), k, v, gate, lam, n_iter, out.data_ptr())
@@ -193,6 +206,7 @@ PyObject *fwd_chunked(PyObject *, PyObject *const *a, Py_ssize_t n) {
         events(d, a[16]);
         d.beta = tk.scalar(a[17], true);
         d.alpha = tk.scalar(a[18], true);
+        const OnStream on(a[15], d, tk.q.get_device());
         const Tensor ws = workspace(d, a[10], chunk, tk.q);
         Tensor out = like(a[7], tk.q);
         Tensor state_out = a[8] == Py_None ? at::empty({B, heads, 2 * dim * dim}, tk.q.options().dtype(at::kFloat)) : THPVariable_Unpack(a[8]);
@@ -220,6 +234,7 @@ PyObject *solve_chunked(PyObject *, PyObject *const *a, Py_ssize_t n) {
         d.state_in = tk.state(a[7], B, heads, dim, true);
         d.device_status = status_word(a[11]);
         d.beta = tk.scalar(a[13], true);
+        const OnStream on(a[12], d, tk.q.get_device());
         const Tensor ws = workspace(d, a[8], chunk, tk.q);
         Tensor out = like(a[6], tk.q);
         const int rc = unlocked([&] { return gka_solve_chunked(&d, tk.q.data_ptr(), k, gate, lam, n_iter, chunk, out.data_ptr()); });

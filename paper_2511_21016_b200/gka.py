@@ -252,7 +252,8 @@ def gka_fwd_chunked(q, k, v, gate, lam, n_iter, chunk=64, out=None, state_out=No
                     fro_out=None, device_status=None, stream=None, profile_events=None, beta=None, alpha=None):
     """Chunk-wise GKA forward.  q,k,v: [B,T,heads,d] (f32 or bf16); gate, lam, beta (optional): [B,T,heads] f32.
 
-    Returns (out, state_out).  Work is enqueued on ``stream`` (default: torch's current stream).
+    Returns (out, state_out).  Work is enqueued on ``stream`` (a cudaStream_t as a number; default: torch's current stream).
+    What is not given is allocated here, for that stream, as inside ``with torch.cuda.stream(stream)``.
     """
     call = (_native or _load_native()).fwd_chunked
     r = call(q, k, v, gate, lam, n_iter, chunk, out, state_out, state_in, workspace, precision, flags, fro_out, device_status,
@@ -352,12 +353,13 @@ def gka_fwd_chunked_noalloc(q, k, v, gate, lam, n_iter, chunk=64, out=None, stat
     _expect("state_out", state_out, torch.float32, (B, heads, 2 * d * d))
     _expect("state_in", state_in, torch.float32, (B, heads, 2 * d * d))
     _check_cuda(q, k, v, gate, lam, out, state_out, state_in)
-    if out is None:
-        out = torch.empty_like(v)
-    if state_out is None:
-        state_out = torch.empty(B, heads, 2 * d * d, dtype=torch.float32, device=q.device)
     if stream is None:
         stream = torch.cuda.current_stream(q.device).cuda_stream
+    with torch.cuda.stream(torch.cuda.ExternalStream(stream, q.device)):
+        if out is None:
+            out = torch.empty_like(v)
+        if state_out is None:
+            state_out = torch.empty(B, heads, 2 * d * d, dtype=torch.float32, device=q.device)
     desc = make_desc(B, T, heads, d, v.shape[-1], _io_code(q), precision, flags, stream, None, state_in)
     rc = load_library().gka_fwd_chunked_noalloc(ctypes.byref(desc), q.data_ptr(), k.data_ptr(),
                                                 v.data_ptr(), gate.data_ptr(), lam.data_ptr(),
