@@ -170,6 +170,18 @@ template <> struct Io<__nv_bfloat16> {
     }
 };
 
+// Programmatic launches.  Every kernel of a call but the validation pass is launched with programmatic stream serialization: its
+// blocks may start while the kernel before it still runs.
+//   - The first kernel of a call waits (griddepcontrol.wait: the kernel before is complete and its writes visible) before its first
+//     access to global memory.
+//   - A call of several kernels: the first one releases its dependents (griddepcontrol.launch_dependents) only behind that wait.
+//     Every later kernel of the call therefore exists only since all work before the call is complete, and may read the call's
+//     inputs ahead of its own wait (fwd_tc_state_kernel behind a summary, fwd_tc_solve_kernel, small_solve), even where the kernel
+//     between them (fwd_scan, small_scan) releases it before it has waited itself.  What the call computes is read behind the wait,
+//     which is also where it is first written over.
+//   - Memory that an earlier kernel may still be writing when this one starts is not read-only for the life of the kernel.  So
+//     it is read by ordinary loads: no ld.global.nc or __ldg, and no __restrict__ on a kernel's pointers, which would let the
+//     compiler use them and move loads ahead of the wait.
 #ifdef __CUDACC__
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return (uint32_t)__cvta_generic_to_shared(p);

@@ -19,14 +19,15 @@ namespace {
 constexpr int kThreads = 256;
 
 
+// (No __restrict__ on the pointers: see gka_common.cuh on programmatic launches.)
 // EXTRA: the instantiation that also serves write strengths and the alpha-connection; the plain step runs the
 // other one (the kernel sits at its register limit).
 template <int D, typename IoT, bool EXTRA>
 __global__ void __launch_bounds__(kThreads, 2)
-decode_kernel(float *__restrict__ state, const IoT *__restrict__ q, const IoT *__restrict__ k,
-              const IoT *__restrict__ v, const float *__restrict__ gate,
-              const float *__restrict__ lam, int n_iter, IoT *__restrict__ out, unsigned flags,
-              const float *__restrict__ beta, const float *__restrict__ alpha, int *__restrict__ device_status) {
+decode_kernel(float *state, const IoT *q, const IoT *k,
+              const IoT *v, const float *gate,
+              const float *lam, int n_iter, IoT *out, unsigned flags,
+              const float *beta, const float *alpha, int *device_status) {
     constexpr int RPT = D / 32;   // rows per thread
     constexpr int CG = D / 32;    // float4 column groups per thread
     extern __shared__ __align__(128) unsigned char smem_raw[];

@@ -12,10 +12,10 @@ constexpr int kThreadsSmall = 128;     // four pairs per block
 
 template <int D, typename IoT>
 __global__ void __launch_bounds__(kThreadsSmall)
-decode_small_kernel(float *__restrict__ state, const IoT *__restrict__ q, const IoT *__restrict__ k,
-                    const IoT *__restrict__ v, const float *__restrict__ gate, const float *__restrict__ lam,
-                    int n_iter, IoT *__restrict__ out, unsigned flags, const float *__restrict__ beta,
-                    const float *__restrict__ alpha, int T, int heads, int npairs) {
+decode_small_kernel(float *state, const IoT *q, const IoT *k,
+                    const IoT *v, const float *gate, const float *lam,
+                    int n_iter, IoT *out, unsigned flags, const float *beta,
+                    const float *alpha, int T, int heads, int npairs) {
     asm volatile("griddepcontrol.wait;" ::: "memory");           // programmatic launch in stream order, as in gka_decode.cu
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int lane = threadIdx.x & 31;

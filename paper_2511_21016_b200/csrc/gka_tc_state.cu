@@ -149,7 +149,7 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const int i = i0 + u * CT;
-                    g[u] = (i < ntok_run) ? __ldg(grun + (size_t)i * a.heads) : 1.f;
+                    g[u] = (i < ntok_run) ? grun[(size_t)i * a.heads] : 1.f;
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) s += fmaxf(log2f(g[u]), -115.f);
@@ -166,7 +166,7 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         // value is used so that nothing waits for the load
         auto load_gate = [&](int n) -> float {
             const int i = n * NT + t;
-            return (t < NT && i < ntok_run) ? ldg_stream_f32(grun + (size_t)i * a.heads) : 1.f;
+            return (t < NT && i < ntok_run) ? ld_stream_f32(grun + (size_t)i * a.heads) : 1.f;
         };
         float g_cur = load_gate(0);
         float prefix = 0.f;                    // log2 decay of the tiles before the current one
@@ -190,7 +190,7 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                 incl += before;
                 // w_j = 2^(decay from token j to the end of the run) = 2^((total - prefix) - incl_j); its root scales the rows
                 float wt = exp2f(0.5f * ((total - prefix) - incl));
-                if (brun) wt *= sqrtf(fmaxf(__ldg(brun + (size_t)(n * NT + t) * a.heads), 0.f));   // write strength
+                if (brun) wt *= sqrtf(fmaxf(brun[(size_t)(n * NT + t) * a.heads], 0.f));   // write strength
                 s_w[t] = wt;
                 prefix += tile_total;
             }
@@ -372,8 +372,8 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             for (int grp = 0; grp < 4; ++grp) {
                 const int tok = 32 * grp + l;
                 if (tok < p.ntok) {
-                    lg[grp] = ldg_stream_f32(a.gate + p.tok0 + (size_t)tok * a.heads);
-                    sb[grp] = a.beta ? fmaxf(ldg_stream_f32(a.beta + p.tok0 + (size_t)tok * a.heads), 0.f) : 1.f;
+                    lg[grp] = ld_stream_f32(a.gate + p.tok0 + (size_t)tok * a.heads);
+                    sb[grp] = a.beta ? fmaxf(ld_stream_f32(a.beta + p.tok0 + (size_t)tok * a.heads), 0.f) : 1.f;
                 }
             }
         };

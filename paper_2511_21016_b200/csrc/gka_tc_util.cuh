@@ -122,10 +122,10 @@ __device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
     return d;
 }
 // Streaming global loads that leave the small L1 (what 228 KB of shared memory leave of it) to the
-// thread-local spill slots.
-__device__ __forceinline__ float ldg_stream_f32(const float *p) {
+// thread-local spill slots.  Ordinary (coherent) loads: see gka_common.cuh on programmatic launches.
+__device__ __forceinline__ float ld_stream_f32(const float *p) {
     float v;
-    asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
 }
 __device__ __forceinline__ float ex2_fast(float x) {

@@ -141,6 +141,17 @@ def test_whole_sequences_as_work_items_cut_nothing(lib, B, T, heads):
         assert not cin and not cout
 
 
+def test_kernels_read_global_memory_with_ordinary_loads():
+    """Kernels start while the kernel before them still runs (programmatic launches), so what they read is not read-only for
+    their lifetime: no non-coherent loads, and no __restrict__ pointers, from which the compiler would make such loads and move
+    them ahead of the wait for the kernel before."""
+    csrc = os.path.join(ROOT, "paper_2511_21016_b200", "csrc")
+    for f in sorted(os.listdir(csrc)):
+        text = re.sub(r"//[^\n]*|/\*.*?\*/", "", open(os.path.join(csrc, f)).read(), flags=re.S)
+        for word in ("__restrict__", "__ldg", "ld.global.nc"):
+            assert word not in text, f"{f}: {word}"
+
+
 def test_missing_library_is_an_error(monkeypatch, tmp_path):
     monkeypatch.setattr(gka, "_lib", None)
     monkeypatch.setattr(gka, "LIB_PATH", str(tmp_path / "nope.so"))
