@@ -495,21 +495,17 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 const TileInfo ti = tile_info(a, t_lo + k);
                 GateScalars *g = &reinterpret_cast<SlotScalars *>(smem + OFF_SC + slot * SC_BYTES)->g[j & 1];
                 float run = 0.f;
-                float ks_g[4], ks_s[4], gv[4], lamv[4], bv[4], av[4];
-#pragma unroll
-                for (int grp = 0; grp < 4; ++grp) {     // (every load before the first store to shared memory)
-                    const int cc = 32 * grp + lane;
-                    const bool in = cc < ti.ntok;       // tokens past the sequence: no decay, unit lambda / strengths
-                    const size_t idx = ti.tok0 + (size_t)cc * a.heads;
-                    gv[grp] = in ? a.gate[idx] : 1.f;
-                    lamv[grp] = in ? a.lam[idx] : 1.f;
-                    bv[grp] = (beta_p && in) ? beta_p[idx] : 1.f;
-                    av[grp] = (alpha_p && in) ? alpha_p[idx] : 1.f;
-                }
+                float ks_g[4], ks_s[4];
 #pragma unroll
                 for (int grp = 0; grp < 4; ++grp) {
                     const int cc = 32 * grp + lane;
-                    const float lgc = fmaxf(log2f(gv[grp]), -115.f);
+                    const bool in = cc < ti.ntok;       // tokens past the sequence: no decay, unit lambda / strengths
+                    const size_t idx = ti.tok0 + (size_t)cc * a.heads;
+                    const float gv = in ? *(a.gate + idx) : 1.f;
+                    const float lamv = in ? *(a.lam + idx) : 1.f;
+                    const float bv = (beta_p && in) ? *(beta_p + idx) : 1.f;
+                    const float av = (alpha_p && in) ? *(alpha_p + idx) : 1.f;
+                    const float lgc = fmaxf(log2f(gv), -115.f);
                     float incl = lgc;
 #pragma unroll
                     for (int o = 1; o < 32; o <<= 1) {
@@ -524,10 +520,10 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     g->ac[cc] = G2c - mc;
                     g->zt[cc] = exp2f(mc);
                     g->iz[cc] = exp2f(-mc);
-                    g->lam[cc] = lamv[grp];
-                    g->al[cc] = av[grp];
+                    g->lam[cc] = lamv;
+                    g->al[cc] = av;
                     ks_g[grp] = G2c;
-                    ks_s[grp] = sqrtf(fmaxf(bv[grp], 0.f));
+                    ks_s[grp] = sqrtf(fmaxf(bv, 0.f));
                 }
                 {
                     // the decay of the whole tile decides how the keys are staged (ti.ntok - 1 is the last token)
