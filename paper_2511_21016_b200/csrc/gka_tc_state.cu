@@ -59,12 +59,24 @@ __device__ __forceinline__ void scale_kv(unsigned char *stage, const float *f, i
     }
 }
 
+// A wait of the block has given up, so products and copies may still be in flight: the products end (a commit by the thread that
+// issued them on a barrier of its own, awaited with a limit) and the copies get time to, before the block gives back its tensor
+// and shared memory.  At the kernels' end, off the path of a call that goes well.
+__device__ __forceinline__ void drain(uint32_t bar) {
+    if (threadIdx.x == CT) {
+        mma_commit(bar);
+        mbar_spin_bounded(bar, 0u);
+    }
+    for (int i = 0; i < 2000; ++i) __nanosleep(1000);
+    __syncthreads();
+}
+
 // ------------------------------------------------------------------------------------------------------------
 // Segment summaries.  The weights are formed in log2 space from the run's total log-decay (one pre-pass over the
 // gates) and a running prefix, so every tile is a pure accumulation into TMEM: no rescaling pass.  The kernel
 // streams K and V once.  A summarised run never holds the last tile of its sequence, so all its tiles are full.
 // ------------------------------------------------------------------------------------------------------------
-enum { SB_KV0 = 0, SB_MMA = NS, SB_COUNT };
+enum { SB_KV0 = 0, SB_MMA = NS, SB_DRAIN, SB_COUNT };
 
 __global__ void __launch_bounds__(kThreadsState, 1)
 fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, FwdArgs a) {
@@ -102,6 +114,10 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     const long long f0 = P.last_run_start(item), f1 = P.lo(item + 1);
     const int ntiles = (int)(f1 - f0);
     const uint32_t base14 = (sb >> 4) & 0x3FFF;
+    auto aborted = [&]() { return *reinterpret_cast<volatile int *>(&s_abort) != 0; };
+    auto wait = [&](int which, uint32_t parity) {     // once a wait has given up the later ones return at once
+        if (!aborted() && !mbar_spin_bounded(bars + 8 * which, parity)) *reinterpret_cast<volatile int *>(&s_abort) = 1;
+    };
 
     if (t >= CT) {
         // ================================ MMA issuing warp ================================
@@ -194,7 +210,7 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                 s_w[t] = wt;
                 prefix += tile_total;
             }
-            if (!mbar_spin_bounded(bars + 8 * (SB_KV0 + n % NS), (uint32_t)((n / NS) & 1))) s_abort = 1;
+            wait(SB_KV0 + n % NS, (uint32_t)((n / NS) & 1));
             asm volatile("bar.sync 1, 512;" ::: "memory");       // weights are published (and the scan scratch is free)
             scale_kv(smem + (size_t)(n % NS) * STAGE, s_w, t);
             fence_async_smem();
@@ -202,12 +218,12 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             asm volatile("bar.sync 3, 544;" ::: "memory");       // hand the tile to the issuing warp
             // the previous tile's products are done: its stage takes the tile after the next
             if (n >= 1) {
-                if (!mbar_spin_bounded(bars + 8 * SB_MMA, (uint32_t)((n - 1) & 1))) s_abort = 1;
-                if (t == 0 && n + 2 < ntiles) issue_tma(n + 2);
+                wait(SB_MMA, (uint32_t)((n - 1) & 1));
+                if (t == 0 && n + 2 < ntiles && !aborted()) issue_tma(n + 2);
             }
             g_cur = g_next;
         }
-        if (ntiles > 0 && !mbar_spin_bounded(bars + 8 * SB_MMA, (uint32_t)((ntiles - 1) & 1))) s_abort = 1;
+        if (ntiles > 0) wait(SB_MMA, (uint32_t)((ntiles - 1) & 1));
         if (t == 0) *reinterpret_cast<volatile int *>(&s_req) = -1;
         asm volatile("bar.sync 3, 544;" ::: "memory");           // releases the issuing warp
         fence_after();
@@ -235,6 +251,7 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     }
     fence_before();
     __syncthreads();
+    if (s_abort != 0) drain(bars + 8 * SB_DRAIN);
     if (t < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
 }
 
@@ -250,7 +267,7 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 // TB_STG0 + stage: one barrier per stage, like the loads.  (With a single barrier the compute warps could complete two
 // phases, tiles m + 1 and m + 2, while the TMA thread was still held up behind tile m's store; the phase parity it
 // then polled looked incomplete, and the compute warps in turn waited for the load that only this thread issues.)
-enum { TB_KV0 = 0, TB_D0 = NS, TB_D1, TB_STG0, TB_COUNT = TB_STG0 + NS };
+enum { TB_KV0 = 0, TB_D0 = NS, TB_D1, TB_DRAIN, TB_STG0, TB_COUNT = TB_STG0 + NS };
 
 template <int PARTS>
 __global__ void __launch_bounds__(kThreadsStateK, 1)
@@ -313,9 +330,9 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         p.tok0 = ((size_t)p.b * a.T + (size_t)p.n * NT) * a.heads + p.h;
         return p;
     };
+    auto aborted = [&]() { return *reinterpret_cast<volatile int *>(&s_abort) != 0; };
     auto wait = [&](int which, uint32_t parity) {     // once a wait has given up the later ones return at once
-        if (*reinterpret_cast<volatile int *>(&s_abort) == 0 && !mbar_spin_bounded(bars + 8 * which, parity))
-            *reinterpret_cast<volatile int *>(&s_abort) = 1;
+        if (!aborted() && !mbar_spin_bounded(bars + 8 * which, parity)) *reinterpret_cast<volatile int *>(&s_abort) = 1;
     };
 
     if (t >= CT + 32) {
@@ -349,6 +366,7 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                 if (m + NS < n_mine) {
                     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the copies have been read
+                    if (aborted()) break;            // (a barrier whose copy never landed takes no second announcement)
                     issue_tma(m + NS);
                 }
             }
@@ -580,6 +598,7 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     }
     fence_before();
     __syncthreads();
+    if (s_abort != 0) drain(bars + 8 * TB_DRAIN);
     if (t < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
 }
 
