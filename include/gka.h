@@ -170,13 +170,14 @@ gka_status gka_decode_tokens(const gka_desc *desc, float *state, const void *q, 
  * any, as well as beta / alpha) stays a device pointer.  The call enqueues host-to-device copies of the
  * five inputs, the forward kernels and device-to-host copies of out (and state_out), and does not
  * synchronise.  Sequences being independent, the batch is cut into up to 8 slices (and the sequences of the last
- * slice into two pieces of whole 128-token tiles, whose state is carried on the device, so that little work is
- * left when the last input byte has arrived) that pass through the
+ * batch entry into pieces of whole 128-token tiles, a half and, where they are long, smaller ones, whose state is carried on the
+ * device, so that little work is left when the last input byte has arrived) that pass through the
  * three stages on three streams (copies in and out on two helper streams the library creates once per
  * device, kernels on desc->stream), so both copy directions and the kernels overlap; work already on
  * desc->stream is waited for, and desc->stream waits for the last copy, so stream order is as if
  * everything ran on desc->stream.  The host buffers must stay valid and unmodified until the stream has
- * passed the call.
+ * passed the call.  Calls from several threads are safe; on one device they share the helper streams and are enqueued one
+ * after the other.
  */
 size_t gka_fwd_host_staging_bytes(const gka_desc *desc);
 gka_status gka_fwd_chunked_host(const gka_desc *desc, void *staging, const void *q, const void *k,

@@ -3,7 +3,6 @@
 #include <stdio.h>
 
 #include <mutex>
-#include <vector>
 
 #include "gka_common.cuh"
 
@@ -197,9 +196,9 @@ gka_status gka_fwd_work_range(const gka_desc *desc, int chunk, int num_items, in
     return GKA_OK;
 }
 
-static gka_status fwd_impl(const gka_desc *desc, const void *q, const void *k, const void *v,
-                           const float *gate, const float *lam, int n_iter, int chunk, void *out,
-                           float *state_out, bool solve_only) {
+// Every argument check of the chunked calls; nothing is launched and no CUDA call made
+static gka_status check_fwd(const gka_desc *desc, const void *q, const void *k, const void *v, const float *gate,
+                            const float *lam, int n_iter, int chunk, const void *out, const float *state_out) {
     gka_status s = check_fwd_shape(desc, chunk);
     if (s != GKA_OK) return s;
     if (!q || !k || !v || !gate || !lam || !out) return GKA_ERR_NULL;
@@ -213,6 +212,14 @@ static gka_status fwd_impl(const gka_desc *desc, const void *q, const void *k, c
     if (!desc->workspace || desc->workspace_bytes < need ||
         (reinterpret_cast<uintptr_t>(desc->workspace) & 255u) != 0)
         return GKA_ERR_WORKSPACE;
+    return GKA_OK;
+}
+
+static gka_status fwd_impl(const gka_desc *desc, const void *q, const void *k, const void *v,
+                           const float *gate, const float *lam, int n_iter, int chunk, void *out,
+                           float *state_out, bool solve_only) {
+    gka_status s = check_fwd(desc, q, k, v, gate, lam, n_iter, chunk, out, state_out);
+    if (s != GKA_OK) return s;
     const int G = gka_fwd_num_work_items(desc, chunk);
     if (G <= 0) return GKA_ERR_CUDA;
 
@@ -350,36 +357,25 @@ size_t gka_fwd_host_staging_bytes(const gka_desc *desc) {
 
 namespace {
 // Helper streams and events of the host-buffer entry point, one set per device, created on first use and
-// kept for the life of the process.
+// kept for the life of the process.  A call holds the mutex while it enqueues: what another call records on the same events
+// must not come between a record and the wait for it.
+constexpr int kMaxJobs = 48;       // 8 batch slices and the pieces of a sequence (at most one per halving of T, and one)
 struct HostPipe {
+    std::mutex mutex;
     cudaStream_t in = nullptr, out = nullptr;
-    cudaEvent_t start = nullptr, done = nullptr;
-    std::vector<cudaEvent_t> copied, computed;
+    cudaEvent_t start = nullptr, done = nullptr, copied[kMaxJobs] = {}, computed[kMaxJobs] = {};
 };
-std::mutex g_pipe_mutex;
-HostPipe g_pipes[64];
+HostPipe g_pipes[kMaxDevices];
 
-cudaError_t get_pipe(int slices, HostPipe **pipe) {
-    int dev = 0;
-    cudaError_t err = cudaGetDevice(&dev);
-    if (err != cudaSuccess) return err;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lock(g_pipe_mutex);
-    HostPipe &hp = g_pipes[dev];
-    if (!hp.in) {
-        if ((err = cudaStreamCreateWithFlags(&hp.in, cudaStreamNonBlocking)) != cudaSuccess) return err;
-        if ((err = cudaStreamCreateWithFlags(&hp.out, cudaStreamNonBlocking)) != cudaSuccess) return err;
-        if ((err = cudaEventCreateWithFlags(&hp.start, cudaEventDisableTiming)) != cudaSuccess) return err;
-        if ((err = cudaEventCreateWithFlags(&hp.done, cudaEventDisableTiming)) != cudaSuccess) return err;
-    }
-    while ((int)hp.copied.size() < slices) {
-        cudaEvent_t e0, e1;
-        if ((err = cudaEventCreateWithFlags(&e0, cudaEventDisableTiming)) != cudaSuccess) return err;
-        if ((err = cudaEventCreateWithFlags(&e1, cudaEventDisableTiming)) != cudaSuccess) return err;
-        hp.copied.push_back(e0);
-        hp.computed.push_back(e1);
-    }
-    *pipe = &hp;
+cudaError_t prepare_pipe(HostPipe &hp, int jobs) {
+    auto stream = [](cudaStream_t &s) { return s ? cudaSuccess : cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking); };
+    auto event = [](cudaEvent_t &e) { return e ? cudaSuccess : cudaEventCreateWithFlags(&e, cudaEventDisableTiming); };
+    cudaError_t err;
+    if ((err = stream(hp.in)) != cudaSuccess || (err = stream(hp.out)) != cudaSuccess || (err = event(hp.start)) != cudaSuccess ||
+        (err = event(hp.done)) != cudaSuccess)
+        return err;
+    for (int i = 0; i < jobs; ++i)
+        if ((err = event(hp.copied[i])) != cudaSuccess || (err = event(hp.computed[i])) != cudaSuccess) return err;
     return cudaSuccess;
 }
 }  // namespace
@@ -415,83 +411,117 @@ gka_status gka_fwd_chunked_host(const gka_desc *desc, void *staging, const void 
     // 20 us of copies and launches).  B = 4, 16 heads, T = 4096, d = 128, bf16: 4.30 ms with two halves, 4.20 with a
     // half and two quarters, 4.22 with one more piece; B = 1: 1.264, 1.189, 1.201 ms (the copies alone: 3.7, 0.95 ms).
     const size_t hh = (size_t)desc->heads;
-    struct Job { int b0, nb, t0, tn; bool first, last; };
-    std::vector<Job> jobs;
+    struct Job {
+        size_t tok0, ntok;                // its tokens are one contiguous range: whole batch entries, or a token range of one entry
+        size_t state0, states;            // offset and size of the entries' states
+        gka_desc sub;
+        float *state;                     // where its final states go on the device
+        bool last;                        // of its sequences
+    };
+    Job jobs[kMaxJobs];
+    int njobs = 0, carry = 0;
+    auto add = [&](int b0, int nb, int t0, int tn) {
+        Job &j = jobs[njobs];
+        const bool first = t0 == 0;
+        j.last = t0 + tn >= desc->T;
+        j.tok0 = ((size_t)b0 * desc->T + t0) * hh;
+        j.ntok = (size_t)nb * tn * hh;
+        j.state0 = (size_t)b0 * hh * st_floats;
+        j.states = (size_t)nb * hh * st_floats;
+        j.sub = *desc;
+        j.sub.B = nb;
+        j.sub.T = tn;
+        // the first piece of a sequence starts from the caller's state (or zero), the others from the state the
+        // piece before left in the carry buffer; the last one writes the caller's state_out
+        if (first) j.sub.state_in = desc->state_in ? desc->state_in + j.state0 : nullptr;
+        else j.sub.state_in = dcarry + (size_t)carry * hh * st_floats;
+        j.state = j.last ? (state_out ? dstate + j.state0 : nullptr) : dcarry + (size_t)(carry ^ 1) * hh * st_floats;
+        if (!j.last) carry ^= 1;
+        if (desc->fro_out) j.sub.fro_out = desc->fro_out + j.tok0;
+        if (desc->beta) j.sub.beta = desc->beta + j.tok0;
+        if (desc->alpha) j.sub.alpha = desc->alpha + j.tok0;
+        if (njobs > 0) j.sub.profile_start = j.sub.profile_stop = nullptr;
+        ++njobs;
+    };
     const int per = (desc->B + 7) / 8;                       // at most 8 batch slices
     const int nslices = (desc->B + per - 1) / per;
     for (int i = 0; i < nslices; ++i) {
         const int b0 = i * per, nb = (b0 + per <= desc->B) ? per : desc->B - b0;
         const bool tail = i + 1 == nslices && desc->T >= 4 * kTile;
-        if (!tail || nb > 1) jobs.push_back({b0, tail ? nb - 1 : nb, 0, desc->T, true, true});
+        if (!tail || nb > 1) add(b0, tail ? nb - 1 : nb, 0, desc->T);
         if (!tail) continue;
         for (int t0 = 0, tn; t0 < desc->T; t0 += tn) {
             const int rest = desc->T - t0, half = (rest / 2 + kTile - 1) / kTile * kTile;     // whole tiles
             const size_t bytes = (size_t)rest * hh * (2 * desc->d_k + desc->d_v) * es;
-            tn = t0 == 0 || (rest >= 8 * kTile && bytes >= (size_t)16 << 20) ? half : rest;
-            jobs.push_back({desc->B - 1, 1, t0, tn, t0 == 0, t0 + tn >= desc->T});
+            tn = njobs + 1 < kMaxJobs && (t0 == 0 || (rest >= 8 * kTile && bytes >= (size_t)16 << 20)) ? half : rest;
+            add(desc->B - 1, 1, t0, tn);
         }
     }
-    const int njobs = (int)jobs.size();
-    HostPipe *hp = nullptr;
-    cudaError_t err = get_pipe(njobs, &hp);
-    if (err != cudaSuccess) return cuda_result(err, "gka_fwd_chunked_host (helper streams)");
-    if ((err = cudaEventRecord(hp->start, stream)) != cudaSuccess ||
-        (err = cudaStreamWaitEvent(hp->in, hp->start, 0)) != cudaSuccess ||
-        (err = cudaStreamWaitEvent(hp->out, hp->start, 0)) != cudaSuccess)
+    // the kernels' part of every job
+    auto call = [&](const Job &j, bool check_only) {
+        const unsigned char *const jq = dq + j.tok0 * desc->d_k * es, *const jk = dk + j.tok0 * desc->d_k * es, *const jv = dv + j.tok0 * desc->d_v * es;
+        const float *const jg = reinterpret_cast<const float *>(dgate + j.tok0 * 4), *const jl = reinterpret_cast<const float *>(dlam + j.tok0 * 4);
+        unsigned char *const jo = dout + j.tok0 * desc->d_v * es;
+        return check_only ? check_fwd(&j.sub, jq, jk, jv, jg, jl, n_iter, chunk, jo, j.state)
+                          : gka_fwd_chunked(&j.sub, jq, jk, jv, jg, jl, n_iter, chunk, jo, j.state);
+    };
+    for (int i = 0; i < njobs; ++i)      // argument errors before the first copy is under way
+        if ((s = call(jobs[i], true)) != GKA_OK) return s;
+
+    int dev = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err == cudaSuccess && (dev < 0 || dev >= kMaxDevices)) err = cudaErrorInvalidDevice;
+    if (err != cudaSuccess) return cuda_result(err, "gka_fwd_chunked_host (device)");
+    HostPipe &hp = g_pipes[dev];
+    std::lock_guard<std::mutex> lock(hp.mutex);
+    if ((err = prepare_pipe(hp, njobs)) != cudaSuccess) return cuda_result(err, "gka_fwd_chunked_host (helper streams)");
+    if ((err = cudaEventRecord(hp.start, stream)) != cudaSuccess ||
+        (err = cudaStreamWaitEvent(hp.in, hp.start, 0)) != cudaSuccess ||
+        (err = cudaStreamWaitEvent(hp.out, hp.start, 0)) != cudaSuccess)
         return cuda_result(err, "gka_fwd_chunked_host (stream ordering)");
+    // an error half way: the caller's stream still waits for what is on the helper streams already
+    auto join = [&] {
+        if (cudaEventRecord(hp.start, hp.in) == cudaSuccess) (void)cudaStreamWaitEvent(stream, hp.start, 0);
+        if (cudaEventRecord(hp.done, hp.out) == cudaSuccess) (void)cudaStreamWaitEvent(stream, hp.done, 0);
+    };
+    auto fail = [&](const char *where) {
+        const gka_status r = cuda_result(err, where);
+        join();
+        return r;
+    };
     auto copy = [&](unsigned char *dst, const void *src, size_t off, size_t bytes, cudaMemcpyKind kind, cudaStream_t on) {
         return kind == cudaMemcpyHostToDevice
                    ? cudaMemcpyAsync(dst + off, static_cast<const unsigned char *>(src) + off, bytes, kind, on)
                    : cudaMemcpyAsync(static_cast<unsigned char *>(const_cast<void *>(src)) + off, dst + off, bytes, kind, on);
     };
     // the per-token scalars of all jobs in one copy each: a copy costs the engine some microseconds whatever its size
-    err = copy(dgate, gate, 0, ng, cudaMemcpyHostToDevice, hp->in);
-    if (err == cudaSuccess) err = copy(dlam, lam, 0, ng, cudaMemcpyHostToDevice, hp->in);
-    if (err != cudaSuccess) return cuda_result(err, "gka_fwd_chunked_host (host-to-device copies)");
+    err = copy(dgate, gate, 0, ng, cudaMemcpyHostToDevice, hp.in);
+    if (err == cudaSuccess) err = copy(dlam, lam, 0, ng, cudaMemcpyHostToDevice, hp.in);
+    if (err != cudaSuccess) return fail("gka_fwd_chunked_host (host-to-device copies)");
     for (int i = 0; i < njobs; ++i) {
         const Job &j = jobs[i];
-        // a job's tokens are one contiguous range: whole batch entries, or a token range of one entry
-        const size_t tok0 = ((size_t)j.b0 * desc->T + j.t0) * hh, ntok = (size_t)j.nb * j.tn * hh;
-        err = copy(dq, q, tok0 * desc->d_k * es, ntok * desc->d_k * es, cudaMemcpyHostToDevice, hp->in);
-        if (err == cudaSuccess) err = copy(dk, k, tok0 * desc->d_k * es, ntok * desc->d_k * es, cudaMemcpyHostToDevice, hp->in);
-        if (err == cudaSuccess) err = copy(dv, v, tok0 * desc->d_v * es, ntok * desc->d_v * es, cudaMemcpyHostToDevice, hp->in);
-        if (err == cudaSuccess) err = cudaEventRecord(hp->copied[i], hp->in);
-        if (err != cudaSuccess) return cuda_result(err, "gka_fwd_chunked_host (host-to-device copies)");
+        err = copy(dq, q, j.tok0 * desc->d_k * es, j.ntok * desc->d_k * es, cudaMemcpyHostToDevice, hp.in);
+        if (err == cudaSuccess) err = copy(dk, k, j.tok0 * desc->d_k * es, j.ntok * desc->d_k * es, cudaMemcpyHostToDevice, hp.in);
+        if (err == cudaSuccess) err = copy(dv, v, j.tok0 * desc->d_v * es, j.ntok * desc->d_v * es, cudaMemcpyHostToDevice, hp.in);
+        if (err == cudaSuccess) err = cudaEventRecord(hp.copied[i], hp.in);
+        if (err != cudaSuccess) return fail("gka_fwd_chunked_host (host-to-device copies)");
     }
-    int carry = 0;
     for (int i = 0; i < njobs; ++i) {
         const Job &j = jobs[i];
-        const size_t tok0 = ((size_t)j.b0 * desc->T + j.t0) * hh, ntok = (size_t)j.nb * j.tn * hh;
-        const size_t ost = (size_t)j.b0 * hh * st_floats;
-        if ((err = cudaStreamWaitEvent(stream, hp->copied[i], 0)) != cudaSuccess)
-            return cuda_result(err, "gka_fwd_chunked_host (stream ordering)");
-        gka_desc sub = *desc;
-        sub.B = j.nb;
-        sub.T = j.tn;
-        // the first piece of a sequence starts from the caller's state (or zero), the others from the state the
-        // piece before left in the carry buffer; the last one writes the caller's state_out
-        if (j.first) sub.state_in = desc->state_in ? desc->state_in + ost : nullptr;
-        else sub.state_in = dcarry + (size_t)carry * hh * st_floats;
-        float *piece_state = j.last ? (state_out ? dstate + ost : nullptr) : dcarry + (size_t)(carry ^ 1) * hh * st_floats;
-        if (!j.last) carry ^= 1;
-        if (desc->fro_out) sub.fro_out = desc->fro_out + tok0;
-        if (desc->beta) sub.beta = desc->beta + tok0;
-        if (desc->alpha) sub.alpha = desc->alpha + tok0;
-        if (i > 0) sub.profile_start = sub.profile_stop = nullptr;
-        s = gka_fwd_chunked(&sub, dq + tok0 * desc->d_k * es, dk + tok0 * desc->d_k * es, dv + tok0 * desc->d_v * es,
-                            reinterpret_cast<const float *>(dgate + tok0 * 4), reinterpret_cast<const float *>(dlam + tok0 * 4),
-                            n_iter, chunk, dout + tok0 * desc->d_v * es, piece_state);
-        if (s != GKA_OK) return s;
-        err = cudaEventRecord(hp->computed[i], stream);
-        if (err == cudaSuccess) err = cudaStreamWaitEvent(hp->out, hp->computed[i], 0);
-        if (err == cudaSuccess) err = copy(dout, out, tok0 * desc->d_v * es, ntok * desc->d_v * es, cudaMemcpyDeviceToHost, hp->out);
+        if ((err = cudaStreamWaitEvent(stream, hp.copied[i], 0)) != cudaSuccess) return fail("gka_fwd_chunked_host (stream ordering)");
+        if ((s = call(j, false)) != GKA_OK) {
+            join();
+            return s;
+        }
+        err = cudaEventRecord(hp.computed[i], stream);
+        if (err == cudaSuccess) err = cudaStreamWaitEvent(hp.out, hp.computed[i], 0);
+        if (err == cudaSuccess) err = copy(dout, out, j.tok0 * desc->d_v * es, j.ntok * desc->d_v * es, cudaMemcpyDeviceToHost, hp.out);
         if (err == cudaSuccess && state_out && j.last)
-            err = cudaMemcpyAsync(state_out + ost, dstate + ost, (size_t)j.nb * hh * st_floats * sizeof(float),
-                                  cudaMemcpyDeviceToHost, hp->out);
-        if (err != cudaSuccess) return cuda_result(err, "gka_fwd_chunked_host (device-to-host copies)");
+            err = cudaMemcpyAsync(state_out + j.state0, dstate + j.state0, j.states * sizeof(float), cudaMemcpyDeviceToHost, hp.out);
+        if (err != cudaSuccess) return fail("gka_fwd_chunked_host (device-to-host copies)");
     }
-    err = cudaEventRecord(hp->done, hp->out);
-    if (err == cudaSuccess) err = cudaStreamWaitEvent(stream, hp->done, 0);
+    err = cudaEventRecord(hp.done, hp.out);
+    if (err == cudaSuccess) err = cudaStreamWaitEvent(stream, hp.done, 0);
     return cuda_result(err, "gka_fwd_chunked_host (stream ordering)");
 }
 

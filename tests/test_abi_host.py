@@ -97,6 +97,25 @@ def test_argument_errors_are_reported_before_any_launch(lib):
     assert lib.gka_decode_tokens(ctypes.byref(dd), ok + 4, ok, ok, ok, ok, ok, 3, ok) == 9
 
 
+def test_host_call_reports_argument_errors_before_any_copy(lib):
+    """The host-buffer call checks what its jobs will be called with before it enqueues the first copy (here, without a
+    device, the first CUDA call would answer 7)."""
+    ok = 256
+    d = gka.make_desc(3, 1000, 2, 64, 64, gka.GKA_BF16)
+    host = lambda desc, n_iter=1, chunk=64: lib.gka_fwd_chunked_host(ctypes.byref(desc), ok, ok, ok, ok, ok, ok, n_iter, chunk, ok, None)
+    assert host(d) == 5                                                    # no workspace
+    d.workspace, d.workspace_bytes = 256, 4096
+    assert host(d) == 5                                                    # workspace too small for a slice
+    d.workspace, d.workspace_bytes = 256 + 16, 1 << 30
+    assert host(d) == 5                                                    # misaligned workspace
+    d.workspace = 256
+    assert host(d, n_iter=-1) == 2
+    d.beta = 257
+    assert host(d) == 9
+    d.beta, d.state_in = None, 260
+    assert host(d) == 9
+
+
 @pytest.mark.parametrize("B,T,heads,G", [(4, 4096, 16, 148), (1, 131072, 32, 148), (1, 256, 2, 4),
                                          (1, 6400, 3, 148), (3, 192, 5, 7), (1, 64, 1, 1)])
 @pytest.mark.parametrize("io", ["bf16", "f32"])

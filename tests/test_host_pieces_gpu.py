@@ -32,3 +32,48 @@ def test_pieces_match_device_call(B, T, heads, d, dtype):
     rel = lambda x, y: float((x.double() - y.cpu().double()).norm() / y.cpu().double().norm())
     assert rel(out, out_ref) < (1e-3 if dtype == torch.bfloat16 else 1e-5)
     assert rel(state, state_ref) < 1e-5
+
+
+def test_calls_from_several_threads():
+    """Host-buffer calls of several threads, each on its own stream with its own buffers, share the helper streams and events of
+    the device: every result as that of a call alone."""
+    import threading
+    B, T, heads, d = 2, 700, 4, 64
+    gen = torch.Generator().manual_seed(5)
+
+    def problem():
+        unit = lambda: torch.nn.functional.normalize(torch.randn(B, T, heads, d, generator=gen), dim=-1).bfloat16().pin_memory()
+        p = dict(args=[unit(), unit(), unit(), torch.sigmoid(torch.randn(B, T, heads, generator=gen) + 3).pin_memory(),
+                       (0.3 + torch.rand(B, T, heads, generator=gen)).pin_memory()],
+                 out=torch.empty(B, T, heads, d, dtype=torch.bfloat16, pin_memory=True), state=torch.empty(B, heads, 2 * d * d, pin_memory=True),
+                 ws=gka.alloc_workspace(B, T, heads, d, "cuda"), stream=torch.cuda.Stream(),
+                 staging=torch.empty(gka.gka_fwd_host_staging_bytes(B, T, heads, d, gka.GKA_BF16), dtype=torch.uint8, device="cuda"))
+        return p
+
+    def call(p):
+        gka.gka_fwd_chunked_host(*p["args"], 4, 64, p["out"], p["state"], staging=p["staging"], workspace=p["ws"], stream=p["stream"].cuda_stream)
+
+    problems = [problem() for _ in range(4)]
+    torch.cuda.synchronize()
+    want = []
+    for p in problems:
+        call(p)
+        torch.cuda.synchronize()
+        want.append((p["out"].clone(), p["state"].clone()))
+    bad = []
+
+    def work(p, w):
+        for _ in range(30):
+            p["out"].zero_()
+            p["state"].zero_()
+            call(p)
+            p["stream"].synchronize()
+            if not (torch.equal(p["out"], w[0]) and torch.equal(p["state"], w[1])):
+                bad.append(1)
+
+    threads = [threading.Thread(target=work, args=a) for a in zip(problems, want)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
