@@ -290,7 +290,8 @@ gka_status gka_decode_step(const gka_desc *desc, float *state, const void *q, co
     if (s != GKA_OK) return s;
     if (!state || !q || !k || !v || !gate || !lam || !out) return GKA_ERR_NULL;
     if (n_iter < 0) return GKA_ERR_SHAPE;
-    if (!aligned16(state) || !aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out))
+    if (!aligned16(state) || !aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out) || !aligned4(gate) ||
+        !aligned4(lam) || !aligned4(desc->beta) || !aligned4(desc->alpha))
         return GKA_ERR_ALIGN;
     cudaError_t err = launch_validate(desc, gate, lam, (size_t)desc->B * desc->heads, reinterpret_cast<cudaStream_t>(desc->stream));
     if (err != cudaSuccess) return cuda_result(err, "gka_decode_step (validation pass)");
@@ -314,7 +315,8 @@ gka_status gka_decode_tokens(const gka_desc *desc, float *state, const void *q, 
     if (s != GKA_OK) return s;
     if (!state || !q || !k || !v || !gate || !lam || !out) return GKA_ERR_NULL;
     if (n_iter < 0 || desc->T < 1) return GKA_ERR_SHAPE;
-    if (!aligned16(state) || !aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out))
+    if (!aligned16(state) || !aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out) || !aligned4(gate) ||
+        !aligned4(lam) || !aligned4(desc->beta) || !aligned4(desc->alpha))
         return GKA_ERR_ALIGN;
     if (desc->T == 1)      // one token: the single-step kernel (same layouts) overlaps the state write-back better
         return gka_decode_step(desc, state, q, k, v, gate, lam, n_iter, out);

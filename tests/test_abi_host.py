@@ -91,6 +91,13 @@ def test_argument_errors_are_reported_before_any_launch(lib):
     assert rc == 9
     rc = lib.gka_decode_step(None, ok, ok, ok, ok, ok, ok, 3, ok)
     assert rc == 1
+    for call in (lib.gka_decode_step, lib.gka_decode_tokens):                # misaligned per-token scalars
+        assert call(ctypes.byref(dd), ok, ok, ok, ok, ok + 2, ok, 3, ok) == 9
+        assert call(ctypes.byref(dd), ok, ok, ok, ok, ok, ok + 1, 3, ok) == 9
+        for name in ("beta", "alpha"):
+            bad = gka.make_desc(4, 2, 2, 128, 128, gka.GKA_BF16)
+            setattr(bad, name, ok + 2)
+            assert call(ctypes.byref(bad), ok, ok, ok, ok, ok, ok, 3, ok) == 9
     d0 = gka.make_desc(4, 0, 2, 128, 128, gka.GKA_BF16)
     assert lib.gka_decode_tokens(ctypes.byref(d0), ok, ok, ok, ok, ok, ok, 3, ok) == 2   # no token
     assert lib.gka_decode_tokens(ctypes.byref(dd), ok, None, ok, ok, ok, ok, 3, ok) == 1
