@@ -202,24 +202,25 @@ const char *gka_status_string(int status);
 const char *gka_last_error_detail(void);
 
 /*
- * Work decomposition of the chunked forward, for callers that size buffers or report launch
- * counts: number of work items (contiguous ranges of the flat chunk list) of the state pass for this
- * descriptor on the current device, or a negative gka_status.  Normally one per SM (fewer for small problems).
- * On the tensor-core path it is pairs / k for a small divisor k of the number of (sequence, head) pairs
- * (k = 1 with fewer pairs than SMs) whenever carrying whole sequences is cheaper than cutting them: no range then
- * starts or ends inside a sequence and no summary or scan kernel runs; with at most half as many work items as
- * SMs the state kernel then runs two thread blocks per work item, one per state matrix.
+ * Work decomposition of the state pass of the tensor-core path, for callers that report launch counts or divide work: number of
+ * work items (contiguous ranges of the flat list of tiles) for this descriptor on the current device, or a negative
+ * gka_status.  Normally one per SM (fewer for small problems).  It is pairs / k for a small divisor k of the number of
+ * (sequence, head) pairs (k = 1 with fewer pairs than SMs) whenever carrying whole sequences is cheaper than cutting them: no
+ * range then starts or ends inside a sequence and no summary or scan kernel runs, and the state kernel runs two thread blocks
+ * per work item with at most half as many work items as SMs, four with at most a quarter (head dimension 128).
+ * fp32 arithmetic splits sequences by rules of its own, which these two functions do not describe: for such a descriptor they
+ * answer with an even split of the list of 64-token chunks into one range per SM (fewer for small problems).
  */
 int gka_fwd_num_work_items(const gka_desc *desc, int chunk);
 
 /*
- * Introspection of the work decomposition (pure host arithmetic, no CUDA call): the flat list of
- * B*heads*ceil(T/chunk) chunks is split into num_items contiguous ranges; item `item` owns chunks
- * [*first_chunk, *end_chunk).  Range sizes differ by at most one chunk; when ceil(T/chunk) is even and
- * there are at least two chunks per item the boundaries are kept at even chunk offsets (the
- * tensor-core kernel works on pairs of chunks) and sizes differ by at most two.  *cut_in / *cut_out
- * tell whether the range starts / ends inside a sequence (then its start state comes from the
- * cross-item scan / its last run is summarised).  Returns GKA_OK or an argument error.
+ * Range `item` of the work decomposition (pure host arithmetic, no CUDA call), in chunks: the flat list of B*heads*ceil(T/chunk)
+ * chunks is split into num_items contiguous ranges; item `item` owns chunks [*first_chunk, *end_chunk).  On the tensor-core path
+ * ranges consist of whole tiles of two chunks (one at the end of a sequence with an odd number of chunks) and their sizes
+ * differ by at most one tile; for fp32 arithmetic they differ by at most one chunk, or by two where the boundaries are kept at even
+ * chunk offsets (ceil(T/chunk) even and at least two chunks per item).  *cut_in / *cut_out tell whether the range starts / ends
+ * inside a sequence (on the tensor-core path its start state then comes from the summaries of the items before it / its last run
+ * is summarised).  Returns GKA_OK or an argument error.
  */
 gka_status gka_fwd_work_range(const gka_desc *desc, int chunk, int num_items, int item,
                               long long *first_chunk, long long *end_chunk, int *cut_in,

@@ -8,7 +8,7 @@
 
 namespace gka {
 
-cudaError_t launch_fwd_tc(const FwdArgs &a, cudaStream_t stream);   // gka_tc.cu
+cudaError_t launch_fwd_tc(const FwdArgs &a, cudaStream_t stream);   // gka_tc_state.cu
 bool fwd_tc_available();
 
 namespace {
@@ -113,7 +113,7 @@ long long work_units(const gka_desc *d) {
     return (long long)d->B * d->heads * (wants_tensor_path(d) ? tiles_of(d->T) : chunks_of(d->T));
 }
 // Upper bound on work items used for sizing (independent of the device).
-int work_items_cap(const gka_desc *d, int chunk) {
+int work_items_cap(const gka_desc *d) {
     const long long nc = work_units(d);
     return (int)(nc < kMaxWorkItems ? nc : kMaxWorkItems);
 }
@@ -143,9 +143,9 @@ const char *gka_status_string(int status) {
 
 size_t gka_fwd_workspace_bytes(const gka_desc *desc, int chunk) {
     if (check_fwd_shape(desc, chunk) != GKA_OK) return 0;
-    if (wants_tensor_path(desc)) return tc_workspace_bytes_for(work_items_cap(desc, chunk), work_units(desc));
+    if (wants_tensor_path(desc)) return tc_workspace_bytes_for(work_items_cap(desc), work_units(desc));
     if (desc->d_k < 64) return small_workspace_bytes_for((long long)desc->B * desc->heads, desc->T, desc->d_k);
-    return workspace_bytes_for(work_items_cap(desc, chunk), desc->d_k, desc->d_v);
+    return workspace_bytes_for(work_items_cap(desc), desc->d_k, desc->d_v);
 }
 
 int gka_fwd_num_work_items(const gka_desc *desc, int chunk) {
@@ -153,7 +153,7 @@ int gka_fwd_num_work_items(const gka_desc *desc, int chunk) {
     if (s != GKA_OK) return -(int)s;
     const int sms = sm_count();
     if (sms <= 0) return -(int)GKA_ERR_CUDA;
-    const int cap = work_items_cap(desc, chunk);
+    const int cap = work_items_cap(desc);
     if (wants_tensor_path(desc)) {
         // Where the ranges cut sequences the summary kernel reads all keys and values once more.  Ranges of whole
         // sequences (pairs / k work items of k sequences each, k the smallest divisor of the number of (sequence, head)
@@ -172,7 +172,7 @@ int gka_fwd_num_work_items(const gka_desc *desc, int chunk) {
             break;
         }
     }
-    return sms < cap ? sms : cap;
+    return sms < cap ? sms : cap;      // (fp32 arithmetic: of an even split of the chunks, which its kernels do not use)
 }
 
 gka_status gka_fwd_work_range(const gka_desc *desc, int chunk, int num_items, int item,
@@ -181,18 +181,21 @@ gka_status gka_fwd_work_range(const gka_desc *desc, int chunk, int num_items, in
     gka_status s = check_fwd_shape(desc, chunk);
     if (s != GKA_OK) return s;
     if (!first_chunk || !end_chunk || !cut_in || !cut_out) return GKA_ERR_NULL;
-    WorkPlan p;
-    const bool tiles = wants_tensor_path(desc);       // that path plans in 128-token tiles = pairs of chunks
-    if (tiles) p.set(desc->B * desc->heads, tiles_of(desc->T), num_items > 0 ? num_items : 1, false);
-    else p.set(desc->B * desc->heads, chunks_of(desc->T), num_items > 0 ? num_items : 1);
-    if (num_items <= 0 || num_items > p.NC || item < 0 || item >= num_items) return GKA_ERR_SHAPE;
-    // a tile is two chunks (the last tile of a sequence with an odd number of chunks holds one)
-    const long long N = chunks_of(desc->T);
-    auto chunk_of = [&](long long f) { return tiles ? (f / p.N) * N + 2 * (f % p.N) : f; };
-    *first_chunk = chunk_of(p.lo(item));
-    *end_chunk = chunk_of(p.lo(item + 1));
-    *cut_in = p.cut_in(item) ? 1 : 0;
-    *cut_out = p.cut_out(item) ? 1 : 0;
+    const long long N = chunks_of(desc->T), NC = (long long)desc->B * desc->heads * N;
+    if (num_items <= 0 || num_items > work_units(desc) || item < 0 || item >= num_items) return GKA_ERR_SHAPE;
+    if (wants_tensor_path(desc)) {       // planned in tiles of two chunks (the last one of a sequence may hold one)
+        WorkPlan p;
+        p.set(desc->B * desc->heads, tiles_of(desc->T), num_items);
+        auto chunk_of = [&](long long f) { return (f / p.N) * N + 2 * (f % p.N); };
+        *first_chunk = chunk_of(p.lo(item));
+        *end_chunk = chunk_of(p.lo(item + 1));
+    } else {                             // an even split of the chunks, in pairs where every sequence and item has whole ones
+        const long long unit = (N % 2 == 0 && 2LL * num_items <= NC) ? 2 : 1;
+        *first_chunk = unit * (item * (NC / unit) / num_items);
+        *end_chunk = unit * ((item + 1) * (NC / unit) / num_items);
+    }
+    *cut_in = *first_chunk % N != 0;
+    *cut_out = *end_chunk % N != 0;
     return GKA_OK;
 }
 
@@ -220,10 +223,8 @@ static gka_status fwd_impl(const gka_desc *desc, const void *q, const void *k, c
                            float *state_out, bool solve_only) {
     gka_status s = check_fwd(desc, q, k, v, gate, lam, n_iter, chunk, out, state_out);
     if (s != GKA_OK) return s;
-    const int G = gka_fwd_num_work_items(desc, chunk);
-    if (G <= 0) return GKA_ERR_CUDA;
 
-    FwdArgs a;
+    FwdArgs a = {};
     a.q = q; a.k = k; a.v = v; a.gate = gate; a.lam = lam; a.out = out;
     a.state_out = state_out;
     a.state_in = desc->state_in;
@@ -236,16 +237,14 @@ static gka_status fwd_impl(const gka_desc *desc, const void *q, const void *k, c
     a.divH.set((unsigned)desc->heads);
     a.n_iter = n_iter;
     a.sms = sm_count();
+    if (a.sms <= 0) return GKA_ERR_CUDA;
     a.flags = desc->flags;
     a.solve_only = solve_only ? 1 : 0;
-    a.start_from_scan = 0;
-    a.state_split = 0;
-    a.after_summary = 0;
     const bool tensor_path = wants_tensor_path(desc) && fwd_tc_available();
-    a.tile_hh = a.tile_hh2 = nullptr;
-    a.tile_hu = nullptr;
     if (tensor_path) {
-        a.plan.set(desc->B * desc->heads, tiles_of(desc->T), G, false);
+        const int G = gka_fwd_num_work_items(desc, chunk);
+        if (G <= 0) return GKA_ERR_CUDA;
+        a.plan.set(desc->B * desc->heads, tiles_of(desc->T), G);
         const TcWorkspace w = carve_tc_workspace(desc->workspace, G, a.plan.NC);
         a.ws.start = w.start;
         a.ws.delta = w.delta;

@@ -1,5 +1,5 @@
 // Shared host/device helpers of the GKA library: work decomposition of the chunked
-// forward, workspace layout, I/O type conversion.  No method arithmetic lives here.
+// forward, workspace layout, I/O type conversion, waits.  No method arithmetic lives here.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -34,35 +34,27 @@ struct FastDiv {
 __host__ __device__ constexpr int chunks_of(int T) { return (T + kChunk - 1) / kChunk; }
 
 // ---------------------------------------------------------------------------------------------
-// Work decomposition.  The B*heads sequences of N = ceil(T/C) chunks each form one flat list of
-// NC = B*heads*N chunks; work item i of G owns the contiguous range [lo(i), lo(i+1)).  A range
-// may cover several sequences and may cut a sequence in the middle.  Where an item's range ends
-// inside a sequence the item's last run is summarised (decay product, delta-H, delta-U) by the
-// summary kernel, the summaries of the items that hold the earlier part of a sequence are folded into
-// the start state of the next item (by a scan kernel on the fp32 path, by the main kernel itself on the
-// tensor-core path), and the main kernel then processes all items independently, carrying (H, U) on
-// chip inside each run.
-// Range boundaries are multiples of `unit` chunks: 2 when every sequence has an even number of chunks
-// and there are at least two chunks per item (the tensor-core kernel pairs chunks into 128-token tiles;
-// even boundaries keep every run an even number of chunks long), else 1.
+// Work decomposition of the state pass on the tensor-core path.  The B*heads sequences of N = ceil(T/128) tiles each form one
+// flat list of NC = B*heads*N tiles; work item i of G owns the contiguous range [lo(i), lo(i+1)).  A range may cover several
+// sequences and may cut a sequence in the middle.  Where an item's range ends inside a sequence the item's last run is
+// summarised (decay product, delta-H, delta-U) by the summary kernel; the summaries of the items that hold the earlier part of a
+// sequence are folded into the start state of the next item, by the state kernel itself or, where many items share a sequence,
+// by a scan kernel before it.  The state kernel then processes all items independently, carrying (H, U) on chip inside each
+// run.  (The fp32 kernels split sequences by rules of their own: gka_recur.cu, gka_fwd_small.cu.)
 // ---------------------------------------------------------------------------------------------
 struct WorkPlan {
-    int BH;        // B * heads
-    int N;         // chunks per sequence
-    long long NC;  // total chunks
+    int N;         // tiles per sequence
+    long long NC;  // total tiles
     int G;         // work items
-    int unit;      // granularity of the range boundaries in chunks (1 or 2)
-    FastDiv divN;  // flat chunk index -> sequence
-    __host__ __device__ long long lo(int i) const { return unit * (((long long)i * (NC / unit)) / G); }
-    __host__ __device__ void set(int bh, int n, int g, bool pairs = true) {
-        BH = bh;
+    FastDiv divN;  // flat tile index -> sequence
+    __host__ __device__ long long lo(int i) const { return ((long long)i * NC) / G; }
+    __host__ __device__ void set(int bh, int n, int g) {
         N = n;
         NC = (long long)bh * n;
         G = g;
         divN.set((unsigned)n);
-        unit = (pairs && n % 2 == 0 && 2LL * g <= NC) ? 2 : 1;
     }
-    // start of the last run of item i (flat chunk index)
+    // start of the last run of item i (flat tile index)
     __host__ __device__ long long last_run_start(int i) const {
         long long l = lo(i), h = lo(i + 1);
         long long s = ((h - 1) / N) * N;
@@ -98,9 +90,8 @@ inline size_t small_workspace_bytes_for(long long pairs, int T, int d) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Tensor-core path (bf16 I/O, d = 128).  Its unit of work is a tile of 128 consecutive tokens of one sequence;
-// a sequence is ceil(T / 128) tiles and the WorkPlan above is then a plan over tiles (N = tiles per sequence,
-// unit 1).  A state kernel walks the plan's items, carries the fp32 (H, U) on chip and stores, for every tile,
+// Tensor-core path (bf16 I/O, d = 128 or 64).  Its unit of work is a tile of 128 consecutive tokens of one sequence.  A state
+// kernel walks the plan's items, carries the fp32 (H, U) on chip and stores, for every tile,
 // the bf16 operand copies of the tile-initial H_0 and U_0 and ||H_0||_F^2; the solve kernel then treats the
 // tiles as independent problems.  Workspace: start states [G][st], summaries [G][st], decay products [G],
 // ||H_0||_F^2 [tiles], bf16 copies [tiles][2][128][128].

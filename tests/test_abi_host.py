@@ -128,7 +128,8 @@ def test_host_call_reports_argument_errors_before_any_copy(lib):
 @pytest.mark.parametrize("io", ["bf16", "f32"])
 def test_work_ranges_partition_the_chunk_list(lib, B, T, heads, G, io):
     """bf16 I/O with head dimension 128 is planned in 128-token tiles (pairs of chunks, the last tile of a
-    sequence with an odd number of chunks holding one), everything else in chunks."""
+    sequence with an odd number of chunks holding one); for everything else the answer is an even split of the chunks (the fp32
+    kernels do not work by it)."""
     N = T // 64
     NC = B * heads * N
     tiles = io == "bf16"

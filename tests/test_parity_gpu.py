@@ -296,7 +296,7 @@ def test_fwd_bf16_native_repeated_calls_are_bit_identical(B, heads, T, d):
 def test_work_items_follow_the_decomposition_rule():
     """Number of work items of the state pass on this device: whole sequences where that is cheaper than cutting them
     (fewer pairs than SMs and short enough sequences; more pairs than SMs with a small divisor), one range per SM
-    otherwise; the fp32 path always takes one range per SM (or one per chunk for small problems)."""
+    otherwise; for fp32 arithmetic, whose kernels split by rules of their own, the answer is an even split of the chunks."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     n = gka.gka_fwd_num_work_items
     assert n(4, 4096, 16, 128) == 64                       # configuration 1: the 64 pairs
