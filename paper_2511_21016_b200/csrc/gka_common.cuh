@@ -179,8 +179,9 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
 }
 
 // 1 / x for x well inside the normal range (the weight schedule of Algorithm 1 divides by 4 - rho^2 omega, between 2 and 4):
-// the hardware's approximation and one Newton step, within one unit in the last place.  Unlike a division it has no rare
-// branch, so the compiler schedules the code around it as one block.
+// the hardware's approximation (relative error at most 2^-23) and one Newton step, whose own error is below 2^-46, so that the last
+// rounding decides: within one unit in the last place.  Unlike a division it has no rare branch, so the compiler schedules the
+// code around it as one block.
 __device__ __forceinline__ float recip(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
