@@ -158,11 +158,16 @@ int gka_fwd_num_work_items(const gka_desc *desc, int chunk) {
         // Where the ranges cut sequences the summary kernel reads all keys and values once more.  Ranges of whole
         // sequences (pairs / k work items of k sequences each, k the smallest divisor of the number of (sequence, head)
         // pairs that leaves at most one item per SM) need no summaries, but may leave SMs idle in the state kernel and
-        // make its run of tiles longer.  Measured per 128-token tile and block: 2.94 us in the state kernel with whole
-        // sequences (2.15 us where two blocks share an item, one per master: at most half as many items as SMs; 1.7 us where four do),
-        // 5.12 us x pairs / SMs for the summary and state kernels with one range per SM, which also cost 36.5 us more
-        // per call (B = 2, 16 heads, T = 4096: 240 -> 220 us with whole sequences; 8 heads, T = 3072: 105.5 -> 91; 16 heads,
-        // T = 4096, just beyond the line: 152.4 in ranges, 153.3 whole).
+        // make its run of tiles longer.  Costs measured at d = 128 per 128-token tile and block: 2.94 us in the state kernel with
+        // whole sequences (2.15 us where two blocks share an item, one per master: at most half as many items as SMs; 1.7 us where
+        // four do), 5.12 us x pairs / SMs for the summary and state kernels with one range per SM, which also cost 36.5 us more
+        // per call.  Both sides, whole sequences against ranges, r = 10:
+        //   d = 128: 16 pairs, 24 tiles each 125 / 138 us, 32 tiles (the line: 36.7) 152 / 152; 32 pairs, 32 tiles 221 / 239, 48
+        //            tiles 321 / 331; 64 pairs, 32 tiles 371 / 416; 256 pairs, 16 tiles 719 / 750
+        //   d = 64:  8 pairs, 16 tiles 64 / 71, 24 tiles 85 / 83; 16 pairs, 22 tiles 101 / 106, 24 tiles (just beyond the line)
+        //            106 / 106, 32 tiles 131 / 118; 32 pairs, 32 tiles 183 / 184, 35 tiles (just beyond) 195 / 192; 64 pairs, 32
+        //            tiles 272 / 301; 256 pairs, 16 tiles 491 / 526
+        // so the same constants serve both (28 shapes at r = 0 and 10: the side taken is never more than 1.8 % the slower one).
         const long long pairs = (long long)desc->B * desc->heads, n = tiles_of(desc->T);
         for (long long k = (pairs + sms - 1) / sms; k <= pairs && k <= 64; ++k) {
             if (pairs % k != 0 || pairs / k > cap) continue;

@@ -87,7 +87,6 @@ __device__ __forceinline__ void mma8_pm_rows(uint32_t d, uint32_t p_tmem, uint32
 }
 
 constexpr uint32_t kIdescKK = make_idesc(128, 128, 0, 0);   // both operands K-major
-constexpr uint32_t kIdescPM = make_idesc(128, 128, 0, 1);   // A from TMEM, B MN-major
 constexpr uint32_t kIdescMM = make_idesc(128, 128, 1, 1);   // both MN-major
 
 #define TMEM_ST8(taddr, r)                                                                                       \

@@ -579,7 +579,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // output stores are complete
             }
         } else if constexpr (!HALF) {
-            // ================================ MMA issuing thread ================================
+            // ================================ MMA issuing thread (128 channels only) ================================
             // Serves the requests of both slots in the order they become ready.  The score tile S is held by a slot
             // from its FROB request until its warps have read the Gram matrix (counted in shared memory), from ITER1 to the issue of
             // ITER2 and from OUT_S to the issue of OUT_O (products run in issue order, so the next owner's score
@@ -601,8 +601,8 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     const uint32_t sbb = bars + 8 * (sl * B_PER_SLOT);
                     const uint32_t sl14 = base14 + ((sl * SLOT_BYTES) >> 4);
                     fence_after();
-                    issue_batch(o, half, sl14 + (BUF_A >> 4), sl14 + (BUF_B >> 4), sl14 + (BUF_C >> 4), tmem + tm_s_of(half, sl),
-                                tmem + tm_r_of(half, sl), tmem + tm_e_of(sl), sbb + 8 * B_MMA_S, sbb + 8 * B_MMA_R, bars + 8 * (B_SC + sl));
+                    issue_batch(o, false, sl14 + (BUF_A >> 4), sl14 + (BUF_B >> 4), sl14 + (BUF_C >> 4), tmem + tm_s_of(false, sl),
+                                tmem + tm_r_of(false, sl), tmem + tm_e_of(sl), sbb + 8 * B_MMA_S, sbb + 8 * B_MMA_R, bars + 8 * (B_SC + sl));
                 };
                 // Bookkeeping of a request of slot sl that has just been issued, together with its follow-up (ITER2 after
                 // ITER1, OUT_O after OUT_S): the slot's next request, counters and tile count.  Returns the counter value
@@ -676,7 +676,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     for (;;) {
                         const int t = 1 - s;
                         const uint32_t s14 = base14 + ((s * SLOT_BYTES) >> 4), t14 = base14 + ((t * SLOT_BYTES) >> 4);
-                        const uint32_t p_kb = s14 + (BUF_A >> 4), p_tmR = tmem + tm_r_of(half, s);
+                        const uint32_t p_kb = s14 + (BUF_A >> 4), p_tmR = tmem + tm_r_of(false, s);
                         const uint32_t p_barR = bars + 8 * (s * B_PER_SLOT + B_MMA_R);
                         const bool t_iter = (t ? left1 : left0) > 0 && (t ? op1 : op0) == OP_ITER1;
                         const uint32_t thr_t = t ? thr1 : thr0;
@@ -695,7 +695,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                         if (gave_up) break;
                         if (o == OP_ITER1) {
                             fence_after();
-                            mma8_pm_rows(p_tmR, tmem + tm_s_of(half, s), p_kb, idesc_r_pm(half));  // ITER2: R += P Khat
+                            mma8_pm_rows(p_tmR, tmem + tm_s_of(false, s), p_kb, idesc_r_pm(false));  // ITER2: R += P Khat
                             mma_commit(p_barR);
                         } else {                                 // OUT_O: the V tile (TMA)
                             wait_bar(bars + 8 * (s * B_PER_SLOT + B_LD_V), til & 1u, abort_addr);
@@ -718,9 +718,9 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                         }
                         // ---- ITER1 of the other slot, at once
                         fence_after();
-                        prod_ek<0>(half, tmem + tm_s_of(half, t), n_tmE, n_kb, kIdescKK);           // S = E Khat^T
+                        prod_ek<0>(false, tmem + tm_s_of(false, t), n_tmE, n_kb, kIdescKK);           // S = E Khat^T
                         mma_commit(bars + 8 * (B_SC + t));
-                        prod_ek<1>(half, tmem + tm_r_of(half, t), n_tmE, n_kb + ((BUF_B - BUF_A) >> 4), idesc_r_kk(half));   // R += E H_0^T
+                        prod_ek<1>(false, tmem + tm_r_of(false, t), n_tmE, n_kb + ((BUF_B - BUF_A) >> 4), idesc_r_kk(false));   // R += E H_0^T
                         if (owner == t) {                        // (its Gram reads are done: it has asked again)
                             if (t) gthr1 += 4u; else gthr0 += 4u;
                             owner = -1;

@@ -52,13 +52,6 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])        \
                  : "r"(taddr)                                                                                             \
                  : "memory")
-#define TMEM_LD2(taddr, r) \
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(taddr) : "memory")
-#define TMEM_LD4(taddr, r)                                                                                    \
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"                                             \
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])                                                         \
-                 : "r"(taddr)                                                                                             \
-                 : "memory")
 #define TMEM_ST16(taddr, r)                                                                                   \
     asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" \
                  ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),   \
@@ -72,22 +65,6 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
                    "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]),            \
                    "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]),            \
                    "=r"(r[30]), "=r"(r[31])                                                                               \
-                 : "r"(taddr)                                                                                             \
-                 : "memory")
-#define TMEM_ST32(taddr, r)                                                                                   \
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"  \
-                 "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),                        \
-                 "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),      \
-                 "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]),          \
-                 "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]),         \
-                 "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])                      \
-                 : "memory")
-// 16 lanes x 32 columns spread over the whole warp: thread l holds rows l/4 and l/4 + 8, and for column
-// block i (8 columns) the pair 2 (l % 4), 2 (l % 4) + 1: r[4 i + 2 h + e] = (row l/4 + 8 h, column 8 i + 2 (l%4) + e)
-#define TMEM_LD_16x256b_x4(taddr, r)                                                                          \
-    asm volatile("tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];" \
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),       \
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])  \
                  : "r"(taddr)                                                                                             \
                  : "memory")
 
@@ -133,14 +110,6 @@ __device__ __forceinline__ float ex2_fast(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-
-// descriptor constants: tile offset and leading-byte-offset field, then the k-step
-__host__ __device__ constexpr uint32_t op_kmaj(uint32_t off) { return (off >> 4) | ((16u >> 4) << 16); }
-__host__ __device__ constexpr uint32_t op_mn(uint32_t off) { return (off >> 4) | ((8192u >> 4) << 16); }
-__host__ __device__ constexpr uint32_t kstep(int ks, int box_bytes) {
-    return (uint32_t)(((ks >> 2) * box_bytes + (ks & 3) * 32) >> 4);
-}
-__host__ __device__ constexpr uint32_t mnstep(int ks) { return (uint32_t)((ks * 2048) >> 4); }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
