@@ -35,8 +35,8 @@
  *   - Supported: d_k == d_v in {16, 32, 64, 128}; chunk == 64; any T >= 1 (a sequence is ceil(T / chunk) chunks, the
  *     last one holds the remaining T mod chunk tokens); n_iter >= 0.
  *   - bf16 I/O with GKA_PREC_NATIVE and T >= 16 runs on the tensor cores (tiles of 128 tokens x 128 channels; head
- *     dimension 64 is zero-extended on chip and skips the zero channels in the contractions over the channels, about
- *     0.83 of the time of 128); f32 I/O, GKA_PREC_HIGH, T < 16 and head dimensions 16 and
+ *     dimension 64 is zero-extended on chip and skips the zero channels in the contractions over the channels: 0.78 of the
+ *     time of 128 at B = 4, 16 heads, T = 4096 and 10 iterations, 0.73 at 30); f32 I/O, GKA_PREC_HIGH, T < 16 and head dimensions 16 and
  *     32 run in fp32 arithmetic on the CUDA cores (16 and 32: an explicit H_t per token in the registers of a few lanes; the
  *     decode calls handle them with one warp per (sequence, head) pair).
  */
@@ -235,7 +235,8 @@ gka_status gka_fwd_work_range(const gka_desc *desc, int chunk, int num_items, in
  *   - Calls no cudaMalloc / cudaFree and no allocating library routine.
  *   - Problems whose scan needs more than the array (gka_fwd_workspace_bytes(desc, chunk) >
  *     gka_noalloc_scratch_bytes()) are rejected with GKA_ERR_WORKSPACE before anything is launched:
- *     fp32 arithmetic: d_k <= 64 fits up to 170 chunks in total (B * heads * ceil(T / chunk)), d_k = 128 up to 42;
+ *     fp32 arithmetic: d_k = 64 fits up to 170 chunks in total (B * heads * ceil(T / 64)), d_k = 128 up to 42; d_k = 32 up to
+ *     2047, d_k = 16 up to 8176 chunks of 32 tokens (B * heads * ceil(T / 32));
  *     bf16 tensor-core path (d_k = 64 or 128): up to 51 tiles of 128 tokens in total (B * heads * ceil(T / 128)).
  *   - The first call on a device looks up the array's device address (cudaGetSymbolAddress) with
  *     that device current; make that first call before any stream capture.

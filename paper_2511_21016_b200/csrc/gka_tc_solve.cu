@@ -39,16 +39,17 @@
 // the first-level instruction cache, so the number of instructions between two hand-overs counts more than their kind.
 // Hence the increment is added to the iterate when it is next unpacked, the diagonal block is masked after the conversion,
 // and there are no separate warps for the scores (as a third party they had to be told whose scores come next, started
-// cold, and shared every scheduler with two update warps).  B = 4, 16 heads, T = 4096, 10 / 30 iterations: 406 / 794 us per
-// call before, 351 / 681 with these.
+// cold, and shared every scheduler with two update warps).  B = 4, 16 heads, T = 4096, 10 / 30 iterations, both builds in turn, 20
+// calls back to back: 406 / 827 us per call before, 354 / 736 with these (413 and 370 at 10 iterations over seconds of
+// calls, where the power cap sets the clock).
 //
 // Head dimension 64 arrives zero-extended to 128 channels (the upper TMA box reads zeros).  The kernel instantiated
 // with HALF leaves out what the zero channels would contribute: contractions over the channels take four k-steps
 // instead of eight, products into R have 64 columns, and the passes of the compute warps stop at channel 64.  R and E then
 // take half of their columns, which leaves room for a score tile per slot: nothing is handed from slot to slot, so a slot is
 // one chain of its four compute warps, and one of their threads issues the slot's products (no issuing thread: a request no
-// longer waits for a thread that serves both slots).  B = 4, 16 heads, T = 2048, 10 / 30 iterations: 179 / 353 us per call with
-// the shared score tile, 153 / 292 with this.
+// longer waits for a thread that serves both slots).  B = 4, 16 heads, T = 2048, 10 / 30 iterations: 177 / 351 us per call with
+// the shared score tile, 152 / 288 with this.
 #include <cuda.h>
 
 #include "gka_common.cuh"

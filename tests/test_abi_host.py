@@ -57,6 +57,16 @@ def test_workspace_bytes_arithmetic(lib):
     assert gka.gka_fwd_workspace_bytes(1, 128, 2, 96) == 0       # unsupported head dim
 
 
+@pytest.mark.parametrize("d,io,tokens,chunks", [(64, gka.GKA_F32, 64, 170), (128, gka.GKA_F32, 64, 42), (32, gka.GKA_F32, 32, 2047),
+                                               (16, gka.GKA_F32, 32, 8176), (64, gka.GKA_BF16, 128, 51), (128, gka.GKA_BF16, 128, 51)])
+def test_builtin_scratch_limits_are_as_stated(lib, d, io, tokens, chunks):
+    """The header states how many chunks (tiles on the tensor-core path) fit the scratch that is built into the library."""
+    limit = lib.gka_noalloc_scratch_bytes()
+    assert gka.gka_fwd_workspace_bytes(1, tokens * chunks, 1, d, io_dtype=io) <= limit
+    assert gka.gka_fwd_workspace_bytes(1, tokens * chunks + 1, 1, d, io_dtype=io) > limit
+    assert gka.gka_fwd_workspace_bytes(chunks, 17, 1, d, io_dtype=io) <= limit < gka.gka_fwd_workspace_bytes(chunks + 1, 17, 1, d, io_dtype=io)
+
+
 def _call_fwd(lib, desc, ptrs, n_iter=1, chunk=64):
     return lib.gka_fwd_chunked(ctypes.byref(desc), *ptrs[:5], n_iter, chunk, *ptrs[5:])
 
