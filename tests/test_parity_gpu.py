@@ -98,17 +98,16 @@ def test_fwd_f32_d128():
 
 
 def test_fwd_f32_items_cut_sequences():
-    """More chunks than SMs, chunk count not a multiple of the item count: every work item starts
-    or ends inside a sequence, so the summary kernel and the cross-item scan carry the state."""
+    """Few long sequences: each is split into many segments whose start states come through the summary and scan kernels."""
     cfg = synth.shrink(SMALL, B=1, heads=3, T=64 * 101, n_iter=2)
     check_fwd(cfg)
 
 
 @pytest.mark.parametrize("io,d", [("f32", 64), ("f32", 128), ("bf16", 128)])
 def test_fwd_slow_fading_state_crosses_many_items(io, d):
-    """Gates close to 1 (sigmoid(N(6,1))): the state of a sequence start is still alive many work items
-    later, so a wrong start state of any item shows (fast-fading gates would hide it).  Several sequences
-    whose boundaries fall inside items."""
+    """Gates close to 1 (sigmoid(N(6,1))): the state of a sequence start is still alive many work items (fp32: segments)
+    later, so a wrong start state of any of them shows (fast-fading gates would hide it).  Several sequences; on the tensor-core
+    path their boundaries fall inside items."""
     cfg = synth.GkaConfig("slow", B=2, heads=3, T=64 * 70, d=d, chunk=64, n_iter=2, io_dtype=io, seed=21,
                           gate_mean=6.0)
     check_fwd(cfg)
@@ -237,7 +236,7 @@ def test_fwd_degenerate_inputs():
     assert np.all(np.isfinite(out))
     assert rel(out, ref["out"]) < TOL_F32
     assert rel(st, ref["state"]) < 1e-5
-    inp["gate"][:, 40, 1] = 0.0                      # exact zero gate: clamped at exp(-80) on device
+    inp["gate"][:, 40, 1] = 0.0                      # exact zero gate
     ref = oracle.fwd(inp["q"], inp["k"], inp["v"], inp["gate"], inp["lam"], 4)
     out, st, fro = run_fwd(inp, 4, False)
     assert np.all(np.isfinite(out)) and rel(out, ref["out"]) < TOL_F32
@@ -274,7 +273,7 @@ def test_fwd_back_to_back_calls_share_a_workspace():
                                          (2, 5, 3840, 128), (4, 40, 200, 128)])
 def test_fwd_bf16_native_repeated_calls_are_bit_identical(B, heads, T, d):
     """The same problem several times over, one workspace: outputs and final states must agree bit for bit in every
-    decomposition of the state pass (whole sequences with one block per master, whole sequences with one block each,
+    decomposition of the state pass (whole sequences with four blocks, with one block per master and with one block each,
     ranges that cut sequences, more pairs than SMs with two whole sequences per work item), and the first call must
     agree with the oracle."""
     cfg = synth.shrink(synth.CONFIGS[1], B=B, heads=heads, T=T, d=d, n_iter=3, seed=31)
@@ -448,7 +447,7 @@ def _beta_for(inp, seed):
 @pytest.mark.parametrize("d", [64, 128])
 def test_fwd_beta_write_f32(d):
     """H_t = gamma_t H_{t-1} + beta_t k k^T, U_t = gamma_t U_{t-1} + beta_t v k^T (Remark on the beta-augmented
-    variant, Section 4.1), fp32 path, sequences cut by work items."""
+    variant, Section 4.1), fp32 path, sequences split into segments."""
     cfg = synth.shrink(synth.CONFIGS[0], d=d, T=384, heads=3)
     inp = synth.make_inputs(cfg)
     beta = _beta_for(inp, 7)
@@ -637,8 +636,8 @@ def test_fwd_bf16_very_short_sequences_under_the_adaptive_rule(T, d):
 # --------------------------------------------------------------------------- head dimensions 16 and 32
 @pytest.mark.parametrize("d,bf16,precision", [(16, False, 0), (32, False, 0), (16, True, 0), (32, True, 0), (32, True, 1)])
 def test_fwd_small_head_dimensions(d, bf16, precision):
-    """Head dimensions 16 and 32 run on the 64-channel fp32 kernels, zero-extended on chip (whatever the I/O dtype and
-    precision): several heads side by side, a ragged last chunk, work items that cut sequences, a caller-supplied
+    """Head dimensions 16 and 32 run on fp32 kernels of their own (whatever the I/O dtype and
+    precision): several heads side by side, many 32-token chunks and a ragged last one, a caller-supplied
     initial state in the caller's d x d layout, write strengths and the alpha-connection; outputs, norms, final state
     and the solve alone against the oracle."""
     B, heads, T = 2, 5, 64 * 40 + 23
