@@ -564,6 +564,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     const TileInfo ti = tile_info(a, t_lo + k);
                     if (!solve_only) {
                         wait_bar(sb + 8 * B_QF, (uint32_t)(j & 1), abort_addr);
+                        if (aborted(abort_addr)) break;
                         mbar_expect_tx(sb + 8 * B_LD_V, 32768u);
                         tma_load_tile3(&tmV, sl + BUF_C, sb + 8 * B_LD_V, ti.h * a.d, tile_x_hi(ti.h, a.d, a.heads), ti.n * NT, ti.b);
                     }
@@ -827,16 +828,17 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             const GateScalars *const gs = &sc->g[j & 1];
             const TileInfo ti = tile_info(a, tile);
             const bool valid = c < ti.ntok;
-            // loads of the slot's next tile, issued by the leader as soon as the buffer's last reader is done
+            // loads of the slot's next tile, issued by the leader as soon as the buffer's last reader is done (none once a wait has
+            // given up: a barrier whose copy never landed takes no second announcement)
             auto load_next_k = [&]() {
-                if (leader && more) {
+                if (leader && more && !aborted(abort_addr)) {
                     const TileInfo tn = tile_info(a, tile + kSlots);
                     mbar_expect_tx(sb + 8 * B_LD_K, 32768u);
                     tma_load_tile3(&tmK, sl + BUF_A, sb + 8 * B_LD_K, tn.h * a.d, tile_x_hi(tn.h, a.d, a.heads), tn.n * NT, tn.b);
                 }
             };
             auto load_next_h = [&]() {
-                if (leader && more) {
+                if (leader && more && !aborted(abort_addr)) {
                     mbar_expect_tx(sb + 8 * B_LD_H, 32768u);
                     tma_load_tile2(&tmS, sl + BUF_B, sb + 8 * B_LD_H, (int)((tile + kSlots) * 256));
                 }
@@ -845,7 +847,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 if (solve_only) {
                     load_next_k();
                     load_next_h();
-                } else if (leader) {
+                } else if (leader && !aborted(abort_addr)) {
                     mbar_expect_tx(sb + 8 * B_LD_U, 32768u);
                     tma_load_tile2(&tmS, sl + BUF_B, sb + 8 * B_LD_U, (int)(tile * 256 + 128));
                 }
