@@ -135,7 +135,9 @@ __global__ void __launch_bounds__(32 * kSumWarps) small_summary(SmallArgs a) {
     if (l == 0) a.decay[(size_t)p.pair * a.chunks + p.chunk] = wt;
 }
 
-// ---- start states in place and the final state: four state elements per thread, blockIdx.y = pair
+// ---- start states in place and the final state: four state elements per thread, blockIdx.y = pair.  Bound by latency: a load
+// behind a store to the same array waits for it, so eight chunks are loaded ahead of their stores (in a loop over the chunks every
+// chunk was a round trip to memory).  64 x 8 pairs, T = 196, d = 16, 30 iterations: 91.7 -> 84.6 us for the call.
 __global__ void small_scan(SmallArgs a, int st, int elements) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -145,12 +147,21 @@ __global__ void small_scan(SmallArgs a, int st, int elements) {
         float4 c = a.state_in ? ld4(a.state_in + (size_t)pair * st + e) : make_float4(0.f, 0.f, 0.f, 0.f);
         float4 *p = reinterpret_cast<float4 *>(a.slot + (size_t)pair * a.chunks * st + e);
         const float *dec = a.decay + (size_t)pair * a.chunks;
-#pragma unroll 8
-        for (int n = 0; n < a.chunks; ++n) {
-            const float4 d = p[(size_t)n * (st / 4)];
-            const float g = dec[n];
-            p[(size_t)n * (st / 4)] = c;
-            c.x = fmaf(g, c.x, d.x); c.y = fmaf(g, c.y, d.y); c.z = fmaf(g, c.z, d.z); c.w = fmaf(g, c.w, d.w);
+        for (int n0 = 0; n0 < a.chunks; n0 += 8) {
+            float4 d[8];
+            float g[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (n0 + i < a.chunks) {
+                    d[i] = p[(size_t)(n0 + i) * (st / 4)];
+                    g[i] = dec[n0 + i];
+                }
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (n0 + i < a.chunks) {
+                    p[(size_t)(n0 + i) * (st / 4)] = c;
+                    c.x = fmaf(g[i], c.x, d[i].x); c.y = fmaf(g[i], c.y, d[i].y); c.z = fmaf(g[i], c.z, d[i].z); c.w = fmaf(g[i], c.w, d[i].w);
+                }
         }
         if (a.state_out) st4(a.state_out + (size_t)pair * st + e, c);
     }
