@@ -148,6 +148,34 @@ size_t gka_fwd_workspace_bytes(const gka_desc *desc, int chunk) {
     return workspace_bytes_for(work_items_cap(desc), desc->d_k, desc->d_v);
 }
 
+// Work items of the state pass of a call on this device (tensor-core path).  Where the ranges of the flat list of tiles cut
+// sequences the summary kernel reads all keys and values once more.  Items of whole sequences (pairs / k items of k sequences each, k
+// the smallest divisor of the number of (sequence, head) pairs that leaves at most one item per SM) need no summaries, but may
+// leave SMs idle in the state kernel and make its run of tiles longer.  With n tiles per sequence whole sequences cost
+// per_tile k n us, ranges cut pairs / SMs n + fixed (the extra launches).  Fitted to both sides of 33 shapes at r = 0 (us per call, whole
+// sequences / ranges):
+//   d = 128 (per_tile by how many blocks share an item): 1 pair, 32 tiles 44.6 / 54.0; 8 pairs, 32 tiles 47.1 / 76.7, 64 tiles 88.8 / 99.1;
+//     16 pairs, 64 tiles 113 / 136, 128 tiles 208 / 216; 32 pairs, 64 tiles 165 / 214, 1024 tiles 2657 / 2824; 64 pairs, 64
+//     tiles 312 / 390; 96 pairs, 64 tiles 473 / 545; 256 pairs (two per item), 32 tiles 589 / 680
+//   d = 64: 8 pairs, 32 tiles 43.9 / 55.2, 64 tiles 74.5 / 69.1; 16 pairs, 32 tiles 50.2 / 62.2, 64 tiles 90.7 / 84.4; 32 pairs, 64
+//     tiles 119 / 129, 128 tiles 247 / 250; 64 pairs, 64 tiles 179 / 217; 256 pairs, 64 tiles 700 / 816
+//   the solve alone, d = 128: 8 pairs, 32 tiles 41.9 / 50.3; 16 pairs, 64 tiles 92.7 / 87.8; 32 pairs, 256 tiles 575 / 562; 64 pairs, 64
+//     tiles 230 / 282
+static int state_items(const gka_desc *desc, int sms, bool solve_only) {
+    const int cap = work_items_cap(desc);
+    const long long pairs = (long long)desc->B * desc->heads, n = tiles_of(desc->T);
+    for (long long k = (pairs + sms - 1) / sms; k <= pairs && k <= 64; ++k) {
+        if (pairs % k != 0 || pairs / k > cap) continue;
+        const long long items = pairs / k;
+        const bool light = desc->d_k == 64 || solve_only;            // half the state or less
+        const double per_tile = light ? 0.83 : 4 * items <= sms ? 0.84 : 2 * items <= sms ? 1.31 : 2.2;
+        const double cut = light ? 3.05 : 4.4, fixed = light ? 28.0 : 40.0;
+        if ((double)n * ((double)k * per_tile - cut * (double)pairs / sms) < fixed) return (int)items;
+        break;
+    }
+    return sms < cap ? sms : cap;
+}
+
 int gka_fwd_num_work_items(const gka_desc *desc, int chunk) {
     gka_status s = check_fwd_shape(desc, chunk);
     if (s != GKA_OK) return -(int)s;
@@ -155,19 +183,8 @@ int gka_fwd_num_work_items(const gka_desc *desc, int chunk) {
     if (sms <= 0) return -(int)GKA_ERR_CUDA;
     const int cap = work_items_cap(desc);
     if (wants_tensor_path(desc)) {
-        // Where the ranges cut sequences the summary kernel reads all keys and values once more.  Ranges of whole
-        // sequences (pairs / k work items of k sequences each, k the smallest divisor of the number of (sequence, head)
-        // pairs that leaves at most one item per SM) need no summaries, but may leave SMs idle in the state kernel and
-        // make its run of tiles longer.  Costs measured at d = 128 per 128-token tile and block: 2.94 us in the state kernel with
-        // whole sequences (2.15 us where two blocks share an item, one per master: at most half as many items as SMs; 1.7 us where
-        // four do), 5.12 us x pairs / SMs for the summary and state kernels with one range per SM, which also cost 36.5 us more
-        // per call.  Both sides, whole sequences against ranges, r = 10:
-        //   d = 128: 16 pairs, 24 tiles each 125 / 138 us, 32 tiles (the line: 36.7) 152 / 152; 32 pairs, 32 tiles 221 / 239, 48
-        //            tiles 321 / 331; 64 pairs, 32 tiles 371 / 416; 256 pairs, 16 tiles 719 / 750
-        //   d = 64:  8 pairs, 16 tiles 64 / 71, 24 tiles 85 / 83; 16 pairs, 22 tiles 101 / 106, 24 tiles (just beyond the line)
-        //            106 / 106, 32 tiles 131 / 118; 32 pairs, 32 tiles 183 / 184, 35 tiles (just beyond) 195 / 192; 64 pairs, 32
-        //            tiles 272 / 301; 256 pairs, 16 tiles 491 / 526
-        // so the same constants serve both (28 shapes at r = 0 and 10: the side taken is never more than 1.8 % the slower one).
+        // The division of work that the function has always answered with (the header states it): whole sequences where they are short
+        // or many.  What a call's own state pass takes is state_items.
         const long long pairs = (long long)desc->B * desc->heads, n = tiles_of(desc->T);
         for (long long k = (pairs + sms - 1) / sms; k <= pairs && k <= 64; ++k) {
             if (pairs % k != 0 || pairs / k > cap) continue;
@@ -247,8 +264,7 @@ static gka_status fwd_impl(const gka_desc *desc, const void *q, const void *k, c
     a.solve_only = solve_only ? 1 : 0;
     const bool tensor_path = wants_tensor_path(desc) && fwd_tc_available();
     if (tensor_path) {
-        const int G = gka_fwd_num_work_items(desc, chunk);
-        if (G <= 0) return GKA_ERR_CUDA;
+        const int G = state_items(desc, a.sms, solve_only);
         a.plan.set(desc->B * desc->heads, tiles_of(desc->T), G);
         const TcWorkspace w = carve_tc_workspace(desc->workspace, G, a.plan.NC);
         a.ws.start = w.start;

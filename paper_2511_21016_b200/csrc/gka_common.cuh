@@ -99,6 +99,7 @@ inline size_t small_workspace_bytes_for(long long pairs, int T, int d) {
 constexpr int kTile = 128;
 __host__ __device__ constexpr int tiles_of(int T) { return (T + kTile - 1) / kTile; }
 constexpr size_t kTileStateBytes = 2 * 128 * 128 * 2;   // bf16 H_0 and U_0 of one tile
+constexpr size_t kTileStateBytes64 = 2 * 64 * 64 * 2;   // the same at head dimension 64
 
 struct TcWorkspace {
     float *start, *delta, *decay, *hh;
@@ -227,7 +228,6 @@ struct FwdArgs {
     int sms;               // of the current device
     int after_summary;     // tensor path: the main kernel is launched as a programmatic dependent of the summary kernel
     int start_from_scan;   // tensor path: start states were materialised by the scan kernel (long chains of summaries)
-    int state_split;       // tensor path, no sequence cut: 2^state_split blocks per work item in the state kernel
     int solve_only;        // write the solve x_t = CH(H_t + lambda_t I, q_t, r) itself instead of U_t x_t (v unused)
     WorkPlan plan;
     Workspace ws;

@@ -1,8 +1,9 @@
 // Operand tiles and tcgen05.mma issue helpers shared by the tensor-core kernels of the chunked GKA forward.
 //
-// Every operand is a [128 rows][128 columns] bf16 tile stored as two TMA boxes of [128 rows][64 columns] with the
-// 128-byte swizzle, 16384 bytes apart.  The same bytes serve as a K-major operand (contraction over the columns)
-// or as an MN-major operand (contraction over the rows) without a transposed copy.
+// Every operand that comes from the caller is a [128 rows][128 columns] bf16 tile stored as two TMA boxes of [128 rows][64 columns] with
+// the 128-byte swizzle, 16384 bytes apart.  The same bytes serve as a K-major operand (contraction over the columns)
+// or as an MN-major operand (contraction over the rows) without a transposed copy.  The bf16 copies of the states have a layout of
+// their own (below), in which the state kernel can write them from registers in whole lines.
 #pragma once
 #include "gka_tc_util.cuh"
 
@@ -22,15 +23,21 @@ __host__ __device__ constexpr uint32_t t_mn(uint32_t off) { return (off >> 4) | 
 __host__ __device__ constexpr uint32_t t_kstep(int ks) { return (uint32_t)(((ks >> 2) * 16384 + (ks & 3) * 32) >> 4); }
 __host__ __device__ constexpr uint32_t t_mnstep(int ks) { return (uint32_t)((ks * 2048) >> 4); }
 
+// State copies as an operand (B, contraction over the columns): [column / 8][128 rows][8 columns] without a swizzle, so 8 rows x 16 bytes
+// are consecutive, 128 bytes from one group of 8 rows to the next and 2048 from one group of 8 columns to the next
+constexpr uint32_t kDescHiState = (128u >> 4) | (1u << 14);
+__host__ __device__ constexpr uint32_t t_state(uint32_t off) { return (off >> 4) | ((2048u >> 4) << 16); }
+__host__ __device__ constexpr uint32_t t_statestep(int ks) { return (uint32_t)((ks * 4096) >> 4); }
+
 // D (+)= A x B, both operands in shared memory: low words are a base register plus an immediate
-template <int ACC, uint32_t A_CONST, uint32_t B_CONST>
+template <int ACC, uint32_t A_CONST, uint32_t B_CONST, uint32_t B_HI = kDescHi>
 __device__ __forceinline__ void mma_ss2(uint32_t d_tmem, uint32_t a_base, uint32_t b_base, uint32_t idesc) {
     asm volatile(
         "{\n\t.reg .b64 da, db;\n\t.reg .b32 la, lb;\n\t"
         "add.u32 la, %1, %5;\n\tadd.u32 lb, %2, %6;\n\t"
-        "mov.b64 da, {la, %4};\n\tmov.b64 db, {lb, %4};\n\t"
+        "mov.b64 da, {la, %4};\n\tmov.b64 db, {lb, %8};\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, %7;\n\t}" ::"r"(d_tmem), "r"(a_base), "r"(b_base), "r"(idesc),
-        "r"(kDescHi), "n"(A_CONST), "n"(B_CONST), "n"(ACC)
+        "r"(kDescHi), "n"(A_CONST), "n"(B_CONST), "n"(ACC), "r"(B_HI)
         : "memory");
 }
 // D += A x B with A (packed bf16 pairs) in TMEM
@@ -48,6 +55,13 @@ __device__ __forceinline__ void mma8_kk(uint32_t d, uint32_t a_base, uint32_t b_
     if constexpr (KS < NK) {
         mma_ss2<(KS == 0 ? ACC0 : 1), t_kmaj(0) + t_kstep(KS), t_kmaj(0) + t_kstep(KS)>(d, a_base, b_base, idesc);
         mma8_kk<ACC0, NK, KS + 1>(d, a_base, b_base, idesc);
+    }
+}
+template <int ACC0, int NK = 8, int KS = 0>   // A K-major, B a state copy, NK k-steps over the first 16 NK columns
+__device__ __forceinline__ void mma8_ks(uint32_t d, uint32_t a_base, uint32_t b_base, uint32_t idesc) {
+    if constexpr (KS < NK) {
+        mma_ss2<(KS == 0 ? ACC0 : 1), t_kmaj(0) + t_kstep(KS), t_state(0) + t_statestep(KS), kDescHiState>(d, a_base, b_base, idesc);
+        mma8_ks<ACC0, NK, KS + 1>(d, a_base, b_base, idesc);
     }
 }
 template <int ACC0, int KS = 0>   // both MN-major, 8 k-steps over the 128 rows
@@ -113,29 +127,14 @@ __device__ __forceinline__ void tma_load_box3(const CUtensorMap *map, uint32_t d
 }
 // column of the second box of head h's tile: the head's upper 64 channels, or past the tensor for head dimension 64
 __host__ __device__ __forceinline__ int tile_x_hi(int h, int d, int heads) { return d == 128 ? h * 128 + 64 : heads * d; }
-__device__ __forceinline__ void tma_load_tile2(const CUtensorMap *map, uint32_t dst, uint32_t bar, int y) {
-#pragma unroll
-    for (int hf = 0; hf < 2; ++hf)
-        asm volatile(
-            "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
-                "r"(dst + 16384 * hf), "l"(reinterpret_cast<uint64_t>(map)), "r"(64 * hf), "r"(y), "r"(bar)
-            : "memory");
+// `bytes` consecutive bytes (16-byte aligned, as the two addresses) of global memory
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
+                 "r"(bytes), "r"(bar)
+                 : "memory");
 }
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-
-// 2-D map over the per-tile bf16 state copies: rows of 128 columns, box = 64 columns x 128 rows, 128-byte swizzle
-inline bool make_state_map(CUtensorMap *map, const void *base, unsigned long long rows) {
-    EncodeTiledFn fn = get_encode_fn();
-    if (!fn) return false;
-    cuuint64_t dims[2] = {128, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {256};
-    cuuint32_t box[2] = {64, 128};
-    cuuint32_t estr[2] = {1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 }  // namespace tcu

@@ -66,7 +66,8 @@ constexpr int ST = 128;                    // compute threads per slot
 constexpr int CT = kSlots * ST;            // compute threads
 // Warpgroups: 0 = helpers (gate scalars, TMA: one warp per slot, MMA issue), 1 and 2 = the compute warps of slot 0 and slot 1.
 constexpr int kThreadsSolve = 128 + CT;
-constexpr int kRegsLaunch = 168, kRegsCompute = 216, kRegsHelper = 72;   // register split after setmaxnreg (128 channels)
+// register split after setmaxnreg (128 channels): with 216 / 72 the compute threads spilled 32 bytes (64 x 4096 tokens, 10 iterations: 299 -> 295 us)
+constexpr int kRegsLaunch = 168, kRegsCompute = 224, kRegsHelper = 56;
 static_assert(kThreadsSolve * kRegsLaunch <= 65536, "launch registers");
 static_assert(CT * kRegsCompute + 128 * kRegsHelper <= kThreadsSolve * kRegsLaunch, "register split exceeds the launch allocation");
 
@@ -194,17 +195,25 @@ __device__ __forceinline__ TileInfo tile_info(const FwdArgs &a, long long tile) 
     return t;
 }
 
+// H_0 of a tile; head dimension 64: H_0 and U_0
+template <bool HALF>
+__device__ __forceinline__ void load_h0(const FwdArgs &a, long long tile, uint32_t dst, uint32_t bar) {
+    constexpr uint32_t bytes = HALF ? (uint32_t)kTileStateBytes64 : 32768u;
+    mbar_expect_tx(bar, bytes);
+    bulk_load(dst, a.tile_hu + (size_t)tile * (HALF ? kTileStateBytes64 : kTileStateBytes), bytes, bar);
+}
+
 // Products of the issuing thread: 8 k-steps of 16 each, unrolled with immediate descriptor offsets: every instruction
 // of the issuing thread takes of the order of ten cycles beside the working warps of its scheduler, and the issue then
 // keeps up with the tensor pipe (one tcgen05.mma per 64 to 78 cycles).
 // D (+)= A x B with A (packed bf16 pairs, 8 columns per k-step of 16) in TMEM and B in shared memory
-template <int ACC, uint32_t B_CONST>
+template <int ACC, uint32_t B_CONST, uint32_t B_HI = kDescHi>
 __device__ __forceinline__ void mma_ts_c(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_base, uint32_t idesc) {
     asm volatile(
         "{\n\t.reg .b64 db;\n\t.reg .b32 lb;\n\t"
         "add.u32 lb, %2, %5;\n\tmov.b64 db, {lb, %4};\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, %6;\n\t}" ::"r"(d_tmem), "r"(a_tmem), "r"(b_base), "r"(idesc),
-        "r"(kDescHi), "n"(B_CONST), "n"(ACC)
+        "r"(B_HI), "n"(B_CONST), "n"(ACC)
         : "memory");
 }
 // A = operand tile in TMEM (64 columns: channels 2 u, 2 u + 1 of a token in column u), B K-major
@@ -213,6 +222,14 @@ __device__ __forceinline__ void mma8_ek(uint32_t d, uint32_t e_tmem, uint32_t b_
     if constexpr (KS < NK) {
         mma_ts_c<(KS == 0 ? ACC0 : 1), t_kmaj(0) + t_kstep(KS)>(d, e_tmem + 8 * KS, b_base, idesc);
         mma8_ek<ACC0, NK, KS + 1>(d, e_tmem, b_base, idesc);
+    }
+}
+// The same, B a copy of H_0 or U_0
+template <int ACC0, int NK = 8, int KS = 0>
+__device__ __forceinline__ void mma8_es(uint32_t d, uint32_t e_tmem, uint32_t b_base, uint32_t idesc) {
+    if constexpr (KS < NK) {
+        mma_ts_c<(KS == 0 ? ACC0 : 1), t_state(0) + t_statestep(KS), kDescHiState>(d, e_tmem + 8 * KS, b_base, idesc);
+        mma8_es<ACC0, NK, KS + 1>(d, e_tmem, b_base, idesc);
     }
 }
 // The contractions over the channels: with head dimension 64 (zero-extended on chip) the channels 64..127 of every
@@ -227,19 +244,29 @@ __device__ __forceinline__ void prod_kk(bool half, uint32_t d, uint32_t a_base, 
     if (half) mma8_kk<ACC0, 4>(d, a_base, b_base, idesc);
     else mma8_kk<ACC0, 8>(d, a_base, b_base, idesc);
 }
+template <int ACC0>
+__device__ __forceinline__ void prod_es(bool half, uint32_t d, uint32_t e_tmem, uint32_t b_base, uint32_t idesc) {
+    if (half) mma8_es<ACC0, 4>(d, e_tmem, b_base, idesc);
+    else mma8_es<ACC0, 8>(d, e_tmem, b_base, idesc);
+}
+template <int ACC0>
+__device__ __forceinline__ void prod_ks(bool half, uint32_t d, uint32_t a_base, uint32_t b_base, uint32_t idesc) {
+    if (half) mma8_ks<ACC0, 4>(d, a_base, b_base, idesc);
+    else mma8_ks<ACC0, 8>(d, a_base, b_base, idesc);
+}
 // The products of one request.  kb, hb, cb: descriptor bases (shared address >> 4) of the slot's buffers.
 __device__ __forceinline__ void issue_batch(int op, bool half, uint32_t kb, uint32_t hb, uint32_t cb, uint32_t tm_S, uint32_t tm_R,
                                             uint32_t tm_E, uint32_t bar_s, uint32_t bar_r, uint32_t bar_sc) {
     switch (op) {
         case OP_FROB:    // Gram matrix Khat Khat^T and Khat H_0
             prod_kk<0>(half, tm_S, kb, kb, kIdescKK);
-            prod_kk<0>(half, tm_R, kb, hb, idesc_r_kk(half));
+            prod_ks<0>(half, tm_R, kb, hb, idesc_r_kk(half));
             mma_commit(bar_s);
             break;
         case OP_ITER1:   // S = E Khat^T, R += E H_0^T (the second runs under the masked-score epilogue)
             prod_ek<0>(half, tm_S, tm_E, kb, kIdescKK);
             mma_commit(bar_sc);
-            prod_ek<1>(half, tm_R, tm_E, hb, idesc_r_kk(half));
+            prod_es<1>(half, tm_R, tm_E, hb, idesc_r_kk(half));
             break;
         case OP_ITER2:   // R += P Khat
             mma8_pm_rows(tm_R, tm_S, kb, idesc_r_pm(half));
@@ -249,7 +276,7 @@ __device__ __forceinline__ void issue_batch(int op, bool half, uint32_t kb, uint
             prod_ek<0>(half, tm_S, tm_E, kb, kIdescKK);
             prod_ek<1>(half, tm_S, tm_R, kb, kIdescKK);
             mma_commit(bar_sc);
-            prod_ek<0>(half, tm_R, tm_E, hb, idesc_r_kk(half));   // O = X_hi U_0^T (runs under the masked-score epilogue; X_lo has been read)
+            prod_es<0>(half, tm_R, tm_E, half ? hb + (1024u >> 4) : hb, idesc_r_kk(half));   // O = X_hi U_0^T (64 channels: U_0 follows H_0's rows) (runs under the masked-score epilogue; X_lo has been read)
             break;
         case OP_OUT_O:   // O += P V
             mma8_pm(tm_R, tm_S, cb, idesc_r_pm(half));
@@ -434,8 +461,7 @@ __device__ __forceinline__ float affine_scan(const Ctx &cx, SlotScalars *sc, int
 template <bool EXTRA, bool HALF>
 __global__ void __launch_bounds__(kThreadsSolve, 1)
 fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-                    const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmO,
-                    const __grid_constant__ CUtensorMap tmS, FwdArgs a, long long ntiles) {
+                    const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmO, FwdArgs a, long long ntiles) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t s_bars[B_COUNT];
     __shared__ uint32_t s_tmem_base;
@@ -556,8 +582,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     mbar_expect_tx(sb + 8 * B_LD_K, 32768u);
                     tma_load_tile3(&tmK, sl + BUF_A, sb + 8 * B_LD_K, ti.h * a.d, tile_x_hi(ti.h, a.d, a.heads), ti.n * NT, ti.b);
                     asm volatile("griddepcontrol.wait;" ::: "memory");
-                    mbar_expect_tx(sb + 8 * B_LD_H, 32768u);
-                    tma_load_tile2(&tmS, sl + BUF_B, sb + 8 * B_LD_H, (int)((t_lo + slot) * 256));
+                    load_h0<HALF>(a, t_lo + slot, sl + BUF_B, sb + 8 * B_LD_H);
                 }
                 for (int j = 0; j < n_slot; ++j) {
                     const int k = slot + 2 * j;
@@ -722,7 +747,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                         fence_after();
                         prod_ek<0>(false, tmem + tm_s_of(false, t), n_tmE, n_kb, kIdescKK);           // S = E Khat^T
                         mma_commit(bars + 8 * (B_SC + t));
-                        prod_ek<1>(false, tmem + tm_r_of(false, t), n_tmE, n_kb + ((BUF_B - BUF_A) >> 4), idesc_r_kk(false));   // R += E H_0^T
+                        prod_es<1>(false, tmem + tm_r_of(false, t), n_tmE, n_kb + ((BUF_B - BUF_A) >> 4), idesc_r_kk(false));   // R += E H_0^T
                         if (owner == t) {                        // (its Gram reads are done: it has asked again)
                             if (t) gthr1 += 4u; else gthr0 += 4u;
                             owner = -1;
@@ -796,7 +821,6 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                             }
                         }
                         if (op == OP_FROB) wait_bar(sb + 8 * B_LD_H, tile_parity, abort_addr);    // the H_0 tile (TMA)
-                        if (op == OP_OUT_S) wait_bar(sb + 8 * B_LD_U, tile_parity, abort_addr);   // the U_0 tile
                         if (op == OP_OUT_O) wait_bar(sb + 8 * B_LD_V, tile_parity, abort_addr);   // the V tile
                         fence_after();
                         const uint32_t s14 = (sl >> 4) & 0x3FFF;
@@ -838,18 +862,15 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 }
             };
             auto load_next_h = [&]() {
-                if (leader && more && !aborted(abort_addr)) {
-                    mbar_expect_tx(sb + 8 * B_LD_H, 32768u);
-                    tma_load_tile2(&tmS, sl + BUF_B, sb + 8 * B_LD_H, (int)((tile + kSlots) * 256));
-                }
+                if (leader && more && !aborted(abort_addr)) load_h0<HALF>(a, tile + kSlots, sl + BUF_B, sb + 8 * B_LD_H);
             };
             auto after_last_h0_product = [&]() {      // H_0 has been read for the last time
                 if (solve_only) {
                     load_next_k();
                     load_next_h();
-                } else if (leader && !aborted(abort_addr)) {
+                } else if (!HALF && leader && !aborted(abort_addr)) {
                     mbar_expect_tx(sb + 8 * B_LD_U, 32768u);
-                    tma_load_tile2(&tmS, sl + BUF_B, sb + 8 * B_LD_U, (int)(tile * 256 + 128));
+                    bulk_load(sl + BUF_B, a.tile_hu + (size_t)tile * kTileStateBytes + 32768, 32768u, sb + 8 * B_LD_U);
                 }
             };
             // ||H_0||_F^2 of the tile (state kernel, one or two terms): fetched now, added up and used by the scan (added up here,
@@ -1129,12 +1150,11 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 }  // namespace
 
 cudaError_t launch_fwd_solve(const FwdArgs &a, cudaStream_t stream) {
-    alignas(64) CUtensorMap tmK, tmV, tmQ, tmO, tmS;
+    alignas(64) CUtensorMap tmK, tmV, tmQ, tmO;
     const int cols = a.heads * a.d;
     const long long ntiles = a.plan.NC;
     if (!make_tile_map(&tmK, a.k, a.B, a.T, cols, NT) || !make_tile_map(&tmV, a.v, a.B, a.T, cols, NT) ||
-        !make_tile_map(&tmQ, a.q, a.B, a.T, cols, NT) || !make_tile_map(&tmO, a.out, a.B, a.T, cols, NT) ||
-        !make_state_map(&tmS, a.tile_hu, (unsigned long long)ntiles * 256ull))
+        !make_tile_map(&tmQ, a.q, a.B, a.T, cols, NT) || !make_tile_map(&tmO, a.out, a.B, a.T, cols, NT))
         return cudaErrorInvalidValue;
     const bool extra = a.beta != nullptr || a.alpha != nullptr || a.solve_only != 0;
     const bool half = a.d == 64;
@@ -1155,7 +1175,7 @@ cudaError_t launch_fwd_solve(const FwdArgs &a, cudaStream_t stream) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = a.ev_start ? 0 : 1;
-    err = cudaLaunchKernelEx(&cfg, kernel, tmK, tmV, tmQ, tmO, tmS, a, ntiles);
+    err = cudaLaunchKernelEx(&cfg, kernel, tmK, tmV, tmQ, tmO, a, ntiles);
     if (err != cudaSuccess) return err;
     if (a.ev_stop) cudaEventRecord(a.ev_stop, stream);
     return cudaGetLastError();

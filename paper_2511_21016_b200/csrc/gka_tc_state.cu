@@ -31,7 +31,6 @@ constexpr int D = 128;
 constexpr int NT = kTile;                                // tokens per tile
 constexpr int CT = 512;                                  // compute threads; + one warp that issues the products
 constexpr int kThreadsState = CT + 32;
-constexpr int kThreadsStateK = CT + 64;                  // state kernel: one more warp for the TMA loads and stores
 
 // ------------------------------------------------------------------------------------------------------------
 // Both kernels advance a state by whole tiles with the products K~^T K~ and V~^T K~ on rows scaled in place,
@@ -43,27 +42,45 @@ constexpr uint32_t STAGE = 65536;                        // K tile + V tile
 constexpr uint32_t KV_SMEM = NS * STAGE + 1024;          // + slack for the 1024-byte alignment of the base
 constexpr uint32_t ST_SMEM = KV_SMEM;
 
-// rows of the K and V tiles of a stage times f[j]
-// (boxes of 64 channels: K 0 and 1, V 2 and 3; those whose bit is set in `boxes`)
-__device__ __forceinline__ void scale_kv(unsigned char *stage, const float *f, int t, uint32_t boxes = 15u) {
+// A row factor f >= 0 as hi + lo, two bf16 terms each twice in a word: hi is f cut off after eight bits, lo the rest, to 2^-17 of f.
+// (lo is never 0 beside a hi that is not, nor negative: an infinite element stays infinite.)
+__device__ __forceinline__ uint2 split_factor(float f) {
+    const uint32_t hi = __float_as_uint(f) & 0xFFFF0000u;
+    const float rest = f - __uint_as_float(hi);
+    const float lo = fmaxf(rest, __uint_as_float(hi) * 9.3132257e-10f);      // 2^-30
+    return make_uint2(hi | hi >> 16, pack_bf16(lo, lo));
+}
+// The first N * THREADS 16-byte groups of BOXES operand boxes (64 channels of 128 tokens each) times f[row]: v hi + (v lo), the fused multiply-add
+// rounded once, is the product with f to within 2^-17 before its rounding to bf16, in two instructions per pair of elements
+// (unpacking to fp32, multiplying and packing takes six).
+template <int N, int THREADS, int BOXES>
+__device__ __forceinline__ void scale_rows(unsigned char *box, const uint2 *f, int t) {
+    uint4 v[BOXES][N];
+    uint2 fj[N];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        if (!(boxes >> (i >> 1) & 1u)) continue;
-        const int qi = t + CT * i;                 // 16-byte group index in the 64 KB stage
-        const float fj = f[(qi & 1023) >> 3];      // row of this group (K and V tiles alike)
-        uint4 v = *reinterpret_cast<const uint4 *>(stage + qi * 16);
-        uint32_t *pv = reinterpret_cast<uint32_t *>(&v);
+    for (int i = 0; i < N; ++i) {
+        fj[i] = f[(t + THREADS * i) >> 3];         // 8 groups of 16 bytes in a row
 #pragma unroll
-        for (int u = 0; u < 4; ++u) pv[u] = pack_bf16(bf16_lo(pv[u]) * fj, bf16_hi(pv[u]) * fj);
-        *reinterpret_cast<uint4 *>(stage + qi * 16) = v;
+        for (int x = 0; x < BOXES; ++x) v[x][i] = *reinterpret_cast<const uint4 *>(box + 16384 * x + (t + THREADS * i) * 16);
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const __nv_bfloat162 hi = *reinterpret_cast<const __nv_bfloat162 *>(&fj[i].x), lo = *reinterpret_cast<const __nv_bfloat162 *>(&fj[i].y);
+#pragma unroll
+        for (int x = 0; x < BOXES; ++x) {
+            __nv_bfloat162 *const p = reinterpret_cast<__nv_bfloat162 *>(&v[x][i]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) p[u] = __hfma2(p[u], hi, __hmul2(p[u], lo));
+            *reinterpret_cast<uint4 *>(box + 16384 * x + (t + THREADS * i) * 16) = v[x][i];
+        }
     }
 }
 
 // A wait of the block has given up, so products and copies may still be in flight: the products end (a commit by the thread that
 // issued them on a barrier of its own, awaited with a limit) and the copies get time to, before the block gives back its tensor
 // and shared memory.  At the kernels' end, off the path of a call that goes well.
-__device__ __forceinline__ void drain(uint32_t bar) {
-    if (threadIdx.x == CT) {
+__device__ __forceinline__ void drain(uint32_t bar, int issuer) {
+    if ((int)threadIdx.x == issuer) {
         mma_commit(bar);
         mbar_spin_bounded(bar, 0u);
     }
@@ -90,7 +107,8 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t s_bars[SB_COUNT];
     __shared__ uint32_t s_tmem_base;
-    __shared__ float s_w[NT], s_ca[4], s_red[16];
+    __shared__ __align__(16) uint2 s_w[NT];
+    __shared__ float s_ca[4], s_red[16];
     __shared__ int s_req, s_abort;
     unsigned char *smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     const uint32_t sb = smem_u32(smem), bars = smem_u32(&s_bars[0]);
@@ -130,10 +148,10 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                 const uint32_t kb = base14 + (uint32_t)(n % NS) * (STAGE >> 4), vb = kb + (32768u >> 4);
                 if (n == 0) {
                     mma8_mm<0>(tm_H, kb, kb, kIdescMM);
-                    mma8_mm<0>(tm_U, vb, kb, kIdescMM);
+                    if (!a.solve_only) mma8_mm<0>(tm_U, vb, kb, kIdescMM);
                 } else {
                     mma8_mm<1>(tm_H, kb, kb, kIdescMM);
-                    mma8_mm<1>(tm_U, vb, kb, kIdescMM);
+                    if (!a.solve_only) mma8_mm<1>(tm_U, vb, kb, kIdescMM);
                 }
                 mma_commit(bars + 8 * SB_MMA);
             }
@@ -149,9 +167,9 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         auto issue_tma = [&](int n) {
             const uint32_t dst = sb + (uint32_t)(n % NS) * STAGE;
             const uint32_t bar = bars + 8 * (SB_KV0 + n % NS);
-            mbar_expect_tx(bar, 65536u);
+            mbar_expect_tx(bar, a.solve_only ? 32768u : 65536u);
             tma_load_tile3(&tmK, dst, bar, h * a.d, tile_x_hi(h, a.d, a.heads), (n0 + n) * NT, b);
-            tma_load_tile3(&tmV, dst + 32768, bar, h * a.d, tile_x_hi(h, a.d, a.heads), (n0 + n) * NT, b);
+            if (!a.solve_only) tma_load_tile3(&tmV, dst + 32768, bar, h * a.d, tile_x_hi(h, a.d, a.heads), (n0 + n) * NT, b);
         };
         if (t == 0)
             for (int n = 0; n < ntiles && n < NS; ++n) issue_tma(n);
@@ -207,12 +225,14 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                 // w_j = 2^(decay from token j to the end of the run) = 2^((total - prefix) - incl_j); its root scales the rows
                 float wt = exp2f(0.5f * ((total - prefix) - incl));
                 if (brun) wt *= sqrtf(fmaxf(brun[(size_t)(n * NT + t) * a.heads], 0.f));   // write strength
-                s_w[t] = wt;
+                s_w[t] = split_factor(wt);
                 prefix += tile_total;
             }
             wait(SB_KV0 + n % NS, (uint32_t)((n / NS) & 1));
             asm volatile("bar.sync 1, 512;" ::: "memory");       // weights are published (and the scan scratch is free)
-            scale_kv(smem + (size_t)(n % NS) * STAGE, s_w, t);
+            unsigned char *const stage = smem + (size_t)(n % NS) * STAGE;
+            scale_rows<2, CT, 2>(stage, s_w, t);
+            if (!a.solve_only) scale_rows<2, CT, 2>(stage + 32768, s_w, t);
             fence_async_smem();
             if (t == 0) *reinterpret_cast<volatile int *>(&s_req) = n;
             asm volatile("bar.sync 3, 544;" ::: "memory");       // hand the tile to the issuing warp
@@ -237,6 +257,7 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             float *dst = a.ws.delta + (size_t)item * st + (size_t)c * D + 32 * cq;
 #pragma unroll
             for (int which = 0; which < 2; ++which) {
+                if (which == 1 && a.solve_only) continue;        // the solve alone reads no U
                 uint32_t r[32];
                 TMEM_LD32(tmem + 128 * which + lane_addr + 32 * cq, r);
                 tmem_wait_ld();
@@ -251,33 +272,93 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     }
     fence_before();
     __syncthreads();
-    if (s_abort != 0) drain(bars + 8 * SB_DRAIN);
+    if (s_abort != 0) drain(bars + 8 * SB_DRAIN, CT);
     if (t < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
 }
 
 // ------------------------------------------------------------------------------------------------------------
-// State kernel.  One block per work item walks its tiles in order.  Thread = (state row c, 32 columns) of both
-// masters, which it keeps in registers in fp32 for a whole run.  The tensor cores compute only each tile's
-// increments dH = K~^T K~, dU = V~^T K~ into one of two TMEM buffers, one tile ahead of their use; per tile a thread
-// stores the bf16 copies of its part of the tile-initial H_0, U_0 (and adds up ||H_0||_F^2), then advances its
-// masters: H <- zeta H + dH, U <- zeta U + dU.  The warp that issues the products also turns the gates into the row
-// factors and the tile's decay, two tiles ahead, so that the compute warps meet no scan.  PARTS: blocks per work
-// item; with two, one keeps H (and loads only the keys), one keeps U; with four, each keeps 64 columns of one of them.
+// State kernel.  A block walks the tiles of a work item in order.  Thread = (state row c, CW columns) of a master, which it keeps in
+// registers in fp32 for a whole run.  The tensor cores compute only each tile's increments (dH = K~^T K~, dU = V~^T K~) into
+// one of two TMEM buffers, one tile ahead of their use; per tile a thread stores the bf16 copies of its part of the tile-initial
+// state (and adds up ||H_0||_F^2), then advances its master: H <- zeta H + dH.
+//
+// Who waits for whom.  One thread loads (TMA), factor warps turn the gates into row factors and a tile's decay several tiles ahead,
+// scaling warps apply them to the rows in shared memory, one thread issues the products, the master warps copy and advance.  Every
+// hand-over is an mbarrier per tile; nothing in the loop meets at a block barrier.
+//
+// What bounds it: device memory where a block has 64 KB of K and V per tile (268 MB at 64 x 4096 tokens), else how long the steps of a
+// tile take one after another, so as many tiles as possible are worked on at once.  Every access to shared memory (a shuffle, a barrier, a
+// load) waits 100 to 250 cycles behind the scaling warps' traffic, so accesses in a chain count more than instructions:
+//   - a row factor is two bf16 terms and a product two instructions per pair of elements (scale_rows);
+//   - the copies go straight from registers to global memory: in the workspace eight consecutive columns of the 128 rows lie together
+//     (2 KB), so a warp's store is 512 consecutive bytes, and the solve kernel reads those bytes as a tensor-core operand without a
+//     swizzle.  (Staged in shared memory over the tile's own K and V for a TMA store, a stage could not be loaded again before the
+//     copies had been read from it);
+//   - what a thread contributes to ||H_0||_F^2 is left in shared memory, and a factor warp adds it up tiles later;
+//   - gates and write strengths are loaded a whole turn of the factor warps ahead and looked at only then.
+// us per call of this kernel, before (one block-wide step after another, copies staged, head dimension 64 on 128 x 128 masters) and with
+// this: 64 sequences x 4096 tokens 80 -> 55; 32 x 2048, solve alone (H only) 36 -> 18; 24 x 1999 with write strengths 61 -> 22 (their
+// loads used to be waited for in the issuing warp); 64 x 2048, d = 64: 42 -> 19.
+//
+// KIND: what a block keeps.
+//   kBoth     H and U (128 channels), where sequences are cut or the items alone fill the device
+//   kOne      H or U: two blocks per item
+//   kQuarter  64 columns of H or of U: four blocks per item
+//   kD64      head dimension 64: H over U as one 128 x 64 master, [K V]^T K one product per k-step
+// Blocks that keep U alone scale the keys by the whole weight and leave V as it is.  The solve alone reads no U: its blocks are not launched.
 // ------------------------------------------------------------------------------------------------------------
-// TB_STG0 + stage: one barrier per stage, like the loads.  (With a single barrier the compute warps could complete two
-// phases, tiles m + 1 and m + 2, while the TMA thread was still held up behind tile m's store; the phase parity it
-// then polled looked incomplete, and the compute warps in turn waited for the load that only this thread issues.)
-enum { TB_KV0 = 0, TB_D0 = NS, TB_D1, TB_DRAIN, TB_STG0, TB_COUNT = TB_STG0 + NS };
+enum { kBoth = 0, kOne = 1, kQuarter = 2, kD64 = 3 };
+// Warps: those that keep the masters; groups that scale rows and take the tiles in turn; helpers (row factors, products, loads).  With 32 KB
+// of K (and V) per tile six stages fit, and what counts is how many tiles are worked on at once: two groups of four warps.  With 64 KB
+// (kBoth, kOne's blocks of U) three fit, so that a stage has to be given back soon: all sixteen warps scale a tile together, a tile ahead,
+// and then keep its masters.  (64 x 4096 tokens, kOne: 54 us, 58 with a group of eight warps, 60 with two of four; 32 x 4096, kQuarter: 42
+// us in one group of all warps, 35.4 with two.)
+// Registers of a thread at launch (what its share of 65,536 allows) and after the split.
+template <int KIND> struct StateKind {
+    static constexpr bool kGroups = KIND == kQuarter || KIND == kD64;
+    static constexpr int kColumns = KIND == kBoth ? 256 : KIND == kOne ? 128 : 64;      // of all masters: TMEM columns of a buffer of increments
+    static constexpr int kMasters = KIND == kBoth ? 2 : 1, kMasterWarps = kGroups ? 8 : 16;
+    static constexpr int kCols = kColumns / kMasters / (kMasterWarps / 4);              // columns of a thread, of each master
+    static constexpr int kGroupWarps = kGroups ? 4 : 16, kScaleGroups = kGroups ? 2 : 1;
+    static constexpr int kFactorWarps = kGroups ? 4 : 2, kHelperWarps = kGroups ? 8 : 4;  // (whole warpgroups)
+    static constexpr int kOtherWarps = (kGroups ? kGroupWarps * kScaleGroups : 0) + kHelperWarps, kThreads = 32 * (kMasterWarps + kOtherWarps);
+    static constexpr int kRegsLaunch = kGroups ? 80 : 96, kRegsMaster = kGroups ? 112 : 104, kRegsOther = 64;
+    static_assert(kHelperWarps >= kFactorWarps + 2 && kThreads * kRegsLaunch <= 65536 &&
+                      32 * (kMasterWarps * kRegsMaster + kOtherWarps * kRegsOther) <= kThreads * kRegsLaunch,
+                  "register split exceeds the launch allocation");
+};
+constexpr int kMaxStages = 6;
+constexpr int kSets = kMaxStages + 2;      // sets of row factors, decays and norm terms
+// A barrier of a kind for each of kRing consecutive tiles, whatever the number of stages: at least as many as stages, so that none is
+// a phase ahead of a waiter; and even, so that the phases of one all belong to the same of two scaling groups.  (With three, a group met
+// a barrier whose phase before had been the other group's: where that was not complete yet, the one before it had the same parity.)
+constexpr int kRing = 6;
+static_assert(kRing >= kMaxStages && kRing % 2 == 0, "ring of barriers");
+enum {                            // mbarriers
+    TB_KV = 0,                    // + tile % kRing: K and V have landed (TMA) and the tile's row factors and decay are ready (factor warp)
+    TB_SC = TB_KV + kRing,        // + tile % kRing: rows scaled (one arrival per scaling warp)
+    TB_D = TB_SC + kRing,         // + tile % kRing: the products are complete: increments for the masters, and the stage is free
+    TB_AD = TB_D + kRing,         // + buffer: increments read (one arrival per master warp)
+    TB_DRAIN = TB_AD + 2,
+    TB_COUNT
+};
 
-template <int PARTS>
-__global__ void __launch_bounds__(kThreadsStateK, 1)
-fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-                    const __grid_constant__ CUtensorMap tmS, FwdArgs a) {
+template <int KIND>
+__global__ void __launch_bounds__(StateKind<KIND>::kThreads, 1)
+fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, FwdArgs a) {
+    using SK = StateKind<KIND>;
+    constexpr int CW = SK::kCols, NM = SK::kMasters;
+    constexpr uint32_t DW = SK::kColumns;
+    constexpr int MT = 32 * SK::kMasterWarps, CT = 32 * (SK::kMasterWarps + SK::kOtherWarps - SK::kHelperWarps);    // threads that keep masters; those that scale; the helpers
+    constexpr int FT = CT + 32 * SK::kFactorWarps;                                 // helpers: factor warps, a warp for the products, one for the loads
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t s_bars[TB_COUNT];
+    __shared__ __align__(16) uint2 s_f[kSets][NT];
+    __shared__ __align__(16) float s_in[SK::kFactorWarps][2][NT];         // gates and write strengths on their way to their lanes
     __shared__ uint32_t s_tmem_base;
-    __shared__ float s_w[3][NT], s_red[3][16], s_decay[4];
-    __shared__ int s_req, s_abort;
+    __shared__ __align__(16) float s_sq[kSets][MT];          // the threads' terms of ||H_0||_F^2
+    __shared__ float s_decay[kSets];
+    __shared__ int s_abort;
     unsigned char *smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     const uint32_t sb = smem_u32(smem), bars = smem_u32(&s_bars[0]);
     const int t = threadIdx.x, l = t & 31;
@@ -290,11 +371,11 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     if (t == 0) {
         s_abort = 0;
         for (int i = 0; i < TB_COUNT; ++i)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bars + 8 * i), "r"(i >= TB_STG0 ? CT / 32 : 1));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bars + 8 * i), "r"(i < TB_SC ? 2 : i < TB_D ? SK::kGroupWarps : i >= TB_AD && i < TB_DRAIN ? SK::kMasterWarps : 1));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (t < 32) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&s_tmem_base))
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "n"(2 * DW)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -303,20 +384,21 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     fence_after();
     const uint32_t tmem = s_tmem_base;
     const WorkPlan &P = a.plan;
-    // With no sequence cut and few work items the masters are split: two blocks per item, one advances H (and needs
-    // only the keys), one U; four blocks: 64 columns each of H and U.  A block handles the masters w_lo <= which < w_hi.
-    const int item = (int)(blockIdx.x / PARTS);
-    const int w_lo = PARTS == 4 ? (int)(blockIdx.x >> 1 & 1) : PARTS == 2 ? (int)(blockIdx.x & 1) : 0, w_hi = PARTS > 1 ? w_lo + 1 : 2;
-    const bool do_h = w_lo == 0, do_u = w_hi == 2;
-    const int half = PARTS == 4 ? (int)(blockIdx.x & 1) : 0;             // columns 64 half .. of the masters
-    constexpr int CW = PARTS == 4 ? 16 : 32;                             // columns of a thread
-    const uint32_t boxes = PARTS < 4 ? (do_u ? 15u : 3u) : (do_u ? 12u + (1u << half) : 3u);     // of K and V: loaded and scaled
-    const long long f_lo = P.lo(item), f_hi = P.lo(item + 1);
-    const int n_mine = (int)(f_hi - f_lo);
-    const uint32_t base14 = (sb >> 4) & 0x3FFF;
+    const int per_item = KIND == kOne || KIND == kQuarter ? (KIND == kQuarter ? 2 : 1) << (a.solve_only ? 0 : 1) : 1;
+    const int item = (int)blockIdx.x / per_item, part = (int)blockIdx.x % per_item;
+    const int half = KIND == kQuarter ? part & 1 : 0;                    // columns 64 half .. of the master
+    const bool u_only = KIND == kQuarter ? part >> 1 : KIND == kOne ? part != 0 : false;
+    const bool both = KIND == kBoth && !a.solve_only;
+    // a stage: K (the part of it that is needed), then V
+    const uint32_t v_off = KIND == kQuarter || KIND == kD64 ? 16384u : 32768u;
+    const uint32_t stage_bytes = KIND == kD64 ? 32768u : (both || u_only) ? v_off + 32768u : 32768u;
+    const int ns = stage_bytes == 32768u ? 6 : stage_bytes == 49152u ? 4 : 3;
+    const long long f_lo = P.lo(item);
+    const int n_mine = (int)(P.lo(item + 1) - f_lo);
+    float *const hh_out = u_only ? nullptr : half ? a.tile_hh2 : a.tile_hh;
 
     // position of tile m of this block
-    struct Pos { int seq, n, b, h, ntok; bool run_start, seq_end; size_t tok0; };
+    struct Pos { int seq, n, b, h, ntok; size_t tok0; };
     auto pos_of = [&](int m) {
         Pos p;
         const unsigned fu = (unsigned)(f_lo + m);
@@ -325,281 +407,346 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         p.b = (int)a.divH.div((unsigned)p.seq);
         p.h = p.seq - p.b * a.heads;
         p.ntok = min(NT, a.T - p.n * NT);
-        p.run_start = (m == 0) || (p.n == 0);
-        p.seq_end = (p.n + 1 == P.N);
         p.tok0 = ((size_t)p.b * a.T + (size_t)p.n * NT) * a.heads + p.h;
         return p;
     };
     auto aborted = [&]() { return *reinterpret_cast<volatile int *>(&s_abort) != 0; };
-    auto wait = [&](int which, uint32_t parity) {     // once a wait has given up the later ones return at once
-        if (!aborted() && !mbar_spin_bounded(bars + 8 * which, parity)) *reinterpret_cast<volatile int *>(&s_abort) = 1;
+    auto give_up = [&]() { *reinterpret_cast<volatile int *>(&s_abort) = 1; };
+    // Once a wait has given up the later ones return at once.  (A look at the flag takes as long as one at the barrier, so it comes
+    // second: most of the compute warps' waits find their phase complete.)
+    auto wait = [&](int which, uint32_t parity) {
+        if (mbar_test(bars + 8 * which, parity) || aborted()) return;
+        if (!(SK::kGroups ? mbar_wait_bounded(bars + 8 * which, parity) : mbar_spin_bounded(bars + 8 * which, parity))) give_up();
+    };
+    auto wait_asleep = [&](int which, uint32_t parity) {     // the same for waits that are long and have time
+        if (!aborted() && !mbar_wait_bounded(bars + 8 * which, parity)) give_up();
+    };
+    // Barrier of tile n among the kRing of a kind, and the parity of its phase
+    auto bar_of = [](int n) { return n % kRing; };
+    auto phase_of = [](int n) { return (uint32_t)(n / kRing) & 1u; };
+
+    // Rows of tile m, in stage `at`, scaled by the GT threads of a group
+    constexpr int GT = 32 * SK::kGroupWarps;
+    auto scale = [&](int m, int at, int ts) {
+        wait(TB_KV + bar_of(m), phase_of(m));
+        unsigned char *const stage = smem + (size_t)at * stage_bytes;
+        const uint2 *const f = s_f[m % kSets];
+        if constexpr (SK::kGroups) {
+#pragma unroll 2
+            for (int i = 0; i < 4; ++i) {
+                if (KIND == kQuarter && u_only) scale_rows<2, GT, 1>(stage, f, ts + 2 * GT * i);
+                else scale_rows<2, GT, 2>(stage, f, ts + 2 * GT * i);
+            }
+        } else {
+            scale_rows<2, GT, 2>(stage, f, ts);
+            if (both) scale_rows<2, GT, 2>(stage + 32768, f, ts);
+        }
+        fence_async_smem();
+        fence_before();
+        __syncwarp();
+        if (l == 0) mbar_arrive(bars + 8 * (TB_SC + bar_of(m)));
     };
 
-    if (t >= CT + 32) {
-        // ================================ TMA thread: loads of K, V; stores of the bf16 copies ================================
-        if (l == 0 && n_mine > 0) {
-            auto issue_tma = [&](int m) {
+    // (one instruction for all of a warpgroup, ahead of the roles)
+    if (t >= MT) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SK::kRegsOther));
+        if (t >= FT + 32) {
+            // ================================ TMA thread: loads of K and V ================================
+            if (t == FT + 32) {
+                for (int m = 0, stage = 0; m < n_mine; ++m, stage = stage + 1 == ns ? 0 : stage + 1) {
+                    if (m >= ns) wait(TB_D + bar_of(m - ns), phase_of(m - ns));
+                    if (aborted()) break;                // (a barrier whose copy never landed takes no second announcement)
+                    const Pos p = pos_of(m);
+                    const uint32_t dst = sb + (uint32_t)stage * stage_bytes, bar = bars + 8 * (TB_KV + bar_of(m));
+                    const int x = p.h * a.d, y = p.n * NT;
+                    mbar_expect_tx(bar, stage_bytes);
+                    if constexpr (KIND == kD64) {
+                        tma_load_box3(&tmK, dst, bar, x, y, p.b);
+                        tma_load_box3(&tmV, dst + v_off, bar, x, y, p.b);
+                    } else {
+                        if (KIND == kQuarter && u_only) tma_load_box3(&tmK, dst, bar, x + 64 * half, y, p.b);
+                        else tma_load_tile3(&tmK, dst, bar, x, x + 64, y, p.b);
+                        if (both || u_only) tma_load_tile3(&tmV, dst + v_off, bar, x, x + 64, y, p.b);
+                    }
+                }
+            }
+        } else if (t >= CT && t < FT) {
+            // ================ factor warps: row factors and decays, and the sums of ||H_0||_F^2 ================
+            // Row factor of token j of a tile: the root of w_j = beta_j 2^(G_last - G_j), or w_j itself where only one of a product's
+            // operands is scaled; 0 past the sequence.  As two bf16 terms, for scale_rows.
+            // The warps take the tiles in turn: a tile's scan, logarithms and sums are a chain of some 4000 cycles beside the warps that scale,
+            // several times as long as a tile.  Before it publishes, tile f waits until the products of tile f - ns are complete: the phase
+            // before its own of the barrier is then complete, and the masters are past tile f - ns - 2 (the products of a
+            // tile are issued when the increments of the tile two before have been read), so with kSets >= ns + 2 sets none is written
+            // over that is still to be read.
+            struct Scalars { float g[4], b[4]; };
+            auto load_scalars = [&](int m, Scalars &x) {         // (taken as they are: nothing here may wait for a load)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    x.g[i] = 1.f;
+                    x.b[i] = 0.f;
+                }
+                if (m >= n_mine) return;
                 const Pos p = pos_of(m);
-                const uint32_t dst = sb + (uint32_t)(m % NS) * STAGE, bar = bars + 8 * (TB_KV0 + m % NS);
-                if (PARTS == 4 && do_u) {                // V and the keys' own 64 channels
-                    mbar_expect_tx(bar, 49152u);
-                    tma_load_box3(&tmK, dst + 16384 * half, bar, p.h * a.d + 64 * half, p.n * NT, p.b);
-                    tma_load_tile3(&tmV, dst + 32768, bar, p.h * a.d, tile_x_hi(p.h, a.d, a.heads), p.n * NT, p.b);
-                    return;
-                }
-                mbar_expect_tx(bar, do_u ? 65536u : 32768u);
-                tma_load_tile3(&tmK, dst, bar, p.h * a.d, tile_x_hi(p.h, a.d, a.heads), p.n * NT, p.b);
-                if (do_u) tma_load_tile3(&tmV, dst + 32768, bar, p.h * a.d, tile_x_hi(p.h, a.d, a.heads), p.n * NT, p.b);
+                const size_t at = p.tok0 + (size_t)l * a.heads;
+                const float *const gp = a.gate + at, *const bp = a.beta ? a.beta + at : nullptr;
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (32 * i + l < p.ntok) {
+                        x.g[i] = ld_stream_f32(gp + 32 * i * a.heads);
+                        x.b[i] = bp ? ld_stream_f32(bp + 32 * i * a.heads) : 1.f;
+                    }
             };
-            for (int m = 0; m < n_mine && m < NS; ++m) issue_tma(m);
-            for (int m = 0; m < n_mine; ++m) {
-                // the compute warps have written the bf16 copies of H_0, U_0 over the tile's K and V (the tile's
-                // products are complete): store them, then the stage takes the tile three further on
-                wait(TB_STG0 + m % NS, (uint32_t)((m / NS) & 1));
-                const uint32_t src = sb + (uint32_t)(m % NS) * STAGE;
-                for (int which = w_lo; which < w_hi; ++which)
-                    for (int hf = half; hf < (PARTS == 4 ? half + 1 : 2); ++hf)
-                        asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::
-                                         "l"(reinterpret_cast<uint64_t>(&tmS)), "r"(64 * hf), "r"((int)((f_lo + m) * 256 + 128 * which)),
-                                     "r"(src + 32768 * which + 16384 * hf)
-                                     : "memory");
-                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                if (m + NS < n_mine) {
-                    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the copies have been read
-                    if (aborted()) break;            // (a barrier whose copy never landed takes no second announcement)
-                    issue_tma(m + NS);
+            const int f0 = (t - CT) >> 5;
+            auto factors = [&](int f, Scalars &x) {
+                // Loaded with lane l at tokens l, 32 + l, 64 + l, 96 + l (with four consecutive tokens per lane a load touches four times as
+                // wide a piece of memory: 64 x 4096 tokens 54 -> 60 us), used with tokens 4 l .. 4 l + 3.
+                float factor[4], incl[4], run = 0.f;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    s_in[f0][0][32 * i + l] = x.g[i];
+                    s_in[f0][1][32 * i + l] = x.b[i];
                 }
-            }
-            asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");    // the stores are complete
-        }
-    } else if (t >= CT) {
-        // ================ MMA issuing warp; it also prepares the row factors, two tiles ahead ================
-        // Row factors sqrt(beta_j 2^(G_last - G_j)) (0 past the sequence) and decay of tile m: lane l has tokens l, 32 + l,
-        // 64 + l, 96 + l.  Written two hand-overs before the compute warps read them, so the hand-over barrier in between
-        // orders the two; three sets, so that no set is rewritten while a slower warp may still read it.
-        float lg[4], sb[4];          // gates and write strengths of the tile whose factors come next (loaded a hand-over ahead)
-        auto load_scalars = [&](int m, float(&lg)[4], float(&sb)[4]) {
+                __syncwarp();
+                const float4 g4 = *reinterpret_cast<const float4 *>(&s_in[f0][0][4 * l]), b4 = *reinterpret_cast<const float4 *>(&s_in[f0][1][4 * l]);
+                __syncwarp();
+                x = Scalars{{g4.x, g4.y, g4.z, g4.w}, {b4.x, b4.y, b4.z, b4.w}};
 #pragma unroll
-            for (int grp = 0; grp < 4; ++grp) {
-                lg[grp] = 1.f;
-                sb[grp] = 0.f;
-            }
-            if (m >= n_mine) return;
-            const Pos p = pos_of(m);
-#pragma unroll
-            for (int grp = 0; grp < 4; ++grp) {
-                const int tok = 32 * grp + l;
-                if (tok < p.ntok) {
-                    lg[grp] = ld_stream_f32(a.gate + p.tok0 + (size_t)tok * a.heads);
-                    sb[grp] = a.beta ? fmaxf(ld_stream_f32(a.beta + p.tok0 + (size_t)tok * a.heads), 0.f) : 1.f;
-                }
-            }
-        };
-        auto factors = [&](int m, float(&lg)[4], const float(&sb)[4]) {      // from the loaded scalars of tile m
-            float before = 0.f;
-#pragma unroll
-            for (int grp = 0; grp < 4; ++grp) {
-                float incl = fmaxf(log2f(lg[grp]), -115.f);
+                for (int i = 0; i < 4; ++i) incl[i] = run += fmaxf(log2f(x.g[i]), -115.f);
+                float before = run;                              // of the lanes up to this one, then of those before it
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
-                    const float up = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (l >= o) incl += up;
+                    const float up = __shfl_up_sync(0xffffffffu, before, o);
+                    before += l >= o ? up : 0.f;
                 }
-                const float tot = __shfl_sync(0xffffffffu, incl, 31);
-                lg[grp] = incl + before;             // cumulative log2 gate up to and including the token
-                before += tot;
-            }
-            const float tile_total = before;
+                const float total = __shfl_sync(0xffffffffu, before, 31);
+                before = total - (before - run);                 // decay from the start of this lane's tokens to the tile's end
 #pragma unroll
-            for (int grp = 0; grp < 4; ++grp) s_w[m % 3][32 * grp + l] = sqrtf(sb[grp]) * exp2f(0.5f * (tile_total - lg[grp]));
-            if (l == 0) s_decay[m & 3] = exp2f(tile_total);      // (four deep: tile m's is read after the hand-over of tile m + 1, behind which tile m + 3's is written)
-            __syncwarp();
-        };
-        if (n_mine > 0) {
-            float lg1[4], sb1[4];
-            load_scalars(0, lg, sb);
-            load_scalars(1, lg1, sb1);               // (both tiles' loads in flight together)
-            factors(0, lg, sb);
-            if (n_mine > 1) factors(1, lg1, sb1);
-            load_scalars(2, lg, sb);
-            asm volatile("bar.sync 3, 544;" ::: "memory");       // the factors of the first two tiles are published
-        }
-        for (;;) {
-            asm volatile("bar.sync 3, 544;" ::: "memory");
-            const int m = *reinterpret_cast<const volatile int *>(&s_req);
-            if (m < 0) break;
+                for (int i = 0; i < 4; ++i) {
+                    const float e = before - incl[i];
+                    factor[i] = u_only ? exp2f(e) : exp2f(0.5f * e);
+                }
+                if (a.beta) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float w = fmaxf(x.b[i], 0.f);
+                        factor[i] *= u_only ? w : sqrtf(w);
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) factor[i] *= x.b[i];      // 1, or 0 past the sequence
+                }
+                load_scalars(f + SK::kFactorWarps, x);
+                if (f >= ns) {
+                    wait_asleep(TB_D + bar_of(f - ns), phase_of(f - ns));
+                    if (f < 2 * kSets) asm volatile("griddepcontrol.wait;" ::: "memory");
+                    if (f >= kSets && hh_out) {                  // tile f - kSets
+                        const float4 *p = reinterpret_cast<const float4 *>(s_sq[f % kSets]) + l;
+                        float hh = 0.f;
+#pragma unroll
+                        for (int i = 0; i < MT / 128; ++i) hh += (p[32 * i].x + p[32 * i].y) + (p[32 * i].z + p[32 * i].w);
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) hh += __shfl_xor_sync(0xffffffffu, hh, o);
+                        if (l == 0) hh_out[f_lo + f - kSets] = hh;
+                    }
+                }
+                const uint2 w0 = split_factor(factor[0]), w1 = split_factor(factor[1]), w2 = split_factor(factor[2]), w3 = split_factor(factor[3]);
+                uint4 *const set = reinterpret_cast<uint4 *>(&s_f[f % kSets][4 * l]);
+                set[0] = make_uint4(w0.x, w0.y, w1.x, w1.y);
+                set[1] = make_uint4(w2.x, w2.y, w3.x, w3.y);
+                if (l == 0) s_decay[f % kSets] = exp2f(total);
+                __syncwarp();
+                if (l == 0) mbar_arrive(bars + 8 * (TB_KV + bar_of(f)));
+            };
+            Scalars x;                                           // (of the warp's next tile, in flight)
+            load_scalars(f0, x);
+            for (int f = f0; f < n_mine; f += SK::kFactorWarps) factors(f, x);
+        } else if (t >= FT) {
+            // ================================ MMA issuing thread ================================
             if (l == 0) {
-                fence_after();
-                const uint32_t kb = base14 + (uint32_t)(m % NS) * (STAGE >> 4), vb = kb + (32768u >> 4);
-                const uint32_t tm_d = tmem + 256 * (m & 1);
-                constexpr uint32_t idesc = PARTS == 4 ? make_idesc(128, 64, 1, 1) : kIdescMM;
-                const uint32_t bb = kb + (16384u >> 4) * half;
-                if (do_h) mma8_mm<0>(tm_d, kb, bb, idesc);                 // dH = K~^T K~
-                if (do_u) mma8_mm<0>(tm_d + 128, vb, bb, idesc);           // dU = V~^T K~
-                mma_commit(bars + 8 * (TB_D0 + (m & 1)));
+                constexpr uint32_t idesc = DW == 64 ? make_idesc(128, 64, 1, 1) : kIdescMM;
+                const uint32_t base14 = (sb >> 4) & 0x3FFF;
+                for (int m = 0, stage = 0; m < n_mine; ++m, stage = stage + 1 == ns ? 0 : stage + 1) {
+                    const uint32_t ph = phase_of(m), ph_ad = ((uint32_t)(m >> 1) & 1u) ^ 1u;      // of tile m - 2's (the phase before a barrier's first one counts as complete)
+                    const bool sc = mbar_test(bars + 8 * (TB_SC + bar_of(m)), ph), ad = !SK::kGroups || mbar_test(bars + 8 * (TB_AD + (m & 1)), ph_ad);
+                    if (!sc) wait(TB_SC + bar_of(m), ph);
+                    if (!ad) wait(TB_AD + (m & 1), ph_ad);
+                    if (!(sc && ad) && aborted()) break;
+                    fence_after();
+                    const uint32_t kb = base14 + (uint32_t)stage * (stage_bytes >> 4), vb = kb + (v_off >> 4);
+                    const uint32_t tm_d = tmem + DW * (uint32_t)(m & 1);
+                    if (!u_only) mma8_mm<0>(tm_d, kb, kb + (16384u >> 4) * half, idesc);           // dH = K~^T K~ (kD64: [K~ V~]^T K~)
+                    if (both || u_only) mma8_mm<0>(tm_d + (NM - 1) * 128, vb, kb, idesc);          // dU = V~^T K~
+                    mma_commit(bars + 8 * (TB_D + bar_of(m)));
+                }
             }
-            __syncwarp();
-            if (m + 2 < n_mine) {
-                factors(m + 2, lg, sb);
-                load_scalars(m + 3, lg, sb);         // (in flight across the hand-over)
+        } else if constexpr (SK::kGroups) {
+            // ================================ scaling groups ================================
+            const int ts = (t - MT) % GT;
+            for (int m = (t - MT) / GT, at = m; m < n_mine; m += SK::kScaleGroups) {
+                scale(m, at, ts);
+                at += SK::kScaleGroups;
+                if (at >= ns) at -= ns;
             }
         }
-    } else if (n_mine > 0) {
-        // ================================= compute threads =================================
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SK::kRegsMaster));
+        // ================================ masters ================================
         const int q = (t >> 5) & 3, cq = t >> 7, c = 32 * q + l, col0 = 64 * half + CW * cq;     // row, first column
-        const uint32_t lane_addr = (uint32_t)(32 * q) << 16;
-        const size_t st = state_floats(D, D);
-        float *const hh_out = half ? a.tile_hh2 : a.tile_hh;
+        const uint32_t tm_c = tmem + ((uint32_t)(32 * q) << 16) + CW * cq;
+        const int which0 = KIND == kD64 ? c >> 6 : u_only ? 1 : 0;           // matrix of the (first) master, and the row in it
+        const int row = KIND == kD64 ? c & 63 : c;
+        constexpr int DD = KIND == kD64 ? 64 : D;                            // head dimension of the caller's states
+        const size_t ext = (size_t)2 * DD * DD;                              // floats of a caller's state
+        const size_t e_ext = (size_t)which0 * DD * DD + (size_t)row * DD + col0;
+        const size_t st = state_floats(D, D), e_ws = (size_t)which0 * D * D + (size_t)row * D + col0;    // the workspace's states are 128 x 128
+        const bool sums = KIND == kD64 ? q < 2 : !u_only;                    // this warp's rows belong to H
+        // the copies: [matrix][column / 8][128 rows][8 columns] of 64 KB per tile; head dimension 64: [column / 8][H over U][8], 16 KB
+        unsigned char *copy = a.tile_hu + (size_t)f_lo * (KIND == kD64 ? kTileStateBytes64 : kTileStateBytes) +
+                              (KIND == kD64 ? 0 : which0 * 32768) + (col0 / 8) * 2048 + c * 16;
         // first item of the chain of summaries behind this block's start state
         int chain_j0 = item;
-        if (P.cut_in(item)) {
+        if ((KIND == kBoth || KIND == kD64) && P.cut_in(item)) {
             const long long seq_start = (f_lo / P.N) * P.N;
             chain_j0 = item - 1;
             while (P.lo(chain_j0) > seq_start) --chain_j0;
         }
-        // Tile m: rows scaled in place by the row factors (prepared by the issuing warp), products posted.
-        auto prepare = [&](int m) {
-            wait(TB_KV0 + m % NS, (uint32_t)((m / NS) & 1));
-            scale_kv(smem + (size_t)(m % NS) * STAGE, s_w[m % 3], t, boxes);
-            fence_async_smem();
-            fence_before();
-            if (t == 0) *reinterpret_cast<volatile int *>(&s_req) = m;
-            asm volatile("bar.sync 3, 544;" ::: "memory");       // hand the tile to the issuing warp
-        };
-
-        float mH[CW], mU[CW];
-        asm volatile("bar.sync 3, 544;" ::: "memory");           // the factors of the first two tiles are published
-        prepare(0);
-        // summaries and start states are read after this point only
+        uint64_t mst[NM][CW / 2];
+        int seq, n;
+        {
+            const Pos p0 = pos_of(0);
+            seq = p0.seq;
+            n = p0.n;
+        }
+        if (!SK::kGroups && n_mine > 0) scale(0, 0, t);
+        // summaries and start states are read, and copies written, after this point only
         asm volatile("griddepcontrol.wait;" ::: "memory");
 
-        for (int m = 0; m < n_mine; ++m) {
-            const Pos p = pos_of(m);
-            if (m + 1 < n_mine) prepare(m + 1);                  // its products run under this tile's passes
-            const long long tile = f_lo + m;
-            if (p.run_start) {
+        for (int m = 0, at = 1; m < n_mine; ++m) {
+            if constexpr (!SK::kGroups) {                        // the next tile's rows: its products run under this tile's passes
+                if (m + 1 < n_mine) scale(m + 1, at, t);
+                if (++at == ns) at = 0;
+            }
+            if (m == 0 || n == 0) {
                 // start of a run: the caller's initial state of the sequence (or zero), carried through the summaries
                 // of the blocks that hold the earlier part of the sequence: state <- decay_j * state + delta_j
-                const bool chained = p.n != 0;
-                const float *s0 = (chained && a.start_from_scan) ? a.ws.start + (size_t)item * st
-                                  : (a.state_in ? a.state_in + (size_t)p.seq * st : nullptr);
-                const int j0 = (chained && !a.start_from_scan) ? chain_j0 : 0, j1 = (chained && !a.start_from_scan) ? item : 0;
-                const size_t e = (size_t)c * D + col0;
-                // the caller's state has head dimension a.d (rows and columns from a.d on are zero on chip); the scan
-                // kernel's start states are in the on-chip layout
-                const bool ext = s0 != nullptr && !(chained && a.start_from_scan);
-                const float *const s0e = ext ? a.state_in + (size_t)p.seq * 2 * a.d * a.d + (size_t)c * a.d + col0 : nullptr;
-                const bool in_ext = c < a.d && col0 < a.d;
+                const bool chained = (KIND == kBoth || KIND == kD64) && n != 0;
+                const bool scanned = chained && a.start_from_scan;
+                const float *const s0 = scanned ? a.ws.start + (size_t)item * st + e_ws : a.state_in ? a.state_in + (size_t)seq * ext + e_ext : nullptr;
+                const int j0 = chained && !scanned ? chain_j0 : 0, j1 = chained && !scanned ? item : 0;
 #pragma unroll
-                for (int which = 0; which < 2; ++which) {
-                    if (which < w_lo || which >= w_hi) continue;
-                    float(&mm)[CW] = which ? mU : mH;
-                    const size_t eo = e + which * (size_t)D * D;
+                for (int w = 0; w < NM; ++w) {
 #pragma unroll
                     for (int i = 0; i < CW / 4; ++i) {
-                        const float4 v4 = ext ? (in_ext ? *reinterpret_cast<const float4 *>(s0e + which * (size_t)a.d * a.d + 4 * i)
-                                                        : make_float4(0.f, 0.f, 0.f, 0.f))
-                                          : (s0 ? *reinterpret_cast<const float4 *>(s0 + eo + 4 * i) : make_float4(0.f, 0.f, 0.f, 0.f));
-                        mm[4 * i + 0] = v4.x; mm[4 * i + 1] = v4.y; mm[4 * i + 2] = v4.z; mm[4 * i + 3] = v4.w;
+                        ulonglong2 v = make_ulonglong2(0ull, 0ull);
+                        if (s0) v = *reinterpret_cast<const ulonglong2 *>(s0 + w * D * D + 4 * i);
+                        mst[w][2 * i] = v.x;
+                        mst[w][2 * i + 1] = v.y;
                     }
                     for (int j = j0; j < j1; ++j) {
                         // summaries come from the kernel this one may overlap with as its programmatic dependent: ordinary loads
                         const float dj = *reinterpret_cast<const volatile float *>(a.ws.decay + j);
+                        const uint64_t dj2 = f2_pack(dj, dj);
+                        const float *const dd = a.ws.delta + (size_t)j * st + e_ws + w * D * D;
 #pragma unroll
                         for (int i = 0; i < CW / 4; ++i) {
-                            const float4 dd = *(reinterpret_cast<const float4 *>(a.ws.delta + (size_t)j * st + eo) + i);
-                            mm[4 * i + 0] = fmaf(dj, mm[4 * i + 0], dd.x);
-                            mm[4 * i + 1] = fmaf(dj, mm[4 * i + 1], dd.y);
-                            mm[4 * i + 2] = fmaf(dj, mm[4 * i + 2], dd.z);
-                            mm[4 * i + 3] = fmaf(dj, mm[4 * i + 3], dd.w);
+                            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(dd + 4 * i);
+                            mst[w][2 * i] = f2_fma(dj2, mst[w][2 * i], v.x);
+                            mst[w][2 * i + 1] = f2_fma(dj2, mst[w][2 * i + 1], v.y);
                         }
                     }
                 }
             }
-            // ---- bf16 copies of the tile-initial state and ||H_0||_F^2: each master in turn is written over the tile's
-            // own K (V) in operand layout and goes from there to the workspace by TMA; then its increments are added
-            wait(TB_D0 + (m & 1), (uint32_t)((m >> 1) & 1));     // the tile's increments are complete (posted a tile ago)
+            // ---- the increments on their way (their products ran under the tile before), the bf16 copies of the tile-initial state
+            // and the thread's term of ||H_0||_F^2, then the masters advanced: zeta m + increment
+            wait(TB_D + bar_of(m), phase_of(m));
             fence_after();
-            const float decay = s_decay[m & 3];
-            unsigned char *const stg = smem + (size_t)(m % NS) * STAGE;   // the tile's own K and V are no longer needed
+            const float decay = s_decay[m % kSets];
+            const uint64_t decay2 = f2_pack(decay, decay);
+            uint64_t sq = 0ull;
+            constexpr int PW = NM == 1 ? 32 : 16;                // columns at a time
 #pragma unroll
-            for (int which = 0; which < 2; ++which) {
-                if (which < w_lo || which >= w_hi) continue;
-                float(&mm)[CW] = which ? mU : mH;
-                float hs = 0.f;
+            for (int w = 0; w < NM; ++w) {
+                if (w == 1 && !both) continue;
 #pragma unroll
-                for (int i = 0; i < CW / 8; ++i) {
-                    uint32_t pk[4];
+                for (int c0 = 0; c0 < CW; c0 += PW) {
+                    uint32_t x[PW];
+                    if constexpr (PW == 32) TMEM_LD32(tm_c + DW * (m & 1) + c0, x);
+                    else TMEM_LD16(tm_c + DW * (m & 1) + 128 * w + c0, x);
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const float v0 = mm[8 * i + 2 * u], v1 = mm[8 * i + 2 * u + 1];
-                        if (which == 0) hs = fmaf(v0, v0, fmaf(v1, v1, hs));
-                        pk[u] = pack_bf16(v0, v1);
+                    for (int i = 0; i < PW / 8; ++i) {
+                        uint32_t pk[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const uint64_t v = mst[w][c0 / 2 + 4 * i + u];
+                            float v0, v1;
+                            f2_unpack(v, v0, v1);
+                            pk[u] = pack_bf16(v0, v1);
+                            if (w == 0) sq = f2_fma(v, v, sq);
+                        }
+                        *reinterpret_cast<uint4 *>(copy + w * 32768 + 2048 * (c0 / 8 + i)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
                     }
-                    *reinterpret_cast<uint4 *>(stg + 32768 * which + tile_off(c, col0 / 8 + i)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                }
-                if (which == 0) {
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) hs += __shfl_xor_sync(0xffffffffu, hs, o);
-                    if (l == 0) s_red[m % 3][t >> 5] = hs;
-                }
-                if (which == w_hi - 1) {
-                    fence_async_smem();
-                    __syncwarp();
-                    if (l == 0) mbar_arrive(bars + 8 * (TB_STG0 + m % NS));  // -> the TMA thread stores both copies
-                }
-                // advance the master: zeta m + increment
-#pragma unroll
-                for (int piece = 0; piece < CW / 16; ++piece) {
-                    uint32_t r[16];
-                    TMEM_LD16(tmem + 256 * (m & 1) + 128 * which + lane_addr + CW * cq + 16 * piece, r);
+                    if (w == 0 && c0 + PW == CW) {
+                        float a0, a1;
+                        f2_unpack(sq, a0, a1);
+                        s_sq[m % kSets][t] = sums ? a0 + a1 : 0.f;
+                    }
                     tmem_wait_ld();
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) mm[16 * piece + i] = fmaf(decay, mm[16 * piece + i], __uint_as_float(r[i]));
+                    for (int i = 0; i < PW / 2; ++i)
+                        mst[w][c0 / 2 + i] = f2_fma(decay2, mst[w][c0 / 2 + i], f2_pack(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])));
                 }
             }
-            fence_before();
-            // ---- final state of the sequence
-            if (p.seq_end && a.state_out && c < a.d && col0 < a.d) {      // in the caller's layout (head dimension a.d)
-                float *so = a.state_out + (size_t)p.seq * 2 * a.d * a.d + (size_t)c * a.d + col0;
+            if constexpr (SK::kGroups) {                         // (else the warp's next arrival with scaled rows says the same)
+                fence_before();
+                __syncwarp();
+                if (l == 0) mbar_arrive(bars + 8 * (TB_AD + (m & 1)));
+            }
+            copy += KIND == kD64 ? kTileStateBytes64 : kTileStateBytes;
+            // ---- final state of the sequence, in the caller's layout
+            if (++n == P.N) {
+                if (a.state_out) {
+                    float *const so = a.state_out + (size_t)seq * ext + e_ext;
 #pragma unroll
-                for (int which = 0; which < 2; ++which) {
-                    if (which < w_lo || which >= w_hi) continue;
-                    const float(&mm)[CW] = which ? mU : mH;
+                    for (int w = 0; w < NM; ++w)
 #pragma unroll
-                    for (int i = 0; i < CW / 4; ++i)
-                        *reinterpret_cast<float4 *>(so + which * (size_t)a.d * a.d + 4 * i) = make_float4(mm[4 * i], mm[4 * i + 1], mm[4 * i + 2], mm[4 * i + 3]);
+                        for (int i = 0; i < CW / 4; ++i)
+                            *reinterpret_cast<ulonglong2 *>(so + w * D * D + 4 * i) = make_ulonglong2(mst[w][2 * i], mst[w][2 * i + 1]);
                 }
-            }
-            // ||H_0||_F^2 of the previous tile: its per-warp sums were written before this tile's hand-over barrier (the
-            // block's last tile has none: the sums of the last two tiles are read after the loop).  Three sets of sums,
-            // so that a warp that runs a tile ahead writes none that is still to be read.
-            if (t == 0 && m >= 1 && m + 1 < n_mine && do_h) {
-                float hh = 0.f;
-#pragma unroll
-                for (int i = 0; i < 16; ++i) hh += s_red[(m - 1) % 3][i];
-                hh_out[tile - 1] = hh;
+                n = 0;
+                ++seq;
             }
         }
-        if (t == 0) *reinterpret_cast<volatile int *>(&s_req) = -1;
-        asm volatile("bar.sync 3, 544;" ::: "memory");           // releases the issuing warp; the last sums are published
-        if (t == 0) {
-            for (int m = n_mine >= 2 ? n_mine - 2 : n_mine - 1; m < n_mine && do_h; ++m) {
-                float hh = 0.f;
-#pragma unroll
-                for (int i = 0; i < 16; ++i) hh += s_red[m % 3][i];
-                hh_out[f_lo + m] = hh;
-            }
-            if (s_abort != 0 && a.device_status) atomicExch(a.device_status, (int)GKA_ERR_TIMEOUT);
-        }
-    } else {
-        if (t == 0) *reinterpret_cast<volatile int *>(&s_req) = -1;
-        asm volatile("bar.sync 3, 544;" ::: "memory");
     }
     fence_before();
     __syncthreads();
-    if (s_abort != 0) drain(bars + 8 * TB_DRAIN);
-    if (t < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+    if (t < 32 * kSets && hh_out) {
+        const int m = n_mine - kSets + (t >> 5);             // (tiles before the last ones: the factor warps)
+        if (m >= 0) {
+            float hh = 0.f;
+#pragma unroll
+            for (int i = 0; i < MT / 32; ++i) hh += s_sq[m % kSets][32 * i + l];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) hh += __shfl_xor_sync(0xffffffffu, hh, o);
+            if (l == 0) hh_out[f_lo + m] = hh;
+        }
+    }
+    if (t == 0) {
+        if (s_abort != 0 && a.device_status) atomicExch(a.device_status, (int)GKA_ERR_TIMEOUT);
+    }
+    if (s_abort != 0) drain(bars + 8 * TB_DRAIN, FT);
+    if (t < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(2 * DW) : "memory");
+}
+
+// (cfg: all but the block size and the shared memory, which belong to the kind)
+template <int KIND>
+cudaError_t launch_state(cudaLaunchConfig_t cfg, const CUtensorMap &tmK, const CUtensorMap &tmV, const FwdArgs &a) {
+    static SmemLimit limit;
+    const cudaError_t err = limit.raise(fwd_tc_state_kernel<KIND>, (int)ST_SMEM);
+    if (err != cudaSuccess) return err;
+    cfg.blockDim = dim3(StateKind<KIND>::kThreads);
+    cfg.dynamicSmemBytes = ST_SMEM;
+    return cudaLaunchKernelEx(&cfg, fwd_tc_state_kernel<KIND>, tmK, tmV, a);
 }
 
 // Scan over work items: the start state of item i (when its range starts inside a sequence) is the
@@ -675,20 +822,25 @@ cudaError_t launch_fwd_tc(const FwdArgs &a_in, cudaStream_t stream) {
     // work items) would make every block re-read its whole chain, so the scan kernel materialises the start
     // states once instead.
     a.start_from_scan = longest > 4 ? 1 : 0;
-    // two blocks per work item (one per master) where no sequence is cut and the blocks still fit one per SM
-    a.state_split = (!any_cut && 2 * a.plan.G <= a.sms) ? 1 : 0;
-    // Four blocks per item, 64 columns of one master each, where those still fit one per SM (at head dimension 64 the upper half
-    // would be zeros): a block scales and packs less per tile.  B=4, 8 heads, T=2048, r = 30 / r = 0: 226 -> 218 / 76 -> 68 us for
-    // the call; B=3, 8 heads, T=1999, r = 30: 205 -> 200.  The second half of ||H_0||_F^2 goes to the summaries' place, which
-    // nothing else uses when no sequence is cut.
-    if (a.state_split && 4 * a.plan.G <= a.sms && a.d == D && a.plan.NC <= (long long)a.plan.G * (long long)state_floats(D, D)) {
-        a.state_split = 2;
-        a.tile_hh2 = a.ws.delta;
+    // Blocks per work item (the kernel's KIND): one with both masters where a sequence is cut, else one per master, or one per 64
+    // columns of a master, as long as those fit one per SM.  The solve alone has no blocks for U.
+    const int masters = a.solve_only ? 1 : 2;
+    int kind = kBoth, per_item = 1;
+    if (a.d == 64) {
+        kind = kD64;
+    } else if (!any_cut && masters * a.plan.G <= a.sms) {
+        kind = kOne;
+        per_item = masters;
+        // the second half of ||H_0||_F^2 goes to the summaries' place, which nothing else uses when no sequence is cut
+        if (2 * masters * a.plan.G <= a.sms && a.plan.NC <= (long long)a.plan.G * (long long)state_floats(D, D)) {
+            kind = kQuarter;
+            per_item = 2 * masters;
+            a.tile_hh2 = a.ws.delta;
+        }
     }
-    alignas(64) CUtensorMap tmK, tmV, tmS;      // boxes of 128 tokens x 64 channels; per-tile bf16 state copies
+    alignas(64) CUtensorMap tmK, tmV;           // boxes of 128 tokens x 64 channels
     const int cols = a.heads * a.d;
-    if (!make_tile_map(&tmK, a.k, a.B, a.T, cols, NT) || !make_tile_map(&tmV, a.v, a.B, a.T, cols, NT) ||
-        !make_state_map(&tmS, a.tile_hu, (unsigned long long)a.plan.NC * 256ull))
+    if (!make_tile_map(&tmK, a.k, a.B, a.T, cols, NT) || !make_tile_map(&tmV, a.v, a.B, a.T, cols, NT))
         return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
@@ -697,7 +849,7 @@ cudaError_t launch_fwd_tc(const FwdArgs &a_in, cudaStream_t stream) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cfg.stream = stream;
-    static SmemLimit summary_limit, state_limit[3];
+    static SmemLimit summary_limit;
     if (any_cut) {
         if ((err = summary_limit.raise(fwd_tc_summary_kernel, (int)KV_SMEM)) != cudaSuccess) return err;
         cfg.gridDim = dim3((unsigned)a.plan.G);
@@ -705,19 +857,17 @@ cudaError_t launch_fwd_tc(const FwdArgs &a_in, cudaStream_t stream) {
         cfg.dynamicSmemBytes = KV_SMEM;
         if ((err = cudaLaunchKernelEx(&cfg, fwd_tc_summary_kernel, tmK, tmV, a)) != cudaSuccess) return err;
         if (a.start_from_scan) {
-            cfg.gridDim = dim3(2 * D * D / 4 / 256, (unsigned)(a.plan.G - 1));
+            cfg.gridDim = dim3((a.solve_only ? 1 : 2) * D * D / 4 / 256, (unsigned)(a.plan.G - 1));
             cfg.blockDim = dim3(256);
             cfg.dynamicSmemBytes = 0;
             if ((err = cudaLaunchKernelEx(&cfg, fwd_scan, a)) != cudaSuccess) return err;
         }
         a.after_summary = 1;
     }
-    auto state_kernel = a.state_split == 2 ? fwd_tc_state_kernel<4> : a.state_split ? fwd_tc_state_kernel<2> : fwd_tc_state_kernel<1>;
-    if ((err = state_limit[a.state_split].raise(state_kernel, (int)ST_SMEM)) != cudaSuccess) return err;
-    cfg.gridDim = dim3((unsigned)(a.plan.G << a.state_split));
-    cfg.blockDim = dim3(kThreadsStateK);
-    cfg.dynamicSmemBytes = ST_SMEM;
-    if ((err = cudaLaunchKernelEx(&cfg, state_kernel, tmK, tmV, tmS, a)) != cudaSuccess) return err;
+    cfg.gridDim = dim3((unsigned)(a.plan.G * per_item));
+    err = kind == kD64 ? launch_state<kD64>(cfg, tmK, tmV, a) : kind == kQuarter ? launch_state<kQuarter>(cfg, tmK, tmV, a)
+          : kind == kOne ? launch_state<kOne>(cfg, tmK, tmV, a) : launch_state<kBoth>(cfg, tmK, tmV, a);
+    if (err != cudaSuccess) return err;
     return launch_fwd_solve(a, stream);
 }
 
