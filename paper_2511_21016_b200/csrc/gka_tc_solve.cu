@@ -882,19 +882,14 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             auto stage_keys = [&](int jj) {
                 wait_bar(sb + 8 * (B_GS0 + (jj & 1)), (uint32_t)((jj >> 1) & 1), abort_addr);
                 wait_bar(sb + 8 * B_LD_K, (uint32_t)(jj & 1), abort_addr);
-                const float fj = sc->g[jj & 1].ks[c];
-                const uint64_t f2 = f2_pack(fj, fj);
+                const uint2 fj = split_factor(sc->g[jj & 1].ks[c]);
 #pragma unroll 1
-                for (int g = 0; g < 2 * NG16; ++g) {             // (rolled: code that runs once per tile is kept small)
-                    uint4 v = *reinterpret_cast<const uint4 *>(bufa + tile_off(c, g));
-                    uint32_t *pv = reinterpret_cast<uint32_t *>(&v);
+                for (int g = 0; g < 2 * NG16; g += 4) {          // (rolled: code that runs once per tile is kept small)
+                    uint4 v[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        float lo, hi;
-                        f2_unpack(f2_mul(f2_pack(bf16_lo(pv[u]), bf16_hi(pv[u])), f2), lo, hi);
-                        pv[u] = pack_bf16(lo, hi);
-                    }
-                    *reinterpret_cast<uint4 *>(bufa + tile_off(c, g)) = v;
+                    for (int u = 0; u < 4; ++u) v[u] = *reinterpret_cast<const uint4 *>(bufa + tile_off(c, g + u));
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) *reinterpret_cast<uint4 *>(bufa + tile_off(c, g + u)) = times_factor(v[u], fj);
                 }
                 fence_async_smem();
             };

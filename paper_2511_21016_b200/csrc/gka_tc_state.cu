@@ -42,17 +42,7 @@ constexpr uint32_t STAGE = 65536;                        // K tile + V tile
 constexpr uint32_t KV_SMEM = NS * STAGE + 1024;          // + slack for the 1024-byte alignment of the base
 constexpr uint32_t ST_SMEM = KV_SMEM;
 
-// A row factor f >= 0 as hi + lo, two bf16 terms each twice in a word: hi is f cut off after eight bits, lo the rest, to 2^-17 of f.
-// (lo is never 0 beside a hi that is not, nor negative: an infinite element stays infinite.)
-__device__ __forceinline__ uint2 split_factor(float f) {
-    const uint32_t hi = __float_as_uint(f) & 0xFFFF0000u;
-    const float rest = f - __uint_as_float(hi);
-    const float lo = fmaxf(rest, __uint_as_float(hi) * 9.3132257e-10f);      // 2^-30
-    return make_uint2(hi | hi >> 16, pack_bf16(lo, lo));
-}
-// The first N * THREADS 16-byte groups of BOXES operand boxes (64 channels of 128 tokens each) times f[row]: v hi + (v lo), the fused multiply-add
-// rounded once, is the product with f to within 2^-17 before its rounding to bf16, in two instructions per pair of elements
-// (unpacking to fp32, multiplying and packing takes six).
+// The first N * THREADS 16-byte groups of BOXES operand boxes (64 channels of 128 tokens each) times f[row]
 template <int N, int THREADS, int BOXES>
 __device__ __forceinline__ void scale_rows(unsigned char *box, const uint2 *f, int t) {
     uint4 v[BOXES][N];
@@ -65,14 +55,8 @@ __device__ __forceinline__ void scale_rows(unsigned char *box, const uint2 *f, i
     }
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-        const __nv_bfloat162 hi = *reinterpret_cast<const __nv_bfloat162 *>(&fj[i].x), lo = *reinterpret_cast<const __nv_bfloat162 *>(&fj[i].y);
 #pragma unroll
-        for (int x = 0; x < BOXES; ++x) {
-            __nv_bfloat162 *const p = reinterpret_cast<__nv_bfloat162 *>(&v[x][i]);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) p[u] = __hfma2(p[u], hi, __hmul2(p[u], lo));
-            *reinterpret_cast<uint4 *>(box + 16384 * x + (t + THREADS * i) * 16) = v[x][i];
-        }
+        for (int x = 0; x < BOXES; ++x) *reinterpret_cast<uint4 *>(box + 16384 * x + (t + THREADS * i) * 16) = times_factor(v[x][i], fj[i]);
     }
 }
 

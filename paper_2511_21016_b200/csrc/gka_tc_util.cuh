@@ -83,6 +83,23 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 }
 __device__ __forceinline__ float bf16_lo(uint32_t p) { return __uint_as_float(p << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t p) { return __uint_as_float(p & 0xFFFF0000u); }
+// A row factor f >= 0 as hi + lo, two bf16 terms each twice in a word: hi is f cut off after eight bits, lo the rest, to 2^-17 of f.
+// (lo is never 0 beside a hi that is not, nor negative: an infinite element stays infinite.)
+__device__ __forceinline__ uint2 split_factor(float f) {
+    const uint32_t hi = __float_as_uint(f) & 0xFFFF0000u;
+    const float rest = f - __uint_as_float(hi);
+    const float lo = fmaxf(rest, __uint_as_float(hi) * 9.3132257e-10f);      // 2^-30
+    return make_uint2(hi | hi >> 16, pack_bf16(lo, lo));
+}
+// Eight bf16 elements times a split factor: v hi + (v lo), the fused multiply-add rounded once, is the product with f to within 2^-17
+// before its rounding to bf16, in two instructions per pair of elements (unpacking to fp32, multiplying and packing takes six).
+__device__ __forceinline__ uint4 times_factor(uint4 v, uint2 f) {
+    const __nv_bfloat162 hi = *reinterpret_cast<const __nv_bfloat162 *>(&f.x), lo = *reinterpret_cast<const __nv_bfloat162 *>(&f.y);
+    __nv_bfloat162 *const p = reinterpret_cast<__nv_bfloat162 *>(&v);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) p[u] = __hfma2(p[u], hi, __hmul2(p[u], lo));
+    return v;
+}
 // Packed pairs of fp32 values in one 64-bit register and the two-wide fp32 arithmetic of sm_100
 __device__ __forceinline__ uint64_t f2_pack(float lo, float hi) {
     uint64_t r;
