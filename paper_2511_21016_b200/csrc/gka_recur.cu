@@ -131,18 +131,18 @@ __device__ __forceinline__ void matvec(const ulonglong2 (&H)[8][Rc<D>::CG], cons
         for (int q = 0; q < Q; ++q) y[Q * p + q] = yp[q];
     }
 }
-// Tokens t0 and t0 + 1 of the batch: row sums v of the thread's block of H, and S[4 t + j] = Gamma[t][j] (k_j . x_t) with kj
-// the columns of key lane / 8: even warps take token t0, odd ones t0 + 1 (no branch: the arithmetic of the pair before is
-// scheduled into this one's).
+// Two tokens of the batch, the warp's own (t0 for even warps, t0 + 1 for odd ones) and the other: row sums v[.][0] and v[.][1] of the
+// thread's block of H, and S[4 t + j] = Gamma[t][j] (k_j . x_t) of the own token with kj the columns of key lane / 8.  (No branch: the
+// arithmetic of the pair before is scheduled into this one's.)
 template <int D>
 __device__ __forceinline__ void pair_sums(const ulonglong2 (&H)[8][Rc<D>::CG], const ulonglong2 (&kj)[Rc<D>::CG], const float *sX,
                                           const float *sGam, float *sS, int t0, float (&v)[8][2]) {
-    const int lane = threadIdx.x & 31, lane8 = lane & 7;
-    const bool odd = (threadIdx.x & 32) != 0;
+    const int lane = threadIdx.x & 31, lane8 = lane & 7, odd = (threadIdx.x >> 5) & 1;
+    const float *const xa_p = sX + (t0 + odd) * D + 4 * lane8, *const xb_p = sX + (t0 + 1 - odd) * D + 4 * lane8;
     uint64_t acc[8][2], dot = 0ull;
 #pragma unroll
     for (int n = 0; n < Rc<D>::CG; ++n) {
-        const ulonglong2 xa = lds2x2(sX + t0 * D + 4 * (lane8 + 8 * n)), xb = lds2x2(sX + (t0 + 1) * D + 4 * (lane8 + 8 * n));
+        const ulonglong2 xa = lds2x2(xa_p + 32 * n), xb = lds2x2(xb_p + 32 * n);
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
             acc[m][0] = n == 0 ? f2_mul(H[m][n].x, xa.x) : f2_fma(H[m][n].x, xa.x, acc[m][0]);
@@ -153,13 +153,13 @@ __device__ __forceinline__ void pair_sums(const ulonglong2 (&H)[8][Rc<D>::CG], c
             acc[m][0] = f2_fma(H[m][n].y, xa.y, acc[m][0]);
             acc[m][1] = f2_fma(H[m][n].y, xb.y, acc[m][1]);
         }
-        dot = f2_fma(kj[n].x, odd ? xb.x : xa.x, dot);
-        dot = f2_fma(kj[n].y, odd ? xb.y : xa.y, dot);
+        dot = f2_fma(kj[n].x, xa.x, dot);
+        dot = f2_fma(kj[n].y, xa.y, dot);
     }
     float s = hsum(dot);
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    const int i = 4 * (t0 + (odd ? 1 : 0)) + (lane >> 3);
+    const int i = 4 * (t0 + odd) + (lane >> 3);
     if (lane8 == 0) sS[i] = sGam[i] * s;
 #pragma unroll
     for (int m = 0; m < 8; ++m)
@@ -383,12 +383,13 @@ __device__ __forceinline__ bool batch(const RecurArgs &a, const Mem<D, IoT> &sm,
             ulonglong2 kj[CG];                               // key (lane / 8), for the pair's products with the keys
 #pragma unroll
             for (int n = 0; n < CG; ++n) kj[n] = lds2x2(sm.K + (lane >> 3) * D + 4 * (lane8 + 8 * n));
+            const bool odd = (warp & 1) != 0;                // v[.][0] is the warp's own token
             float v0[8][2], v1[8][2];
             auto finish = [&](int t0, float (&v)[8][2], float4 sa, float4 sb) {
                 float y[2];
                 reduce_rows<2>(v, y);
-                advance(t0, y[0], sa);
-                advance(t0 + 1, y[1], sb);
+                advance(t0, odd ? y[1] : y[0], sa);
+                advance(t0 + 1, odd ? y[0] : y[1], sb);
             };
             // products of the tokens t1, t1 + 1 beside the update of the tokens t0, t0 + 1
             auto region = [&](int t1, float (&v1)[8][2], int t0, float (&v0)[8][2]) {
