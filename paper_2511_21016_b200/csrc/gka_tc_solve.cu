@@ -413,10 +413,25 @@ __device__ __forceinline__ void p_epilogue_t(const Ctx &cx, const GateScalars *g
     }
     tmem_wait_st();
 }
-template <bool KEYF, bool AHEAD>
+// The epilogues of strongly decaying tiles, which most calls never run, as functions: inlined they lie between the others' code (what
+// the warps execute does not fit the first-level instruction cache, and neighbours of it are fetched too).  The read's as a function:
+// 64 x 2048 tokens, d = 64: 117.8 -> 116.3 us, nothing else changes; an iteration's too: with beta, alpha or for the solve alone 197.7
+// -> 194.0 (24 x 1999, 30 iterations) and 185.5 -> 183.0 (32 x 2048), but in the plain kernel at 128 channels a call there costs spills
+// (349 -> 350, 131072 tokens 5700 -> 5740), so there it stays inlined.
+template <bool KEYF>
+__device__ __noinline__ void p_epilogue_exact(uint32_t tm_s, int q, int l, const GateScalars *gs, float ac_c, const DiagMasks *dm) {
+    Ctx cx;
+    cx.tm_s = tm_s;
+    cx.q = q;
+    cx.l = l;
+    p_epilogue_t<true, KEYF, false>(cx, gs, ac_c, *dm);
+}
+template <bool KEYF, bool AHEAD, bool CALL>
 __device__ __forceinline__ void p_epilogue(const Ctx &cx, const GateScalars *gs, bool exact, float ac_c, const DiagMasks &dm) {
-    if (exact) p_epilogue_t<true, KEYF, AHEAD>(cx, gs, ac_c, dm);
-    else p_epilogue_t<false, KEYF, AHEAD>(cx, gs, ac_c, dm);
+    if (exact) {
+        if constexpr (CALL) p_epilogue_exact<KEYF>(cx.tm_s, cx.q, cx.l, gs, ac_c, &dm);
+        else p_epilogue_t<true, KEYF, AHEAD>(cx, gs, ac_c, dm);
+    } else p_epilogue_t<false, KEYF, AHEAD>(cx, gs, ac_c, dm);
 }
 
 // Sum over one 32-key block of the squared Gram entries of the earlier keys (decayed when the keys are not
@@ -992,7 +1007,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 const float beta = omega - 1.f, cz = czb * omega;
                 const uint64_t beta2 = f2_pack(beta, beta), cz2 = f2_pack(cz, cz), lz2 = f2_pack(lz, lz);
                 wait_scores();                                   // the masked scores
-                p_epilogue<false, !HALF>(cx, gs, exact, exact ? gs->ac[c] : 0.f, dm);
+                p_epilogue<false, !HALF, EXTRA>(cx, gs, exact, exact ? gs->ac[c] : 0.f, dm);
                 fence_before();
                 request(OP_ITER2, 0u);
                 wait_r();
@@ -1096,7 +1111,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             request(OP_OUT_S, (uint32_t)(j & 1));
             wait_scores();
             load_next_k();                                       // its products were the last readers of the keys
-            p_epilogue<true, !HALF>(cx, gs, exact, exact ? gs->ac[c] : 0.f, dm);
+            p_epilogue<true, !HALF, true>(cx, gs, exact, exact ? gs->ac[c] : 0.f, dm);
             fence_before();
             request(OP_OUT_O, (uint32_t)(j & 1));
             // (the values stay as loaded: their row factor sqrt(beta_j) 2^(-G_j / 2) rides on the masked scores)
