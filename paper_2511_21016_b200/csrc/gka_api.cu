@@ -152,11 +152,11 @@ size_t gka_fwd_workspace_bytes(const gka_desc *desc, int chunk) {
 // sequences the summary kernel reads all keys and values once more.  Items of whole sequences (pairs / k items of k sequences each, k
 // the smallest divisor of the number of (sequence, head) pairs that leaves at most one item per SM) need no summaries, but may
 // leave SMs idle in the state kernel and make its run of tiles longer.  With n tiles per sequence whole sequences cost
-// per_tile k n us, ranges cut pairs / SMs n + fixed (the extra launches).  Fitted to both sides of 33 shapes at r = 0 (us per call, whole
+// per_tile k n us, ranges cut pairs / SMs n + fixed (the extra launches).  Fitted to both sides of 28 shapes at r = 0 (us per call, whole
 // sequences / ranges):
-//   d = 128 (per_tile by how many blocks share an item): 1 pair, 32 tiles 44.6 / 54.0; 8 pairs, 32 tiles 47.1 / 76.7, 64 tiles 88.8 / 99.1;
-//     16 pairs, 64 tiles 113 / 136, 128 tiles 208 / 216; 32 pairs, 64 tiles 165 / 214, 1024 tiles 2657 / 2824; 64 pairs, 64
-//     tiles 312 / 390; 96 pairs, 64 tiles 473 / 545; 256 pairs (two per item), 32 tiles 589 / 680
+//   d = 128 (per_tile by how many blocks share an item): 1 pair, 32 tiles 48.3 / 53.9; 8 pairs, 32 tiles 52.0 / 76.4, 64 tiles 98.2 / 98.8;
+//     16 pairs, 64 tiles 122 / 135, 128 tiles 228 / 213; 32 pairs, 64 tiles 172 / 210, 1024 tiles 2824 / 2809; 64 pairs, 64
+//     tiles 339 / 398; 96 pairs, 64 tiles 482 / 538; 256 pairs (two per item), 32 tiles 579 / 673
 //   d = 64: 8 pairs, 32 tiles 43.9 / 55.2, 64 tiles 74.5 / 69.1; 16 pairs, 32 tiles 50.2 / 62.2, 64 tiles 90.7 / 84.4; 32 pairs, 64
 //     tiles 119 / 129, 128 tiles 247 / 250; 64 pairs, 64 tiles 179 / 217; 256 pairs, 64 tiles 700 / 816
 //   the solve alone, d = 128: 8 pairs, 32 tiles 41.9 / 50.3; 16 pairs, 64 tiles 92.7 / 87.8; 32 pairs, 256 tiles 575 / 562; 64 pairs, 64
@@ -168,8 +168,8 @@ static int state_items(const gka_desc *desc, int sms, bool solve_only) {
         if (pairs % k != 0 || pairs / k > cap) continue;
         const long long items = pairs / k;
         const bool light = desc->d_k == 64 || solve_only;            // half the state or less
-        const double per_tile = light ? 0.83 : 4 * items <= sms ? 0.84 : 2 * items <= sms ? 1.31 : 2.2;
-        const double cut = light ? 3.05 : 4.4, fixed = light ? 28.0 : 40.0;
+        const double per_tile = light ? 0.83 : 4 * items <= sms ? 0.95 : 2 * items <= sms ? 1.42 : 2.2;
+        const double cut = light ? 3.05 : 4.2, fixed = light ? 28.0 : 40.0;
         if ((double)n * ((double)k * per_tile - cut * (double)pairs / sms) < fixed) return (int)items;
         break;
     }

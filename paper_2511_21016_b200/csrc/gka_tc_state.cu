@@ -281,22 +281,24 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 //   - what a thread contributes to ||H_0||_F^2 is left in shared memory, and a factor warp adds it up tiles later;
 //   - gates and write strengths are loaded a whole turn of the factor warps ahead and looked at only then.
 // us per call of this kernel, before (one block-wide step after another, copies staged, head dimension 64 on 128 x 128 masters) and with
-// this: 64 sequences x 4096 tokens 80 -> 55; 32 x 2048, solve alone (H only) 36 -> 18; 24 x 1999 with write strengths 61 -> 22 (their
-// loads used to be waited for in the issuing warp); 64 x 2048, d = 64: 42 -> 19.
+// this: 64 sequences x 4096 tokens 80 -> 60; 32 x 2048, solve alone (H only) 36 -> 18; 24 x 1999 with write strengths 61 -> 25 (their
+// loads used to be waited for in the issuing warp); 64 x 2048, d = 64: 42 -> 20.
 //
 // KIND: what a block keeps.
 //   kBoth     H and U (128 channels), where sequences are cut or the items alone fill the device
 //   kOne      H or U: two blocks per item
 //   kQuarter  64 columns of H or of U: four blocks per item
 //   kD64      head dimension 64: H over U as one 128 x 64 master, [K V]^T K one product per k-step
-// Blocks that keep U alone scale the keys by the whole weight and leave V as it is.  The solve alone reads no U: its blocks are not launched.
+// H and U are made from the same rounded keys, whichever block makes them.  (The whole weight on K, and V as it is, halves the scaling of a
+// block of U and brings U itself closer, 1.4e-3 against 2.0e-3, but the read U x meets an H of other keys: 4.9e-3 -> 5.7e-3 at 3 heads x
+// 1999 tokens, 30 iterations.)  The solve alone reads no U: its blocks are not launched.
 // ------------------------------------------------------------------------------------------------------------
 enum { kBoth = 0, kOne = 1, kQuarter = 2, kD64 = 3 };
 // Warps: those that keep the masters; groups that scale rows and take the tiles in turn; helpers (row factors, products, loads).  With 32 KB
 // of K (and V) per tile six stages fit, and what counts is how many tiles are worked on at once: two groups of four warps.  With 64 KB
 // (kBoth, kOne's blocks of U) three fit, so that a stage has to be given back soon: all sixteen warps scale a tile together, a tile ahead,
-// and then keep its masters.  (64 x 4096 tokens, kOne: 54 us, 58 with a group of eight warps, 60 with two of four; 32 x 4096, kQuarter: 42
-// us in one group of all warps, 35.4 with two.)
+// and then keep its masters.  (With V left unscaled in the blocks of U: 64 x 4096 tokens, kOne: 54 us, 58 with a group of eight warps, 60
+// with two of four; 32 x 4096, kQuarter: 42 us in one group of all warps, 35.4 with two.)
 // Registers of a thread at launch (what its share of 65,536 allows) and after the split.
 template <int KIND> struct StateKind {
     static constexpr bool kGroups = KIND == kQuarter || KIND == kD64;
@@ -418,12 +420,12 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         if constexpr (SK::kGroups) {
 #pragma unroll 2
             for (int i = 0; i < 4; ++i) {
-                if (KIND == kQuarter && u_only) scale_rows<2, GT, 1>(stage, f, ts + 2 * GT * i);
+                if (KIND == kQuarter && u_only) scale_rows<2, GT, 3>(stage, f, ts + 2 * GT * i);
                 else scale_rows<2, GT, 2>(stage, f, ts + 2 * GT * i);
             }
         } else {
             scale_rows<2, GT, 2>(stage, f, ts);
-            if (both) scale_rows<2, GT, 2>(stage + 32768, f, ts);
+            if (both || u_only) scale_rows<2, GT, 2>(stage + 32768, f, ts);
         }
         fence_async_smem();
         fence_before();
@@ -456,8 +458,7 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             }
         } else if (t >= CT && t < FT) {
             // ================ factor warps: row factors and decays, and the sums of ||H_0||_F^2 ================
-            // Row factor of token j of a tile: the root of w_j = beta_j 2^(G_last - G_j), or w_j itself where only one of a product's
-            // operands is scaled; 0 past the sequence.  As two bf16 terms, for scale_rows.
+            // Row factor of token j of a tile: the root of w_j = beta_j 2^(G_last - G_j); 0 past the sequence.  As two bf16 terms, for scale_rows.
             // The warps take the tiles in turn: a tile's scan, logarithms and sums are a chain of some 4000 cycles beside the warps that scale,
             // several times as long as a tile.  Before it publishes, tile f waits until the products of tile f - ns are complete: the phase
             // before its own of the barrier is then complete, and the masters are past tile f - ns - 2 (the products of a
@@ -508,13 +509,13 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const float e = before - incl[i];
-                    factor[i] = u_only ? exp2f(e) : exp2f(0.5f * e);
+                    factor[i] = exp2f(0.5f * e);
                 }
                 if (a.beta) {
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         const float w = fmaxf(x.b[i], 0.f);
-                        factor[i] *= u_only ? w : sqrtf(w);
+                        factor[i] *= sqrtf(w);
                     }
                 } else {
 #pragma unroll
