@@ -233,7 +233,7 @@ __device__ __forceinline__ void store_rows(IoT *dst, const uint64_t (&o)[R / 2])
 }
 
 // Blocks of two warps, 8 warps per SM: with 12 (168 registers, some spilled) this kernel took 95 us instead of 80 at 64 x 8 pairs,
-// T = 196, d = 16, 30 iterations (multiply-add pipe 69 % of active cycles; the call: 91 us, 3997 us before on the chunk-wise kernel
+// T = 196, d = 16, 30 iterations (multiply-add pipe 69 % of active cycles; the call: 84 us, 3997 us before on the chunk-wise kernel
 // zero-extended to 64 channels).
 constexpr int kSolveWarps = 2;
 constexpr int kSolveBlocks = 4;

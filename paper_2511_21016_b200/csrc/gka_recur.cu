@@ -25,9 +25,10 @@
 // segment, and a block of a later part first folds the tokens of its segment that come before it.
 //
 // Measured, before (chunk-wise fp32 kernels; one token at a time for decoding) and with these kernels: B=2, 8 heads, T=8192,
-// d=128, f32, r=8: 3209 -> 2075 us; 64 x 32 pairs, 8 tokens, d=128, bf16, r=10: 425 -> 286 us; B=1, 2 heads, T=256, d=64, f32,
-// r=8: 118.5 -> 29 us (there: three dependent launches and the chain of batches).  Tried: scalar instead of two-wide
-// multiply-adds +10 %, the batch's constants in shared memory +8 %, rolled loops +3 %.
+// d=128, f32, r=8: 3209 -> 1945 us; 64 x 32 pairs, 8 tokens, d=128, bf16, r=10: 425 -> 267 us; B=1, 2 heads, T=256, d=64, f32,
+// r=8: 118.5 -> 25.5 us (there: three dependent launches and the chain of batches).  Tried: scalar instead of two-wide
+// multiply-adds +10 %, the batch's constants in shared memory +8 %, rolled loops +3 %, both tokens of a pair updated in two-wide
+// registers +5 % (fewer instructions, a longer chain), two-wide multiply-adds in recur_summary 228 -> 260 us.
 #include "gka_common.cuh"
 #include "gka_tc_util.cuh"
 
@@ -133,7 +134,8 @@ __device__ __forceinline__ void matvec(const ulonglong2 (&H)[8][Rc<D>::CG], cons
 }
 // Two tokens of the batch, the warp's own (t0 for even warps, t0 + 1 for odd ones) and the other: row sums v[.][0] and v[.][1] of the
 // thread's block of H, and S[4 t + j] = Gamma[t][j] (k_j . x_t) of the own token with kj the columns of key lane / 8.  (No branch: the
-// arithmetic of the pair before is scheduled into this one's.)
+// arithmetic of the pair before is scheduled into this one's.  No selects: choosing the own token's words of two operands was 16
+// instructions per pair; 64 x 32 pairs, 8 tokens 287.6 -> 268.1 us, 2 x 8 pairs, T = 8192 2071 -> 1952.)
 template <int D>
 __device__ __forceinline__ void pair_sums(const ulonglong2 (&H)[8][Rc<D>::CG], const ulonglong2 (&kj)[Rc<D>::CG], const float *sX,
                                           const float *sGam, float *sS, int t0, float (&v)[8][2]) {

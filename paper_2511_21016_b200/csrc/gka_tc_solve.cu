@@ -49,7 +49,8 @@
 // take half of their columns, which leaves room for a score tile per slot: nothing is handed from slot to slot, so a slot is
 // one chain of its four compute warps, and one of their threads issues the slot's products (no issuing thread: a request no
 // longer waits for a thread that serves both slots).  B = 4, 16 heads, T = 2048, 10 / 30 iterations: 177 / 351 us per call with
-// the shared score tile, 152 / 288 with this.
+// the shared score tile, 152 / 288 with this (121 at 10 with the present state kernel).  Two threads per token, each with half of the
+// channels and every other key block, measured slower (117.4 -> 120.4).
 #include <cuda.h>
 
 #include "gka_common.cuh"
