@@ -84,11 +84,11 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 __device__ __forceinline__ float bf16_lo(uint32_t p) { return __uint_as_float(p << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t p) { return __uint_as_float(p & 0xFFFF0000u); }
 // A row factor f >= 0 as hi + lo, two bf16 terms each twice in a word: hi is f cut off after eight bits, lo the rest, to 2^-17 of f.
-// (lo is never 0 beside a hi that is not, nor negative: an infinite element stays infinite.)
+// (lo is never 0 beside a hi that is not, nor negative, so an infinite element stays infinite: where the rest is 0 or rounds to 0, lo is
+// the smallest bf16 number, which is also the smallest hi other than 0.)
 __device__ __forceinline__ uint2 split_factor(float f) {
     const uint32_t hi = __float_as_uint(f) & 0xFFFF0000u;
-    const float rest = f - __uint_as_float(hi);
-    const float lo = fmaxf(rest, __uint_as_float(hi) * 9.3132257e-10f);      // 2^-30
+    const float lo = fmaxf(f - __uint_as_float(hi), fminf(__uint_as_float(hi), 9.1835496e-41f));      // 2^-133
     return make_uint2(hi | hi >> 16, pack_bf16(lo, lo));
 }
 // Eight bf16 elements times a split factor: v hi + (v lo), the fused multiply-add rounded once, is the product with f to within 2^-17
