@@ -94,7 +94,8 @@ inline size_t small_workspace_bytes_for(long long pairs, int T, int d) {
 // kernel walks the plan's items, carries the fp32 (H, U) on chip and stores, for every tile,
 // the bf16 operand copies of the tile-initial H_0 and U_0 and ||H_0||_F^2; the solve kernel then treats the
 // tiles as independent problems.  Workspace: start states [G][st], summaries [G][st], decay products [G],
-// ||H_0||_F^2 [tiles], bf16 copies [tiles][2][128][128].
+// ||H_0||_F^2 [tiles], bf16 copies [tiles][H, U][column / 8][row][8 columns], 128 x 128 or 64 x 64 (room for the former either way).
+// The solve alone writes and reads nothing of U: half of each copy, summary and start state stays as it was.
 // ---------------------------------------------------------------------------------------------
 constexpr int kTile = 128;
 __host__ __device__ constexpr int tiles_of(int T) { return (T + kTile - 1) / kTile; }

@@ -23,11 +23,11 @@ __host__ __device__ constexpr uint32_t t_mn(uint32_t off) { return (off >> 4) | 
 __host__ __device__ constexpr uint32_t t_kstep(int ks) { return (uint32_t)(((ks >> 2) * 16384 + (ks & 3) * 32) >> 4); }
 __host__ __device__ constexpr uint32_t t_mnstep(int ks) { return (uint32_t)((ks * 2048) >> 4); }
 
-// State copies as an operand (B, contraction over the columns): [column / 8][128 rows][8 columns] without a swizzle, so 8 rows x 16 bytes
-// are consecutive, 128 bytes from one group of 8 rows to the next and 2048 from one group of 8 columns to the next
+// State copies as an operand (B, contraction over the columns): [column / 8][rows][8 columns] without a swizzle, so 8 rows x 16 bytes are
+// consecutive, 128 bytes from one group of 8 rows to the next and 16 x rows from one group of 8 columns to the next.  A matrix has as many
+// rows as columns: 16 per k-step of its NK.
 constexpr uint32_t kDescHiState = (128u >> 4) | (1u << 14);
-__host__ __device__ constexpr uint32_t t_state(uint32_t off) { return (off >> 4) | ((2048u >> 4) << 16); }
-__host__ __device__ constexpr uint32_t t_statestep(int ks) { return (uint32_t)((ks * 4096) >> 4); }
+template <int NK> __host__ __device__ constexpr uint32_t t_state(int ks) { return (uint32_t)((ks * 512 * NK) >> 4) | ((256u * NK >> 4) << 16); }
 
 // D (+)= A x B, both operands in shared memory: low words are a base register plus an immediate
 template <int ACC, uint32_t A_CONST, uint32_t B_CONST, uint32_t B_HI = kDescHi>
@@ -60,7 +60,7 @@ __device__ __forceinline__ void mma8_kk(uint32_t d, uint32_t a_base, uint32_t b_
 template <int ACC0, int NK = 8, int KS = 0>   // A K-major, B a state copy, NK k-steps over the first 16 NK columns
 __device__ __forceinline__ void mma8_ks(uint32_t d, uint32_t a_base, uint32_t b_base, uint32_t idesc) {
     if constexpr (KS < NK) {
-        mma_ss2<(KS == 0 ? ACC0 : 1), t_kmaj(0) + t_kstep(KS), t_state(0) + t_statestep(KS), kDescHiState>(d, a_base, b_base, idesc);
+        mma_ss2<(KS == 0 ? ACC0 : 1), t_kmaj(0) + t_kstep(KS), t_state<NK>(KS), kDescHiState>(d, a_base, b_base, idesc);
         mma8_ks<ACC0, NK, KS + 1>(d, a_base, b_base, idesc);
     }
 }

@@ -196,10 +196,10 @@ __device__ __forceinline__ TileInfo tile_info(const FwdArgs &a, long long tile) 
     return t;
 }
 
-// H_0 of a tile; head dimension 64: H_0 and U_0
+// H_0 of a tile; head dimension 64: and U_0 behind it, which nobody has written for the solve alone
 template <bool HALF>
-__device__ __forceinline__ void load_h0(const FwdArgs &a, long long tile, uint32_t dst, uint32_t bar) {
-    constexpr uint32_t bytes = HALF ? (uint32_t)kTileStateBytes64 : 32768u;
+__device__ __forceinline__ void load_h0(const FwdArgs &a, long long tile, uint32_t dst, uint32_t bar, bool h_only) {
+    const uint32_t bytes = !HALF ? 32768u : h_only ? (uint32_t)kTileStateBytes64 / 2 : (uint32_t)kTileStateBytes64;
     mbar_expect_tx(bar, bytes);
     bulk_load(dst, a.tile_hu + (size_t)tile * (HALF ? kTileStateBytes64 : kTileStateBytes), bytes, bar);
 }
@@ -229,7 +229,7 @@ __device__ __forceinline__ void mma8_ek(uint32_t d, uint32_t e_tmem, uint32_t b_
 template <int ACC0, int NK = 8, int KS = 0>
 __device__ __forceinline__ void mma8_es(uint32_t d, uint32_t e_tmem, uint32_t b_base, uint32_t idesc) {
     if constexpr (KS < NK) {
-        mma_ts_c<(KS == 0 ? ACC0 : 1), t_state(0) + t_statestep(KS), kDescHiState>(d, e_tmem + 8 * KS, b_base, idesc);
+        mma_ts_c<(KS == 0 ? ACC0 : 1), t_state<NK>(KS), kDescHiState>(d, e_tmem + 8 * KS, b_base, idesc);
         mma8_es<ACC0, NK, KS + 1>(d, e_tmem, b_base, idesc);
     }
 }
@@ -277,7 +277,7 @@ __device__ __forceinline__ void issue_batch(int op, bool half, uint32_t kb, uint
             prod_ek<0>(half, tm_S, tm_E, kb, kIdescKK);
             prod_ek<1>(half, tm_S, tm_R, kb, kIdescKK);
             mma_commit(bar_sc);
-            prod_es<0>(half, tm_R, tm_E, half ? hb + (1024u >> 4) : hb, idesc_r_kk(half));   // O = X_hi U_0^T (64 channels: U_0 follows H_0's rows) (runs under the masked-score epilogue; X_lo has been read)
+            prod_es<0>(half, tm_R, tm_E, half ? hb + (8192u >> 4) : hb, idesc_r_kk(half));   // O = X_hi U_0^T (64 channels: U_0 follows H_0) (runs under the masked-score epilogue; X_lo has been read)
             break;
         case OP_OUT_O:   // O += P V
             mma8_pm(tm_R, tm_S, cb, idesc_r_pm(half));
@@ -598,7 +598,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     mbar_expect_tx(sb + 8 * B_LD_K, 32768u);
                     tma_load_tile3(&tmK, sl + BUF_A, sb + 8 * B_LD_K, ti.h * a.d, tile_x_hi(ti.h, a.d, a.heads), ti.n * NT, ti.b);
                     asm volatile("griddepcontrol.wait;" ::: "memory");
-                    load_h0<HALF>(a, t_lo + slot, sl + BUF_B, sb + 8 * B_LD_H);
+                    load_h0<HALF>(a, t_lo + slot, sl + BUF_B, sb + 8 * B_LD_H, solve_only);
                 }
                 for (int j = 0; j < n_slot; ++j) {
                     const int k = slot + 2 * j;
@@ -878,7 +878,7 @@ fwd_tc_solve_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 }
             };
             auto load_next_h = [&]() {
-                if (leader && more && !aborted(abort_addr)) load_h0<HALF>(a, tile + kSlots, sl + BUF_B, sb + 8 * B_LD_H);
+                if (leader && more && !aborted(abort_addr)) load_h0<HALF>(a, tile + kSlots, sl + BUF_B, sb + 8 * B_LD_H, solve_only);
             };
             auto after_last_h0_product = [&]() {      // H_0 has been read for the last time
                 if (solve_only) {

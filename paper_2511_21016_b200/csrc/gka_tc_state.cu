@@ -274,8 +274,8 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 // tile take one after another, so as many tiles as possible are worked on at once.  Every access to shared memory (a shuffle, a barrier, a
 // load) waits 100 to 250 cycles behind the scaling warps' traffic, so accesses in a chain count more than instructions:
 //   - a row factor is two bf16 terms and a product two instructions per pair of elements (scale_rows);
-//   - the copies go straight from registers to global memory: in the workspace eight consecutive columns of the 128 rows lie together
-//     (2 KB), so a warp's store is 512 consecutive bytes, and the solve kernel reads those bytes as a tensor-core operand without a
+//   - the copies go straight from registers to global memory: in the workspace eight consecutive columns of a matrix's rows lie
+//     together, so a warp's store is 512 consecutive bytes, and the solve kernel reads those bytes as a tensor-core operand without a
 //     swizzle.  (Staged in shared memory over the tile's own K and V for a TMA store, a stage could not be loaded again before the
 //     copies had been read from it);
 //   - what a thread contributes to ||H_0||_F^2 is left in shared memory, and a factor warp adds it up tiles later;
@@ -289,11 +289,15 @@ fwd_tc_summary_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 //   kOne      H or U: two blocks per item
 //   kQuarter  64 columns of H or of U: four blocks per item
 //   kD64      head dimension 64: H over U as one 128 x 64 master, [K V]^T K one product per k-step
+//   kD64H     the same for the solve alone: H only.  The product keeps its 128 rows, the upper 64 of them made of zeros that lie behind the
+//             stages (its A operand's second 64 columns are at a distance that the descriptor gives), and their master warps have nothing to do.
+//             Whole call, before (as kD64 with K in V's place, its copies of U included) and with it: 32 x 2048, r = 30: 137.2 -> 134.7 us,
+//             r = 0: 30.5 -> 28.0; 64 x 4096, r = 10: 196.4 -> 191.6; 256 x 1024: 191.7 -> 189.6
 // H and U are made from the same rounded keys, whichever block makes them.  (The whole weight on K, and V as it is, halves the scaling of a
 // block of U and brings U itself closer, 1.4e-3 against 2.0e-3, but the read U x meets an H of other keys: 4.9e-3 -> 5.7e-3 at 3 heads x
-// 1999 tokens, 30 iterations.)  The solve alone reads no U: its blocks are not launched.
+// 1999 tokens, 30 iterations.)  The solve alone keeps no U: no block of U is launched, kBoth skips it, kD64H has no room for it.
 // ------------------------------------------------------------------------------------------------------------
-enum { kBoth = 0, kOne = 1, kQuarter = 2, kD64 = 3 };
+enum { kBoth = 0, kOne = 1, kQuarter = 2, kD64 = 3, kD64H = 4 };
 // Warps: those that keep the masters; groups that scale rows and take the tiles in turn; helpers (row factors, products, loads).  With 32 KB
 // of K (and V) per tile six stages fit, and what counts is how many tiles are worked on at once: two groups of four warps.  With 64 KB
 // (kBoth, kOne's blocks of U) three fit, so that a stage has to be given back soon: all sixteen warps scale a tile together, a tile ahead,
@@ -301,9 +305,10 @@ enum { kBoth = 0, kOne = 1, kQuarter = 2, kD64 = 3 };
 // with two of four; 32 x 4096, kQuarter: 42 us in one group of all warps, 35.4 with two.)
 // Registers of a thread at launch (what its share of 65,536 allows) and after the split.
 template <int KIND> struct StateKind {
-    static constexpr bool kGroups = KIND == kQuarter || KIND == kD64;
+    static constexpr bool kIs64 = KIND == kD64 || KIND == kD64H, kGroups = KIND == kQuarter || kIs64;
     static constexpr int kColumns = KIND == kBoth ? 256 : KIND == kOne ? 128 : 64;      // of all masters: TMEM columns of a buffer of increments
     static constexpr int kMasters = KIND == kBoth ? 2 : 1, kMasterWarps = kGroups ? 8 : 16;
+    static constexpr int kKeepers = KIND == kD64H ? kMasterWarps / 2 : kMasterWarps;    // master warps that have rows to keep
     static constexpr int kCols = kColumns / kMasters / (kMasterWarps / 4);              // columns of a thread, of each master
     static constexpr int kGroupWarps = kGroups ? 4 : 16, kScaleGroups = kGroups ? 2 : 1;
     static constexpr int kFactorWarps = kGroups ? 4 : 2, kHelperWarps = kGroups ? 8 : 4;  // (whole warpgroups)
@@ -314,6 +319,8 @@ template <int KIND> struct StateKind {
                   "register split exceeds the launch allocation");
 };
 constexpr int kMaxStages = 6;
+constexpr uint32_t kZeros = kMaxStages * 16384;          // kD64H: 16 KB of zeros behind the stages of 16 KB
+static_assert(kZeros + 16384 + 1024 <= ST_SMEM, "shared memory of kD64H");
 constexpr int kSets = kMaxStages + 2;      // sets of row factors, decays and norm terms
 // A barrier of a kind for each of kRing consecutive tiles, whatever the number of stages: at least as many as stages, so that none is
 // a phase ahead of a waiter; and even, so that the phases of one all belong to the same of two scaling groups.  (With three, a group met
@@ -357,13 +364,18 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     if (t == 0) {
         s_abort = 0;
         for (int i = 0; i < TB_COUNT; ++i)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bars + 8 * i), "r"(i < TB_SC ? 2 : i < TB_D ? SK::kGroupWarps : i >= TB_AD && i < TB_DRAIN ? SK::kMasterWarps : 1));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bars + 8 * i), "r"(i < TB_SC ? 2 : i < TB_D ? SK::kGroupWarps : i >= TB_AD && i < TB_DRAIN ? SK::kKeepers : 1));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (t < 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "n"(2 * DW)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if constexpr (KIND == kD64H) {
+        for (int i = t; i < 1024; i += SK::kThreads) *reinterpret_cast<uint4 *>(smem + kZeros + 16 * i) = make_uint4(0u, 0u, 0u, 0u);
+        for (int i = t; i < kSets * MT; i += SK::kThreads) (&s_sq[0][0])[i] = 0.f;         // (the terms of the warps without rows stay 0)
+        fence_async_smem();
     }
     fence_before();
     __syncthreads();
@@ -377,8 +389,8 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     const bool both = KIND == kBoth && !a.solve_only;
     // a stage: K (the part of it that is needed), then V
     const uint32_t v_off = KIND == kQuarter || KIND == kD64 ? 16384u : 32768u;
-    const uint32_t stage_bytes = KIND == kD64 ? 32768u : (both || u_only) ? v_off + 32768u : 32768u;
-    const int ns = stage_bytes == 32768u ? 6 : stage_bytes == 49152u ? 4 : 3;
+    const uint32_t stage_bytes = KIND == kD64H ? 16384u : KIND == kD64 ? 32768u : (both || u_only) ? v_off + 32768u : 32768u;
+    const int ns = stage_bytes <= 32768u ? kMaxStages : stage_bytes == 49152u ? 4 : 3;
     const long long f_lo = P.lo(item);
     const int n_mine = (int)(P.lo(item + 1) - f_lo);
     float *const hh_out = u_only ? nullptr : half ? a.tile_hh2 : a.tile_hh;
@@ -417,7 +429,10 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         wait(TB_KV + bar_of(m), phase_of(m));
         unsigned char *const stage = smem + (size_t)at * stage_bytes;
         const uint2 *const f = s_f[m % kSets];
-        if constexpr (SK::kGroups) {
+        if constexpr (KIND == kD64H) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) scale_rows<4, GT, 1>(stage, f, ts + 4 * GT * i);
+        } else if constexpr (SK::kGroups) {
 #pragma unroll 2
             for (int i = 0; i < 4; ++i) {
                 if (KIND == kQuarter && u_only) scale_rows<2, GT, 3>(stage, f, ts + 2 * GT * i);
@@ -446,9 +461,9 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     const uint32_t dst = sb + (uint32_t)stage * stage_bytes, bar = bars + 8 * (TB_KV + bar_of(m));
                     const int x = p.h * a.d, y = p.n * NT;
                     mbar_expect_tx(bar, stage_bytes);
-                    if constexpr (KIND == kD64) {
+                    if constexpr (SK::kIs64) {
                         tma_load_box3(&tmK, dst, bar, x, y, p.b);
-                        tma_load_box3(&tmV, dst + v_off, bar, x, y, p.b);
+                        if (KIND == kD64) tma_load_box3(&tmV, dst + v_off, bar, x, y, p.b);
                     } else {
                         if (KIND == kQuarter && u_only) tma_load_box3(&tmK, dst, bar, x + 64 * half, y, p.b);
                         else tma_load_tile3(&tmK, dst, bar, x, x + 64, y, p.b);
@@ -560,7 +575,9 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     fence_after();
                     const uint32_t kb = base14 + (uint32_t)stage * (stage_bytes >> 4), vb = kb + (v_off >> 4);
                     const uint32_t tm_d = tmem + DW * (uint32_t)(m & 1);
-                    if (!u_only) mma8_mm<0>(tm_d, kb, kb + (16384u >> 4) * half, idesc);           // dH = K~^T K~ (kD64: [K~ V~]^T K~)
+                    // (kD64H: the second half of A's columns from the zeros instead of 16384 bytes on; the distance stands in bits 16 to 29)
+                    const uint32_t ka = KIND == kD64H ? kb + (((kZeros - 16384u - (uint32_t)stage * stage_bytes) >> 4) << 16) : kb;
+                    if (!u_only) mma8_mm<0>(tm_d, ka, kb + (16384u >> 4) * half, idesc);           // dH = K~^T K~ (kD64: [K~ V~]^T K~)
                     if (both || u_only) mma8_mm<0>(tm_d + (NM - 1) * 128, vb, kb, idesc);          // dU = V~^T K~
                     mma_commit(bars + 8 * (TB_D + bar_of(m)));
                 }
@@ -579,19 +596,20 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         // ================================ masters ================================
         const int q = (t >> 5) & 3, cq = t >> 7, c = 32 * q + l, col0 = 64 * half + CW * cq;     // row, first column
         const uint32_t tm_c = tmem + ((uint32_t)(32 * q) << 16) + CW * cq;
-        const int which0 = KIND == kD64 ? c >> 6 : u_only ? 1 : 0;           // matrix of the (first) master, and the row in it
-        const int row = KIND == kD64 ? c & 63 : c;
-        constexpr int DD = KIND == kD64 ? 64 : D;                            // head dimension of the caller's states
+        const int which0 = SK::kIs64 ? c >> 6 : u_only ? 1 : 0;              // matrix of the (first) master, and the row in it
+        const int row = SK::kIs64 ? c & 63 : c;
+        constexpr int DD = SK::kIs64 ? 64 : D;                               // head dimension of the caller's states
+        const int n_keep = KIND == kD64H && q >= 2 ? 0 : n_mine;             // tiles that this warp has rows of
         const size_t ext = (size_t)2 * DD * DD;                              // floats of a caller's state
         const size_t e_ext = (size_t)which0 * DD * DD + (size_t)row * DD + col0;
         const size_t st = state_floats(D, D), e_ws = (size_t)which0 * D * D + (size_t)row * D + col0;    // the workspace's states are 128 x 128
-        const bool sums = KIND == kD64 ? q < 2 : !u_only;                    // this warp's rows belong to H
-        // the copies: [matrix][column / 8][128 rows][8 columns] of 64 KB per tile; head dimension 64: [column / 8][H over U][8], 16 KB
-        unsigned char *copy = a.tile_hu + (size_t)f_lo * (KIND == kD64 ? kTileStateBytes64 : kTileStateBytes) +
-                              (KIND == kD64 ? 0 : which0 * 32768) + (col0 / 8) * 2048 + c * 16;
+        const bool sums = SK::kIs64 ? q < 2 : !u_only;                       // this warp's rows belong to H
+        // the copies: [H, U][column / 8][row][8 columns], 64 KB per tile, 16 KB at head dimension 64
+        unsigned char *copy = a.tile_hu + (size_t)f_lo * (SK::kIs64 ? kTileStateBytes64 : kTileStateBytes) +
+                              which0 * (2 * DD * DD) + (col0 / 8) * (16 * DD) + row * 16;
         // first item of the chain of summaries behind this block's start state
         int chain_j0 = item;
-        if ((KIND == kBoth || KIND == kD64) && P.cut_in(item)) {
+        if ((KIND == kBoth || SK::kIs64) && P.cut_in(item)) {
             const long long seq_start = (f_lo / P.N) * P.N;
             chain_j0 = item - 1;
             while (P.lo(chain_j0) > seq_start) --chain_j0;
@@ -607,7 +625,7 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         // summaries and start states are read, and copies written, after this point only
         asm volatile("griddepcontrol.wait;" ::: "memory");
 
-        for (int m = 0, at = 1; m < n_mine; ++m) {
+        for (int m = 0, at = 1; m < n_keep; ++m) {
             if constexpr (!SK::kGroups) {                        // the next tile's rows: its products run under this tile's passes
                 if (m + 1 < n_mine) scale(m + 1, at, t);
                 if (++at == ns) at = 0;
@@ -615,7 +633,7 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             if (m == 0 || n == 0) {
                 // start of a run: the caller's initial state of the sequence (or zero), carried through the summaries
                 // of the blocks that hold the earlier part of the sequence: state <- decay_j * state + delta_j
-                const bool chained = (KIND == kBoth || KIND == kD64) && n != 0;
+                const bool chained = (KIND == kBoth || SK::kIs64) && n != 0;
                 const bool scanned = chained && a.start_from_scan;
                 const float *const s0 = scanned ? a.ws.start + (size_t)item * st + e_ws : a.state_in ? a.state_in + (size_t)seq * ext + e_ext : nullptr;
                 const int j0 = chained && !scanned ? chain_j0 : 0, j1 = chained && !scanned ? item : 0;
@@ -624,11 +642,11 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 #pragma unroll
                     for (int i = 0; i < CW / 4; ++i) {
                         ulonglong2 v = make_ulonglong2(0ull, 0ull);
-                        if (s0) v = *reinterpret_cast<const ulonglong2 *>(s0 + w * D * D + 4 * i);
+                        if (s0 && (w == 0 || both)) v = *reinterpret_cast<const ulonglong2 *>(s0 + w * D * D + 4 * i);      // (the solve alone: nobody has written U's)
                         mst[w][2 * i] = v.x;
                         mst[w][2 * i + 1] = v.y;
                     }
-                    for (int j = j0; j < j1; ++j) {
+                    for (int j = j0; j < j1 && (w == 0 || both); ++j) {
                         // summaries come from the kernel this one may overlap with as its programmatic dependent: ordinary loads
                         const float dj = *reinterpret_cast<const volatile float *>(a.ws.decay + j);
                         const uint64_t dj2 = f2_pack(dj, dj);
@@ -669,7 +687,7 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                             pk[u] = pack_bf16(v0, v1);
                             if (w == 0) sq = f2_fma(v, v, sq);
                         }
-                        *reinterpret_cast<uint4 *>(copy + w * 32768 + 2048 * (c0 / 8 + i)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                        *reinterpret_cast<uint4 *>(copy + w * 32768 + 16 * DD * (c0 / 8 + i)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
                     }
                     if (w == 0 && c0 + PW == CW) {
                         float a0, a1;
@@ -687,7 +705,7 @@ fwd_tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 __syncwarp();
                 if (l == 0) mbar_arrive(bars + 8 * (TB_AD + (m & 1)));
             }
-            copy += KIND == kD64 ? kTileStateBytes64 : kTileStateBytes;
+            copy += SK::kIs64 ? kTileStateBytes64 : kTileStateBytes;
             // ---- final state of the sequence, in the caller's layout
             if (++n == P.N) {
                 if (a.state_out) {
@@ -812,7 +830,7 @@ cudaError_t launch_fwd_tc(const FwdArgs &a_in, cudaStream_t stream) {
     const int masters = a.solve_only ? 1 : 2;
     int kind = kBoth, per_item = 1;
     if (a.d == 64) {
-        kind = kD64;
+        kind = a.solve_only ? kD64H : kD64;
     } else if (!any_cut && masters * a.plan.G <= a.sms) {
         kind = kOne;
         per_item = masters;
@@ -850,7 +868,7 @@ cudaError_t launch_fwd_tc(const FwdArgs &a_in, cudaStream_t stream) {
         a.after_summary = 1;
     }
     cfg.gridDim = dim3((unsigned)(a.plan.G * per_item));
-    err = kind == kD64 ? launch_state<kD64>(cfg, tmK, tmV, a) : kind == kQuarter ? launch_state<kQuarter>(cfg, tmK, tmV, a)
+    err = kind == kD64H ? launch_state<kD64H>(cfg, tmK, tmV, a) : kind == kD64 ? launch_state<kD64>(cfg, tmK, tmV, a) : kind == kQuarter ? launch_state<kQuarter>(cfg, tmK, tmV, a)
           : kind == kOne ? launch_state<kOne>(cfg, tmK, tmV, a) : launch_state<kBoth>(cfg, tmK, tmV, a);
     if (err != cudaSuccess) return err;
     return launch_fwd_solve(a, stream);
