@@ -218,6 +218,26 @@ def make_fwd_inputs_device(cfg, device, seed):
     return dict(q=q, k=k, v=v, gate=gate, lam=lam)
 
 
+def kernel_launches(gka, call):
+    """Kernels that one call launches: the call is captured into a graph, which is not run, and its kernel nodes are counted."""
+    import ctypes
+
+    import torch
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    lib = gka.load_library()          # (its symbols include those of the CUDA runtime that it is linked to)
+    raw, n = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t(0)
+    assert lib.cudaGraphGetNodes(raw, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert lib.cudaGraphGetNodes(raw, nodes, ctypes.byref(n)) == 0
+    kernels, kind = 0, ctypes.c_int(-1)
+    for node in nodes:
+        assert lib.cudaGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        kernels += kind.value == 0    # cudaGraphNodeTypeKernel
+    return kernels
+
+
 def time_forward(gka, dev, cfg, n_iter, flags, steps, warmup, peaks, stream, new_event, flush, world, device):
     """K timed calls of the chunk-wise forward (L2 flushed between calls, CUDA events on the launch stream, every
     call exactly as a user's), then a separate pass of bracketed launches that times the dominant kernel alone."""
@@ -260,6 +280,7 @@ def time_forward(gka, dev, cfg, n_iter, flags, steps, warmup, peaks, stream, new
     torch.cuda.synchronize()
     assert int(status.item()) == 0, "a device-side bounded wait timed out"
     kernel_ms = statistics.mean(a.elapsed_time(b) for a, b in kev)
+    launches = kernel_launches(gka, fwd)
     n_chunks = cfg.B * cfg.heads * ((cfg.T + cfg.chunk - 1) // cfg.chunk)
     n_tiles = cfg.B * cfg.heads * ((cfg.T + 127) // 128)
     flops_solve = fwd_flops(n_chunks, n_iter, cfg.chunk, cfg.d, part="solve")
@@ -275,7 +296,7 @@ def time_forward(gka, dev, cfg, n_iter, flags, steps, warmup, peaks, stream, new
                 "whole_call_frac": flops_all / (ms_per_step * 1e-3) / 1e12 / peaks["bf16_tflops"],
                 "frac_of_nominal_2250": achieved_tf / 2250.0}
     return dict(ms_per_step=ms_per_step, value=tokens_per_step / (ms_per_step * 1e-3), roofline=roofline, wall=wall,
-                fwd=fwd, ws=ws, status=status)
+                launches=launches, fwd=fwd, ws=ws, status=status)
 
 
 def run_ours(args):
@@ -371,9 +392,6 @@ def run_ours(args):
     e2e_value = tokens_per_step / (e2e_ms * 1e-3)
 
     work_items = gka.gka_fwd_num_work_items(cfg.B, cfg.T, cfg.heads, cfg.d)
-    any_cut = any(gka.gka_fwd_work_range(cfg.B, cfg.T, cfg.heads, cfg.d, work_items, i)[3]
-                  for i in range(work_items))
-    launches_per_step = 3 if any_cut else 2     # (segment summaries,) state kernel, solve kernel
 
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K, "warmup": W,
@@ -385,7 +403,7 @@ def run_ours(args):
                    "batch_per_gpu": cfg.B},
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "ms_per_step": e2e_ms},
-        "gpu_launches": launches_per_step * K,
+        "gpu_launches": head["launches"] * K,
         "roofline": roofline,
         "clocks": clocks,
         "wall_s_timed_region": wall,
@@ -404,7 +422,7 @@ def run_ours(args):
                            "steps": K2, "config": {"workload": "cfg1 shapes at the paper's setting", "B": cfg.B,
                                                    "heads": cfg.heads, "T": cfg.T, "d": cfg.d, "n_iter": 30,
                                                    "lam": "adaptive, a = 0.02", "io_dtype": cfg.io_dtype},
-                           "roofline": r30["roofline"], "gpu_launches": launches_per_step * K2}
+                           "roofline": r30["roofline"], "gpu_launches": r30["launches"] * K2}
         del r30, dev30
         # ---- head dimension 64 on configuration 1's shapes (the tensor path's four-k-step instantiation), inputs drawn
         # on the device; no ncu capture of this instantiation exists, so its traffic is not reported
@@ -419,7 +437,7 @@ def run_ours(args):
                                "steps": K4, "config": {"workload": "cfg1 shapes at head dimension 64", "B": cfg64.B,
                                                        "heads": cfg64.heads, "T": cfg64.T, "d": 64, "n_iter": cfg64.n_iter,
                                                        "io_dtype": cfg64.io_dtype, "inputs": "drawn on the device"},
-                               "roofline": r64["roofline"], "gpu_launches": launches_per_step * K4}
+                               "roofline": r64["roofline"], "gpu_launches": r64["launches"] * K4}
             del r64, dev64
             torch.cuda.empty_cache()
         # ---- long context (configuration 3), inputs drawn on the device
@@ -432,7 +450,7 @@ def run_ours(args):
                                 "steps": K3, "config": {"workload": cfg3.name, "B": cfg3.B, "heads": cfg3.heads,
                                                         "T": cfg3.T, "d": cfg3.d, "n_iter": cfg3.n_iter,
                                                         "io_dtype": cfg3.io_dtype, "inputs": "drawn on the device"},
-                                "roofline": r3["roofline"], "gpu_launches": 3 * K3}
+                                "roofline": r3["roofline"], "gpu_launches": r3["launches"] * K3}
             del r3, dev3
             torch.cuda.empty_cache()
 
