@@ -202,12 +202,12 @@ const char *gka_status_string(int status);
 const char *gka_last_error_detail(void);
 
 /*
- * A work decomposition of the flat list of tiles of the tensor-core path, for callers that divide work: number of
- * work items (contiguous ranges of that list) for this descriptor on the current device, or a negative
+ * Work decomposition of the state pass of gka_fwd_chunked on the tensor-core path, for callers that report launch counts or divide
+ * work: number of work items (contiguous ranges of the flat list of tiles) for this descriptor on the current device, or a negative
  * gka_status.  Normally one per SM (fewer for small problems).  It is pairs / k for a small divisor k of the number of
- * (sequence, head) pairs (k = 1 with fewer pairs than SMs) where sequences are short or many: no range then starts or ends inside a
- * sequence.  The state pass of a call works on such ranges too, but takes whole sequences in more cases than this function
- * (wherever that is the quicker way); where it cuts none, no summary or scan kernel runs.
+ * (sequence, head) pairs (k = 1 with fewer pairs than SMs) wherever carrying whole sequences is the quicker way: no range then starts or
+ * ends inside a sequence and no summary or scan kernel runs.  (gka_solve_chunked, which keeps half of the state, weighs the two
+ * ways with times of its own and may take the other one.)
  * fp32 arithmetic splits sequences by rules of its own, which these two functions do not describe: for such a descriptor they
  * answer with an even split of the list of 64-token chunks into one range per SM (fewer for small problems).
  */

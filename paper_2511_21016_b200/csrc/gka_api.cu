@@ -181,20 +181,9 @@ int gka_fwd_num_work_items(const gka_desc *desc, int chunk) {
     if (s != GKA_OK) return -(int)s;
     const int sms = sm_count();
     if (sms <= 0) return -(int)GKA_ERR_CUDA;
+    if (wants_tensor_path(desc)) return state_items(desc, sms, false);
     const int cap = work_items_cap(desc);
-    if (wants_tensor_path(desc)) {
-        // The division of work that the function has always answered with (the header states it): whole sequences where they are short
-        // or many.  What a call's own state pass takes is state_items.
-        const long long pairs = (long long)desc->B * desc->heads, n = tiles_of(desc->T);
-        for (long long k = (pairs + sms - 1) / sms; k <= pairs && k <= 64; ++k) {
-            if (pairs % k != 0 || pairs / k > cap) continue;
-            const long long items = pairs / k;
-            const double per_tile = 4 * items <= sms && desc->d_k == 128 ? 1.7 : 2 * items <= sms ? 2.15 : 2.94;
-            if ((double)n * ((double)k * per_tile - 5.12 * (double)pairs / sms) < 36.5) return (int)items;
-            break;
-        }
-    }
-    return sms < cap ? sms : cap;      // (fp32 arithmetic: of an even split of the chunks, which its kernels do not use)
+    return sms < cap ? sms : cap;      // of an even split of the chunks, which the fp32 kernels do not use
 }
 
 gka_status gka_fwd_work_range(const gka_desc *desc, int chunk, int num_items, int item,

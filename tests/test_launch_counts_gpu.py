@@ -31,3 +31,17 @@ def test_kernels_of_a_decode_step():
     state = torch.zeros(2, 4, 2 * 128 * 128, device=DEV)
     out = gka.gka_decode_step(state, *x, 1)
     assert kernel_launches(gka, lambda: gka.gka_decode_step(state, *x, 1, out=out)) == 1
+
+
+@pytest.mark.parametrize("d", [128, 64])
+@pytest.mark.parametrize("heads,tiles", [(1, 10), (1, 42), (1, 46), (10, 30), (10, 58), (10, 61), (16, 64), (40, 139), (40, 142)])
+def test_work_items_are_those_of_a_call(heads, tiles, d):
+    """Where the library answers with ranges that cut sequences a call has summaries, and where it answers with whole ones none."""
+    T = 128 * tiles
+    x = inputs((1, T, heads), d)
+    ws = gka.alloc_workspace(1, T, heads, d, torch.device(DEV))
+    out, st = gka.gka_fwd_chunked(*x, 0, workspace=ws)
+    G = gka.gka_fwd_num_work_items(1, T, heads, d)
+    cut = any(gka.gka_fwd_work_range(1, T, heads, d, G, i)[3] for i in range(G))
+    kernels = kernel_launches(gka, lambda: gka.gka_fwd_chunked(*x, 0, out=out, state_out=st, workspace=ws))
+    assert (kernels > 2) == cut
