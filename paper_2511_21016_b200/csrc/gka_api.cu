@@ -152,8 +152,8 @@ size_t gka_fwd_workspace_bytes(const gka_desc *desc, int chunk) {
 // sequences the summary kernel reads all keys and values once more.  Items of whole sequences (pairs / k items of k sequences each, k
 // the smallest divisor of the number of (sequence, head) pairs that leaves at most one item per SM) need no summaries, but may
 // leave SMs idle in the state kernel and make its run of tiles longer.  With n tiles per sequence whole sequences cost
-// per_tile k n us, ranges cut pairs / SMs n + fixed (the extra launches).  Fitted to both sides of 28 shapes at r = 0 (us per call, whole
-// sequences / ranges):
+// per_tile k n us, ranges cut pairs / SMs n + fixed (the extra launches).  Fitted to both sides of these shapes at r = 0 (us per call,
+// whole sequences / ranges):
 //   d = 128 (per_tile by how many blocks share an item): 1 pair, 32 tiles 48.3 / 53.9; 8 pairs, 32 tiles 52.0 / 76.4, 64 tiles 98.2 / 98.8;
 //     16 pairs, 64 tiles 122 / 135, 128 tiles 228 / 213; 32 pairs, 64 tiles 172 / 210, 1024 tiles 2824 / 2809; 64 pairs, 64
 //     tiles 339 / 398; 96 pairs, 64 tiles 482 / 538; 256 pairs (two per item), 32 tiles 579 / 673
@@ -161,6 +161,12 @@ size_t gka_fwd_workspace_bytes(const gka_desc *desc, int chunk) {
 //     tiles 119 / 129, 128 tiles 247 / 250; 64 pairs, 64 tiles 179 / 217; 256 pairs, 64 tiles 700 / 816
 //   the solve alone, d = 128: 8 pairs, 32 tiles 41.9 / 50.3; 16 pairs, 64 tiles 92.7 / 87.8; 32 pairs, 256 tiles 575 / 562; 64 pairs, 64
 //     tiles 230 / 282
+//   more than two sequences per item, where the launches of the ranges hide behind the kernels before and no scan runs: d = 128, 155 pairs
+//     (five per item) 16 tiles 226 / 236, 32 tiles 427 / 427, 64 tiles 846 / 832, 110 tiles 1514 / 1450; 161 pairs (seven), 16 tiles
+//     264 / 241; 312 pairs (three), 16 tiles 415 / 432; 352 pairs (four), 16 tiles 484 / 468 (the wrong side, as 32 tiles 929 / 911);
+//     d = 64, 155 pairs, 8 tiles 90 / 80, 16 tiles 158 / 131; 312 pairs, 16 tiles 226 / 254; 352 pairs 266 / 287; the solve alone,
+//     d = 128, 155 pairs, 8 tiles 98 / 93, 16 tiles 194 / 175; 312 pairs, 16 tiles 320 / 335; d = 64, 155 pairs, 8 tiles 60 / 61, 16 tiles
+//     128 / 112.  (With the same fixed as for fewer sequences 161 pairs of 8 tiles at d = 64 took the side that costs a third more.)
 static int state_items(const gka_desc *desc, int sms, bool solve_only) {
     const int cap = work_items_cap(desc);
     const long long pairs = (long long)desc->B * desc->heads, n = tiles_of(desc->T);
@@ -169,7 +175,7 @@ static int state_items(const gka_desc *desc, int sms, bool solve_only) {
         const long long items = pairs / k;
         const bool light = desc->d_k == 64 || solve_only;            // half the state or less
         const double per_tile = light ? 0.83 : 4 * items <= sms ? 0.95 : 2 * items <= sms ? 1.42 : 2.2;
-        const double cut = light ? 3.05 : 4.2, fixed = light ? 28.0 : 40.0;
+        const double cut = light ? 3.05 : 4.2, fixed = k > 2 ? (light ? 4.0 : 18.0) : light ? 28.0 : 40.0;
         if ((double)n * ((double)k * per_tile - cut * (double)pairs / sms) < fixed) return (int)items;
         break;
     }

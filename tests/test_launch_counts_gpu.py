@@ -34,7 +34,8 @@ def test_kernels_of_a_decode_step():
 
 
 @pytest.mark.parametrize("d", [128, 64])
-@pytest.mark.parametrize("heads,tiles", [(1, 10), (1, 42), (1, 46), (10, 30), (10, 58), (10, 61), (16, 64), (40, 139), (40, 142)])
+@pytest.mark.parametrize("heads,tiles", [(1, 10), (1, 42), (1, 46), (10, 30), (10, 58), (10, 61), (16, 64), (40, 139), (40, 142),
+                                         (155, 16), (155, 24)])
 def test_work_items_are_those_of_a_call(heads, tiles, d):
     """Where the library answers with ranges that cut sequences a call has summaries, and where it answers with whole ones none."""
     T = 128 * tiles

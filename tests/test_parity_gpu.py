@@ -304,6 +304,8 @@ def test_work_items_follow_the_decomposition_rule():
         assert n(16, 2048, 16, 128) == 128                 # 256 pairs: 128 items of two sequences
         assert n(2, 3840, 5, 128) == 10                    # 10 pairs of 30 tiles: whole, four blocks each
         assert n(2, 128 * 61, 5, 128) == 148               # 10 pairs of 61 tiles: cut
+        assert n(1, 2048, 155, 128) == 31 and n(1, 2048, 155, 64) == 148     # 155 pairs, five whole sequences per item or cut
+        assert n(13, 2048, 24, 128) == 104                 # 312 pairs: three whole sequences per item
     assert n(4, 4096, 16, 128, io_dtype=gka.GKA_F32) == min(sms, 4 * 16 * 64)
     for B, T, heads in ((4, 4096, 16), (16, 2048, 16), (2, 640, 5)):
         G = n(B, T, heads, 128)
