@@ -103,12 +103,12 @@ def test_fwd_f32_items_cut_sequences():
     check_fwd(cfg)
 
 
-@pytest.mark.parametrize("io,d", [("f32", 64), ("f32", 128), ("bf16", 128)])
-def test_fwd_slow_fading_state_crosses_many_items(io, d):
+@pytest.mark.parametrize("io,d,T", [("f32", 64, 64 * 70), ("f32", 128, 64 * 70), ("bf16", 128, 64 * 70), ("bf16", 128, 128 * 56)])
+def test_fwd_slow_fading_state_crosses_many_items(io, d, T):
     """Gates close to 1 (sigmoid(N(6,1))): the state of a sequence start is still alive many work items (fp32: segments)
     later, so a wrong start state of any of them shows (fast-fading gates would hide it).  Several sequences; on the tensor-core
-    path their boundaries fall inside items."""
-    cfg = synth.GkaConfig("slow", B=2, heads=3, T=64 * 70, d=d, chunk=64, n_iter=2, io_dtype=io, seed=21,
+    path, of 35 tiles each they are carried whole, of 56 their boundaries fall inside items."""
+    cfg = synth.GkaConfig("slow", B=2, heads=3, T=T, d=d, chunk=64, n_iter=2, io_dtype=io, seed=21,
                           gate_mean=6.0)
     check_fwd(cfg)
 
@@ -216,10 +216,11 @@ def test_fwd_adaptive_lambda_mode_bf16(T, n_iter):
     assert rel(out, ref["out"]) <= 5e-3
 
 
-def test_fwd_bf16_native_paper_iteration_count():
-    """30 iterations (the paper's setting in every experiment) on configuration-1-like inputs, sequences cut by
+@pytest.mark.parametrize("T", [64 * 70, 128 * 56])
+def test_fwd_bf16_native_paper_iteration_count(T):
+    """30 iterations (the paper's setting in every experiment) on configuration-1-like inputs, sequences carried whole and cut by
     work items: tensor-core path against the oracle."""
-    cfg = synth.shrink(synth.CONFIGS[1], B=2, heads=3, T=64 * 70, n_iter=30)
+    cfg = synth.shrink(synth.CONFIGS[1], B=2, heads=3, T=T, n_iter=30)
     e = check_fwd(cfg)
     print("bf16 native r=30 rel L2 (out, state, fro, worst tile):", e)
 
@@ -242,19 +243,21 @@ def test_fwd_degenerate_inputs():
     assert np.all(np.isfinite(out)) and rel(out, ref["out"]) < TOL_F32
 
 
-def test_fwd_is_deterministic():
-    cfg = synth.shrink(synth.CONFIGS[1], B=1, heads=3, T=64 * 60, n_iter=3)
+@pytest.mark.parametrize("T", [64 * 60, 128 * 56])      # whole sequences, and cut ones
+def test_fwd_is_deterministic(T):
+    cfg = synth.shrink(synth.CONFIGS[1], B=1, heads=3, T=T, n_iter=3)
     inp = synth.make_inputs(cfg)
     a = run_fwd(inp, 3, True)
     b = run_fwd(inp, 3, True)
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
 
 
-def test_fwd_back_to_back_calls_share_a_workspace():
+@pytest.mark.parametrize("T", [64 * 60, 128 * 61])      # whole sequences, and cut ones
+def test_fwd_back_to_back_calls_share_a_workspace(T):
     """Two different problems enqueued back to back on one stream with the same workspace: the second result must not
     see the first call's segment summaries (the main kernel starts under the summary kernel's tail and waits for the
     summaries only where it reads them)."""
-    cfg = synth.shrink(synth.CONFIGS[1], B=2, heads=5, T=64 * 60, n_iter=3)
+    cfg = synth.shrink(synth.CONFIGS[1], B=2, heads=5, T=T, n_iter=3)
     a = synth.make_inputs(cfg)
     b = synth.make_inputs(synth.shrink(cfg, seed=77))
     ws = gka.alloc_workspace(cfg.B, cfg.T, cfg.heads, cfg.d, DEV)
@@ -270,7 +273,7 @@ def test_fwd_back_to_back_calls_share_a_workspace():
 
 
 @pytest.mark.parametrize("B,heads,T,d", [(2, 5, 640, 128), (2, 5, 640, 64), (1, 40, 2000, 128), (8, 16, 1000, 128),
-                                         (2, 5, 3840, 128), (4, 40, 200, 128)])
+                                         (2, 5, 3840, 128), (4, 40, 200, 128), (2, 5, 128 * 61, 128), (2, 5, 128 * 56, 64)])
 def test_fwd_bf16_native_repeated_calls_are_bit_identical(B, heads, T, d):
     """The same problem several times over, one workspace: outputs and final states must agree bit for bit in every
     decomposition of the state pass (whole sequences with four blocks, with one block per master and with one block each,
@@ -414,10 +417,11 @@ def test_solve_f32_matches_the_oracle_iterates(d, n_iter):
     assert rel(x, ref) <= TOL_F32
 
 
-@pytest.mark.parametrize("n_iter", [0, 1, 10])
-def test_solve_bf16_native_matches_the_oracle_iterates(n_iter):
-    """Tensor-core path; several work items cut the sequences so the start states come through the summaries."""
-    cfg = synth.shrink(synth.CONFIGS[1], B=2, heads=3, T=64 * 70)
+@pytest.mark.parametrize("n_iter,T", [(0, 64 * 70), (1, 64 * 70), (10, 64 * 70), (0, 128 * 48), (10, 128 * 48)])
+def test_solve_bf16_native_matches_the_oracle_iterates(n_iter, T):
+    """Tensor-core path; sequences carried whole (35 tiles), and cut by work items so that the start states come through the
+    summaries (48 tiles)."""
+    cfg = synth.shrink(synth.CONFIGS[1], B=2, heads=3, T=T)
     inp = synth.make_inputs(cfg)
     rng = np.random.default_rng(6)
     rhs = synth.round_bf16(rng.standard_normal(inp["q"].shape).astype(np.float32))
@@ -556,6 +560,7 @@ def test_decode_alpha_connection():
 @pytest.mark.parametrize("bf16,d,B,heads,T", [
     (True, 128, 2, 3, 1), (True, 128, 2, 3, 63), (True, 128, 1, 2, 65), (True, 128, 2, 2, 127), (True, 128, 2, 3, 129),
     (True, 128, 3, 2, 64 * 5 + 17), (True, 128, 1, 3, 64 * 70 + 33), (True, 128, 1, 1, 64 * 301 + 1),
+    (True, 128, 1, 3, 128 * 56 + 33),
     (False, 64, 2, 3, 1), (False, 64, 2, 2, 50), (False, 128, 2, 3, 100), (False, 128, 1, 5, 64 * 5 + 17),
     (True, 64, 2, 2, 64 * 3 + 5)])
 def test_fwd_ragged_sequence_length(bf16, d, B, heads, T):

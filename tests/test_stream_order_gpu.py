@@ -21,7 +21,9 @@ def draw(shape, d, dtype, gen):
     (32, torch.bfloat16, 0, 8, 8, 500), (64, torch.float32, 0, 1, 2, 256), (64, torch.float32, 0, 30, 16, 7),
     (128, torch.float32, 0, 1, 3, 1000), (128, torch.bfloat16, gka.GKA_PREC_HIGH, 2, 4, 300),
     (128, torch.bfloat16, 0, 1, 2, 500),        # whole sequences as work items
-    (128, torch.bfloat16, 0, 2, 5, 3840),       # ranges that cut sequences
+    (128, torch.bfloat16, 0, 2, 5, 3840),       # whole sequences, four blocks each
+    (128, torch.bfloat16, 0, 2, 5, 128 * 61),   # ranges that cut sequences
+    (128, torch.bfloat16, 0, 1, 40, 128 * 142), # ... so few of a sequence that the state kernel folds their summaries
     (128, torch.bfloat16, 0, 1, 1, 16384),      # ... over so many items that the scan kernel runs
     (64, torch.bfloat16, 0, 3, 4, 1000)])
 def test_unsynchronised_chain_matches_one_call_at_a_time(d, dtype, precision, B, heads, T):
