@@ -419,6 +419,9 @@ __device__ __forceinline__ void p_epilogue_t(const Ctx &cx, const GateScalars *g
 // 64 x 2048 tokens, d = 64: 117.8 -> 116.3 us, nothing else changes; an iteration's too: with beta, alpha or for the solve alone 197.7
 // -> 194.0 (24 x 1999, 30 iterations) and 185.5 -> 183.0 (32 x 2048), but in the plain kernel at 128 channels a call there costs spills
 // (349 -> 350, 131072 tokens 5700 -> 5740), so there it stays inlined.
+// What such tiles cost (gates of mean 1 or less before the sigmoid instead of 2): 64 x 4096 tokens, 10 iterations 330 -> 464 us per call; 24 x
+// 1999, 30 iterations 196 -> 272; 32 x 2048, the solve alone 184 -> 287; 64 x 2048, d = 64 117 -> 171.  All inlined they take 460, 272,
+// 294 and 170: the functions cost them up to 1 %, and save the solve alone 2.
 template <bool KEYF>
 __device__ __noinline__ void p_epilogue_exact(uint32_t tm_s, int q, int l, const GateScalars *gs, float ac_c, const DiagMasks *dm) {
     Ctx cx;

@@ -92,7 +92,11 @@ __device__ __forceinline__ uint2 split_factor(float f) {
     return make_uint2(hi | hi >> 16, pack_bf16(lo, lo));
 }
 // Eight bf16 elements times a split factor: v hi + (v lo), the fused multiply-add rounded once, is the product with f to within 2^-17
-// before its rounding to bf16, in two instructions per pair of elements (unpacking to fp32, multiplying and packing takes six).
+// before its rounding to bf16, in two instructions per pair of elements (unpacking to fp32, multiplying and packing takes six).  The
+// elements are rounded to 2^-9 either way, and about one in a hundred rounds to the other side.  Errors of a call against fp64 over 72
+// drawn cases, with fp32 factors and with these: outputs 4.006e-3 and 4.005e-3 (10 to 30 iterations), 3.541e-3 and 3.535e-3 (every option),
+// 4.452e-3 and 4.441e-3 (slow gates), 3.745e-3 and 3.749e-3 (64 channels); the solve alone 1.852e-3 and 1.851e-3; H 1.905e-3 both,
+// U 1.953e-3 and 1.954e-3.
 __device__ __forceinline__ uint4 times_factor(uint4 v, uint2 f) {
     const __nv_bfloat162 hi = *reinterpret_cast<const __nv_bfloat162 *>(&f.x), lo = *reinterpret_cast<const __nv_bfloat162 *>(&f.y);
     __nv_bfloat162 *const p = reinterpret_cast<__nv_bfloat162 *>(&v);
