@@ -35,8 +35,8 @@
  *   - Supported: d_k == d_v in {16, 32, 64, 128}; chunk == 64; any T >= 1 (a sequence is ceil(T / chunk) chunks, the
  *     last one holds the remaining T mod chunk tokens); n_iter >= 0.
  *   - bf16 I/O with GKA_PREC_NATIVE and T >= 16 runs on the tensor cores (tiles of 128 tokens x 128 channels; head
- *     dimension 64 is zero-extended on chip and skips the zero channels in the contractions over the channels: 0.78 of the
- *     time of 128 at B = 4, 16 heads, T = 4096 and 10 iterations, 0.73 at 30); f32 I/O, GKA_PREC_HIGH, T < 16 and head dimensions 16 and
+ *     dimension 64 is zero-extended on chip and skips the zero channels in the contractions over the channels: 0.65 to 0.71 of
+ *     the time of 128 at B = 4, 16 heads, T = 4096 and 10 iterations, 0.63 at 30); f32 I/O, GKA_PREC_HIGH, T < 16 and head dimensions 16 and
  *     32 run in fp32 arithmetic on the CUDA cores (16 and 32: an explicit H_t per token in the registers of a few lanes; the
  *     decode calls handle them with one warp per (sequence, head) pair).
  */
